@@ -38,6 +38,463 @@ f32_project_kernel(const float* __restrict__ X, const float* W0, const float* W1
     }
 }
 
+// ---------------------------------------------------------------- tiled kernels
+// Two fp32 multiply-accumulates in one instruction, each rounded as fmaf rounds it.
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float v) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+// Asynchronous copies global -> shared (4 and 16 bytes) and the waits for them.
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Projection, tiled: BM x BN outputs per CTA, TM x TN per thread (rows strided by BM / TM, columns in groups of four),
+// operands staged GP_STAGES deep with asynchronous copies.  Every output is the same chain of fmaf over k = 0, 1, ...
+// as in f32_project_kernel, so the results are bitwise the same.  Needs D and N to be multiples of 4.
+constexpr int GP_BK = 32, GP_LDA = GP_BK + 4, GP_STAGES = 3;
+template <int BM, int BN, int TM, int TN>
+struct GPCfg {
+    static constexpr int TX = BN / TN, TY = BM / TM, THREADS = TX * TY;
+    static constexpr int A_FLOATS = BM * GP_LDA, B_FLOATS = GP_BK * BN, STAGE = A_FLOATS + B_FLOATS;
+    static constexpr int SMEM = GP_STAGES * STAGE * (int)sizeof(float);
+};
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__(GPCfg<BM, BN, TM, TN>::THREADS, 2)
+f32_project_tiled_kernel(const float* __restrict__ X, const float* W0, const float* W1, const float* W2, float* O0,
+                         float* O1, float* O2, int rows, int D, int N, const float* __restrict__ R, DeviceCounters* dc) {
+    using C = GPCfg<BM, BN, TM, TN>;
+    static_assert(C::TX % 8 == 0 && C::TY % 4 == 0 && TN % 4 == 0, "a warp is 4 x 8 threads");
+    extern __shared__ float4 gp_smem4[];
+    float* sm = reinterpret_cast<float*>(gp_smem4);
+    const float* W = blockIdx.z == 0 ? W0 : (blockIdx.z == 1 ? W1 : W2);
+    float* O = blockIdx.z == 0 ? O0 : (blockIdx.z == 1 ? O1 : O2);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tx = (warp % (C::TX / 8)) * 8 + (lane & 7), ty = (warp / (C::TX / 8)) * 4 + (lane >> 3);
+    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int nk = (D + GP_BK - 1) / GP_BK;
+
+    auto load = [&](int kt) {       // k-step kt: rows beyond the matrix are clamped, columns of k beyond D skipped
+        float* a = sm + (kt % GP_STAGES) * C::STAGE;
+        float* b = a + C::A_FLOATS;
+        const int k0 = kt * GP_BK;
+        for (int t = tid; t < BM * (GP_BK / 4); t += C::THREADS) {
+            const int r = t / (GP_BK / 4), c = (t % (GP_BK / 4)) * 4;
+            if (k0 + c < D) cp_async16(a + r * GP_LDA + c, X + (size_t)min(m0 + r, rows - 1) * D + k0 + c);
+        }
+        for (int t = tid; t < GP_BK * (BN / 4); t += C::THREADS) {
+            const int k = t / (BN / 4), c = (t % (BN / 4)) * 4;
+            if (k0 + k < D) cp_async16(b + k * BN + c, W + (size_t)(k0 + k) * N + min(n0 + c, N - 4));
+        }
+    };
+    unsigned long long acc[TM][TN / 2] = {};
+#pragma unroll
+    for (int s = 0; s < GP_STAGES - 1; ++s) {
+        if (s < nk) load(s);
+        cp_async_commit();
+    }
+    for (int kt = 0; kt < nk; ++kt) {
+        cp_async_wait_group<GP_STAGES - 2>();
+        __syncthreads();            // step kt has landed, and step kt - 1's buffer is free
+        if (kt + GP_STAGES - 1 < nk) load(kt + GP_STAGES - 1);
+        cp_async_commit();
+        const float* a = sm + (kt % GP_STAGES) * C::STAGE + ty * GP_LDA;
+        const float* b = sm + (kt % GP_STAGES) * C::STAGE + C::A_FLOATS + 4 * tx;
+        const int kn = min(GP_BK, D - kt * GP_BK);
+#pragma unroll 2
+        for (int k = 0; k < kn; k += 4) {
+            float4 av[TM];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a + i * C::TY * GP_LDA + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                ulonglong2 bv[TN / 4];
+#pragma unroll
+                for (int g = 0; g < TN / 4; ++g) bv[g] = *reinterpret_cast<const ulonglong2*>(b + (k + kk) * BN + g * 4 * C::TX);
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const unsigned long long x = dup2(kk == 0 ? av[i].x : kk == 1 ? av[i].y : kk == 2 ? av[i].z : av[i].w);
+#pragma unroll
+                    for (int g = 0; g < TN / 4; ++g) { fma2(acc[i][2 * g], x, bv[g].x); fma2(acc[i][2 * g + 1], x, bv[g].y); }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int r = m0 + ty + i * C::TY;
+        if (r >= rows) continue;
+#pragma unroll
+        for (int g = 0; g < TN / 4; ++g) {
+            const int c = n0 + 4 * tx + g * 4 * C::TX;
+            if (c >= N) continue;
+            const float2 lo = unpack2(acc[i][2 * g]), hi = unpack2(acc[i][2 * g + 1]);
+            float4 o = make_float4(lo.x, lo.y, hi.x, hi.y);
+            if (R) {
+                const float4 x = *reinterpret_cast<const float4*>(R + (size_t)r * N + c);
+                o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
+            }
+            *reinterpret_cast<float4*>(O + (size_t)r * N + c) = o;
+        }
+    }
+    if (tid == 0)
+        atomicAdd(&dc->proj_macs, (unsigned long long)min(BM, rows - m0) * min(BN, N - n0) * D);
+}
+
+// Attention, tiled: a CTA of four warps works on BR = 64 / KS query rows of one (batch, head) and walks the keys in
+// blocks of 64 staged in shared memory.  A warp owns 16 rows and 64 / KS keys of every block: two half-warps of 16
+// lanes, lane (ty, tx) holding rows ty + 2 i (i < 8) and keys tx + 16 u (u < 4 / KS) of S, and output columns 4 tx .. + 3
+// (and 64 + 4 tx .. + 3).  With KS > 1 the KS warps of a row group see different keys of each block and are merged
+// once at the end.
+//
+// Element-exact skipping: lim_i is the last key of the warp's share that row i keeps; groups of 16 keys that a whole
+// warp keeps run without tests, groups that nobody keeps are passed over, the rest is predicated weight by weight.  The
+// same limits bound phase 3.
+//
+// Shared-memory rows hold 64 DG floats as 16-byte chunks, chunk c of row r at c ^ (r % 8): 16-byte reads of 8 rows in
+// the same column, or of 8 neighbouring columns of one row, touch every bank once.
+constexpr int FA_THREADS = 128, FA_BC = 64;
+
+template <int DG> __device__ __forceinline__ int fa_off(int row, int chunk) { return row * (64 * DG) + ((chunk ^ (row & 7)) << 2); }
+
+template <int DG, int KS>
+struct FACfg {
+    static constexpr int BR = 64 / KS, U = 4 / KS, KW = FA_BC / KS;     // rows per CTA; key groups and keys of a warp
+    static constexpr int Q_FLOATS = BR * 64 * DG, KV_FLOATS = FA_BC * 64 * DG, P_FLOATS = 4 * 16 * KW;
+    static constexpr int SMEM = (Q_FLOATS + 2 * KV_FLOATS + P_FLOATS) * (int)sizeof(float);
+    static constexpr int PCH = KW / 4;                                  // 16-byte chunks of a row of P
+};
+// P of a warp: 16 rows of KW weights, chunks permuted like the tiles above as far as a row has chunks
+template <int DG, int KS> __device__ __forceinline__ int fa_poff(int row, int chunk) {
+    using C = FACfg<DG, KS>;
+    return row * C::KW + ((chunk ^ (row & (C::PCH >= 8 ? 7 : C::PCH - 1))) << 2);
+}
+
+// Rows r0 .. r0 + nrows - 1 of one head into a tile (rows beyond n stay as they are; nothing reads them).
+template <int DG>
+__device__ __forceinline__ void fa_load(float* tile, const float* src, int r0, int nrows, int n, size_t ld, int d4) {
+    for (int t = threadIdx.x; t < nrows * 16 * DG; t += FA_THREADS) {
+        const int r = t / (16 * DG), c = t % (16 * DG);
+        if (c < d4 && r0 + r < n) cp_async16(tile + fa_off<DG>(r, c), src + (size_t)(r0 + r) * ld + 4 * c);
+    }
+}
+
+// acc[i][u] (+)= q_i . k_u, sums of even and odd components side by side.  EDGE: only the weights with keep true.
+template <int DG, int U, bool EDGE>
+__device__ __forceinline__ void fa_scores(unsigned long long (&acc)[8][U], const float* Q, const float* K, int qrow, int krow,
+                                          int d4, const int (&lim)[8], int tx, int minlim, int maxlim) {
+#pragma unroll 4
+    for (int c = 0; c < d4; ++c) {
+        ulonglong2 k[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) k[u] = *reinterpret_cast<const ulonglong2*>(K + fa_off<DG>(krow + 16 * u, c));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(Q + fa_off<DG>(qrow + 2 * i, c));
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (EDGE) {
+                    if (16 * u > maxlim) continue;                                  // (same for the whole warp)
+                    if (16 * u + 15 > minlim && tx + 16 * u > lim[i]) continue;
+                }
+                fma2(acc[i][u], q.x, k[u].x);
+                fma2(acc[i][u], q.y, k[u].y);
+            }
+        }
+    }
+}
+
+// MODE 0: the three phases for FULL / MASKED.  MODE 2: phases 2 and 3 of the symmetric scheme, scores read from S.
+template <int DG, int KS, int MODE>
+__global__ void __launch_bounds__(FA_THREADS, DG == 1 ? 3 : 2)
+f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
+                 float* __restrict__ out, const float* __restrict__ S, int n, int H, int d, float scale, int masked,
+                 DeviceCounters* dc) {
+    using C = FACfg<DG, KS>;
+    constexpr int U = C::U;
+    extern __shared__ float4 fa_smem4[];
+    float* Qs = reinterpret_cast<float*>(fa_smem4);
+    float* Ks = Qs + C::Q_FLOATS;
+    float* Vs = Ks + C::KV_FLOATS;
+    float* Ps = Vs + C::KV_FLOATS;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
+    const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
+    const int rb = masked ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // the longest rows first
+    const int r0 = rb * C::BR;
+    const int rg = warp / KS, kw = (warp % KS) * C::KW;                 // the warp's row group and first key of a block
+    const int qrow = 16 * rg + ty, row = r0 + qrow;                     // row i of the lane: + 2 i
+    const int wr0 = r0 + 16 * rg;                                       // first row of the warp
+    const size_t ld = (size_t)H * d;
+    const size_t base = ((size_t)b * n) * ld + (size_t)h * d;
+    const int d4 = d >> 2;
+    const int kend = masked ? min(r0 + C::BR, n) : n;                   // keys that some row of the CTA keeps
+    const int nblk = (kend + FA_BC - 1) / FA_BC;
+    const float* Sh = MODE == 2 ? S + (size_t)bh * n * n : nullptr;
+    float* Pw = Ps + warp * 16 * C::KW;
+    const bool act0 = tx < d4, act1 = DG == 2 && 16 + tx < d4;          // output columns this lane owns
+
+    if (MODE != 2) {
+        fa_load<DG>(Qs, Q + base, r0, C::BR, n, ld, d4);
+        fa_load<DG>(Ks, K + base, 0, FA_BC, n, ld, d4);
+    }
+    cp_async_commit();
+
+    float m[8], l[8];
+    unsigned long long o[8][2 * DG] = {};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+    unsigned long long dots = 0, wts = 0;                               // weights of this lane; of its rows in phase 3
+
+    for (int jb = 0; jb < nblk; ++jb) {
+        const int k0 = jb * FA_BC + kw;                                 // first key of the warp's share
+        int lim[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) lim[i] = row + 2 * i >= n ? -1 : min(masked ? row + 2 * i : n - 1, n - 1) - k0;
+        const int last = min(wr0 + 15, n - 1);                          // last row of the warp that exists
+        const int maxlim = wr0 >= n ? -1 : (masked ? last : n - 1) - k0;
+        const int minlim = wr0 + 15 >= n ? -1 : (masked ? wr0 : n - 1) - k0;
+        const bool whole = minlim >= C::KW - 1;
+
+        float s[8][U];
+        if (MODE != 2) cp_async_wait_all();
+        __syncthreads();            // K_j has landed; every warp is done with V_{j-1}
+        fa_load<DG>(Vs, V + base, jb * FA_BC, FA_BC, n, ld, d4);
+        cp_async_commit();
+        // ---- phase 1 (Eq. 1)
+        if (MODE == 2) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    s[i][u] = tx + 16 * u <= lim[i] ? __ldg(Sh + (size_t)(row + 2 * i) * n + k0 + tx + 16 * u) : -INFINITY;
+        } else {
+            unsigned long long acc[8][U] = {};
+            if (whole) {
+                fa_scores<DG, U, false>(acc, Qs, Ks, qrow, kw + tx, d4, lim, tx, minlim, maxlim);
+                dots += 8 * U;
+            } else if (maxlim >= 0) {
+                fa_scores<DG, U, true>(acc, Qs, Ks, qrow, kw + tx, d4, lim, tx, minlim, maxlim);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float2 f = unpack2(acc[i][u]);
+                    s[i][u] = (f.x + f.y) * scale;
+                    if (!whole) {
+                        const bool keep = tx + 16 * u <= lim[i];
+                        s[i][u] = keep ? s[i][u] : -INFINITY;
+                        dots += keep;
+                    }
+                }
+        }
+        // ---- phase 2 (Eq. 2): running row maximum and sum; the sum stays per lane until the end
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float mx = s[i][0];
+#pragma unroll
+            for (int u = 1; u < U; ++u) mx = fmaxf(mx, s[i][u]);
+#pragma unroll
+            for (int off = 8; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            mx = fmaxf(mx, m[i]);
+            const float sub = mx == -INFINITY ? 0.f : mx;               // (no finite score yet: every weight is 0)
+            if (mx != m[i]) {
+                const float alpha = expf(m[i] - mx);
+                m[i] = mx;
+                l[i] *= alpha;
+                const unsigned long long a2 = dup2(alpha);
+#pragma unroll
+                for (int g = 0; g < 2 * DG; ++g) asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(o[i][g]) : "l"(a2));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (whole || tx + 16 * u <= lim[i]) {
+                    const float e = expf(s[i][u] - sub);
+                    l[i] += e;
+                    Pw[fa_poff<DG, KS>(ty + 2 * i, (tx >> 2) + 4 * u) + (tx & 3)] = e;
+                }
+            }
+            if (tx == 0) wts += min(max(lim[i] + 1, 0), C::KW);
+        }
+        cp_async_wait_all();
+        __syncthreads();            // V_j has landed, P is written; every warp is done with K_j
+        if (MODE != 2 && jb + 1 < nblk) fa_load<DG>(Ks, K + base, (jb + 1) * FA_BC, FA_BC, n, ld, d4);
+        cp_async_commit();
+        // ---- phase 3 (Eq. 3): keys in order, the warp's columns of V against its weights
+        if (act0) {
+            const int jfull = whole ? C::KW : (minlim + 1 > 0 ? (minlim + 1) & ~3 : 0);
+            const float* vb = Vs + kw * 64 * DG;                        // (kw is a multiple of 16: rows keep their phase)
+            for (int j = 0; j < jfull; j += 4) {
+                float4 p[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) p[i] = *reinterpret_cast<const float4*>(Pw + fa_poff<DG, KS>(ty + 2 * i, j >> 2));
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    ulonglong2 v[DG];
+                    v[0] = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j + jj, tx));
+                    if (DG == 2 && act1) v[DG - 1] = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j + jj, 16 + tx));
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const unsigned long long w = dup2(jj == 0 ? p[i].x : jj == 1 ? p[i].y : jj == 2 ? p[i].z : p[i].w);
+                        fma2(o[i][0], w, v[0].x);
+                        fma2(o[i][1], w, v[0].y);
+                        if (DG == 2 && act1) {
+                            fma2(o[i][2 * DG - 2], w, v[DG - 1].x);
+                            fma2(o[i][2 * DG - 1], w, v[DG - 1].y);
+                        }
+                    }
+                }
+            }
+            if (!whole) {
+                const int jend = min(maxlim + 1, C::KW);
+#pragma unroll 1
+                for (int j = jfull; j < jend; ++j) {
+                    const ulonglong2 v0 = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j, tx));
+                    ulonglong2 v1 = v0;
+                    if (DG == 2 && act1) v1 = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j, 16 + tx));
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        if (j > lim[i]) continue;
+                        const unsigned long long w = dup2(Pw[fa_poff<DG, KS>(ty + 2 * i, j >> 2) + (j & 3)]);
+                        fma2(o[i][0], w, v0.x);
+                        fma2(o[i][1], w, v0.y);
+                        if (DG == 2 && act1) { fma2(o[i][2 * DG - 2], w, v1.x); fma2(o[i][2 * DG - 1], w, v1.y); }
+                    }
+                }
+            }
+        }
+    }
+    // ---- row sums over the 16 lanes of a row, the division of Eq. 2, output
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int off = 8; off; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+    if (KS == 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (row + 2 * i >= n) continue;
+            const float inv = 1.f / l[i];
+            float* dst = out + base + (size_t)(row + 2 * i) * ld + 4 * tx;
+#pragma unroll
+            for (int g = 0; g < DG; ++g) {
+                if (!(g == 0 ? act0 : act1)) continue;
+                const float2 lo = unpack2(o[i][2 * g]), hi = unpack2(o[i][2 * g + 1]);
+                *reinterpret_cast<float4*>(dst + 64 * g) = make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv);
+            }
+        }
+    } else {
+        // the KS partial results of a row, brought to their common maximum and added up
+        __syncthreads();            // every warp is done with V and P
+        float* part = Ks;           // [KS][BR][64 DG], over the K tile
+        float* ml = Ps;             // [KS][BR] maxima, then [KS][BR] sums
+        const int ks = warp % KS;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = qrow + 2 * i;
+#pragma unroll
+            for (int g = 0; g < DG; ++g) {
+                const float2 lo = unpack2(o[i][2 * g]), hi = unpack2(o[i][2 * g + 1]);
+                *reinterpret_cast<float4*>(part + (size_t)(ks * C::BR + r) * 64 * DG + 64 * g + 4 * tx) = make_float4(lo.x, lo.y, hi.x, hi.y);
+            }
+            if (tx == 0) { ml[ks * C::BR + r] = m[i]; ml[KS * C::BR + ks * C::BR + r] = l[i]; }
+        }
+        __syncthreads();
+        for (int t = tid; t < C::BR * d4; t += FA_THREADS) {
+            const int r = t / d4, c = t - r * d4;
+            if (r0 + r >= n) continue;
+            float mx = -INFINITY;
+#pragma unroll
+            for (int k = 0; k < KS; ++k) mx = fmaxf(mx, ml[k * C::BR + r]);
+            float sum = 0.f;
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                const float mk = ml[k * C::BR + r];
+                if (mk == -INFINITY && ml[KS * C::BR + k * C::BR + r] == 0.f) continue;      // no key of this share counts
+                const float w = mk == mx ? 1.f : expf(mk - mx);
+                const float4 f = *reinterpret_cast<const float4*>(part + (size_t)(k * C::BR + r) * 64 * DG + 4 * c);
+                sum = fmaf(w, ml[KS * C::BR + k * C::BR + r], sum);
+                y.x = fmaf(w, f.x, y.x); y.y = fmaf(w, f.y, y.y); y.z = fmaf(w, f.z, y.z); y.w = fmaf(w, f.w, y.w);
+            }
+            const float inv = 1.f / sum;
+            *reinterpret_cast<float4*>(out + base + (size_t)(r0 + r) * ld + 4 * c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+        }
+    }
+    // ---- census
+    for (int off = 16; off; off >>= 1) {
+        dots += __shfl_xor_sync(0xffffffffu, dots, off);
+        wts += __shfl_xor_sync(0xffffffffu, wts, off);
+    }
+    if (lane == 0) {
+        if (MODE != 2 && dots) atomicAdd(&dc->qk_macs, dots * (unsigned long long)d);
+        if (wts) { atomicAdd(&dc->pv_macs, wts * (unsigned long long)d); atomicAdd(&dc->exps, wts); }
+    }
+}
+
+// Phase 1 of the symmetric scheme, tiled: one CTA per 64 x 64 block at or below the diagonal; S_ij for j <= i is computed
+// once and stored at (i, j) and, through shared memory, at its mirror (j, i).
+template <int DG>
+__global__ void __launch_bounds__(FA_THREADS)
+f32_sym_scores_kernel(const float* __restrict__ X, float* __restrict__ S, int n, int H, int d, float scale, DeviceCounters* dc) {
+    extern __shared__ float4 fa_smem4[];
+    float* Qs = reinterpret_cast<float*>(fa_smem4);
+    float* Ks = Qs + 64 * 64 * DG;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
+    const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
+    int I = 0, t = blockIdx.y;
+    while (t > I) { t -= I + 1; ++I; }
+    const int r0 = 64 * I, c0 = 64 * t;
+    const size_t ld = (size_t)H * d, base = ((size_t)b * n) * ld + (size_t)h * d;
+    fa_load<DG>(Qs, X + base, r0, 64, n, ld, d >> 2);
+    fa_load<DG>(Ks, X + base, c0, 64, n, ld, d >> 2);
+    cp_async_wait_all();
+    __syncthreads();
+    const int qrow = 16 * warp + ty, row = r0 + qrow, wr0 = r0 + 16 * warp;
+    int lim[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) lim[i] = row + 2 * i >= n ? -1 : row + 2 * i - c0;
+    const int maxlim = wr0 >= n ? -1 : min(wr0 + 15, n - 1) - c0, minlim = wr0 + 15 >= n ? -1 : wr0 - c0;
+    unsigned long long acc[8][4] = {}, dots = 0;
+    if (minlim >= 63) fa_scores<DG, 4, false>(acc, Qs, Ks, qrow, tx, d >> 2, lim, tx, minlim, maxlim);
+    else if (maxlim >= 0) fa_scores<DG, 4, true>(acc, Qs, Ks, qrow, tx, d >> 2, lim, tx, minlim, maxlim);
+    __syncthreads();                // the operand tiles become the block's staging buffer, [64][65]
+    float* Sh = S + (size_t)bh * n * n;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float2 f = unpack2(acc[i][u]);
+            const float v = (f.x + f.y) * scale;
+            const int j = tx + 16 * u;
+            if (j > lim[i]) continue;
+            Qs[(qrow + 2 * i) * 65 + j] = v;
+            Sh[(size_t)(row + 2 * i) * n + c0 + j] = v;
+            ++dots;
+        }
+    __syncthreads();
+    for (int e = tid; e < 64 * 64; e += FA_THREADS) {       // mirror: row c0 + j, columns r0 + i
+        const int j = e >> 6, i = e & 63;
+        if (r0 + i < n && c0 + j < r0 + i) Sh[(size_t)(c0 + j) * n + r0 + i] = Qs[i * 65 + j];
+    }
+    for (int off = 16; off; off >>= 1) dots += __shfl_xor_sync(0xffffffffu, dots, off);
+    if (lane == 0 && dots) atomicAdd(&dc->qk_macs, dots * (unsigned long long)d);
+}
+
 constexpr int ROWS_PER_BLOCK = 4;  // one warp per query row
 constexpr int KEY_TILE = 32;
 
@@ -364,15 +821,6 @@ f32_fused_layer_kernel(const float* __restrict__ X, const float* __restrict__ Wq
     if (tid == 0) atomicAdd(&dc->proj_macs, (unsigned long long)nW * n * D * d);
 }
 
-// Asynchronous copies global -> shared (4 and 16 bytes) and the wait for all of a thread's copies.
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // The same layer spread over a cluster of C CTAs (FULL and MASKED): 4-row tiles are dealt to the CTAs in turn (tile ti
 // belongs to CTA ti % C, which balances the masked scheme's growing rows), each CTA projects q, k, v of its own rows,
 // the CTAs read one another's k and v through distributed shared memory, and each finishes phases 1-3 for its rows.
@@ -549,8 +997,41 @@ size_t attn_smem_bytes(int n, int d) {
 
 }  // namespace
 
+namespace {
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+template <int BM, int BN, int TM, int TN>
+cudaError_t launch_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
+                           const float* residual, DeviceCounters* dc, cudaStream_t stream) {
+    using C = GPCfg<BM, BN, TM, TN>;
+    const dim3 grid((N + BN - 1) / BN, (rows + BM - 1) / BM, nW);
+    f32_project_tiled_kernel<BM, BN, TM, TN><<<grid, C::THREADS, C::SMEM, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2],
+                                                                                    rows, D, N, residual, dc);
+    return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
                         int N, const float* residual, DeviceCounters* dc, cudaStream_t stream) {
+    bool tiled = D % 4 == 0 && N % 4 == 0 && aligned16(X) && aligned16(residual);      // 16-byte rows
+    for (int w = 0; w < nW; ++w) tiled = tiled && aligned16(W[w]) && aligned16(out[w]);
+    // (grid.y holds 65535 row tiles)
+    if (tiled && (rows + 31) / 32 <= 65535) {
+        static DeviceSetup setup;
+        const int sms = device_setup(&setup, [] {
+            cudaError_t e = cudaFuncSetAttribute(f32_project_tiled_kernel<128, 128, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 GPCfg<128, 128, 8, 8>::SMEM);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(f32_project_tiled_kernel<64, 64, 4, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         GPCfg<64, 64, 4, 8>::SMEM);
+            return e;
+        }, "fp32 projection set-up");
+        if (sms <= 0) return cudaErrorUnknown;
+        auto tiles = [&](int t) { return (long long)((rows + t - 1) / t) * ((N + t - 1) / t) * nW; };
+        if (tiles(128) >= sms) return launch_project<128, 128, 8, 8>(X, W, out, nW, rows, D, N, residual, dc, stream);
+        if (tiles(64) >= sms) return launch_project<64, 64, 4, 8>(X, W, out, nW, rows, D, N, residual, dc, stream);
+        return launch_project<32, 32, 2, 4>(X, W, out, nW, rows, D, N, residual, dc, stream);
+    }
     dim3 block(PROJ_TILE, PROJ_TILE), grid((N + PROJ_TILE - 1) / PROJ_TILE, (rows + PROJ_TILE - 1) / PROJ_TILE, nW);
     f32_project_kernel<<<grid, block, 0, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);
     return cudaGetLastError();
@@ -605,8 +1086,58 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
     return cudaGetLastError();
 }
 
+namespace {
+template <int DG, int KS, int MODE>
+cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n, int d,
+                         float scale, int masked, DeviceCounters* dc, cudaStream_t stream) {
+    using C = FACfg<DG, KS>;
+    static DeviceSetup setup;
+    if (device_setup(&setup, [] {
+            return cudaFuncSetAttribute(f32_flash_kernel<DG, KS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, FACfg<DG, KS>::SMEM);
+        }, "fp32 attention set-up") <= 0)
+        return cudaErrorUnknown;
+    const dim3 grid(B * H, (n + C::BR - 1) / C::BR);
+    f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc);
+    return cudaGetLastError();
+}
+template <int DG, int MODE>
+cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n,
+                               int d, float scale, int masked, DeviceCounters* dc, cudaStream_t stream) {
+#ifdef PSA_FA_KS
+    return launch_flash<DG, PSA_FA_KS, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+#endif
+    static DeviceSetup setup;
+    const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
+    if (sms <= 0) return cudaErrorUnknown;
+    auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
+    if (ctas(64) >= sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+    if (ctas(32) >= sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+    return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+}
+template <int DG>
+cudaError_t tiled_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H, int n, int d,
+                            float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+    if (scheme != PSA_SYMMETRIC)
+        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, stream);
+    constexpr int SMEM = 2 * 64 * 64 * DG * (int)sizeof(float);
+    static DeviceSetup setup;
+    if (device_setup(&setup, [] {
+            return cudaFuncSetAttribute(f32_sym_scores_kernel<DG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        }, "fp32 scores set-up") <= 0)
+        return cudaErrorUnknown;
+    const int T = (n + 63) / 64;
+    f32_sym_scores_kernel<DG><<<dim3(B * H, T * (T + 1) / 2), FA_THREADS, SMEM, stream>>>(Q, S, n, H, d, scale, dc);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, stream);
+}
+}  // namespace
+
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H,
                           int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+    if (d % 4 == 0 && (long long)B * H <= 0x7fffffff && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(out))      // 16-byte rows
+        return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream)
+                       : tiled_attention<2>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
     dim3 grid((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, H, B), block(ROWS_PER_BLOCK * 32);
     const size_t smem = attn_smem_bytes(n, d);
     if (scheme == PSA_SYMMETRIC) {

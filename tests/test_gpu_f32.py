@@ -94,3 +94,60 @@ def test_host_entry_matches_device_entry():
     binding.psa_attention_host(*host, 1, binding.MASKED, out_h)
     out_d = binding.psa_attention_f32(*[t.cuda() for t in host], 1, binding.MASKED)
     assert torch.equal(out_h, out_d.cpu())
+
+
+# The tiled kernels walk keys in blocks of 64 and rows in tiles of 64, 32 or 16 (fewer rows per CTA when a call has few
+# heads), heads of up to 64 and up to 128 columns: the shapes put n one below, at and one above those edges, and B * H on
+# both sides of the switches between row tiles.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.SYMMETRIC, oracle.MASKED])
+@pytest.mark.parametrize("B,H,n,d", [(1, 1, 1, 4), (1, 2, 15, 64), (1, 1, 17, 128), (2, 1, 63, 68), (1, 3, 64, 100),
+                                     (1, 2, 65, 64), (3, 16, 129, 20), (4, 40, 33, 128), (3, 25, 96, 64), (1, 1, 1000, 128)])
+def test_core_at_tile_edges(scheme, B, H, n, d):
+    rng = np.random.default_rng(7 * n + d)
+    Q, K, V = (rng.standard_normal((B, n, H, d)).astype(np.float32) for _ in range(3))
+    if scheme == oracle.SYMMETRIC:
+        out = binding.psa_attention_core(_dev(Q), None, None, scheme)
+        ref, cnt = oracle.attention_core(Q, Q, Q, scheme)
+    else:
+        out = binding.psa_attention_core(_dev(Q), _dev(K), _dev(V), scheme)
+        ref, cnt = oracle.attention_core(Q, K, V, scheme)
+    assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= TOL_F32
+    _check_counts(cnt, 0)
+
+
+# Rows that keep only scores of -inf so far (their first blocks weigh nothing), and infinite and NaN scores, come out as
+# in the plain softmax: finite where the row has a finite score, NaN where the plain form divides 0 by 0 or meets NaN.
+@pytest.mark.parametrize("n,H", [(200, 1), (200, 80)])
+def test_core_with_infinite_scores(n, H):
+    rng = np.random.default_rng(3)
+    Q = np.abs(rng.standard_normal((1, n, H, 16))).astype(np.float32) + 0.1
+    K = rng.standard_normal((1, n, H, 16)).astype(np.float32)
+    V = rng.standard_normal((1, n, H, 16)).astype(np.float32)
+    K[0, :130, :, 0] = -np.inf          # scores of keys 0-129 are -inf in every row
+    Q[0, 7, :, 0] = np.nan
+    out = binding.psa_attention_core(_dev(Q), _dev(K), _dev(V), binding.FULL).cpu().numpy()[0].reshape(n, H, 16)
+    with np.errstate(invalid="ignore"):
+        s = np.einsum("ihd,jhd->hij", Q[0].astype(np.float64), K[0].astype(np.float64)) / 4.0
+        w = np.exp(s - s.max(-1, keepdims=True))
+        ref = np.einsum("hij,jhd->ihd", w / w.sum(-1, keepdims=True), V[0].astype(np.float64))
+    assert np.array_equal(np.isnan(out), np.isnan(ref)) and np.isnan(out[7]).all()
+    keep = np.arange(n) != 7
+    assert np.abs(out[keep] - ref[keep]).max() <= TOL_F32
+    masked = binding.psa_attention_core(_dev(Q), _dev(K), _dev(V), binding.MASKED).cpu().numpy()[0].reshape(n, H, 16)
+    assert np.isnan(masked[:130]).all() and np.isfinite(masked[130:]).all()
+
+
+# Tile sizes of the projection (128, 64 and 32, by how many tiles the call has) and the general kernel where a row is not a
+# multiple of 16 bytes: ragged rows, columns and k.
+@pytest.mark.parametrize("rows,D,H,d", [(1, 4, 1, 4), (33, 36, 3, 20), (300, 100, 9, 68), (1100, 68, 12, 100), (1100, 66, 12, 100)])
+def test_projection_tiles(rows, D, H, d):
+    rng = np.random.default_rng(rows + d)
+    X = (rng.standard_normal((1, 1, D)) * 0.5).astype(np.float32).repeat(rows, 0)       # rows sequences of one vector:
+    X *= np.linspace(0.5, 1.5, rows, dtype=np.float32)[:, None, None]                   # y = v, the projection itself
+    W = (rng.standard_normal((D, H * d)) / np.sqrt(D)).astype(np.float32)
+    Wo = (rng.standard_normal((H * d, D)) / np.sqrt(H * d)).astype(np.float32)
+    out = binding.psa_attention_block(_dev(X), _dev(W), _dev(W), _dev(W), _dev(Wo), H, binding.FULL, residual=_dev(X * 2))
+    ref = X.astype(np.float64) @ W.astype(np.float64) @ Wo.astype(np.float64) + 2.0 * X
+    assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= TOL_F32
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got["proj_macs"] == 4 * rows * D * H * d
