@@ -1110,8 +1110,11 @@ cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, f
     const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
     if (sms <= 0) return cudaErrorUnknown;
     auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
-    if (ctas(64) >= sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
-    if (ctas(32) >= sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+    // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs:
+    // measured, two resident CTAs per SM are where the line lies (us for KS = 1 / 2 / 4).  80 tiles of 64 rows: 208 / 144 /
+    // 112; 256 tiles, masked, d = 128: 268 / 216 / 252; 384 tiles: 137 / 155 / 180.
+    if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+    if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
     return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
 }
 template <int DG>
