@@ -1,21 +1,28 @@
-// Attention core of the bf16 path: dispatch, and the two kernels of the symmetric scheme (paper Sec. 4).
+// Attention core of the bf16 path: dispatch, and the kernel of the symmetric scheme (paper Sec. 4).
 //
 // With query = key = value = X the weight matrix before the softmax is symmetric, w'_ij = w'_ji (paper
 // Eq. 4), and the paper computes one member of each pair and reuses it.  On this machine the reuse goes
-// through memory:
+// through memory, inside one persistent kernel: the CTA that works on 128-row tile I computes the blocks
+// (I, J), J <= I, on the tensor core, uses them and hands those with J < I on through the scratch; for
+// J > I it takes block (J, I) from there, transposed.  A block is written once and read once, and since a
+// tile uses its computed blocks first and the handed-on ones after them, in the order of J, the tiles of a
+// head run in step: block (J, I) is finished at step I of tile J and needed at step J of tile I, usually
+// while it is still in L2.
 //
-//   sym_scores_kernel   phase 1, one CTA per unordered pair of 128-row tiles {I, J}, J <= I: the block
-//                       S_IJ = scale * X_I X_J^T on the tensor core, written ONCE to the scratch.  Blocks
-//                       above the diagonal are neither computed nor stored.
-//   sym_attn_kernel     phases 2 and 3 per 128-row tile: the row of blocks S_I,* is fetched into shared
-//                       memory -- block (I, J) as stored for J <= I, block (J, I) read transposed for
-//                       J > I (the reuse) -- then softmax and O += P V as in the fused kernel of the other
-//                       schemes (two threads per row, P written to TMEM as bf16, V = X staged by TMA,
-//                       accumulator O in TMEM, the division of Eq. 2 applied once to the output row).
+// A work item is a row tile of one head.  Items are numbered with the last tile of a head first and taken
+// from a device counter in that order, so an item only ever waits for items that were taken before it: the
+// oldest unfinished item waits for nobody.
 //
-// The scratch holds, per head, the T(T+1)/2 blocks at or below the block diagonal, each as one contiguous
-// 64 KB image of its shared-memory form (four [128 rows x 32 fp32] sub-tiles in the 128-byte swizzle), so
-// that a block moves between shared and global memory as one bulk copy of consecutive bytes.
+// Roles of a CTA (352 threads): warp 0 takes items and loads operand tiles and handed-on blocks, warp 1 issues
+// the MMAs, warps 2-9 do the softmax and the output (a warp owns 16 rows, quad layout of sm100.cuh), warp 10
+// announces finished blocks to the other CTAs.  One row tile at a time, but with two score buffers and two
+// weight buffers in tensor memory (S0 S1 | P0 P1 | O): S of the next block is there when the softmax of
+// the current one ends, PV of a block runs under the softmax of the next, and the eight softmax warps drift
+// apart by up to a block, which keeps the special-function pipe busy while some of them are at their loads.
+//
+// What bounds it: softmax (1024 cycles of exponentials per block) and, in step with it, the operands of one row
+// tile per SM: 32 KB of X per block, 64 KB of scores stored or loaded for all but the diagonal one.  Measured
+// (L2 flushed, B = 64, H = 16, n = 1024, d_k = 128): @@MEASURED@@
 //
 // The fused persistent kernel of the FULL and MASKED schemes is in psa_attn_persist.cu.
 #include "psa_internal.h"
@@ -28,173 +35,113 @@ namespace psa {
 
 namespace {
 
-constexpr int S_SUB_BYTES = 128 * 32 * 4;       // one [128 rows x 32 fp32] sub-tile of a score block, 128-byte rows
-constexpr int S_BLOCK_BYTES = 4 * S_SUB_BYTES;  // one 128 x 128 fp32 score block: 64 KB
-#ifndef PSA_SYM_COPIES
-#define PSA_SYM_COPIES 4
-#endif
-constexpr int S_COPIES = PSA_SYM_COPIES;        // bulk copies a block is moved in
+constexpr int S_BLOCK_BYTES = 128 * 128 * 4;    // one 128 x 128 fp32 score block of the scratch: 64 KB
+constexpr int S_HALF_BYTES = S_BLOCK_BYTES / 2; // 64 of its rows = 64 key columns of the tile that reads it transposed
+constexpr int SYM_WARPS = SOFTMAX_WARPS_PER_TILE;                    // 8
+constexpr int SYM_PUBLISHER = CTRL_WARPS + SYM_WARPS;                // warp that announces finished blocks
+constexpr int SYM_THREADS = 32 * (SYM_PUBLISHER + 1);                // 352
+constexpr int SYM_ITEM_READERS = SYM_WARPS + 2;                      // softmax warps, MMA issuer, publisher
 
 template <int D>
 struct SymCfg {
     static constexpr int SUB = D / 64;                  // 64-column sub-tiles per 128-row tile of X
     static constexpr int TILE_BYTES = 128 * D * 2;      // one X tile (bf16)
-    static constexpr int VSTAGES = D == 128 ? 2 : 4;
-    static constexpr int SMEM = 2 * S_BLOCK_BYTES + VSTAGES * TILE_BYTES + 1024;
-    static constexpr int TMEM_P = 0, TMEM_O = 64;       // P (64 columns: 128 keys as bf16 pairs) | O (D columns)
-    static constexpr int SCORES_SMEM = (S_BLOCK_BYTES > 2 * TILE_BYTES ? S_BLOCK_BYTES : 2 * TILE_BYTES) + 1024;
+    static constexpr int XST = D == 128 ? 3 : 4;        // X tiles in flight: PV of a block, S of the next, one loading
+    static constexpr int MST = D == 128 ? 2 : 4;        // half blocks of handed-on scores in flight
+    static constexpr int STAGE_BYTES = 16 * 64 * 2;     // a softmax warp's output staging buffer
+    static constexpr int SMEM = (1 + XST) * TILE_BYTES + MST * S_HALF_BYTES + SYM_WARPS * STAGE_BYTES + 1024;
+    static constexpr int TMEM_S = 0, TMEM_P = 256, TMEM_O = 384;
 };
 
 struct SymMaps {
-    CUtensorMap x;     // X as [batch, n, H*d] bf16, boxes of 128 rows x 64 columns
-    CUtensorMap o;     // output, like x
+    CUtensorMap x;     // X as [batch, n, heads, d] bf16, boxes of 128 rows x 64 columns
+    CUtensorMap o;     // output, boxes of 16 rows
 };
 
 struct SymBars {
-    uint64_t s_full[2], s_free[2];
-    uint64_t v_full[4], v_empty[4];
-    uint64_t p_ready[2], o_done[2];
+    uint64_t item_full[2], item_empty[2];
+    uint64_t q_full, q_empty;
+    uint64_t x_full[4], x_empty[4], m_full[4], m_empty[4];
+    uint64_t s_full[2], s_free[2], p_ready[2], o_done[2];
 };
 
-// Phase 1 of the symmetric scheme (paper Sec. 4.1): one CTA per unordered tile pair {I, J}, J <= I, computes
-// S_IJ = scale * X_I X_J^T once and stores it at block (I, J) of the scratch; the mirror block (J, I) is never
-// formed: its readers take (I, J) transposed.
-template <int D>
-__global__ void __launch_bounds__(128)
-sym_scores_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, int n, int H, int bh0, float scale,
-                  DeviceCounters* dc) {
-    constexpr int SUB = D / 64, TILE_BYTES = 128 * D * 2;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sA = smem;
-    uint8_t* sB = smem + TILE_BYTES;
-    uint8_t* sS = smem;                  // the finished block is staged over the operand tiles
-    __shared__ uint64_t full_bar, acc_bar;
-    __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_flag;
+// The scratch of a head is one 64 KB block per tile pair (I, J), J <= I, numbered I (I + 1) / 2 + J.  Diagonal blocks are
+// never handed on; the place of block (0, 0) holds the head's flags instead: flag I = blocks that tile I has handed on.  The
+// first head's place also holds, behind its T flags, the work counter of the launch.
+__device__ __forceinline__ float* sym_head(float* Sg, int hl, int np) { return Sg + (size_t)hl * np * (S_BLOCK_BYTES / 4); }
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int T = row_tiles(n);
-    const int np = sym_pairs(T);
-    const int hl = blockIdx.x / np;                 // head inside this pass
-    int I, J;
-    sym_pair(blockIdx.x - hl * np, &I, &J);
-    const int bh = bh0 + hl, b = bh / H, h = bh - b * H;
-    const int pair = blockIdx.x - hl * np;           // = I (I + 1) / 2 + J: the block's place in the head's scratch
-
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
-        mbar_init(&full_bar, 1);
-        mbar_init(&acc_bar, 1);
-        fence_mbar_init();
-    }
-    if (warp == 0) { tmem_alloc(&tmem_base_s, 128); tmem_relinquish(); }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base_s;
-    volatile int* abortp = &abort_flag;
-
-    if (threadIdx.x == 0) {
-        mbar_arrive_expect_tx(&full_bar, 2 * TILE_BYTES);
-        for (int u = 0; u < SUB; ++u) {
-            tma_load_4d(sA + u * 16384, &maps.x, &full_bar, 64 * u, h, I * TILE, b);
-            tma_load_4d(sB + u * 16384, &maps.x, &full_bar, 64 * u, h, J * TILE, b);
-        }
-        if (mbar_wait(&full_bar, 0, abortp)) {
-            tc_fence_after();
-            const uint32_t idesc = umma_idesc_bf16(128, 128, UMMA_K_MAJOR, UMMA_K_MAJOR);
-            const uint32_t a = smem_u32(sA), bb = smem_u32(sB);
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                const uint32_t off = (kk >> 2) * 16384 + (kk & 3) * 32;
-                umma_ss(tmem, umma_desc_kmajor(a + off), umma_desc_kmajor(bb + off), idesc, kk != 0);
-            }
-            umma_commit(&acc_bar);
-            atomicAdd(&dc->qk_macs, (unsigned long long)TILE * TILE * D);
-        } else {
-            mbar_wait_drain(&full_bar, 0);
-        }
-    }
-    __syncwarp();
-    const bool ready = mbar_wait(&acc_bar, 0, abortp);
-    if (__syncthreads_and(ready)) {
-        // every MMA has read its operands: the block goes to shared memory as four [128 x 32] fp32 sub-tiles in
-        // the 128-byte swizzle, each thread its own row, and from there to the scratch as one bulk copy
-        tc_fence_after();
-        const int r = warp * 32 + lane;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 4; ++c0) {
-            uint32_t v[32];
-            tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + 32 * c0, v);
-            tc_wait_ld();
-#pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                float4 f;
-                f.x = __uint_as_float(v[4 * g]) * scale;     f.y = __uint_as_float(v[4 * g + 1]) * scale;
-                f.z = __uint_as_float(v[4 * g + 2]) * scale; f.w = __uint_as_float(v[4 * g + 3]) * scale;
-                *reinterpret_cast<float4*>(sS + c0 * S_SUB_BYTES + swz128_offset(r, g)) = f;
-            }
-        }
-        fence_async_smem();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float* dst = Sg + ((size_t)hl * np + pair) * (S_BLOCK_BYTES / 4);
-            for (int u = 0; u < S_COPIES; ++u)
-                bulk_store_1d(dst + u * (S_BLOCK_BYTES / S_COPIES / 4), sS + u * (S_BLOCK_BYTES / S_COPIES), S_BLOCK_BYTES / S_COPIES);
-            tma_store_commit();
-            tma_store_wait_read();   // shared memory may be released; the writes complete on their own
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (threadIdx.x == 0 && abort_flag) atomicExch(&dc->status, (int)PSA_ERR_TIMEOUT);
-    if (warp == 0) tmem_dealloc(tmem, 128);
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
+__device__ __forceinline__ void st_release(int* p, int v) { asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ int ld_acquire_cta(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_cta(int* p, int v) { asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory"); }
 
-// Phases 2 and 3 of the symmetric scheme for one 128-row tile of one head: softmax over the stored scores and
-// O = P X.  320 threads: warp 0 = producer (score blocks and X tiles, bulk / TMA copies), warp 1 = MMA issuer,
-// warps 2-9 = softmax and epilogue, two threads per row.  The kernel is bound by the arrival of its score blocks
-// (64 KB per 128 x 128 weights), so these are double-buffered: block j + 1 is in flight while block j is in the
-// softmax, and a buffer is released as soon as its scores are in registers.
-constexpr int SYM_THREADS = 32 * (CTRL_WARPS + SOFTMAX_WARPS_PER_TILE);   // 320
+// Bounded wait until read() >= target.
+template <class Read>
+__device__ __forceinline__ bool wait_at_least(Read read, int target, volatile int* abort_flag) {
+    if (read() >= target) return true;
+    const uint64_t t0 = globaltimer_ns();
+    while (read() < target) {
+        if (*abort_flag) return false;
+        if (globaltimer_ns() - t0 > PSA_WAIT_LIMIT_NS) { *abort_flag = 1; return false; }
+        __nanosleep(64);
+    }
+    return true;
+}
 
 template <int D>
 __global__ void __launch_bounds__(SYM_THREADS, 1)
-sym_attn_kernel(const __grid_constant__ SymMaps maps, const float* __restrict__ Sg, int n, int H, int bh0,
+sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, int n, int H, int bh0, int nitems, float sl2,
                 DeviceCounters* dc) {
     using Cfg = SymCfg<D>;
-    constexpr int VST = Cfg::VSTAGES;
+    constexpr int XST = Cfg::XST, MST = Cfg::MST;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sS = smem;                                  // two 64 KB score blocks (stages)
-    uint8_t* sV = smem + 2 * S_BLOCK_BYTES;              // VSTAGES tiles of X
+    uint8_t* sQ = smem;                                          // the row tile
+    uint8_t* sX = sQ + Cfg::TILE_BYTES;                          // XST column tiles
+    uint8_t* sM = sX + XST * Cfg::TILE_BYTES;                    // MST half blocks of handed-on scores
+    uint8_t* sStage = sM + MST * S_HALF_BYTES;                   // output staging
     __shared__ SymBars bars;
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_flag;
-    __shared__ float xch_max[2][2][128];      // [block parity][column half][row]
-    __shared__ float xch_sum[2][128];         // [column half][row]
+    __shared__ int item_ring[2];
+    __shared__ int stored[SYM_WARPS];                            // blocks whose scores a softmax warp has stored, all items
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int T = row_tiles(n);
     const int np = sym_pairs(T);
-    const int hl = blockIdx.x / T;                       // head inside this pass
-    const int It = blockIdx.x - hl * T;                  // row tile
-    const int bh = bh0 + hl;
-    const int b = bh / H, h = bh - b * H;
+    int* work_counter = reinterpret_cast<int*>(Sg) + T;
+    // item -> head inside this pass and row tile, the last tile of a head first
+    auto item_head = [&](int idx) { return idx / T; };
+    auto item_tile = [&](int idx, int hl) { return T - 1 - (idx - hl * T); };
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&bars.s_full[s], 1);
-            mbar_init(&bars.s_free[s], 32 * SOFTMAX_WARPS_PER_TILE);
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(&bars.item_full[t], 1);
+            mbar_init(&bars.item_empty[t], SYM_ITEM_READERS);
+            mbar_init(&bars.s_full[t], 1);
+            mbar_init(&bars.s_free[t], SYM_WARPS);               // one arrival per softmax warp
+            mbar_init(&bars.p_ready[t], SYM_WARPS);
+            mbar_init(&bars.o_done[t], 1);
         }
-        mbar_init(&bars.p_ready[0], 32 * SOFTMAX_WARPS_PER_TILE);
-        mbar_init(&bars.o_done[0], 1);
-        for (int s = 0; s < 4; ++s) { mbar_init(&bars.v_full[s], 1); mbar_init(&bars.v_empty[s], 1); }
+        mbar_init(&bars.q_full, 1);
+        mbar_init(&bars.q_empty, 1);
+        for (int s = 0; s < 4; ++s) {
+            mbar_init(&bars.x_full[s], 1); mbar_init(&bars.x_empty[s], 1);
+            mbar_init(&bars.m_full[s], 1); mbar_init(&bars.m_empty[s], SYM_WARPS);
+        }
         fence_mbar_init();
     }
-    if (warp == 1) { tmem_alloc(&tmem_base_s, 256); tmem_relinquish(); }
+    if (threadIdx.x < SYM_WARPS) stored[threadIdx.x] = 0;
+    if (warp == 1) { tmem_alloc(&tmem_base_s, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -203,209 +150,349 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, const float* __restrict__ 
 
     if (warp == 0) {
         if (lane == 0) {
-            // ------------------------------------------------------------ producer
-            int s_loads = 0, v_loads = 0;
+            // ------------------------------------------------------------ work items, X tiles, handed-on score blocks
+            uint32_t xc = 0, mc = 0, qc = 0;         // X tiles, half blocks and row tiles requested so far
             bool ok = true;
-            for (int j = 0; j < T && ok; ++j) {
-                const int st = j & 1;
-                // a stage is free once the softmax threads have taken block j - 2 into registers
-                if (j >= 2) ok = mbar_wait(&bars.s_free[st], ((j >> 1) - 1) & 1, abortp);
+            int idx = atomicAdd(work_counter, 1);
+            for (uint32_t it = 0; ok; ++it) {
+                const int slot = it & 1;
+                if (it >= 2) ok = mbar_wait(&bars.item_empty[slot], ((it >> 1) - 1) & 1, abortp);
                 if (!ok) break;
-                const int bi = j <= It ? It : j, bj = j <= It ? j : It;      // stored block (row tile, column tile)
-                const float* src = Sg + ((size_t)hl * np + bi * (bi + 1) / 2 + bj) * (S_BLOCK_BYTES / 4);
-                mbar_arrive_expect_tx(&bars.s_full[st], S_BLOCK_BYTES);
-                for (int u = 0; u < S_COPIES; ++u)      // several copies in flight move a block faster than one
-                    bulk_load_1d(sS + st * S_BLOCK_BYTES + u * (S_BLOCK_BYTES / S_COPIES), src + u * (S_BLOCK_BYTES / S_COPIES / 4),
-                                 S_BLOCK_BYTES / S_COPIES, &bars.s_full[st]);
-                ++s_loads;
-                const int s = j % VST;
-                if (j >= VST) ok = mbar_wait(&bars.v_empty[s], ((j / VST) - 1) & 1, abortp);
-                if (!ok) break;
-                mbar_arrive_expect_tx(&bars.v_full[s], Cfg::TILE_BYTES);
-                for (int u = 0; u < Cfg::SUB; ++u)
-                    tma_load_4d(sV + s * Cfg::TILE_BYTES + u * 16384, &maps.x, &bars.v_full[s], 64 * u, h, j * TILE, b);
-                ++v_loads;
+                item_ring[slot] = idx < nitems ? idx : -1;
+                mbar_arrive(&bars.item_full[slot]);
+                if (idx >= nitems) break;
+                const int hl = item_head(idx), It = item_tile(idx, hl);
+                const int bh = bh0 + hl, b = bh / H, h = bh - b * H;
+                float* head = sym_head(Sg, hl, np);
+                const int* flags = reinterpret_cast<const int*>(head);
+                int next = 0;
+                for (int j = 0; j < T && ok; ++j) {
+                    const int s = xc % XST;
+                    if (xc >= (uint32_t)XST) ok = mbar_wait(&bars.x_empty[s], ((xc / XST) - 1) & 1, abortp);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(&bars.x_full[s], Cfg::TILE_BYTES);
+                    for (int u = 0; u < Cfg::SUB; ++u)
+                        tma_load_4d(sX + s * Cfg::TILE_BYTES + u * 16384, &maps.x, &bars.x_full[s], 64 * u, h, j * TILE, b);
+                    ++xc;
+                    if (j == 0) {
+                        if (qc > 0) ok = mbar_wait(&bars.q_empty, (qc - 1) & 1, abortp);
+                        if (!ok) break;
+                        mbar_arrive_expect_tx(&bars.q_full, Cfg::TILE_BYTES);
+                        for (int u = 0; u < Cfg::SUB; ++u) tma_load_4d(sQ + u * 16384, &maps.x, &bars.q_full, 64 * u, h, It * TILE, b);
+                        ++qc;
+                        next = atomicAdd(work_counter, 1);       // (behind the item's first loads)
+                    }
+                    if (j <= It) continue;
+                    // block (j, It), handed on by the CTA that works on tile j: present once its flag counts past It.  The
+                    // stores behind the flag were ordinary ones, the copies below go through the asynchronous proxy.
+                    ok = wait_at_least([&] { return ld_acquire(flags + j); }, It + 1, abortp);
+                    if (!ok) break;
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                    const float* src = head + (size_t)(j * (j + 1) / 2 + It) * (S_BLOCK_BYTES / 4);
+                    for (int half = 0; half < 2 && ok; ++half) {
+                        const int ms = mc % MST;
+                        if (mc >= (uint32_t)MST) ok = mbar_wait(&bars.m_empty[ms], ((mc / MST) - 1) & 1, abortp);
+                        if (!ok) break;
+                        mbar_arrive_expect_tx(&bars.m_full[ms], S_HALF_BYTES);
+                        for (int u = 0; u < 2; ++u)
+                            bulk_load_1d(sM + ms * S_HALF_BYTES + u * (S_HALF_BYTES / 2), src + half * (S_HALF_BYTES / 4) + u * (S_HALF_BYTES / 8),
+                                         S_HALF_BYTES / 2, &bars.m_full[ms]);
+                        ++mc;
+                    }
+                }
+                idx = next;
             }
             if (*abortp) {  // let copies already issued land before shared memory is released
-                for (int c = max(0, s_loads - 2); c < s_loads; ++c) mbar_wait_drain(&bars.s_full[c & 1], (c >> 1) & 1);
-                for (int c = max(0, v_loads - VST); c < v_loads; ++c) mbar_wait_drain(&bars.v_full[c % VST], (c / VST) & 1);
+                if (qc > 0) mbar_wait_drain(&bars.q_full, (qc - 1) & 1);
+                for (uint32_t c = xc > (uint32_t)XST ? xc - XST : 0; c < xc; ++c) mbar_wait_drain(&bars.x_full[c % XST], (c / XST) & 1);
+                for (uint32_t c = mc > (uint32_t)MST ? mc - MST : 0; c < mc; ++c) mbar_wait_drain(&bars.m_full[c % MST], (c / MST) & 1);
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            // ------------------------------------------------------------ MMA issuer: O (+)= P X_j (phase 3, Eq. 3)
+            // ------------------------------------------------------------ MMA issuer
+            // Per item S_0 .. S_It (phase 1, Eq. 1) and PV_0 .. PV_{T-1} (phase 3, Eq. 3), each S one block ahead of its PV;
+            // the first S of the next item goes ahead of the last PV of this one.
+            const uint32_t idescS = umma_idesc_bf16(128, 128, UMMA_K_MAJOR, UMMA_K_MAJOR);
             const uint32_t idescO = umma_idesc_bf16(128, D, UMMA_K_MAJOR, UMMA_MN_MAJOR);
-            const uint32_t v_lo = umma_desc_lo_mnmajor(smem_u32(sV), 16384);
-            const uint32_t dO = tmem + Cfg::TMEM_O, aP = tmem + Cfg::TMEM_P;
-            unsigned long long pv_blocks = 0;
+            const uint32_t q_lo = umma_desc_lo_kmajor(smem_u32(sQ)), k_lo = umma_desc_lo_kmajor(smem_u32(sX));
+            const uint32_t v_lo = umma_desc_lo_mnmajor(smem_u32(sX), 16384);
+            uint32_t sc = 0, pc = 0, xbase = 0, it = 0;      // S and PV issued so far; ring position of the item's first X tile
             bool ok = true;
-            for (int j = 0; j < T && ok; ++j) {
-                const int sv = j % VST;
-                ok = mbar_wait(&bars.v_full[sv], (j / VST) & 1, abortp) && mbar_wait(&bars.p_ready[0], j & 1, abortp);
-                if (!ok) break;
+            auto take = [&]() -> int {                        // next item: index, -1 at the end, -2 when a wait ran out
+                if (!mbar_wait(&bars.item_full[it & 1], (it >> 1) & 1, abortp)) return -2;
+                const int idx = item_ring[it & 1];
+                mbar_arrive(&bars.item_empty[it & 1]);
+                ++it;
+                return idx;
+            };
+            auto issue_S = [&](uint32_t xpos, bool first, bool last) -> bool {
+                if (first && !mbar_wait(&bars.q_full, (it - 1) & 1, abortp)) return false;
+                if (!mbar_wait(&bars.x_full[xpos % XST], (xpos / XST) & 1, abortp)) return false;
+                if (sc >= 2 && !mbar_wait(&bars.s_free[sc & 1], ((sc >> 1) - 1) & 1, abortp)) return false;
                 tc_fence_after();
-                const uint32_t v = v_lo + sv * (Cfg::TILE_BYTES >> 4);
-                if (j == 0) {
+                const uint32_t k = k_lo + (xpos % XST) * (Cfg::TILE_BYTES >> 4), dS = tmem + Cfg::TMEM_S + (sc & 1) * 128;
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        umma_ts(dO, aP + kk * 8, umma_desc_join(v + kk * (2048 >> 4), UMMA_DESC_HI_SW128), idescO, kk != 0);
-                } else {
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        umma_ts(dO, aP + kk * 8, umma_desc_join(v + kk * (2048 >> 4), UMMA_DESC_HI_SW128), idescO, 1);
+                for (int kk = 0; kk < D / 16; ++kk) {
+                    const uint32_t off = ((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
+                    umma_ss(dS, umma_desc_join(q_lo + off, UMMA_DESC_HI_SW128), umma_desc_join(k + off, UMMA_DESC_HI_SW128), idescS, kk != 0);
                 }
-                ++pv_blocks;
-                umma_commit(&bars.o_done[0]);
-                umma_commit(&bars.v_empty[sv]);
+                umma_commit(&bars.s_full[sc & 1]);
+                if (last) umma_commit(&bars.q_empty);
+                ++sc;
+                return true;
+            };
+            int idx = take();
+            int It = idx >= 0 ? item_tile(idx, item_head(idx)) : 0;
+            if (idx >= 0) ok = issue_S(0, true, It == 0);
+            while (idx >= 0 && ok) {
+                int idx_next = -1, It_next = 0;
+                for (int j = 0; j < T; ++j) {
+                    if (j < It) {
+                        ok = issue_S(xbase + j + 1, false, j + 1 == It);
+                    } else if (j == T - 1) {
+                        idx_next = take();
+                        if (idx_next == -2) ok = false;
+                        if (idx_next >= 0) {
+                            It_next = item_tile(idx_next, item_head(idx_next));
+                            ok = issue_S(xbase + T, true, It_next == 0);
+                        }
+                    }
+                    const uint32_t xpos = xbase + j;
+                    if (ok && j > It) ok = mbar_wait(&bars.x_full[xpos % XST], (xpos / XST) & 1, abortp);
+                    if (ok) ok = mbar_wait(&bars.p_ready[pc & 1], (pc >> 1) & 1, abortp);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t v = v_lo + (xpos % XST) * (Cfg::TILE_BYTES >> 4);
+                    const uint32_t aP = tmem + Cfg::TMEM_P + (pc & 1) * 64, dO = tmem + Cfg::TMEM_O;
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)
+                        umma_ts(dO, aP + kk * 8, umma_desc_join(v + kk * (2048 >> 4), UMMA_DESC_HI_SW128), idescO, (j != 0 || kk != 0) ? 1u : 0u);
+                    umma_commit(&bars.o_done[pc & 1]);
+                    umma_commit(&bars.x_empty[xpos % XST]);
+                    ++pc;
+                }
+                xbase += T;
+                idx = idx_next;
+                It = It_next;
             }
-            if (pv_blocks) {
-                atomicAdd(&dc->pv_macs, pv_blocks * (unsigned long long)TILE * TILE * D);
-                atomicAdd(&dc->exps, pv_blocks * (unsigned long long)(TILE * TILE));
+            const unsigned long long block_macs = (unsigned long long)TILE * TILE * D;
+            if (sc) atomicAdd(&dc->qk_macs, sc * block_macs);
+            if (pc) {
+                atomicAdd(&dc->pv_macs, pc * block_macs);
+                atomicAdd(&dc->exps, pc * (unsigned long long)(TILE * TILE));
             }
+        }
+    } else if (warp == SYM_PUBLISHER) {
+        // ------------------------------------------------------------ announces blocks handed on
+        // Lane w < 8 watches softmax warp w.  A block is complete when all eight have stored their rows; the fence orders
+        // their stores, observed through shared memory, before the flag.
+        int done = 0;                                           // blocks announced in earlier items
+        for (uint32_t it = 0;; ++it) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&bars.item_full[it & 1], (it >> 1) & 1, abortp))) break;
+            const int idx = item_ring[it & 1];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.item_empty[it & 1]);
+            if (idx < 0) break;
+            const int hl = item_head(idx), It = item_tile(idx, hl);
+            int* flag = reinterpret_cast<int*>(sym_head(Sg, hl, np)) + It;
+            int sent = 0;
+            bool ok = true;
+            while (sent < It) {
+                const int* mine = &stored[lane & (SYM_WARPS - 1)];
+                ok = __all_sync(0xffffffffu, wait_at_least([&] { return ld_acquire_cta(mine); }, done + sent + 1, abortp));
+                if (!ok) break;
+                const int ready = __reduce_min_sync(0xffffffffu, ld_acquire_cta(mine)) - done;    // may have moved on
+                sent = min(ready, It);
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence();
+                    st_release(flag, sent);
+                }
+            }
+            if (!ok) break;
+            done += It;
         }
     } else {
         // ------------------------------------------------------------ softmax + epilogue
-        // Two threads share a query row; thread `part` owns block columns [64 part, 64 part + 64).
-        constexpr int CPT = 128 / TPR, NCH = CPT / 32, OPT = D / TPR;
-        constexpr float sl2 = LOG2E;                          // the stored scores carry the 1/sqrt(d) factor already
-        const int sw = warp - CTRL_WARPS;
-        const int part = sw >> 2;                               // which share of the row's columns
+        const int wq = warp - CTRL_WARPS;                       // softmax warp 0-7
         const int q = warp & 3;                                 // TMEM lane quarter this warp may access
-        const int r = q * 32 + lane;                            // row inside the tile = TMEM lane
-        const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
-        const uint32_t tO = tmem + Cfg::TMEM_O + lane_off + part * OPT;
-        const uint32_t tP = tmem + Cfg::TMEM_P + lane_off;
-        const int pair_bar = 1 + q;                             // named barrier of the two warps sharing rows
-        const int tile_bar = 9;                                 // named barrier of all softmax warps
-        const int col_base = part * CPT;
-        float m_run = -INFINITY, l_run = 0.f;
+        const int kw = 2 * q + (wq >> 2);                       // its group of 16 rows inside the tile
+        const int row0 = 16 * kw;
+        const int cq = 2 * (lane & 3);                          // the thread's first column inside every group of 8
+        const uint32_t lane_off = static_cast<uint32_t>(row0) << 16;
+        const uint32_t tO = tmem + Cfg::TMEM_O + lane_off;
+        uint8_t* stage = sStage + wq * Cfg::STAGE_BYTES;
+        // Place of a score in a handed-on block, in floats.  The block is laid out for the threads that read it transposed:
+        // element (r, c) of the writer is row c, key r of the reader, and the reader's fragments (sm100.cuh) are stored as
+        // [key half][16-row group][row A / B][key group of 8][lane][2 keys].  For a writer thread everything but the
+        // constants below is a compile-time offset, and a warp's store fills whole 32-byte sectors.
+        const int put = (kw >> 2) * 8192 + 2 * (kw & 3) * 64 + (4 * cq + (lane >> 3)) * 2 + ((lane >> 2) & 1);
+        const int get = kw * 1024 + lane * 2;
+        uint32_t blk = 0, sc = 0, mc = 0;                       // blocks, computed blocks and half blocks so far, all items
+        int nstored = 0;
+        bool store_pending = false;                             // a TMA store of this warp may still be reading `stage`
         bool ok = true;
-        for (int j = 0; j < T; ++j) {
-            const uint8_t* sblock = sS + (j & 1) * S_BLOCK_BYTES;
-            ok = mbar_wait(&bars.s_full[j & 1], (j >> 1) & 1, abortp);
-            ok = __all_sync(0xffffffffu, ok);
-            // keys beyond the sequence (ragged last block) carry no weight; `cb` = last kept column
-            const int nvalid = min(TILE, n - j * TILE);
-            const bool ragged = nvalid < TILE;
-            const int cb = nvalid - 1;
-            float mx = -INFINITY;
-            uint32_t sreg[NCH][32];
-            if (ok) {
-                // ---- this thread's 64 scores: from the block as stored (column tile j at or below the row tile), or
-                // from the mirror block (j, I) read down its columns (the reused half)
+        for (uint32_t it = 0; ok; ++it) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&bars.item_full[it & 1], (it >> 1) & 1, abortp));
+            if (!ok) break;
+            const int idx = item_ring[it & 1];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.item_empty[it & 1]);
+            if (idx < 0) break;
+            const int hl = item_head(idx), It = item_tile(idx, hl);
+            float* own = sym_head(Sg, hl, np) + (size_t)(It * (It + 1) / 2) * (S_BLOCK_BYTES / 4);
+            float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;       // running maxima (log2 units) and row sums
+            for (int j = 0; j < T; ++j, ++blk) {
+                uint32_t s0[32], s1[32];
                 if (j <= It) {
+                    // ---- a block computed here
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bars.s_full[sc & 1], (sc >> 1) & 1, abortp));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t tS = tmem + Cfg::TMEM_S + (sc & 1) * 128 + lane_off;
+                    tmem_ld_quad64(tS, s0);
+                    tmem_ld_quad64(tS + 64, s1);
+                    tc_wait_ld();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bars.s_free[sc & 1]);
+                    ++sc;
+                    if (j < It) {                               // the mirror block's tile needs it
+                        float* dst = own + (size_t)j * (S_BLOCK_BYTES / 4) + put;
 #pragma unroll
-                    for (int c = 0; c < NCH; ++c) {
-                        const uint8_t* sub = sblock + ((col_base >> 5) + c) * S_SUB_BYTES;
+                        for (int g = 0; g < 8; ++g)
 #pragma unroll
-                        for (int g = 0; g < 8; ++g) {
-                            const float4 f = *reinterpret_cast<const float4*>(sub + swz128_offset(r, g));
-                            sreg[c][4 * g] = __float_as_uint(f.x); sreg[c][4 * g + 1] = __float_as_uint(f.y);
-                            sreg[c][4 * g + 2] = __float_as_uint(f.z); sreg[c][4 * g + 3] = __float_as_uint(f.w);
-                        }
+                            for (int e = 0; e < 4; ++e) {       // e: column parity, row A / B
+                                const int off = (g >> 1) * 1024 + (g & 1) * 512 + (e >> 1) * 64 + (e & 1) * 8;
+                                dst[off] = __uint_as_float(s0[4 * g + e]);
+                                dst[off + 4096] = __uint_as_float(s1[4 * g + e]);
+                            }
+                        __syncwarp();
+                        if (lane == 0) st_release_cta(&stored[wq], ++nstored);
                     }
                 } else {
-                    const uint8_t* sub = sblock + q * S_SUB_BYTES + (lane & 3) * 4;   // rows of the mirror block = my columns
+                    // ---- a block computed by the CTA of tile j, read transposed
 #pragma unroll
-                    for (int c = 0; c < NCH; ++c)
+                    for (int half = 0; half < 2; ++half, ++mc) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&bars.m_full[mc % MST], (mc / MST) & 1, abortp));
+                        if (!ok) break;
+                        const float* src = reinterpret_cast<const float*>(sM + (mc % MST) * S_HALF_BYTES) + get;
+                        uint32_t (&s)[32] = half ? s1 : s0;
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            sreg[c][i] = *reinterpret_cast<const uint32_t*>(sub + swz128_offset(col_base + 32 * c + i, lane >> 2));
+                        for (int g = 0; g < 8; ++g) {
+                            const uint2 a = *reinterpret_cast<const uint2*>(src + 64 * g);
+                            const uint2 bb = *reinterpret_cast<const uint2*>(src + 512 + 64 * g);
+                            s[4 * g] = a.x; s[4 * g + 1] = a.y; s[4 * g + 2] = bb.x; s[4 * g + 3] = bb.y;
+                        }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&bars.m_empty[mc % MST]);
+                    }
+                    if (!ok) break;
                 }
+                // ---- keys beyond the sequence (ragged last block) carry no weight
+                const int nvalid = n - j * TILE;
+                if (nvalid < TILE) {
+                    mask_quad64(s0, cq, nvalid - 1, nvalid - 1);
+                    mask_quad64(s1, 64 + cq, nvalid - 1, nvalid - 1);
+                }
+                float bA = -INFINITY, bB = -INFINITY;
+                max_quad64(s0, bA, bB);
+                max_quad64(s1, bA, bB);
+                bA = quad_max(bA) * sl2;
+                bB = quad_max(bB) * sl2;
+                float alphaA = 1.f, alphaB = 1.f;
+                if (bA > mA + RESCALE_THRESHOLD) {   // also taken on the first block (m = -inf)
+                    alphaA = ex2_mufu(mA - bA);
+                    mA = bA;
+                }
+                if (bB > mB + RESCALE_THRESHOLD) {
+                    alphaB = ex2_mufu(mB - bB);
+                    mB = bB;
+                }
+                // ---- P = exp2(S*sl2 - m) as bf16; its buffer is free behind the PV before the previous one
+                const uint32_t tP = tmem + Cfg::TMEM_P + (blk & 1) * 64 + lane_off;
+                float sumA = 0.f, sumB = 0.f;
+                uint32_t pk[16];
+                exp_quad64(s0, sl2, -mA, -mB, pk, sumA, sumB);
+                if (blk >= 2) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bars.o_done[blk & 1], ((blk >> 1) - 1) & 1, abortp));
+                    if (!ok) break;
+                    tc_fence_after();
+                }
+                tmem_st_quad32(tP, pk);
+                exp_quad64(s1, sl2, -mA, -mB, pk, sumA, sumB);
+                tmem_st_quad32(tP + 32, pk);
+                lA = fmaf(lA, alphaA, sumA);
+                lB = fmaf(lB, alphaB, sumB);
+                if (j > 0 && __any_sync(0xffffffffu, alphaA != 1.f || alphaB != 1.f)) {   // rare: a row maximum grew by > 2^8
+                    const int nA = __popc(__ballot_sync(0xffffffffu, (lane & 3) == 0 && alphaA != 1.f));
+                    const int nB = __popc(__ballot_sync(0xffffffffu, (lane & 3) == 0 && alphaB != 1.f));
+                    if (lane == 0) atomicAdd(&dc->rescales, (unsigned long long)(nA + nB));
+                    // O is at rest once the PV before this block's has committed
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bars.o_done[(blk - 1) & 1], ((blk - 1) >> 1) & 1, abortp));
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int c = 0; c < D / 64; ++c) {
+                        uint32_t v[32];
+                        tmem_ld_quad64(tO + 64 * c, v);
+                        tc_wait_ld();
 #pragma unroll
-                for (int c = 0; c < NCH; ++c)
-                    mx = ragged ? max_chunk32<true>(sreg[c], col_base + 32 * c, cb, mx)
-                                : max_chunk32<false>(sreg[c], col_base + 32 * c, r, mx);
+                        for (int g = 0; g < 8; ++g) {
+                            v[4 * g] = __float_as_uint(__uint_as_float(v[4 * g]) * alphaA);
+                            v[4 * g + 1] = __float_as_uint(__uint_as_float(v[4 * g + 1]) * alphaA);
+                            v[4 * g + 2] = __float_as_uint(__uint_as_float(v[4 * g + 2]) * alphaB);
+                            v[4 * g + 3] = __float_as_uint(__uint_as_float(v[4 * g + 3]) * alphaB);
+                        }
+                        tmem_st_quad64(tO + 64 * c, v);
+                    }
+                }
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars.p_ready[blk & 1]);
             }
-            // the scores are in registers: the stage may take block j + 2
-            mbar_arrive(&bars.s_free[j & 1]);
-            // the two threads of a row exchange their half-row maxima (and leave together if either gave up a wait)
-            xch_max[j & 1][part][r] = mx;
-            ok = named_bar_all(ok, pair_bar, 64);
             if (!ok) break;
-            mx = fmaxf(mx, xch_max[j & 1][part ^ 1][r]);
-            const float mx2 = mx * sl2;
-            float alpha = 1.f;
-            if (mx2 > m_run + RESCALE_THRESHOLD) {   // also taken on the first block (m_run = -inf)
-                alpha = ex2_mufu(m_run - mx2);
-                m_run = mx2;
-            }
-            // P and O are still in use by PV_{j-1} until its commit.  A wait given up here is not acted on
-            // before the next pair barrier, so that the two threads of a row stay together.
-            if (j > 0) {
-                ok = mbar_wait(&bars.o_done[0], (j - 1) & 1, abortp);
-                ok = __all_sync(0xffffffffu, ok);
-                tc_fence_after();
-            }
-            // ---- P = exp2(S * log2 e - m) as bf16 into TMEM
-            float rowsum = 0.f;
-            if (ok) {
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    uint32_t pk[16];
-                    const int kc = col_base + 32 * c;            // first key column of the chunk
-                    rowsum += ragged ? exp_chunk32<true>(sreg[c], sl2, -m_run, kc, cb, pk)
-                                     : exp_chunk32<false>(sreg[c], sl2, -m_run, kc, r, pk);
-                    tmem_st16(tP + (kc >> 1), pk);
-                }
-            }
-            l_run = fmaf(l_run, alpha, rowsum);
-            if (ok && j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {   // rare: a row maximum grew by > 2^8
-                const unsigned grown = __ballot_sync(0xffffffffu, alpha != 1.f);
-                if (part == 0 && lane == 0) atomicAdd(&dc->rescales, (unsigned long long)__popc(grown));
-#pragma unroll
-                for (int c = 0; c < OPT / 32; ++c) {
-                    uint32_t v[32];
-                    tmem_ld32(tO + 32 * c, v);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
-                    tmem_st32(tO + 32 * c, v);
-                }
-            }
-            tc_wait_st();
-            tc_fence_before();
-            mbar_arrive(&bars.p_ready[0]);
-        }
-        if (ok) ok = mbar_wait(&bars.o_done[0], (T - 1) & 1, abortp);
-        xch_sum[part][r] = l_run;
-        if (named_bar_all(ok, tile_bar, 32 * SOFTMAX_WARPS_PER_TILE)) {
-            // ---- epilogue: y = O / l (the division of Eq. 2, applied once per output row); the first score stage,
-            // which no copy targets any more, stages the bf16 tile for the TMA store
+            ok = __all_sync(0xffffffffu, mbar_wait(&bars.o_done[(blk - 1) & 1], ((blk - 1) >> 1) & 1, abortp));
+            if (!ok) break;
+            // ---- epilogue: y = O / l (the division of Eq. 2, applied once per output row), bf16, 64 columns at a time.  (The
+            // next write to O, PV_0 of the next item, waits for that item's first P from every warp.)
             tc_fence_after();
-            const float inv = 1.f / (l_run + xch_sum[part ^ 1][r]);
-            uint8_t* stage = sS;
+            const int bh = bh0 + hl, b = bh / H, h = bh - b * H;
+            const float invA = 1.f / quad_sum(lA), invB = 1.f / quad_sum(lB);
 #pragma unroll
-            for (int c = 0; c < OPT / 32; ++c) {
-                const int col = part * OPT + 32 * c;       // first of 32 output columns handled here
+            for (int u = 0; u < Cfg::SUB; ++u) {
                 uint32_t v[32];
-                tmem_ld32(tO + 32 * c, v);
+                tmem_ld_quad64(tO + 64 * u, v);
                 tc_wait_ld();
-                uint8_t* sub = stage + (col / 64) * 16384;
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    uint4 o;
-                    o.x = pack_bf16x2(__uint_as_float(v[g * 8 + 0]) * inv, __uint_as_float(v[g * 8 + 1]) * inv);
-                    o.y = pack_bf16x2(__uint_as_float(v[g * 8 + 2]) * inv, __uint_as_float(v[g * 8 + 3]) * inv);
-                    o.z = pack_bf16x2(__uint_as_float(v[g * 8 + 4]) * inv, __uint_as_float(v[g * 8 + 5]) * inv);
-                    o.w = pack_bf16x2(__uint_as_float(v[g * 8 + 6]) * inv, __uint_as_float(v[g * 8 + 7]) * inv);
-                    *reinterpret_cast<uint4*>(sub + swz128_offset(r, (col % 64) / 8 + g)) = o;
+                if (store_pending) {        // the store that last used the buffer must have read it
+                    if (lane == 0) tma_store_wait_read();
+                    __syncwarp();
                 }
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    const uint32_t a = pack_bf16x2(__uint_as_float(v[4 * g]) * invA, __uint_as_float(v[4 * g + 1]) * invA);
+                    const uint32_t bb = pack_bf16x2(__uint_as_float(v[4 * g + 2]) * invB, __uint_as_float(v[4 * g + 3]) * invB);
+                    *reinterpret_cast<uint32_t*>(stage + swz128_offset(lane >> 2, g) + 2 * cq) = a;
+                    *reinterpret_cast<uint32_t*>(stage + swz128_offset((lane >> 2) + 8, g) + 2 * cq) = bb;
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_4d(&maps.o, stage, 64 * u, h, It * TILE + row0, b);
+                    tma_store_commit();
+                }
+                store_pending = true;
             }
-            fence_async_smem();
-            named_bar_sync(tile_bar, 32 * SOFTMAX_WARPS_PER_TILE);
-            if (sw == 0 && lane == 0) {
-                for (int u = 0; u < Cfg::SUB; ++u)
-                    tma_store_4d(&maps.o, stage + u * 16384, 64 * u, h, It * TILE, b);
-                tma_store_commit();
-                tma_store_wait_read();   // smem may be released; the writes complete on their own
-            }
+            tc_fence_before();
         }
+        if (store_pending && lane == 0) tma_store_wait_read();   // shared memory may be released; the writes complete on their own
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) atomicExch(&dc->status, (int)PSA_ERR_TIMEOUT);
-    if (warp == 1) tmem_dealloc(tmem, 256);
+    if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
 // Heads per pass: as many as the scratch cap allows, in passes of equal size (the scratch is reused from pass
@@ -422,30 +509,32 @@ int sym_heads_per_pass(int B, int H, int n) {
     return (int)((all + passes - 1) / passes);
 }
 
-// D: head size the kernels work with (64 or 128); d <= D: the tensors' head size (see the 4-D tensor maps).
+// D: head size the kernel works with (64 or 128); d <= D: the tensors' head size (see the 4-D tensor maps).
 template <int D>
 int launch_symmetric(const void* X, void* out, float* S, int B, int H, int n, int d, float scale, DeviceCounters* dc,
                      cudaStream_t stream) {
     using Cfg = SymCfg<D>;
     static DeviceSetup setup;
-    if (device_setup(&setup, [] {
-            cudaError_t e = cudaFuncSetAttribute(sym_attn_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SymCfg<D>::SMEM);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(sym_scores_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SymCfg<D>::SCORES_SMEM);
-            return e;
-        }, "cudaFuncSetAttribute(symmetric attention)") <= 0)
-        return PSA_ERR_CUDA;
-    const int T = row_tiles(n), np = sym_pairs(T);
+    const int sm_count = device_setup(&setup, [] {
+        return cudaFuncSetAttribute(sym_attn_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SymCfg<D>::SMEM);
+    }, "cudaFuncSetAttribute(symmetric attention)");
+    if (sm_count <= 0) return PSA_ERR_CUDA;
+    const int T = row_tiles(n);
+    const size_t head_bytes = (size_t)sym_pairs(T) * S_BLOCK_BYTES;
     const int hp = sym_heads_per_pass(B, H, n);
     SymMaps maps;
-    if (!make_tensor_map_bf16_4d(&maps.x, X, B, n, H, d, 128) || !make_tensor_map_bf16_4d(&maps.o, out, B, n, H, d, 128))
+    if (!make_tensor_map_bf16_4d(&maps.x, X, B, n, H, d, 128) || !make_tensor_map_bf16_4d(&maps.o, out, B, n, H, d, 16))
         return PSA_ERR_CUDA;
     for (int bh0 = 0; bh0 < B * H; bh0 += hp) {
         const int heads = min(hp, B * H - bh0);
-        sym_scores_kernel<D><<<heads * np, 128, Cfg::SCORES_SMEM, stream>>>(maps, S, n, H, bh0, scale, dc);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) { set_cuda_error(e, "sym_scores_kernel launch"); return PSA_ERR_CUDA; }
-        sym_attn_kernel<D><<<heads * T, SYM_THREADS, Cfg::SMEM, stream>>>(maps, S, n, H, bh0, dc);
+        if ((long long)heads * T > 0x7fffffffLL - 2 * sm_count) return PSA_ERR_SHAPE;      // (the work counter runs past the list)
+        const int nitems = heads * T;
+        // flags of every head and the work counter (the diagonal block whose place they take has room for 16384)
+        const size_t flag_bytes = (size_t)(T + 1) * sizeof(int);
+        cudaError_t e = heads == 1 ? cudaMemsetAsync(S, 0, flag_bytes, stream)
+                                   : cudaMemset2DAsync(S, head_bytes, 0, flag_bytes, heads, stream);
+        if (e != cudaSuccess) { set_cuda_error(e, "symmetric scheme: clearing the flags"); return PSA_ERR_CUDA; }
+        sym_attn_kernel<D><<<min(nitems, sm_count), SYM_THREADS, Cfg::SMEM, stream>>>(maps, S, n, H, bh0, nitems, scale * LOG2E, dc);
         e = cudaGetLastError();
         if (e != cudaSuccess) { set_cuda_error(e, "sym_attn_kernel launch"); return PSA_ERR_CUDA; }
     }
