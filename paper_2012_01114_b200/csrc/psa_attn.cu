@@ -9,9 +9,9 @@
 // head run in step: block (J, I) is finished at step I of tile J and needed at step J of tile I, usually
 // while it is still in L2.
 //
-// A work item is a row tile of one head.  Items are numbered with the last tile of a head first and taken
-// from a device counter in that order, so an item only ever waits for items that were taken before it: the
-// oldest unfinished item waits for nobody.
+// A work item is a row tile of one head.  Items are numbered group of heads by group of heads, inside a group
+// the last tiles of all its heads first, and taken from a device counter in that order, so an item only ever
+// waits for items that were taken before it: the oldest unfinished item waits for nobody.
 //
 // Roles of a CTA (352 threads): warp 0 takes items and loads operand tiles and handed-on blocks, warp 1 issues
 // the MMAs, warps 2-9 do the softmax and the output (a warp owns 16 rows, quad layout of sm100.cuh), warp 10
@@ -22,7 +22,9 @@
 //
 // What bounds it: softmax (1024 cycles of exponentials per block) and, in step with it, the operands of one row
 // tile per SM: 32 KB of X per block, 64 KB of scores stored or loaded for all but the diagonal one.  Measured
-// (L2 flushed, B = 64, H = 16, n = 1024, d_k = 128): @@MEASURED@@
+// (L2 flushed, B = 64, H = 16, n = 1024, d_k = 128): 1430 us as two kernels through 36 blocks written and 64 read
+// per head, 955 us as one with 28 and 28.  An SM spends 4000 cycles per block; clock stamps of a softmax warp put
+// 950 of them in the exponentials, 550 in the stores of computed blocks, 1000 in waits for handed-on ones.
 //
 // The fused persistent kernel of the FULL and MASKED schemes is in psa_attn_persist.cu.
 #include "psa_internal.h"
@@ -46,7 +48,7 @@ template <int D>
 struct SymCfg {
     static constexpr int SUB = D / 64;                  // 64-column sub-tiles per 128-row tile of X
     static constexpr int TILE_BYTES = 128 * D * 2;      // one X tile (bf16)
-    static constexpr int XST = D == 128 ? 3 : 4;        // X tiles in flight: PV of a block, S of the next, one loading
+    static constexpr int XST = D == 128 ? 3 : 4;        // X tiles in flight: PV of a block, S of the next, one loading (2: 5 % slower)
     static constexpr int MST = D == 128 ? 2 : 4;        // half blocks of handed-on scores in flight
     static constexpr int STAGE_BYTES = 16 * 64 * 2;     // a softmax warp's output staging buffer
     static constexpr int SMEM = (1 + XST) * TILE_BYTES + MST * S_HALF_BYTES + SYM_WARPS * STAGE_BYTES + 1024;
@@ -98,7 +100,7 @@ __device__ __forceinline__ bool wait_at_least(Read read, int target, volatile in
 
 template <int D>
 __global__ void __launch_bounds__(SYM_THREADS, 1)
-sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, int n, int H, int bh0, int nitems, float sl2,
+sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, int n, int H, int bh0, int heads, int group, float sl2,
                 DeviceCounters* dc) {
     using Cfg = SymCfg<D>;
     constexpr int XST = Cfg::XST, MST = Cfg::MST;
@@ -117,10 +119,15 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int T = row_tiles(n);
     const int np = sym_pairs(T);
+    const int nitems = heads * T;
     int* work_counter = reinterpret_cast<int*>(Sg) + T;
-    // item -> head inside this pass and row tile, the last tile of a head first
-    auto item_head = [&](int idx) { return idx / T; };
-    auto item_tile = [&](int idx, int hl) { return T - 1 - (idx - hl * T); };
+    // item -> head inside this pass and row tile: groups of heads, in a group the last tiles of all heads first
+    auto item_work = [&](int idx, int& hl, int& It) {
+        const int g = idx / (group * T), first = g * group, size = min(group, heads - first);
+        const int off = idx - first * T, r = off / size;
+        hl = first + off - r * size;
+        It = T - 1 - r;
+    };
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -161,7 +168,8 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                 item_ring[slot] = idx < nitems ? idx : -1;
                 mbar_arrive(&bars.item_full[slot]);
                 if (idx >= nitems) break;
-                const int hl = item_head(idx), It = item_tile(idx, hl);
+                int hl, It;
+                item_work(idx, hl, It);
                 const int bh = bh0 + hl, b = bh / H, h = bh - b * H;
                 float* head = sym_head(Sg, hl, np);
                 const int* flags = reinterpret_cast<const int*>(head);
@@ -180,8 +188,9 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                         mbar_arrive_expect_tx(&bars.q_full, Cfg::TILE_BYTES);
                         for (int u = 0; u < Cfg::SUB; ++u) tma_load_4d(sQ + u * 16384, &maps.x, &bars.q_full, 64 * u, h, It * TILE, b);
                         ++qc;
-                        next = atomicAdd(work_counter, 1);       // (behind the item's first loads)
                     }
+                    // the next item, as late as its answer's way allows: items then start in the order of their numbers
+                    if (j == max(T - 3, 0)) next = atomicAdd(work_counter, 1);
                     if (j <= It) continue;
                     // block (j, It), handed on by the CTA that works on tile j: present once its flag counts past It.  The
                     // stores behind the flag were ordinary ones, the copies below go through the asynchronous proxy.
@@ -212,7 +221,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
         if (lane == 0) {
             // ------------------------------------------------------------ MMA issuer
             // Per item S_0 .. S_It (phase 1, Eq. 1) and PV_0 .. PV_{T-1} (phase 3, Eq. 3), each S one block ahead of its PV;
-            // the first S of the next item goes ahead of the last PV of this one.
+            // the first S of the next item runs under the output of this one.
             const uint32_t idescS = umma_idesc_bf16(128, 128, UMMA_K_MAJOR, UMMA_K_MAJOR);
             const uint32_t idescO = umma_idesc_bf16(128, D, UMMA_K_MAJOR, UMMA_MN_MAJOR);
             const uint32_t q_lo = umma_desc_lo_kmajor(smem_u32(sQ)), k_lo = umma_desc_lo_kmajor(smem_u32(sX));
@@ -243,21 +252,13 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                 return true;
             };
             int idx = take();
-            int It = idx >= 0 ? item_tile(idx, item_head(idx)) : 0;
+            int hl, It = 0;
+            if (idx >= 0) item_work(idx, hl, It);
             if (idx >= 0) ok = issue_S(0, true, It == 0);
             while (idx >= 0 && ok) {
                 int idx_next = -1, It_next = 0;
                 for (int j = 0; j < T; ++j) {
-                    if (j < It) {
-                        ok = issue_S(xbase + j + 1, false, j + 1 == It);
-                    } else if (j == T - 1) {
-                        idx_next = take();
-                        if (idx_next == -2) ok = false;
-                        if (idx_next >= 0) {
-                            It_next = item_tile(idx_next, item_head(idx_next));
-                            ok = issue_S(xbase + T, true, It_next == 0);
-                        }
-                    }
+                    if (j < It) ok = issue_S(xbase + j + 1, false, j + 1 == It);
                     const uint32_t xpos = xbase + j;
                     if (ok && j > It) ok = mbar_wait(&bars.x_full[xpos % XST], (xpos / XST) & 1, abortp);
                     if (ok) ok = mbar_wait(&bars.p_ready[pc & 1], (pc >> 1) & 1, abortp);
@@ -271,6 +272,13 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                     umma_commit(&bars.o_done[pc & 1]);
                     umma_commit(&bars.x_empty[xpos % XST]);
                     ++pc;
+                }
+                if (!ok) break;
+                idx_next = take();
+                if (idx_next == -2) break;
+                if (idx_next >= 0) {
+                    item_work(idx_next, hl, It_next);
+                    ok = issue_S(xbase + T, true, It_next == 0);
                 }
                 xbase += T;
                 idx = idx_next;
@@ -294,7 +302,8 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.item_empty[it & 1]);
             if (idx < 0) break;
-            const int hl = item_head(idx), It = item_tile(idx, hl);
+            int hl, It;
+                item_work(idx, hl, It);
             int* flag = reinterpret_cast<int*>(sym_head(Sg, hl, np)) + It;
             int sent = 0;
             bool ok = true;
@@ -323,12 +332,12 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
         const uint32_t lane_off = static_cast<uint32_t>(row0) << 16;
         const uint32_t tO = tmem + Cfg::TMEM_O + lane_off;
         uint8_t* stage = sStage + wq * Cfg::STAGE_BYTES;
-        // Place of a score in a handed-on block, in floats.  The block is laid out for the threads that read it transposed:
-        // element (r, c) of the writer is row c, key r of the reader, and the reader's fragments (sm100.cuh) are stored as
-        // [key half][16-row group][row A / B][key group of 8][lane][2 keys].  For a writer thread everything but the
-        // constants below is a compile-time offset, and a warp's store fills whole 32-byte sectors.
-        const int put = (kw >> 2) * 8192 + 2 * (kw & 3) * 64 + (4 * cq + (lane >> 3)) * 2 + ((lane >> 2) & 1);
-        const int get = kw * 1024 + lane * 2;
+        // Place of a score in a handed-on block, in floats: [16-row group of the writer][column half][group of 8 columns]
+        // [chunk][column parity][row A / B].  A writer thread stores its four scores of a column group as one 16-byte chunk;
+        // element (r, c) is row c, key r of the reader, which takes keys r and r + 8 as 8 bytes.  Chunk numbers are permuted
+        // (bits of r: 2-1, bits of c: 2-1, bit 0 of r, from the lowest up) so that a half-warp reads 8 different ones.
+        const int put = kw * 2048 + 4 * ((lane >> 3) | ((lane & 3) << 2) | (((lane >> 2) & 1) << 4));
+        const int get = (kw >> 2) * 1024 + (kw & 3) * 256 + 4 * ((lane & 3) | ((lane >> 3) << 2)) + 2 * ((lane >> 2) & 1);
         uint32_t blk = 0, sc = 0, mc = 0;                       // blocks, computed blocks and half blocks so far, all items
         int nstored = 0;
         bool store_pending = false;                             // a TMA store of this warp may still be reading `stage`
@@ -340,7 +349,8 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.item_empty[it & 1]);
             if (idx < 0) break;
-            const int hl = item_head(idx), It = item_tile(idx, hl);
+            int hl, It;
+                item_work(idx, hl, It);
             float* own = sym_head(Sg, hl, np) + (size_t)(It * (It + 1) / 2) * (S_BLOCK_BYTES / 4);
             float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;       // running maxima (log2 units) and row sums
             for (int j = 0; j < T; ++j, ++blk) {
@@ -361,13 +371,10 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                     if (j < It) {                               // the mirror block's tile needs it
                         float* dst = own + (size_t)j * (S_BLOCK_BYTES / 4) + put;
 #pragma unroll
-                        for (int g = 0; g < 8; ++g)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {       // e: column parity, row A / B
-                                const int off = (g >> 1) * 1024 + (g & 1) * 512 + (e >> 1) * 64 + (e & 1) * 8;
-                                dst[off] = __uint_as_float(s0[4 * g + e]);
-                                dst[off + 4096] = __uint_as_float(s1[4 * g + e]);
-                            }
+                        for (int g = 0; g < 8; ++g) {
+                            *reinterpret_cast<uint4*>(dst + 128 * g) = make_uint4(s0[4 * g], s0[4 * g + 2], s0[4 * g + 1], s0[4 * g + 3]);
+                            *reinterpret_cast<uint4*>(dst + 1024 + 128 * g) = make_uint4(s1[4 * g], s1[4 * g + 2], s1[4 * g + 1], s1[4 * g + 3]);
+                        }
                         __syncwarp();
                         if (lane == 0) st_release_cta(&stored[wq], ++nstored);
                     }
@@ -380,11 +387,13 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                         const float* src = reinterpret_cast<const float*>(sM + (mc % MST) * S_HALF_BYTES) + get;
                         uint32_t (&s)[32] = half ? s1 : s0;
 #pragma unroll
-                        for (int g = 0; g < 8; ++g) {
-                            const uint2 a = *reinterpret_cast<const uint2*>(src + 64 * g);
-                            const uint2 bb = *reinterpret_cast<const uint2*>(src + 512 + 64 * g);
-                            s[4 * g] = a.x; s[4 * g + 1] = a.y; s[4 * g + 2] = bb.x; s[4 * g + 3] = bb.y;
-                        }
+                        for (int g = 0; g < 4; ++g)             // keys 16 g .. 16 g + 15 of the half, row A / B, key parity
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const uint2 v = *reinterpret_cast<const uint2*>(src + 2048 * g + 128 * (e >> 1) + 64 * (e & 1));
+                                s[8 * g + e] = v.x;
+                                s[8 * g + 4 + e] = v.y;
+                            }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars.m_empty[mc % MST]);
                     }
@@ -509,6 +518,13 @@ int sym_heads_per_pass(int B, int H, int n) {
     return (int)((all + passes - 1) / passes);
 }
 
+// Heads per group of the item list: the tiles of one head are started a group apart.  A tile needs its first handed-on block
+// one step after its neighbour has computed it, so tiles that start together wait for one another; started 256 / T items
+// apart (two steps, on 148 CTAs) they do not, and a head's scratch still lives briefly enough to stay in L2.  Measured for
+// 64 / 128 / 256 / 512 / 1024 items (us; n = 256, 1024, 4096 at d_k = 128): 106 99 89 87 87, 279 270 249 252 258, 948 949 937
+// 959 961.
+constexpr int SYM_GROUP_ITEMS = 256;
+
 // D: head size the kernel works with (64 or 128); d <= D: the tensors' head size (see the 4-D tensor maps).
 template <int D>
 int launch_symmetric(const void* X, void* out, float* S, int B, int H, int n, int d, float scale, DeviceCounters* dc,
@@ -534,7 +550,7 @@ int launch_symmetric(const void* X, void* out, float* S, int B, int H, int n, in
         cudaError_t e = heads == 1 ? cudaMemsetAsync(S, 0, flag_bytes, stream)
                                    : cudaMemset2DAsync(S, head_bytes, 0, flag_bytes, heads, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "symmetric scheme: clearing the flags"); return PSA_ERR_CUDA; }
-        sym_attn_kernel<D><<<min(nitems, sm_count), SYM_THREADS, Cfg::SMEM, stream>>>(maps, S, n, H, bh0, nitems, scale * LOG2E, dc);
+        sym_attn_kernel<D><<<min(nitems, sm_count), SYM_THREADS, Cfg::SMEM, stream>>>(maps, S, n, H, bh0, heads, min(heads, max(1, SYM_GROUP_ITEMS / T)), scale * LOG2E, dc);
         e = cudaGetLastError();
         if (e != cudaSuccess) { set_cuda_error(e, "sym_attn_kernel launch"); return PSA_ERR_CUDA; }
     }

@@ -161,11 +161,6 @@ __device__ __forceinline__ void bulk_load_1d(void* smem_dst, const void* gmem_sr
                  "l"(reinterpret_cast<uint64_t>(gmem_src)), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-__device__ __forceinline__ void bulk_store_1d(void* gmem_dst, const void* smem_src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(reinterpret_cast<uint64_t>(gmem_dst)),
-                 "r"(smem_u32(smem_src)), "r"(bytes)
-                 : "memory");
-}
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -190,15 +185,9 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 enum : uint32_t { UMMA_K_MAJOR = 0, UMMA_MN_MAJOR = 1 };
 enum : uint32_t { UMMA_SWIZZLE_128B = 2 };
 
-// Shared-memory matrix descriptor: start address, leading / stride byte offsets (16-byte units),
-// descriptor version 1 (sm_100), swizzle mode in the top three bits.
-__device__ __forceinline__ uint64_t umma_smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16) |
-           (static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32) | (1ull << 46) |
-           (static_cast<uint64_t>(UMMA_SWIZZLE_128B) << 61);
-}
-// K-major operand tile [rows x 64] bf16, 128-byte swizzle: 8-row groups are 1024 bytes apart.
-__device__ __forceinline__ uint64_t umma_desc_kmajor(uint32_t saddr) { return umma_smem_desc(saddr, 16, 1024); }
+// Shared-memory matrix descriptor: start address, leading / stride byte offsets (16-byte units), descriptor version 1
+// (sm_100), swizzle mode in the top three bits.  A K-major operand tile is [rows x 64] bf16 with its 8-row groups 1024 bytes
+// apart; an MN-major one has 64-element blocks `mn_block_bytes` apart.
 // Cheap descriptor arithmetic for the MMA-issuing thread.  The thread that issues tcgen05.mma is a
 // single lane; every instruction it spends per MMA delays the tensor pipe (a 128x128x16 MMA runs
 // for 64 cycles).  A descriptor is therefore split into its two 32-bit halves: the high half is a
@@ -261,26 +250,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
-        "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
-        "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
-
 // 16 lanes x 64 consecutive 32-bit columns in the "quad" layout: the calling warp reads lanes L .. L+15 (L = the lane
 // field of taddr, a multiple of 16 inside the warp's quarter); thread t holds, for g = 0 .. 7,
 //     r[4g + 0], r[4g + 1]   lane L + t/4,      columns 8g + 2(t%4), 8g + 2(t%4) + 1

@@ -197,3 +197,21 @@ def test_keys_equal_values(scheme, B, H, n, d):
     # two distinct tensors with the same contents take the two-ring path: bitwise the same result
     out2 = binding.psa_attention_core(q, k, k.clone(), scheme)
     assert torch.equal(out.view(torch.int16), out2.view(torch.int16))
+
+
+# The symmetric kernel hands score blocks from CTA to CTA: one, two and more row tiles per head (one tile hands nothing on),
+# ragged last tiles, more work items than SMs, and a head count that leaves a partial group at the end of the item list
+# (256 / row tiles heads per group).  Run twice: the flags of the first call must not satisfy the second.
+@pytest.mark.parametrize("B,H,n,d", [(10, 30, 100, 64), (11, 14, 200, 128), (9, 10, 300, 64), (3, 11, 1100, 32), (1, 1, 2500, 128)])
+def test_symmetric_blocks_handed_on(B, H, n, d):
+    xv, xb = inputs.tensor(3 * n + d, 4, (B, n, H, d), 1.0, "bf16")
+    ref, _ = oracle.attention_core(xv, xv, xv, oracle.SYMMETRIC)
+    first = None
+    for call in range(2):
+        out = binding.psa_attention_core(_dev_bf16(xb), None, None, binding.SYMMETRIC)
+        st, got = binding.psa_last_issued()
+        assert st == binding.OK and got == binding.psa_skip_count(B, H, n, 0, d, binding.SYMMETRIC, binding.BF16)
+        # outputs reach 4 and more (a row's own key dominates): half a bf16 step of the output itself on top
+        assert (np.abs(_to_f64(out).reshape(ref.shape) - ref) <= TOL_BF16 + 2.0 ** -8 * np.abs(ref)).all()
+        assert first is None or torch.equal(first.view(torch.int16), out.view(torch.int16))
+        first = out
