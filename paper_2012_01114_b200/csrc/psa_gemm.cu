@@ -2,12 +2,18 @@
 //     C_w[M, N] = A[M, K] * B_w[K, N] (+ R[M, N]),  w < nW,  bf16 row-major operands, fp32 accumulation in TMEM;
 // the optional residual R is added in the epilogue (the output projection of the attention block).
 //
-// Persistent kernel, one CTA per SM, walking 128 x 256 output tiles (all three weight matrices in one
-// launch).  Warp 0 streams operand tiles with TMA into a shared-memory ring, warp 1 issues tcgen05 MMAs
-// (A K-major, B in its natural row-major form = MN-major) into one of two 256-column TMEM accumulators,
-// warps 2-5 drain the other accumulator (TMEM -> registers -> bf16 -> swizzled shared memory -> TMA
-// store, 64 columns at a time through two staging buffers so that the stores overlap the conversion),
-// so that a tile's epilogue runs under the next tile's main loop.
+// Persistent kernel over output tiles of 128 CTAS rows by BN columns (all weight matrices in one launch).  CTAS = 2: a
+// cluster of two CTAs works on one tile with cta_group::2 MMAs; each CTA holds 128 rows of A and of the accumulator and
+// one half of the B columns.  Per CTA, warp 0 streams operand tiles with TMA into a shared-memory ring, warp 1 (of the
+// first CTA) issues the MMAs (A K-major, B in its natural row-major form = MN-major) into one of two accumulators in
+// TMEM, the other warps drain the other accumulator: a warp takes 32 rows by 64 columns at a time (TMEM -> registers ->
+// bf16 -> a swizzled buffer of its own -> TMA store), so that no warp waits for another and a tile's epilogue runs under
+// the next tile's main loop.
+//
+// What bounds it: a CTA of its own needs 48 KB of operands per 64-deep k-step for a 128 x 256 tile and an SM takes about 64
+// bytes per cycle from L2: 740 cycles measured for 512 cycles of MMA (1.56 PFLOP/s over the chip).  A pair shares B, 32 KB per
+// CTA and k-step, and takes 650 (1.79 PFLOP/s); M = 8192, N = 3 x 768: K = 3072 84.7 us with lone CTAs, 78.2 with pairs.  About
+// 12 us do not scale with K: launch, first operands from DRAM, last epilogue.
 #include <stdio.h>
 
 #include <mutex>
@@ -81,20 +87,22 @@ bool make_tensor_map_bf16_4d(CUtensorMap* map, const void* base, uint64_t batch,
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int NSUB = BN / 64;                  // 64-column sub-tiles of B and C per tile
-#ifndef PSA_GEMM_STAGES
-#define PSA_GEMM_STAGES 4
-#endif
-constexpr int STAGES = PSA_GEMM_STAGES;
+constexpr int BM = 128, BK = 64;               // rows of a CTA, depth of a k-step
 constexpr int A_BYTES = BM * BK * 2;           // 16 KB, K-major [128 x 64]
 constexpr int B_SUB_BYTES = BK * 64 * 2;       // 8 KB, one [64 k-rows x 64 n] sub-tile
-constexpr int B_BYTES = NSUB * B_SUB_BYTES;    // 32 KB
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES; // 48 KB
-constexpr int OUT_BYTES = 2 * BM * 64 * 2;      // 32 KB output staging: two swizzled [128 x 64] sub-tiles used in turn
-constexpr int GEMM_THREADS = 192;
-constexpr int GEMM_SMEM = STAGES * STAGE_BYTES + OUT_BYTES + 1024;  // + slack for 1024-byte alignment
-constexpr int TMEM_COLS = 2 * BN;              // two accumulators
+constexpr int C_BUF_BYTES = 32 * 64 * 2;       // one staging buffer: 32 rows x 64 columns, bf16
+
+template <int CTAS, int BN>
+struct GCfg {
+    static constexpr int NSUB = BN / 64;                       // 64-column sub-tiles of C per tile
+    static constexpr int BSUB = NSUB / CTAS;                   // 64-column sub-tiles of B that a CTA loads
+    static constexpr int STAGE_BYTES = A_BYTES + BSUB * B_SUB_BYTES;
+    static constexpr int EPI_WARPS = 4;                        // (eight: 0.8 us more per launch, nothing gained)
+    static constexpr int STAGES = 192 * 1024 / STAGE_BYTES;
+    static constexpr int THREADS = 64 + 32 * EPI_WARPS;
+    static constexpr int SMEM = STAGES * STAGE_BYTES + EPI_WARPS * 2 * C_BUF_BYTES + 1024;     // + slack for 1024-byte alignment
+    static constexpr int TMEM_COLS = 2 * BN;                   // two accumulators
+};
 
 struct GemmMaps {
     CUtensorMap a;
@@ -107,18 +115,21 @@ struct TileCoord {
 };
 // Tile t of the launch: column tiles fastest, then row tiles, then the weight matrix, so that CTAs
 // working side by side share the A row panel in L2.
-__device__ __forceinline__ TileCoord tile_coord(int t, int mt, int nt) {
+__device__ __forceinline__ TileCoord tile_coord(int t, int mt, int nt, int bm, int bn) {
     TileCoord c;
-    c.n0 = (t % nt) * BN;
+    c.n0 = (t % nt) * bn;
     const int r = t / nt;
-    c.m0 = (r % mt) * BM;
+    c.m0 = (r % mt) * bm;
     c.w = r / mt;
     return c;
 }
 
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+template <int CTAS, int BN>
+__global__ void __launch_bounds__(GCfg<CTAS, BN>::THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int nW, const uint16_t* __restrict__ R,
                  DeviceCounters* dc) {
+    using Cfg = GCfg<CTAS, BN>;
+    constexpr int STAGES = Cfg::STAGES, STAGE_BYTES = Cfg::STAGE_BYTES, NSUB = Cfg::NSUB;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* stage_out = smem + STAGES * STAGE_BYTES;
@@ -127,19 +138,27 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = CTAS == 2 ? (int)cluster_ctarank() : 0;   // the first CTA of a pair issues its MMAs
+    const int unit = blockIdx.x / CTAS, units = gridDim.x / CTAS;
     const int nk = (K + BK - 1) / BK;
-    const int mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
+    const int mt = (M + CTAS * BM - 1) / (CTAS * BM), nt = (N + BN - 1) / BN;
     const int ntiles = mt * nt * nW;
 
+    // full_bar and acc_empty of the first CTA serve the pair; empty_bar and acc_full exist in both and are completed in
+    // both by one commit
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 128); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], CTAS * Cfg::EPI_WARPS); }
         fence_mbar_init();
     }
-    if (warp == 1) { tmem_alloc(&tmem_base_s, TMEM_COLS); tmem_relinquish(); }
+    if (warp == 1) {
+        if constexpr (CTAS == 2) { tmem_alloc_pair(&tmem_base_s, Cfg::TMEM_COLS); tmem_relinquish_pair(); }
+        else { tmem_alloc(&tmem_base_s, Cfg::TMEM_COLS); tmem_relinquish(); }
+    }
     tc_fence_before();
     __syncthreads();
+    if constexpr (CTAS == 2) cluster_sync();       // the partner's barriers are initialised
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
     volatile int* abortp = &abort_flag;
@@ -148,36 +167,48 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
     grid_dependency_wait();
 
     if (warp == 0 && lane == 0) {
-        // ---- TMA producer: k-steps of all this CTA's tiles, numbered g = 0, 1, ... through the ring
+        // ---- TMA producer: k-steps of all this CTA's tiles, numbered g = 0, 1, ... through the ring.  The two CTAs of a pair
+        // fill their halves of a stage on their own; the first CTA's barrier collects the bytes of both.
         int g = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-            const TileCoord c = tile_coord(t, mt, nt);
+        for (int t = unit; t < ntiles && ok; t += units) {
+            const TileCoord c = tile_coord(t, mt, nt, CTAS * BM, BN);
+            const int m0 = c.m0 + rank * BM, n0 = c.n0 + rank * Cfg::BSUB * 64;
             for (int kt = 0; kt < nk; ++kt, ++g) {
                 const int s = g % STAGES;
                 if (g >= STAGES && !mbar_wait(&empty_bar[s], ((g / STAGES) - 1) & 1, abortp)) { ok = false; break; }
                 uint8_t* sA = smem + s * STAGE_BYTES;
                 uint8_t* sB = sA + A_BYTES;
-                mbar_arrive_expect_tx(&full_bar[s], STAGE_BYTES);
-                tma_load_2d(sA, &maps.a, &full_bar[s], kt * BK, c.m0);
+                if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], CTAS * STAGE_BYTES);
+                if constexpr (CTAS == 2) {
+                    const uint32_t bar = cluster_map(&full_bar[s], 0);
+                    tma_load_2d_pair(sA, &maps.a, bar, kt * BK, m0);
 #pragma unroll
-                for (int u = 0; u < NSUB; ++u)
-                    tma_load_2d(sB + u * B_SUB_BYTES, &maps.b[c.w], &full_bar[s], c.n0 + 64 * u, kt * BK);
+                    for (int u = 0; u < Cfg::BSUB; ++u)
+                        tma_load_2d_pair(sB + u * B_SUB_BYTES, &maps.b[c.w], bar, n0 + 64 * u, kt * BK);
+                } else {
+                    tma_load_2d(sA, &maps.a, &full_bar[s], kt * BK, m0);
+#pragma unroll
+                    for (int u = 0; u < Cfg::BSUB; ++u)
+                        tma_load_2d(sB + u * B_SUB_BYTES, &maps.b[c.w], &full_bar[s], n0 + 64 * u, kt * BK);
+                }
             }
         }
-        if (*abortp) {  // let copies already in flight land before the CTA goes away
+        // Let copies already in flight land before the CTA goes away.  (A pair's copies are all seen by the first CTA's
+        // barriers, and neither CTA leaves before the other.)
+        if (*abortp && rank == 0) {
             for (int k = max(0, g - STAGES); k < g; ++k) mbar_wait_drain(&full_bar[k % STAGES], (k / STAGES) & 1);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && lane == 0 && rank == 0) {
         // ---- MMA issuer
-        const uint32_t idesc = umma_idesc_bf16(BM, BN, UMMA_K_MAJOR, UMMA_MN_MAJOR);
+        const uint32_t idesc = umma_idesc_bf16(CTAS * BM, BN, UMMA_K_MAJOR, UMMA_MN_MAJOR);
         // descriptor low words of stage 0; a stage or k-step is a constant added to them (sm100.cuh)
         const uint32_t a_lo0 = umma_desc_lo_kmajor(smem_u32(smem));
         const uint32_t b_lo0 = umma_desc_lo_mnmajor(smem_u32(smem + A_BYTES), B_SUB_BYTES);
         unsigned long long macs = 0;
         int g = 0, i = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
+        for (int t = unit; t < ntiles && ok; t += units, ++i) {
             const int buf = i & 1;
             if (i >= 2) ok = mbar_wait(&acc_empty[buf], ((i >> 1) - 1) & 1, abortp);   // epilogue drained it
             if (!ok) break;
@@ -189,68 +220,87 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a_lo = a_lo0 + s * (STAGE_BYTES >> 4), b_lo = b_lo0 + s * (STAGE_BYTES >> 4);
+                auto mma = [&](int k, uint32_t accumulate) {
+                    const uint64_t a = umma_desc_join(a_lo + k * (32 >> 4), UMMA_DESC_HI_SW128);
+                    const uint64_t b = umma_desc_join(b_lo + k * (2048 >> 4), UMMA_DESC_HI_SW128);
+                    if constexpr (CTAS == 2) umma_ss_pair(acc, a, b, idesc, accumulate);
+                    else umma_ss(acc, a, b, idesc, accumulate);
+                };
                 if (kt == 0) {
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        umma_ss(acc, umma_desc_join(a_lo + k * (32 >> 4), UMMA_DESC_HI_SW128),
-                                umma_desc_join(b_lo + k * (2048 >> 4), UMMA_DESC_HI_SW128), idesc, k != 0);
+                    for (int k = 0; k < BK / 16; ++k) mma(k, k != 0);
                 } else {
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        umma_ss(acc, umma_desc_join(a_lo + k * (32 >> 4), UMMA_DESC_HI_SW128),
-                                umma_desc_join(b_lo + k * (2048 >> 4), UMMA_DESC_HI_SW128), idesc, 1);
+                    for (int k = 0; k < BK / 16; ++k) mma(k, 1);
                 }
-                umma_commit(&empty_bar[s]);
+                if constexpr (CTAS == 2) umma_commit_pair(&empty_bar[s]);
+                else umma_commit(&empty_bar[s]);
             }
             if (!ok) break;
-            umma_commit(&acc_full[buf]);
-            const TileCoord c = tile_coord(t, mt, nt);
-            macs += (unsigned long long)min(BM, M - c.m0) * min(BN, N - c.n0) * K;
+            if constexpr (CTAS == 2) umma_commit_pair(&acc_full[buf]);
+            else umma_commit(&acc_full[buf]);
+            const TileCoord c = tile_coord(t, mt, nt, CTAS * BM, BN);
+            macs += (unsigned long long)min(CTAS * BM, M - c.m0) * min(BN, N - c.n0) * K;
         }
         if (macs) atomicAdd(&dc->proj_macs, macs);
-    }
-    else if (warp >= 2) {
-        // ---- epilogue: 4 warps, warp q owns TMEM lanes 32q .. 32q+31 = output rows
+    } else if (warp >= 2) {
+        // ---- epilogue: warp q owns TMEM lanes 32q .. 32q+31 = output rows
         const int q = warp & 3;
-        const int row = q * 32 + lane;
-        int i = 0;
-        bool ok = true;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
+        uint8_t* buffers = stage_out + (warp - 2) * 2 * C_BUF_BYTES;
+        const uint32_t empty0 = CTAS == 2 ? cluster_map(&acc_empty[0], 0) : 0, empty1 = CTAS == 2 ? cluster_map(&acc_empty[1], 0) : 0;
+        int i = 0, stores = 0;
+        for (int t = unit; t < ntiles; t += units, ++i) {
             const int buf = i & 1;
-            if (ok) ok = mbar_wait(&acc_full[buf], (i >> 1) & 1, abortp);
-            const TileCoord c = tile_coord(t, mt, nt);
-            bool live = true;
+            const TileCoord c = tile_coord(t, mt, nt, CTAS * BM, BN);
+            const int row0 = c.m0 + rank * BM + 32 * q, row = row0 + lane;
+            bool ready = false, ok = true;
 #pragma unroll 1
             for (int u = 0; u < NSUB; ++u) {
-                // The tile leaves in 64-column sub-tiles through two staging buffers used in turn: while the TMA store
-                // of one reads its buffer, the next sub-tile is converted into the other.
-                // This barrier is uniform across the four warps; it also orders the store that last used this buffer
-                // (warp 2 lane 0 waited for it to have read the buffer) before the writes below.
-                if (!named_bar_all(ok, 1, 128)) { live = false; break; }
-                tc_fence_after();
-                uint8_t* sub = stage_out + (u & 1) * 16384;
+                const int col = c.n0 + 64 * u;
+                // residual input: C = A B + R, added in fp32 before the rounding to bf16 (R is [M, N] bf16, row-major);
+                // it is on its way while the tile is still being computed
+                uint4 x[8];
+                const bool res = R && row < M && col < N;
+                if (res) {
+                    const uint4* rp = reinterpret_cast<const uint4*>(R + (size_t)row * N + col);
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) x[g] = __ldg(rp + g);
+                }
+                if (!ready) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (i >> 1) & 1, abortp));
+                    if (!ok) break;
+                    tc_fence_after();
+                    ready = true;
+                }
                 uint32_t r[2][32];
                 const uint32_t src = tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * BN + u * 64;
                 tmem_ld32(src, r[0]);
                 tmem_ld32(src + 32, r[1]);
                 tc_wait_ld();
-                if (R) {
-                    // residual input: C = A B + R, added in fp32 before the rounding to bf16 (R is [M, N] bf16, row-major)
-                    const int grow = c.m0 + row, gcol = c.n0 + 64 * u;
-                    if (grow < M && gcol < N) {
-                        const uint4* rp = reinterpret_cast<const uint4*>(R + (size_t)grow * N + gcol);
+                if (u == NSUB - 1) {                    // the accumulator may be overwritten by tile i + 2
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (CTAS == 2) mbar_arrive_cluster(buf ? empty1 : empty0);
+                        else mbar_arrive(&acc_empty[buf]);
+                    }
+                }
+                if (res) {
 #pragma unroll
-                        for (int g = 0; g < 8; ++g) {
-                            const uint4 x = __ldg(rp + g);
-                            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+                    for (int g = 0; g < 8; ++g) {
+                        const uint32_t w[4] = {x[g].x, x[g].y, x[g].z, x[g].w};
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                uint32_t* dst = &r[g >> 2][(g & 3) * 8 + 2 * e];
-                                dst[0] = __float_as_uint(__uint_as_float(dst[0]) + __uint_as_float(w[e] << 16));
-                                dst[1] = __float_as_uint(__uint_as_float(dst[1]) + __uint_as_float(w[e] & 0xffff0000u));
-                            }
+                        for (int e = 0; e < 4; ++e) {
+                            uint32_t* dst = &r[g >> 2][(g & 3) * 8 + 2 * e];
+                            dst[0] = __float_as_uint(__uint_as_float(dst[0]) + __uint_as_float(w[e] << 16));
+                            dst[1] = __float_as_uint(__uint_as_float(dst[1]) + __uint_as_float(w[e] & 0xffff0000u));
                         }
                     }
+                }
+                uint8_t* sub = buffers + (stores & 1) * C_BUF_BYTES;
+                if (stores >= 2) {                      // the store before the last must have read this buffer
+                    if (lane == 0) tma_store_wait_read_1();
+                    __syncwarp();
                 }
 #pragma unroll
                 for (int c0 = 0; c0 < 2; ++c0) {
@@ -261,30 +311,69 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
                         v.y = pack_bf16x2(__uint_as_float(r[c0][g * 8 + 2]), __uint_as_float(r[c0][g * 8 + 3]));
                         v.z = pack_bf16x2(__uint_as_float(r[c0][g * 8 + 4]), __uint_as_float(r[c0][g * 8 + 5]));
                         v.w = pack_bf16x2(__uint_as_float(r[c0][g * 8 + 6]), __uint_as_float(r[c0][g * 8 + 7]));
-                        *reinterpret_cast<uint4*>(sub + swz128_offset(row, c0 * 4 + g)) = v;
+                        *reinterpret_cast<uint4*>(sub + swz128_offset(lane, c0 * 4 + g)) = v;
                     }
                 }
-                if (u == NSUB - 1) {
-                    tc_fence_before();
-                    mbar_arrive(&acc_empty[buf]);      // the accumulator may be overwritten by tile i + 2
-                }
                 fence_async_smem();
-                named_bar_sync(2, 128);
-                if (warp == 2 && lane == 0) {
-                    const int col = c.n0 + 64 * u;
-                    if (col < N) tma_store_2d(&maps.c[c.w], sub, col, c.m0);
-                    tma_store_commit();                // (an empty group when the sub-tile lies beyond N)
-                    tma_store_wait_read_1();           // the OTHER buffer, stored one sub-tile ago, may be rewritten
+                __syncwarp();
+                if (lane == 0) {
+                    if (col < N && row0 < M) tma_store_2d(&maps.c[c.w], sub, col, row0);
+                    tma_store_commit();                // (an empty group when the sub-tile lies outside the matrix)
                 }
+                ++stores;
             }
-            if (!live) { ok = false; break; }
+            if (!ok) break;
         }
-        if (warp == 2 && lane == 0) tma_store_wait_all();
+        if (lane == 0) tma_store_wait_read();      // shared memory may be released; the writes complete on their own
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) atomicExch(&dc->status, (int)PSA_ERR_TIMEOUT);
-    if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
+    if constexpr (CTAS == 2) {
+        __syncwarp();
+        cluster_sync();                 // MMAs, arrivals and copies that involve the partner are over in both CTAs
+        tc_fence_after();
+        if (warp == 1) tmem_dealloc_pair(tmem, Cfg::TMEM_COLS);
+    } else {
+        if (warp == 1) tmem_dealloc(tmem, Cfg::TMEM_COLS);
+    }
+}
+
+template <int CTAS, int BN>
+int launch_gemm(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N, const void* residual,
+                int sm_count, DeviceCounters* dc, cudaStream_t stream) {
+    using Cfg = GCfg<CTAS, BN>;
+    static DeviceSetup setup;
+    if (device_setup(&setup, [] {
+            return cudaFuncSetAttribute(gemm_bf16_kernel<CTAS, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<CTAS, BN>::SMEM);
+        }, "gemm set-up") <= 0)
+        return PSA_ERR_CUDA;
+    GemmMaps maps;
+    if (!make_tensor_map_bf16(&maps.a, A, M, K, (uint64_t)K * 2, BM, BK)) return PSA_ERR_CUDA;
+    for (int w = 0; w < 3; ++w) {
+        const int src = w < nW ? w : 0;
+        if (!make_tensor_map_bf16(&maps.b[w], Bw[src], K, N, (uint64_t)N * 2, BK, 64)) return PSA_ERR_CUDA;
+        if (!make_tensor_map_bf16(&maps.c[w], C[src], M, N, (uint64_t)N * 2, 32, 64)) return PSA_ERR_CUDA;
+    }
+    const int ntiles = ((M + CTAS * BM - 1) / (CTAS * BM)) * ((N + BN - 1) / BN) * nW;
+    const int units = ntiles < sm_count / CTAS ? ntiles : sm_count / CTAS;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(units * CTAS);
+    cfg.blockDim = dim3(Cfg::THREADS);
+    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = CTAS;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = CTAS == 2 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_bf16_kernel<CTAS, BN>, maps, M, N, K, nW, static_cast<const uint16_t*>(residual), dc);
+    if (e != cudaSuccess) { set_cuda_error(e, "gemm_bf16_kernel launch"); return PSA_ERR_CUDA; }
+    return PSA_OK;
 }
 
 }  // namespace
@@ -292,32 +381,22 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
 int bf16_project(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N,
                  const void* residual, DeviceCounters* dc, cudaStream_t stream) {
     static DeviceSetup setup;
-    const int sm_count = device_setup(&setup, [] {
-        return cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
-    }, "gemm set-up");
-    if (sm_count <= 0) return PSA_ERR_CUDA;
-    GemmMaps maps;
-    if (!make_tensor_map_bf16(&maps.a, A, M, K, (uint64_t)K * 2, BM, BK)) return PSA_ERR_CUDA;
-    for (int w = 0; w < 3; ++w) {
-        const int src = w < nW ? w : 0;
-        if (!make_tensor_map_bf16(&maps.b[w], Bw[src], K, N, (uint64_t)N * 2, BK, 64)) return PSA_ERR_CUDA;
-        if (!make_tensor_map_bf16(&maps.c[w], C[src], M, N, (uint64_t)N * 2, BM, 64)) return PSA_ERR_CUDA;
-    }
-    const int ntiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN) * nW;
-    const int grid = ntiles < sm_count ? ntiles : sm_count;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(GEMM_THREADS);
-    cfg.dynamicSmemBytes = GEMM_SMEM;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_bf16_kernel, maps, M, N, K, nW, static_cast<const uint16_t*>(residual), dc);
-    if (e != cudaSuccess) { set_cuda_error(e, "gemm_bf16_kernel launch"); return PSA_ERR_CUDA; }
-    return PSA_OK;
+    const int sms = device_setup(&setup, [] { return cudaSuccess; }, "gemm set-up");
+    if (sms <= 0) return PSA_ERR_CUDA;
+    // The tile with the shortest estimated run: start and last epilogue plus rounds of tiles over the SMs times their k-steps, in
+    // cycles as measured (K = 64 .. 3072).  A pair of CTAs takes 650 cycles per k-step of a 256 x 256 tile where a lone CTA
+    // takes 740 for 128 x 256, but its launch costs 2 us more; narrow tiles pay where wide ones leave SMs idle.  Projections
+    // with N = 768, K = 768 (us, pair / 256 / 128 columns): 200 rows 14.5 14.1 12.1, 600 rows 14.5 14.0 12.6, 2000 rows
+    // 16.2 14.5 16.7, 4096 rows 20.9 20.4 24.8, 8192 rows 30.5 32.4 41.1; K = 3072, 8192 rows 78.2 87.1 126.
+    const long long nk = (K + BK - 1) / BK;
+    auto cost = [&](int ctas, int bn, long long step, long long fixed) {
+        const long long tiles = (long long)((M + ctas * BM - 1) / (ctas * BM)) * ((N + bn - 1) / bn) * nW, slots = sms / ctas;
+        return fixed + ((tiles + slots - 1) / slots) * (nk * step);
+    };
+    const long long pair = cost(2, 256, 650, 7200), wide = cost(1, 256, 740, 3000), narrow = cost(1, 128, 570, 1500);
+    if (narrow <= wide && narrow <= pair) return launch_gemm<1, 128>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+    if (wide <= pair) return launch_gemm<1, 256>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+    return launch_gemm<2, 256>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
 }
 
 }  // namespace psa

@@ -160,3 +160,26 @@ def test_block_residual_must_not_be_the_output():
     with pytest.raises(binding.PsaError) as ei:
         binding.psa_attention_block(x, w, w, w, wo, H, oracle.FULL, out=out, residual=out)
     assert ei.value.status == binding.ERR_SCHEME_ARGS
+
+
+# The projection kernel has three tiles (128 x 128, 128 x 256, and 256 x 256 over a pair of CTAs), chosen by how many of
+# them the call has.  Sequences of one vector make the layer the projection itself (y = v) and the block y Wo + residual:
+# rows around the tile edges and the switches, ragged column tiles, one and many k-steps.
+@pytest.mark.parametrize("rows,D,H,d", [(1, 64, 1, 64), (129, 128, 2, 64), (257, 192, 5, 64), (1000, 320, 3, 128), (2000, 768, 12, 64),
+                                        (4096, 64, 12, 64), (5000, 1024, 7, 64), (9000, 1600, 13, 64), (300, 64, 20, 128)])
+def test_projection_tile_choices(rows, D, H, d):
+    g = torch.Generator(device="cuda").manual_seed(rows + D)
+    X = torch.randn(rows, 1, D, device="cuda", generator=g).bfloat16()
+    W = [(torch.randn(D, H * d, device="cuda", generator=g) * D ** -0.5).bfloat16() for _ in range(3)]
+    Wo = (torch.randn(H * d, D, device="cuda", generator=g) * (H * d) ** -0.5).bfloat16()
+    y = binding.psa_attention(X, *W, H, binding.FULL)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got["proj_macs"] == 3 * rows * D * H * d
+    ref = X.double().view(rows, D) @ W[2].double()
+    # one rounding to bf16 of a sum of K products in fp32 (|q|, |k| = O(1): the single weight is exactly 1)
+    assert ((y.double().view(rows, -1) - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-4).all()
+    z = binding.psa_attention_block(X, *W, Wo, H, binding.FULL, residual=X)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got["proj_macs"] == 4 * rows * D * H * d
+    zref = y.double().view(rows, -1) @ Wo.double() + X.double().view(rows, D)
+    assert ((z.double().view(rows, -1) - zref).abs() <= 2.0 ** -8 * zref.abs() + 1e-4).all()
