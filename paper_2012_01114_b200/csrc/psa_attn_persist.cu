@@ -130,8 +130,8 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
     const uint32_t tmem = tmem_base_s;
     volatile int* abortp = &abort_flag;
     // Everything above (barriers, TMEM) overlaps the end of the kernel before this one in the stream; global memory
-    // is touched only from here on.
-    grid_launch_dependents();
+    // is touched only from here on.  The kernel after this one is let in when a CTA's work is done: let in at once, its
+    // waiting CTAs cost a layer of n = 512 0.9 us (31.8 -> 30.9) and a block of n = 1024 1.4 us.
     grid_dependency_wait();
     // the counter block of the NEXT call on this workspace is cleared here, off that call's critical path
     if (threadIdx.x == 0 && blockIdx.x == 0 && dc_next) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};
@@ -627,6 +627,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
             idx = idx_next;
             work = work_next;
         }
+        if (sw == 0 && lane == 0) grid_launch_dependents();
         if (store_pending && lane == 0) tma_store_wait_read();   // shared memory may be released; the writes complete on their own
     }
     tc_fence_before();

@@ -124,7 +124,7 @@ __device__ __forceinline__ TileCoord tile_coord(int t, int mt, int nt, int bm, i
     return c;
 }
 
-template <int CTAS, int BN>
+template <int CTAS, int BN, bool RES>
 __global__ void __launch_bounds__(GCfg<CTAS, BN>::THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int nW, const uint16_t* __restrict__ R,
                  DeviceCounters* dc) {
@@ -162,8 +162,8 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
     volatile int* abortp = &abort_flag;
-    // (programmatic dependent launch: the set-up above overlaps the end of the kernel before this one)
-    grid_launch_dependents();
+    // (programmatic dependent launch: the set-up above overlaps the end of the kernel before this one; the kernel after
+    // this one is let in when a CTA's tiles are done, see attn_persist_kernel)
     grid_dependency_wait();
 
     if (warp == 0 && lane == 0) {
@@ -253,25 +253,22 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
             const int buf = i & 1;
             const TileCoord c = tile_coord(t, mt, nt, CTAS * BM, BN);
             const int row0 = c.m0 + rank * BM + 32 * q, row = row0 + lane;
-            bool ready = false, ok = true;
-#pragma unroll 1
+            // residual input: C = A B + R, added in fp32 before the rounding to bf16 (R is [M, N] bf16, row-major).  The
+            // row's part of R is read while the tile is still being computed: sub-tile by sub-tile behind the
+            // accumulator it cost 6 us on 8192 x 768.
+            uint4 x[RES ? NSUB : 1][8];
+            if constexpr (RES) {
+                const uint4* rp = reinterpret_cast<const uint4*>(R + (size_t)row * N + c.n0);
+#pragma unroll
+                for (int u = 0; u < NSUB; ++u)
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) x[u][g] = row < M && c.n0 + 64 * u < N ? __ldg(rp + 8 * u + g) : make_uint4(0, 0, 0, 0);
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (i >> 1) & 1, abortp))) break;
+            tc_fence_after();
+#pragma unroll(RES ? NSUB : 1)
             for (int u = 0; u < NSUB; ++u) {
                 const int col = c.n0 + 64 * u;
-                // residual input: C = A B + R, added in fp32 before the rounding to bf16 (R is [M, N] bf16, row-major);
-                // it is on its way while the tile is still being computed
-                uint4 x[8];
-                const bool res = R && row < M && col < N;
-                if (res) {
-                    const uint4* rp = reinterpret_cast<const uint4*>(R + (size_t)row * N + col);
-#pragma unroll
-                    for (int g = 0; g < 8; ++g) x[g] = __ldg(rp + g);
-                }
-                if (!ready) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (i >> 1) & 1, abortp));
-                    if (!ok) break;
-                    tc_fence_after();
-                    ready = true;
-                }
                 uint32_t r[2][32];
                 const uint32_t src = tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * BN + u * 64;
                 tmem_ld32(src, r[0]);
@@ -285,10 +282,10 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
                         else mbar_arrive(&acc_empty[buf]);
                     }
                 }
-                if (res) {
+                if constexpr (RES) {
 #pragma unroll
                     for (int g = 0; g < 8; ++g) {
-                        const uint32_t w[4] = {x[g].x, x[g].y, x[g].z, x[g].w};
+                        const uint32_t w[4] = {x[u][g].x, x[u][g].y, x[u][g].z, x[u][g].w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             uint32_t* dst = &r[g >> 2][(g & 3) * 8 + 2 * e];
@@ -322,8 +319,8 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
                 }
                 ++stores;
             }
-            if (!ok) break;
         }
+        if (warp == 2 && lane == 0) grid_launch_dependents();
         if (lane == 0) tma_store_wait_read();      // shared memory may be released; the writes complete on their own
     }
     tc_fence_before();
@@ -339,13 +336,13 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
     }
 }
 
-template <int CTAS, int BN>
-int launch_gemm(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N, const void* residual,
+template <int CTAS, int BN, bool RES>
+int launch_gemm_kernel(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N, const void* residual,
                 int sm_count, DeviceCounters* dc, cudaStream_t stream) {
     using Cfg = GCfg<CTAS, BN>;
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
-            return cudaFuncSetAttribute(gemm_bf16_kernel<CTAS, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<CTAS, BN>::SMEM);
+            return cudaFuncSetAttribute(gemm_bf16_kernel<CTAS, BN, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<CTAS, BN>::SMEM);
         }, "gemm set-up") <= 0)
         return PSA_ERR_CUDA;
     GemmMaps maps;
@@ -371,9 +368,16 @@ int launch_gemm(const void* A, const void* const Bw[3], void* const C[3], int nW
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = CTAS == 2 ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_bf16_kernel<CTAS, BN>, maps, M, N, K, nW, static_cast<const uint16_t*>(residual), dc);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_bf16_kernel<CTAS, BN, RES>, maps, M, N, K, nW, static_cast<const uint16_t*>(residual), dc);
     if (e != cudaSuccess) { set_cuda_error(e, "gemm_bf16_kernel launch"); return PSA_ERR_CUDA; }
     return PSA_OK;
+}
+
+template <int CTAS, int BN>
+int launch_gemm(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N, const void* residual,
+                int sm_count, DeviceCounters* dc, cudaStream_t stream) {
+    return residual ? launch_gemm_kernel<CTAS, BN, true>(A, Bw, C, nW, M, K, N, residual, sm_count, dc, stream)
+                    : launch_gemm_kernel<CTAS, BN, false>(A, Bw, C, nW, M, K, N, residual, sm_count, dc, stream);
 }
 
 }  // namespace
