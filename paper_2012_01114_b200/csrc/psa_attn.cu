@@ -49,8 +49,8 @@ struct SymCfg {
     static constexpr int SUB = D / 64;                  // 64-column sub-tiles per 128-row tile of X
     static constexpr int TILE_BYTES = 128 * D * 2;      // one X tile (bf16)
     static constexpr int XST = D == 128 ? 3 : 4;        // X tiles in flight: PV of a block, S of the next, one loading (2: 5 % slower)
-    static constexpr int MST = D == 128 ? 2 : 4;        // half blocks of handed-on scores in flight
-    static constexpr int STAGE_BYTES = 16 * 64 * 2;     // a softmax warp's output staging buffer
+    static constexpr int MST = D == 128 ? 2 : 3;        // half blocks of handed-on scores in flight
+    static constexpr int STAGE_BYTES = 16 * 64 * 4;     // a softmax warp's buffer for scores and outputs on their way out
     static constexpr int SMEM = (1 + XST) * TILE_BYTES + MST * S_HALF_BYTES + SYM_WARPS * STAGE_BYTES + 1024;
     static constexpr int TMEM_S = 0, TMEM_P = 256, TMEM_O = 384;
 };
@@ -193,7 +193,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                     if (j == max(T - 3, 0)) next = atomicAdd(work_counter, 1);
                     if (j <= It) continue;
                     // block (j, It), handed on by the CTA that works on tile j: present once its flag counts past It.  The
-                    // stores behind the flag were ordinary ones, the copies below go through the asynchronous proxy.
+                    // flag is an ordinary load, the copies below go through the asynchronous proxy.
                     ok = wait_at_least([&] { return ld_acquire(flags + j); }, It + 1, abortp);
                     if (!ok) break;
                     asm volatile("fence.proxy.async;" ::: "memory");
@@ -293,8 +293,8 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
         }
     } else if (warp == SYM_PUBLISHER) {
         // ------------------------------------------------------------ announces blocks handed on
-        // Lane w < 8 watches softmax warp w.  A block is complete when all eight have stored their rows; the fence orders
-        // their stores, observed through shared memory, before the flag.
+        // Lane w < 8 watches softmax warp w.  A block is complete when all eight report their copies out as complete; the fence
+        // orders those, observed through shared memory, before the flag.
         int done = 0;                                           // blocks announced in earlier items
         for (uint32_t it = 0;; ++it) {
             if (!__all_sync(0xffffffffu, mbar_wait(&bars.item_full[it & 1], (it >> 1) & 1, abortp))) break;
@@ -334,13 +334,31 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
         uint8_t* stage = sStage + wq * Cfg::STAGE_BYTES;
         // Place of a score in a handed-on block, in floats: [16-row group of the writer][column half][group of 8 columns]
         // [chunk][column parity][row A / B].  A writer thread stores its four scores of a column group as one 16-byte chunk;
-        // element (r, c) is row c, key r of the reader, which takes keys r and r + 8 as 8 bytes.  Chunk numbers are permuted
-        // (bits of r: 2-1, bits of c: 2-1, bit 0 of r, from the lowest up) so that a half-warp reads 8 different ones.
-        const int put = kw * 2048 + 4 * ((lane >> 3) | ((lane & 3) << 2) | (((lane >> 2) & 1) << 4));
-        const int get = (kw >> 2) * 1024 + (kw & 3) * 256 + 4 * ((lane & 3) | ((lane >> 3) << 2)) + 2 * ((lane >> 2) & 1);
+        // element (r, c) is row c, key r of the reader, which takes keys r and r + 8 as 8 bytes.  With r2 r1 r0 the row and c1 c0
+        // the column pair inside an 8 x 8 square, the chunk's number is (r2, r1, r2 ^ r0, r1 ^ c1, c0): the 8 lanes of a
+        // writing phase and the 16 of a reading one then touch every bank once.
+        const int put = 4 * ((lane & 1) | ((lane ^ (lane >> 2)) & 2) | ((lane ^ (lane >> 2)) & 4) | (lane & 24));
+        const int get_chunk = ((lane >> 3) & 1) | (((lane ^ (lane >> 4)) & 1) << 1) | ((lane & 2) << 1) | ((lane & 1) << 3) | ((lane & 2) << 3);
+        const int get = (kw >> 2) * 1024 + (kw & 3) * 256 + 2 * ((lane >> 2) & 1);
+        const int get_even = get + 4 * get_chunk, get_odd = get + 4 * (get_chunk ^ 4);      // rows r with r0 = 0, 1
         uint32_t blk = 0, sc = 0, mc = 0;                       // blocks, computed blocks and half blocks so far, all items
         int nstored = 0;
-        bool store_pending = false;                             // a TMA store of this warp may still be reading `stage`
+        bool handed = false;                                    // the block before was handed on and not yet reported
+        // Half a block's scores of this warp (16 rows, 64 columns) go out through its buffer as one bulk copy.  (Stored from the
+        // registers they take the warps 1100 cycles per block, an SM's way out being 64 bytes wide.)
+        auto hand_on = [&](const uint32_t (&s)[32], float* dst) {
+            if (lane == 0) tma_store_wait_read();               // whatever used the buffer last
+            __syncwarp();
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+                *reinterpret_cast<uint4*>(stage + 512 * g + 4 * put) = make_uint4(s[4 * g], s[4 * g + 2], s[4 * g + 1], s[4 * g + 3]);
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                bulk_store_1d(dst, stage, Cfg::STAGE_BYTES);
+                tma_store_commit();
+            }
+        };
         bool ok = true;
         for (uint32_t it = 0; ok; ++it) {
             ok = __all_sync(0xffffffffu, mbar_wait(&bars.item_full[it & 1], (it >> 1) & 1, abortp));
@@ -351,7 +369,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
             if (idx < 0) break;
             int hl, It;
                 item_work(idx, hl, It);
-            float* own = sym_head(Sg, hl, np) + (size_t)(It * (It + 1) / 2) * (S_BLOCK_BYTES / 4);
+            float* own = sym_head(Sg, hl, np) + (size_t)(It * (It + 1) / 2) * (S_BLOCK_BYTES / 4) + kw * 2048;
             float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;       // running maxima (log2 units) and row sums
             for (int j = 0; j < T; ++j, ++blk) {
                 uint32_t s0[32], s1[32];
@@ -368,29 +386,24 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bars.s_free[sc & 1]);
                     ++sc;
-                    if (j < It) {                               // the mirror block's tile needs it
-                        float* dst = own + (size_t)j * (S_BLOCK_BYTES / 4) + put;
-#pragma unroll
-                        for (int g = 0; g < 8; ++g) {
-                            *reinterpret_cast<uint4*>(dst + 128 * g) = make_uint4(s0[4 * g], s0[4 * g + 2], s0[4 * g + 1], s0[4 * g + 3]);
-                            *reinterpret_cast<uint4*>(dst + 1024 + 128 * g) = make_uint4(s1[4 * g], s1[4 * g + 2], s1[4 * g + 1], s1[4 * g + 3]);
-                        }
-                        __syncwarp();
-                        if (lane == 0) st_release_cta(&stored[wq], ++nstored);
+                    if (handed) {                               // the previous block's last stores are complete by now
+                        if (lane == 0) { tma_store_wait_all(); st_release_cta(&stored[wq], ++nstored); }
+                        handed = false;
                     }
+                    if (j < It) hand_on(s0, own + (size_t)j * (S_BLOCK_BYTES / 4));
                 } else {
                     // ---- a block computed by the CTA of tile j, read transposed
 #pragma unroll
                     for (int half = 0; half < 2; ++half, ++mc) {
                         ok = __all_sync(0xffffffffu, mbar_wait(&bars.m_full[mc % MST], (mc / MST) & 1, abortp));
                         if (!ok) break;
-                        const float* src = reinterpret_cast<const float*>(sM + (mc % MST) * S_HALF_BYTES) + get;
+                        const float* src = reinterpret_cast<const float*>(sM + (mc % MST) * S_HALF_BYTES);
                         uint32_t (&s)[32] = half ? s1 : s0;
 #pragma unroll
                         for (int g = 0; g < 4; ++g)             // keys 16 g .. 16 g + 15 of the half, row A / B, key parity
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
-                                const uint2 v = *reinterpret_cast<const uint2*>(src + 2048 * g + 128 * (e >> 1) + 64 * (e & 1));
+                                const uint2 v = *reinterpret_cast<const uint2*>(src + ((e & 1) ? get_odd : get_even) + 2048 * g + 128 * (e >> 1));
                                 s[8 * g + e] = v.x;
                                 s[8 * g + 4 + e] = v.y;
                             }
@@ -424,6 +437,10 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                 float sumA = 0.f, sumB = 0.f;
                 uint32_t pk[16];
                 exp_quad64(s0, sl2, -mA, -mB, pk, sumA, sumB);
+                if (j < It) {
+                    hand_on(s1, own + (size_t)j * (S_BLOCK_BYTES / 4) + 1024);
+                    handed = true;
+                }
                 if (blk >= 2) {
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars.o_done[blk & 1], ((blk >> 1) - 1) & 1, abortp));
                     if (!ok) break;
@@ -475,28 +492,28 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
                 uint32_t v[32];
                 tmem_ld_quad64(tO + 64 * u, v);
                 tc_wait_ld();
-                if (store_pending) {        // the store that last used the buffer must have read it
+                if (u == 0) {               // whatever used the buffer last must have been read
                     if (lane == 0) tma_store_wait_read();
                     __syncwarp();
                 }
+                uint8_t* sub = stage + u * (16 * 64 * 2);
 #pragma unroll
                 for (int g = 0; g < 8; ++g) {
                     const uint32_t a = pack_bf16x2(__uint_as_float(v[4 * g]) * invA, __uint_as_float(v[4 * g + 1]) * invA);
                     const uint32_t bb = pack_bf16x2(__uint_as_float(v[4 * g + 2]) * invB, __uint_as_float(v[4 * g + 3]) * invB);
-                    *reinterpret_cast<uint32_t*>(stage + swz128_offset(lane >> 2, g) + 2 * cq) = a;
-                    *reinterpret_cast<uint32_t*>(stage + swz128_offset((lane >> 2) + 8, g) + 2 * cq) = bb;
+                    *reinterpret_cast<uint32_t*>(sub + swz128_offset(lane >> 2, g) + 2 * cq) = a;
+                    *reinterpret_cast<uint32_t*>(sub + swz128_offset((lane >> 2) + 8, g) + 2 * cq) = bb;
                 }
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_4d(&maps.o, stage, 64 * u, h, It * TILE + row0, b);
+                    tma_store_4d(&maps.o, sub, 64 * u, h, It * TILE + row0, b);
                     tma_store_commit();
                 }
-                store_pending = true;
             }
             tc_fence_before();
         }
-        if (store_pending && lane == 0) tma_store_wait_read();   // shared memory may be released; the writes complete on their own
+        if (lane == 0) tma_store_wait_read();   // shared memory may be released; the writes complete on their own
     }
     tc_fence_before();
     __syncthreads();
