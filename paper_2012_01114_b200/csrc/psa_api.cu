@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "psa_internal.h"
@@ -29,6 +30,8 @@ struct Context {
     // call's first kernel.  `clean_ws` is the workspace whose block `next_block` is known to be clear.
     char* clean_ws = nullptr;
     int next_block = 0;
+    // Streams and events of the entry points on host buffers, created by the first such call and kept.
+    struct HostPipe* pipe = nullptr;
     std::vector<cudaEvent_t> prof_events;  // 3 per profiled call
     int prof_calls = 0, prof_max = 0;
     psa_counts last_useful = {0, 0, 0, 0, 0, 0};
@@ -46,9 +49,18 @@ Context* current_ctx() {
     return &g_ctxs[dev];
 }
 
+constexpr size_t HOST_CHUNK_BYTES = 3 << 20;    // see psa_attention_host
+constexpr int HOST_CHUNKS = 8;                  // most parts a batch on host buffers is worked off in
+struct HostPipe {
+    cudaStream_t in = nullptr, out = nullptr;
+    cudaEvent_t start = nullptr, weights = nullptr, loaded[HOST_CHUNKS] = {}, computed[HOST_CHUNKS] = {}, stored = nullptr;
+};
+
 constexpr size_t COUNTER_BYTES = 256;          // two counter blocks
 constexpr size_t COUNTER_BLOCK_BYTES = 128;
-static_assert(sizeof(DeviceCounters) <= COUNTER_BLOCK_BYTES, "counter block too small");
+constexpr size_t CURSOR_OFFSET = 64;           // work counters of a call in several parts, behind the counters
+static_assert(sizeof(DeviceCounters) <= CURSOR_OFFSET, "counter block too small");
+static_assert(CURSOR_OFFSET + HOST_CHUNKS * sizeof(unsigned int) <= COUNTER_BLOCK_BYTES, "counter block too small");
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -104,6 +116,28 @@ WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme
     return L;
 }
 
+HostPipe* acquire_pipe(Context& cx) {
+    if (cx.pipe) return cx.pipe;
+    HostPipe* p = new (std::nothrow) HostPipe;
+    if (!p) { set_error_text("out of host memory"); return nullptr; }
+    cudaError_t e = cudaStreamCreateWithFlags(&p->in, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->out, cudaStreamNonBlocking);
+    auto event = [&](cudaEvent_t* ev) { if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming); };
+    event(&p->start); event(&p->weights); event(&p->stored);
+    for (int c = 0; c < HOST_CHUNKS; ++c) { event(&p->loaded[c]); event(&p->computed[c]); }
+    if (e == cudaSuccess) return cx.pipe = p;
+    set_cuda_error(e, "streams of the host entry points");
+    if (p->in) cudaStreamDestroy(p->in);
+    if (p->out) cudaStreamDestroy(p->out);
+    for (cudaEvent_t ev : {p->start, p->weights, p->stored}) if (ev) cudaEventDestroy(ev);
+    for (int c = 0; c < HOST_CHUNKS; ++c) {
+        if (p->loaded[c]) cudaEventDestroy(p->loaded[c]);
+        if (p->computed[c]) cudaEventDestroy(p->computed[c]);
+    }
+    delete p;
+    return nullptr;
+}
+
 // Returns the base of a workspace of at least `bytes`, or nullptr (error text set).
 char* acquire_ws(Context& cx, size_t bytes) {
     if (cx.user_ws && cx.user_bytes >= bytes) return static_cast<char*>(cx.user_ws);
@@ -132,18 +166,59 @@ void useful_counts(int batch, int heads, int n, int d_model, int d_k, int scheme
     c->proj_macs = with_proj ? nproj * (uint64_t)batch * N * (uint64_t)d_model * (uint64_t)heads * d : 0;
 }
 
+// The kernels of one layer (or, without projections, of one attention core) over `batch` sequences.  q, k, v: the workspace's
+// projections (with_proj), written here; `cursor`: work counter of the fused bf16 kernel, zero when it starts; `dc_next`: see
+// Context (may be null).  `between`, if given, is recorded between projections and attention.
+int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K, const void* V,
+                  int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out, cudaStream_t stream,
+                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, DeviceCounters* dc, unsigned int* cursor,
+                  DeviceCounters* dc_next, cudaEvent_t between) {
+    const float scale = 1.0f / sqrtf((float)d_k);
+    const int nW = scheme == PSA_SYMMETRIC ? 1 : 3;
+    cudaError_t e = cudaSuccess;
+    if (with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme)) {
+        // a small fp32 layer runs as one launch; q, k, v never leave shared memory
+        if (between) cudaEventRecord(between, stream);
+        e = f32_fused_layer(static_cast<const float*>(X), static_cast<const float*>(Wq), static_cast<const float*>(Wk),
+                            static_cast<const float*>(Wv), static_cast<float*>(out), batch, heads, n, d_model, d_k, scale,
+                            scheme, dc, dc_next, stream);
+        if (e != cudaSuccess) { set_cuda_error(e, "f32_fused_layer"); return PSA_ERR_CUDA; }
+        return PSA_OK;
+    }
+    if (with_proj) {
+        const void* Ws[3] = {Wq, nW == 3 ? Wk : Wq, nW == 3 ? Wv : Wq};
+        if (dtype == PSA_F32) {
+            float* const outs[3] = {static_cast<float*>(qkv[0]), static_cast<float*>(qkv[1]), static_cast<float*>(qkv[2])};
+            e = f32_project(static_cast<const float*>(X), reinterpret_cast<const float* const*>(Ws), outs, nW, batch * n, d_model,
+                            heads * d_k, nullptr, dc, stream);
+            if (e != cudaSuccess) { set_cuda_error(e, "f32_project"); return PSA_ERR_CUDA; }
+        } else {
+            int rc = bf16_project(X, Ws, qkv, nW, batch * n, d_model, heads * d_k, nullptr, dc, stream);
+            if (rc != PSA_OK) return rc;
+        }
+        Q = qkv[0]; K = qkv[1]; V = qkv[2];
+    }
+    if (between) cudaEventRecord(between, stream);
+    if (dtype == PSA_F32) {
+        e = f32_attention(static_cast<const float*>(Q), static_cast<const float*>(K), static_cast<const float*>(V),
+                          static_cast<float*>(out), S, batch, heads, n, d_k, scale, scheme, dc, stream);
+        if (e != cudaSuccess) { set_cuda_error(e, "f32_attention"); return PSA_ERR_CUDA; }
+        return PSA_OK;
+    }
+    return bf16_attention(Q, K, V, out, S, s_bytes, batch, heads, n, d_k, scale, scheme, dc, cursor, dc_next, stream);
+}
+
 int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K,
               const void* V, int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out,
               cudaStream_t stream, bool with_proj, char* ws, const WsLayout& L) {
     // the paths whose last kernel clears the other counter block: the fused bf16 kernel and the one-launch fp32 layer
-    const bool fused_f32 = with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme);
-    const bool turns = (dtype == PSA_BF16 && scheme != PSA_SYMMETRIC && d_k <= 128) || fused_f32;
+    const bool turns = (dtype == PSA_BF16 && scheme != PSA_SYMMETRIC && d_k <= 128) ||
+                       (with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme));
     int block = 0;
-    cudaError_t e = cudaSuccess;
     if (turns && cx.clean_ws == ws) {
         block = cx.next_block;
     } else {
-        e = cudaMemsetAsync(ws, 0, 2 * COUNTER_BLOCK_BYTES, stream);
+        const cudaError_t e = cudaMemsetAsync(ws, 0, 2 * COUNTER_BLOCK_BYTES, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync(counters)"); return PSA_ERR_CUDA; }
     }
     cx.clean_ws = nullptr;           // until this call's kernels are known to be queued
@@ -152,8 +227,6 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     cx.last_dc = dc;
     memset(&cx.last_useful, 0, sizeof(psa_counts));
     useful_counts(batch, heads, n, d_model, d_k, scheme, with_proj, &cx.last_useful);
-    const float scale = 1.0f / sqrtf((float)d_k);
-    const int nW = scheme == PSA_SYMMETRIC ? 1 : 3;
     cudaEvent_t* pev = nullptr;
     if (cx.prof_calls < cx.prof_max) pev = &cx.prof_events[3 * cx.prof_calls++];
     struct EventTail {  // records the closing event on every exit path
@@ -161,39 +234,10 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
         ~EventTail() { if (ev) cudaEventRecord(ev[2], st); }
     } tail{pev, stream};
     if (pev) cudaEventRecord(pev[0], stream);
-    if (fused_f32) {
-        // a small fp32 layer runs as one launch; q, k, v never leave shared memory
-        if (pev) cudaEventRecord(pev[1], stream);
-        e = f32_fused_layer(static_cast<const float*>(X), static_cast<const float*>(Wq), static_cast<const float*>(Wk),
-                            static_cast<const float*>(Wv), static_cast<float*>(out), batch, heads, n, d_model, d_k, scale,
-                            scheme, dc, dc_next, stream);
-        if (e != cudaSuccess) { set_cuda_error(e, "f32_fused_layer"); return PSA_ERR_CUDA; }
-        cx.clean_ws = ws;               // the other block will be clear once this call has run
-        cx.next_block = block ^ 1;
-        return PSA_OK;
-    }
-    if (with_proj) {
-        void* outs[3] = {ws + L.q, ws + L.k, ws + L.v};
-        const void* Ws[3] = {Wq, nW == 3 ? Wk : Wq, nW == 3 ? Wv : Wq};
-        if (dtype == PSA_F32) {
-            e = f32_project(static_cast<const float*>(X), reinterpret_cast<const float* const*>(Ws),
-                            reinterpret_cast<float* const*>(outs), nW, batch * n, d_model, heads * d_k, nullptr, dc, stream);
-            if (e != cudaSuccess) { set_cuda_error(e, "f32_project"); return PSA_ERR_CUDA; }
-        } else {
-            int rc = bf16_project(X, Ws, outs, nW, batch * n, d_model, heads * d_k, nullptr, dc, stream);
-            if (rc != PSA_OK) return rc;
-        }
-        Q = ws + L.q; K = ws + L.k; V = ws + L.v;
-    }
-    if (pev) cudaEventRecord(pev[1], stream);
+    void* const qkv[3] = {ws + L.q, ws + L.k, ws + L.v};
     float* S = scheme == PSA_SYMMETRIC ? reinterpret_cast<float*>(ws + L.s) : nullptr;
-    if (dtype == PSA_F32) {
-        e = f32_attention(static_cast<const float*>(Q), static_cast<const float*>(K), static_cast<const float*>(V),
-                          static_cast<float*>(out), S, batch, heads, n, d_k, scale, scheme, dc, stream);
-        if (e != cudaSuccess) { set_cuda_error(e, "f32_attention"); return PSA_ERR_CUDA; }
-        return PSA_OK;
-    }
-    const int rc = bf16_attention(Q, K, V, out, S, L.s_bytes, batch, heads, n, d_k, scale, scheme, dc, dc_next, stream);
+    const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
+                                 qkv, S, L.s_bytes, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
     if (rc == PSA_OK && turns) {        // the other block will be clear once this call has run
         cx.clean_ws = ws;
         cx.next_block = block ^ 1;
@@ -310,21 +354,92 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     char* ws = acquire_ws(cx, L.total);
     if (!ws) return PSA_ERR_WORKSPACE;
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
-    const size_t xb = (size_t)batch * n * d_model * es, wb = (size_t)d_model * heads * d_k * es;
-    const size_t ob = (size_t)batch * n * heads * d_k * es;
-    cudaError_t e = cudaMemcpyAsync(ws + L.xs, X_host, xb, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.wq, Wq_host, wb, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess && scheme != PSA_SYMMETRIC) {
-        e = cudaMemcpyAsync(ws + L.wk, Wk_host, wb, cudaMemcpyHostToDevice, stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.wv, Wv_host, wb, cudaMemcpyHostToDevice, stream);
+    const size_t xb = (size_t)n * d_model * es, wb = (size_t)d_model * heads * d_k * es, ob = (size_t)n * heads * d_k * es;   // per sequence; per matrix
+    // The batch is worked off in parts of at least HOST_CHUNK_BYTES in and out, so that the copies of one part run under the
+    // copies and kernels of the others (both directions of the link are busy at once).
+    const int parts = (int)std::max<size_t>(1, std::min<size_t>(std::min(batch, HOST_CHUNKS), batch * (xb + ob) / HOST_CHUNK_BYTES));
+    // (a call that is being timed runs in one part, and so does one whose score scratch, sized for the batch's passes, is
+    // smaller than a part's passes would have it)
+    const bool scratch_fits = dtype != PSA_BF16 || scheme != PSA_SYMMETRIC ||
+                              bf16_symmetric_scratch_bytes((batch + parts - 1) / parts, heads, n) <= L.s_bytes;
+    HostPipe* pipe = nullptr;
+    if (parts > 1 && scratch_fits && cx.prof_calls >= cx.prof_max) {
+        pipe = acquire_pipe(cx);
+        if (!pipe) return PSA_ERR_CUDA;
     }
-    if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpyAsync(H2D)"); return PSA_ERR_CUDA; }
-    rc = run_layer(cx, ws + L.xs, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, batch, heads, n, d_model,
-                   d_k, scheme, dtype, ws + L.outs, stream, true, ws, L);
+    const bool sym = scheme == PSA_SYMMETRIC;
+    if (!pipe) {
+        cudaError_t e = cudaMemcpyAsync(ws + L.xs, X_host, batch * xb, cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.wq, Wq_host, wb, cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess && !sym) {
+            e = cudaMemcpyAsync(ws + L.wk, Wk_host, wb, cudaMemcpyHostToDevice, stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.wv, Wv_host, wb, cudaMemcpyHostToDevice, stream);
+        }
+        if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpyAsync(H2D)"); return PSA_ERR_CUDA; }
+        rc = run_layer(cx, ws + L.xs, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, batch, heads, n, d_model,
+                       d_k, scheme, dtype, ws + L.outs, stream, true, ws, L);
+        if (rc != PSA_OK) return rc;
+        e = cudaMemcpyAsync(out_host, ws + L.outs, batch * ob, cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpyAsync(D2H)/sync"); return PSA_ERR_CUDA; }
+        return PSA_OK;
+    }
+    // In parts: copies in on one stream, kernels on the caller's, copies out on another.  The counters of all parts go to one
+    // block; the work counter of each has a place of its own behind them.  All copies in are queued before the first copy
+    // out: with pageable buffers a copy may hold the calling thread until it is done.
+    const char* what = "ordering the streams of a host call";
+    cudaError_t e = cudaEventRecord(pipe->start, stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->start, 0);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->out, pipe->start, 0);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, 2 * COUNTER_BLOCK_BYTES, stream);
+    cx.clean_ws = nullptr;
+    DeviceCounters* dc = reinterpret_cast<DeviceCounters*>(ws);
+    cx.last_dc = dc;
+    memset(&cx.last_useful, 0, sizeof(psa_counts));
+    useful_counts(batch, heads, n, d_model, d_k, scheme, true, &cx.last_useful);
+    if (e == cudaSuccess) {
+        what = "cudaMemcpyAsync(H2D)";
+        e = cudaMemcpyAsync(ws + L.wq, Wq_host, wb, cudaMemcpyHostToDevice, pipe->in);
+        if (e == cudaSuccess && !sym) e = cudaMemcpyAsync(ws + L.wk, Wk_host, wb, cudaMemcpyHostToDevice, pipe->in);
+        if (e == cudaSuccess && !sym) e = cudaMemcpyAsync(ws + L.wv, Wv_host, wb, cudaMemcpyHostToDevice, pipe->in);
+    }
+    auto first = [&](int c) { return (int)((long long)batch * c / parts); };      // first sequence of part c
+    for (int c = 0; c < parts && e == cudaSuccess; ++c) {
+        const size_t b0 = first(c), nb = first(c + 1) - b0;
+        e = cudaMemcpyAsync(ws + L.xs + b0 * xb, static_cast<const char*>(X_host) + b0 * xb, nb * xb, cudaMemcpyHostToDevice, pipe->in);
+        if (e == cudaSuccess) e = cudaEventRecord(pipe->loaded[c], pipe->in);
+    }
+    for (int c = 0; c < parts && e == cudaSuccess && rc == PSA_OK; ++c) {
+        const size_t b0 = first(c), nb = first(c + 1) - b0;
+        what = "ordering the streams of a host call";
+        e = cudaStreamWaitEvent(stream, pipe->loaded[c], 0);
+        if (e != cudaSuccess) break;
+        void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
+        rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
+                           d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,
+                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, dc,
+                           reinterpret_cast<unsigned int*>(ws + CURSOR_OFFSET) + c, nullptr, nullptr);
+        if (rc != PSA_OK) break;
+        e = cudaEventRecord(pipe->computed[c], stream);
+    }
+    for (int c = 0; c < parts && e == cudaSuccess && rc == PSA_OK; ++c) {
+        const size_t b0 = first(c), nb = first(c + 1) - b0;
+        what = "cudaMemcpyAsync(D2H)";
+        e = cudaStreamWaitEvent(pipe->out, pipe->computed[c], 0);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(static_cast<char*>(out_host) + b0 * ob, ws + L.outs + b0 * ob, nb * ob, cudaMemcpyDeviceToHost, pipe->out);
+    }
+    if (e == cudaSuccess && rc == PSA_OK) e = cudaEventRecord(pipe->stored, pipe->out);
+    if (e == cudaSuccess && rc == PSA_OK) e = cudaStreamWaitEvent(stream, pipe->stored, 0);
+    if (e == cudaSuccess && rc == PSA_OK) {
+        e = cudaStreamSynchronize(stream);
+    } else {            // nothing of this call may touch the caller's buffers after it has returned
+        cudaStreamSynchronize(pipe->in);
+        cudaStreamSynchronize(stream);
+        cudaStreamSynchronize(pipe->out);
+    }
     if (rc != PSA_OK) return rc;
-    e = cudaMemcpyAsync(out_host, ws + L.outs, ob, cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpyAsync(D2H)/sync"); return PSA_ERR_CUDA; }
+    if (e != cudaSuccess) { set_cuda_error(e, what); return PSA_ERR_CUDA; }
     return PSA_OK;
 }
 

@@ -76,7 +76,7 @@ template <int D> __host__ __device__ constexpr int item_readers() { return (D ==
 template <int D, bool KVS>
 __global__ void __launch_bounds__(persist_threads<D>(), 1)
 attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ SchedParams sp, int H, int scheme,
-                    int nitems, float sl2, DeviceCounters* dc, DeviceCounters* dc_next) {
+                    int nitems, float sl2, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next) {
     using Cfg = PCfg<D>;
     constexpr bool SEP = Cfg::SEP_P;
     constexpr int VST = Cfg::VSTAGES;
@@ -184,7 +184,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
                             if (!ok) break;
                         }
                         // the next item's index is fetched behind the item's first loads and long before it is needed
-                        if (p == 1) next = (int)gridDim.x + (int)atomicAdd(&dc->next_item, 1u);
+                        if (p == 1) next = (int)gridDim.x + (int)atomicAdd(cursor, 1u);
                     }
                 } else {
                     for (int j = 0; j < maxkv && ok; ++j) {
@@ -222,7 +222,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
                         }
                         // the next item's index is fetched behind the item's first loads (the atomic's round trip of about
                         // a thousand cycles would otherwise delay them) and long before it is needed
-                        if (j == 0) next = (int)gridDim.x + (int)atomicAdd(&dc->next_item, 1u);
+                        if (j == 0) next = (int)gridDim.x + (int)atomicAdd(cursor, 1u);
                     }
                 }
                 idx = next;
@@ -640,7 +640,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
 // between d and D are zero-filled by the loads and dropped by the stores).
 template <int D, bool KVS>
 int launch_persist(const void* Q, const void* K, const void* V, void* out, int B, int H, int n, int d, float scale,
-                   int scheme, DeviceCounters* dc, DeviceCounters* dc_next, cudaStream_t stream) {
+                   int scheme, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next, cudaStream_t stream) {
     using Cfg = PCfg<D>;
     static DeviceSetup setup;
     const int sm_count = device_setup(&setup, [] {
@@ -669,25 +669,25 @@ int launch_persist(const void* Q, const void* K, const void* V, void* out, int B
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_persist_kernel<D, KVS>, maps, sp, H, scheme, (int)nitems,
-                                             scale * LOG2E, dc, dc_next);
+                                             scale * LOG2E, dc, cursor, dc_next);
     if (e != cudaSuccess) { set_cuda_error(e, "attn_persist_kernel launch"); return PSA_ERR_CUDA; }
     return PSA_OK;
 }
 
 }  // namespace
 
-// FULL and MASKED schemes.  `dc->next_item` must be zero when the kernel starts (the per-call clearing of the
+// FULL and MASKED schemes.  `*cursor` must be zero when the kernel starts (the per-call clearing of the
 // counter block does that); the kernel is launched once per call.
 int bf16_attention_persist(const void* Q, const void* K, const void* V, void* out, int B, int H, int n, int d,
-                           float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next, cudaStream_t stream) {
+                           float scale, int scheme, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next, cudaStream_t stream) {
     if (scheme != PSA_FULL && scheme != PSA_MASKED) return PSA_ERR_SCHEME_ARGS;
     if (d < 8 || d > 128 || d % 8) return PSA_ERR_UNSUPPORTED;
     if (K == V) {     // one tensor for keys and values: each key tile is loaded once
-        if (d <= 64) return launch_persist<64, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, dc_next, stream);
-        return launch_persist<128, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, dc_next, stream);
+        if (d <= 64) return launch_persist<64, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
+        return launch_persist<128, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
     }
-    if (d <= 64) return launch_persist<64, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, dc_next, stream);
-    return launch_persist<128, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, dc_next, stream);
+    if (d <= 64) return launch_persist<64, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
+    return launch_persist<128, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
 }
 
 }  // namespace psa

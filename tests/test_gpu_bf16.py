@@ -215,3 +215,29 @@ def test_symmetric_blocks_handed_on(B, H, n, d):
         assert (np.abs(_to_f64(out).reshape(ref.shape) - ref) <= TOL_BF16 + 2.0 ** -8 * np.abs(ref)).all()
         assert first is None or torch.equal(first.view(torch.int16), out.view(torch.int16))
         first = out
+
+
+# Host buffers of some size are worked off in parts of the batch (3 MB in and out each, at most 8), copies and kernels of
+# different parts at the same time: batches that do not divide evenly, one sequence per part, all schemes, wide heads,
+# pinned and pageable buffers; results, census and repeated calls as from one part on the device.
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("scheme,B,H,n,D,d", [(binding.FULL, 5, 12, 512, 768, 64), (binding.MASKED, 19, 4, 1000, 512, 128),
+                                              (binding.SYMMETRIC, 7, 8, 700, 512, 64), (binding.MASKED, 3, 4, 1500, 768, 192),
+                                              (binding.FULL, 2, 16, 2048, 1024, 64)])
+def test_host_batch_in_parts(scheme, B, H, n, D, d, pinned):
+    g = torch.Generator().manual_seed(B + n)
+    sym = scheme == binding.SYMMETRIC
+
+    def host(*shape, scale=1.0):
+        t = (torch.randn(*shape, generator=g) * scale).bfloat16()
+        return t.pin_memory() if pinned else t
+    X = host(B, n, D)
+    W = [host(D, H * d, scale=D ** -0.5) for _ in range(1 if sym else 3)] + ([None, None] if sym else [])
+    ref = binding.psa_attention(X.cuda(), *[None if w is None else w.cuda() for w in W], H, scheme).cpu()
+    for call in range(2):
+        out = torch.full((B, n, H * d), float("nan"), dtype=torch.bfloat16)
+        out = out.pin_memory() if pinned else out
+        binding.psa_attention_host(X, *W, H, scheme, out)
+        assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
+        st, got = binding.psa_last_issued()
+        assert st == binding.OK and got == binding.psa_skip_count(B, H, n, D, d, scheme, binding.BF16)
