@@ -211,8 +211,8 @@ int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv,
 int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K,
               const void* V, int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out,
               cudaStream_t stream, bool with_proj, char* ws, const WsLayout& L) {
-    // the paths whose last kernel clears the other counter block: the fused bf16 kernel and the one-launch fp32 layer
-    const bool turns = (dtype == PSA_BF16 && scheme != PSA_SYMMETRIC && d_k <= 128) ||
+    // the paths whose last kernel clears the other counter block: the fused bf16 kernels and the one-launch fp32 layer
+    const bool turns = (dtype == PSA_BF16 && scheme != PSA_SYMMETRIC) ||
                        (with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme));
     int block = 0;
     if (turns && cx.clean_ws == ws) {

@@ -145,3 +145,19 @@ def test_wide_heads_with_one_tensor_for_keys_and_values():
     ref, _ = oracle.attention_core(vq, vk, vk, oracle.MASKED)
     err = np.abs(_f64(out) - ref)
     assert (err <= TOL_BF16 + 2.0 ** -8 * np.abs(ref)).all(), err.max()
+
+
+# The wide kernel (128 < d_k <= 256) walks a work list with a CTA per SM: one block per item, more items than SMs, ragged last
+# tiles, and repeated calls (the work counter and the census start from zero each time).
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("B,H,n,d", [(1, 1, 1, 136), (20, 10, 100, 256), (3, 31, 260, 160), (2, 3, 1029, 256)])
+def test_wide_heads_work_list(scheme, B, H, n, d):
+    vals, bits = zip(*(inputs.tensor(5 * n + d, 4 + i, (B, n, H, d), 1.0, "bf16") for i in range(3)))
+    dev = [torch.from_numpy(np.ascontiguousarray(b).view(np.int16)).cuda().view(torch.bfloat16) for b in bits]
+    ref, _ = oracle.attention_core(*vals, scheme)
+    for call in range(3):
+        out = binding.psa_attention_core(*dev, scheme)
+        st, got = binding.psa_last_issued()
+        assert st == binding.OK and got == binding.psa_skip_count(B, H, n, 0, d, scheme, binding.BF16)
+        err = np.abs(out.float().cpu().numpy().astype(np.float64).reshape(ref.shape) - ref)
+        assert (err <= 2e-2 + 2.0 ** -8 * np.abs(ref)).all()
