@@ -4,6 +4,8 @@
 // the throughput path is the bf16 tensor-core one.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "psa_internal.h"
 
 namespace psa {
@@ -166,57 +168,71 @@ f32_project_tiled_kernel(const float* __restrict__ X, const float* W0, const flo
 // warp keeps run without tests, groups that nobody keeps are passed over, the rest is predicated weight by weight.  The
 // same limits bound phase 3.
 //
-// Shared-memory rows hold 64 DG floats as 16-byte chunks, chunk c of row r at c ^ (r % 8): 16-byte reads of 8 rows in
-// the same column, or of 8 neighbouring columns of one row, touch every bank once.
+// What bounds it: the fp32 pipe (100-105 multiply-accumulates per clock and SM measured in chains, 128 nominal) and, level with
+// it, instruction issue: phase 1 pairs components in two-wide fma, which leaves issue slots to its loads; phase 3 would have to
+// double every weight into a pair and runs on plain fma.  Measured (us, one warp per row before): 48 heads of n = 512, d = 64,
+// full 1554 -> 117; 16 heads of n = 1024, d = 128, masked 2003 -> 172; in a large call 61 multiply-accumulates per clock and SM.
+//
+// Shared memory, so that no address needs arithmetic in the inner loops: K rows are padded by 16 bytes (16 rows are read at
+// once), Q rows keep 16-byte chunk c at c ^ (row & 1) (rows of both half-warps are read at once), V rows are plain.
 constexpr int FA_THREADS = 128, FA_BC = 64;
-
-template <int DG> __device__ __forceinline__ int fa_off(int row, int chunk) { return row * (64 * DG) + ((chunk ^ (row & 7)) << 2); }
 
 template <int DG, int KS>
 struct FACfg {
+    static constexpr int DP = 64 * DG, KP = DP + 4;                     // row pitches of Q and V, of K, in floats
     static constexpr int BR = 64 / KS, U = 4 / KS, KW = FA_BC / KS;     // rows per CTA; key groups and keys of a warp
-    static constexpr int Q_FLOATS = BR * 64 * DG, KV_FLOATS = FA_BC * 64 * DG, P_FLOATS = 4 * 16 * KW;
-    static constexpr int SMEM = (Q_FLOATS + 2 * KV_FLOATS + P_FLOATS) * (int)sizeof(float);
-    static constexpr int PCH = KW / 4;                                  // 16-byte chunks of a row of P
+    static constexpr int PP = KW % 32 == 0 && !(DG == 2 && KS == 1) ? KW + 16 : KW;    // row pitch of P (the exception: room for two CTAs)
+    static constexpr int Q_FLOATS = BR * DP, K_FLOATS = FA_BC * KP, V_FLOATS = FA_BC * DP, P_FLOATS = 4 * 16 * PP;
+    static constexpr int SMEM = (Q_FLOATS + K_FLOATS + V_FLOATS + P_FLOATS) * (int)sizeof(float);
 };
-// P of a warp: 16 rows of KW weights, chunks permuted like the tiles above as far as a row has chunks
-template <int DG, int KS> __device__ __forceinline__ int fa_poff(int row, int chunk) {
-    using C = FACfg<DG, KS>;
-    return row * C::KW + ((chunk ^ (row & (C::PCH >= 8 ? 7 : C::PCH - 1))) << 2);
-}
 
-// Rows r0 .. r0 + nrows - 1 of one head into a tile (rows beyond n stay as they are; nothing reads them).
-template <int DG>
-__device__ __forceinline__ void fa_load(float* tile, const float* src, int r0, int nrows, int n, size_t ld, int d4) {
-    for (int t = threadIdx.x; t < nrows * 16 * DG; t += FA_THREADS) {
-        const int r = t / (16 * DG), c = t % (16 * DG);
-        if (c < d4 && r0 + r < n) cp_async16(tile + fa_off<DG>(r, c), src + (size_t)(r0 + r) * ld + 4 * c);
+// Rows r0 .. r0 + ROWS - 1 of one head into a tile of row pitch PITCH (rows beyond n stay as they are; nothing reads them).
+template <int DG, int ROWS, int PITCH, bool SWAP>
+__device__ __forceinline__ void fa_load(float* tile, const float* src, int r0, int n, size_t ld, int d4) {
+    const int c = threadIdx.x % (16 * DG), r = threadIdx.x / (16 * DG);
+    constexpr int STEP = FA_THREADS / (16 * DG);
+    if (c >= d4) return;
+    const float* p = src + (size_t)(r0 + r) * ld + 4 * c;
+    float* dst = tile + r * PITCH;
+#pragma unroll
+    for (int k = 0; k < ROWS / STEP; ++k) {
+        if (r0 + r + k * STEP < n) cp_async16(dst + k * STEP * PITCH + 4 * (SWAP ? c ^ ((r + k * STEP) & 1) : c), p + (size_t)(k * STEP) * ld);
     }
 }
 
-// acc[i][u] (+)= q_i . k_u, sums of even and odd components side by side.  EDGE: only the weights with keep true.
+// acc[i][u] += q_i . k_u, sums of even and odd components side by side.  q: row ty of the warp's rows, k: row tx of its keys.
+// EDGE: only the weights that are kept.
 template <int DG, int U, bool EDGE>
-__device__ __forceinline__ void fa_scores(unsigned long long (&acc)[8][U], const float* Q, const float* K, int qrow, int krow,
-                                          int d4, const int (&lim)[8], int tx, int minlim, int maxlim) {
-#pragma unroll 4
-    for (int c = 0; c < d4; ++c) {
-        ulonglong2 k[U];
+__device__ __forceinline__ void fa_scores(unsigned long long (&acc)[8][U], const float* q, const float* k, int d4, int tx, int ty,
+                                          const int (&lim)[8], int minlim, int maxlim) {
+    constexpr int DP = 64 * DG, KP = DP + 4;
+    auto step = [&](const float* qc, const float* kc) {
+        ulonglong2 kv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) k[u] = *reinterpret_cast<const ulonglong2*>(K + fa_off<DG>(krow + 16 * u, c));
+        for (int u = 0; u < U; ++u) kv[u] = *reinterpret_cast<const ulonglong2*>(kc + 16 * u * KP);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(Q + fa_off<DG>(qrow + 2 * i, c));
+            const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(qc + 2 * i * DP);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (EDGE) {
                     if (16 * u > maxlim) continue;                                  // (same for the whole warp)
                     if (16 * u + 15 > minlim && tx + 16 * u > lim[i]) continue;
                 }
-                fma2(acc[i][u], q.x, k[u].x);
-                fma2(acc[i][u], q.y, k[u].y);
+                fma2(acc[i][u], qv.x, kv[u].x);
+                fma2(acc[i][u], qv.y, kv[u].y);
             }
         }
+    };
+    const float* qe = q + 4 * ty;           // chunks of even number of this lane's rows, and of odd number
+    const float* qo = q - 4 * ty;
+    int c = 0;
+#pragma unroll 1
+    for (; c + 1 < d4; c += 2) {
+        step(qe + 4 * c, k + 4 * c);
+        step(qo + 4 * c + 4, k + 4 * c + 4);
     }
+    if (c < d4) step(qe + 4 * c, k + 4 * c);
 }
 
 // MODE 0: the three phases for FULL / MASKED.  MODE 2: phases 2 and 3 of the symmetric scheme, scores read from S.
@@ -230,8 +246,8 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     extern __shared__ float4 fa_smem4[];
     float* Qs = reinterpret_cast<float*>(fa_smem4);
     float* Ks = Qs + C::Q_FLOATS;
-    float* Vs = Ks + C::KV_FLOATS;
-    float* Ps = Vs + C::KV_FLOATS;
+    float* Vs = Ks + C::K_FLOATS;
+    float* Ps = Vs + C::V_FLOATS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
     const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
     const int rb = masked ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // the longest rows first
@@ -245,135 +261,150 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     const int kend = masked ? min(r0 + C::BR, n) : n;                   // keys that some row of the CTA keeps
     const int nblk = (kend + FA_BC - 1) / FA_BC;
     const float* Sh = MODE == 2 ? S + (size_t)bh * n * n : nullptr;
-    float* Pw = Ps + warp * 16 * C::KW;
+    float* Pw = Ps + warp * 16 * C::PP;
+    const float* Pr = Pw + ty * C::PP;                                  // row i of the lane: + 2 i PP
+    const float* vb = Vs + kw * C::DP + 4 * tx;
     const bool act0 = tx < d4, act1 = DG == 2 && 16 + tx < d4;          // output columns this lane owns
 
     if (MODE != 2) {
-        fa_load<DG>(Qs, Q + base, r0, C::BR, n, ld, d4);
-        fa_load<DG>(Ks, K + base, 0, FA_BC, n, ld, d4);
+        fa_load<DG, C::BR, C::DP, true>(Qs, Q + base, r0, n, ld, d4);
+        fa_load<DG, FA_BC, C::KP, false>(Ks, K + base, 0, n, ld, d4);
     }
     cp_async_commit();
 
-    float m[8], l[8];
-    unsigned long long o[8][2 * DG] = {};
+    float m[8], l[8], o[8][4 * DG];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
-    unsigned long long dots = 0, wts = 0;                               // weights of this lane; of its rows in phase 3
+    for (int i = 0; i < 8; ++i) {
+        m[i] = -INFINITY; l[i] = 0.f;
+#pragma unroll
+        for (int g = 0; g < 4 * DG; ++g) o[i][g] = 0.f;
+    }
+    unsigned int dots = 0, wts = 0;                                     // weights of this lane; of its rows in phase 3
 
     for (int jb = 0; jb < nblk; ++jb) {
         const int k0 = jb * FA_BC + kw;                                 // first key of the warp's share
-        int lim[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) lim[i] = row + 2 * i >= n ? -1 : min(masked ? row + 2 * i : n - 1, n - 1) - k0;
         const int last = min(wr0 + 15, n - 1);                          // last row of the warp that exists
         const int maxlim = wr0 >= n ? -1 : (masked ? last : n - 1) - k0;
         const int minlim = wr0 + 15 >= n ? -1 : (masked ? wr0 : n - 1) - k0;
-        const bool whole = minlim >= C::KW - 1;
 
-        float s[8][U];
         if (MODE != 2) cp_async_wait_all();
         __syncthreads();            // K_j has landed; every warp is done with V_{j-1}
-        fa_load<DG>(Vs, V + base, jb * FA_BC, FA_BC, n, ld, d4);
+        fa_load<DG, FA_BC, C::DP, false>(Vs, V + base, jb * FA_BC, n, ld, d4);
         cp_async_commit();
-        // ---- phase 1 (Eq. 1)
-        if (MODE == 2) {
+        auto block = [&](auto edge_tag) {
+            constexpr bool EDGE = decltype(edge_tag)::value;
+            int lim[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 8; ++i) lim[i] = !EDGE ? C::KW - 1 : row + 2 * i >= n ? -1 : min(masked ? row + 2 * i : n - 1, n - 1) - k0;
+            float s[8][U];
+            // ---- phase 1 (Eq. 1)
+            if (MODE == 2) {
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    s[i][u] = tx + 16 * u <= lim[i] ? __ldg(Sh + (size_t)(row + 2 * i) * n + k0 + tx + 16 * u) : -INFINITY;
-        } else {
-            unsigned long long acc[8][U] = {};
-            if (whole) {
-                fa_scores<DG, U, false>(acc, Qs, Ks, qrow, kw + tx, d4, lim, tx, minlim, maxlim);
-                dots += 8 * U;
-            } else if (maxlim >= 0) {
-                fa_scores<DG, U, true>(acc, Qs, Ks, qrow, kw + tx, d4, lim, tx, minlim, maxlim);
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        s[i][u] = !EDGE || tx + 16 * u <= lim[i] ? __ldg(Sh + (size_t)(row + 2 * i) * n + k0 + tx + 16 * u) : -INFINITY;
+            } else {
+                unsigned long long acc[8][U] = {};
+                if (!EDGE || maxlim >= 0)
+                    fa_scores<DG, U, EDGE>(acc, Qs + qrow * C::DP, Ks + (kw + tx) * C::KP, d4, tx, ty, lim, minlim, maxlim);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const float2 f = unpack2(acc[i][u]);
+                        s[i][u] = (f.x + f.y) * scale;
+                        if (EDGE) {
+                            const bool keep = tx + 16 * u <= lim[i];
+                            s[i][u] = keep ? s[i][u] : -INFINITY;
+                            dots += keep;
+                        }
+                    }
+                if (!EDGE) dots += 8 * U;
             }
+            // ---- phase 2 (Eq. 2): running row maximum and sum; the sum stays per lane until the end
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 8; ++i) {
+                float mx = s[i][0];
+#pragma unroll
+                for (int u = 1; u < U; ++u) mx = fmaxf(mx, s[i][u]);
+#pragma unroll
+                for (int off = 8; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                mx = fmaxf(mx, m[i]);
+                const float sub = mx == -INFINITY ? 0.f : mx;           // (no finite score yet: every weight is 0)
+                if (mx != m[i]) {
+                    const float alpha = expf(m[i] - mx);
+                    m[i] = mx;
+                    l[i] *= alpha;
+#pragma unroll
+                    for (int g = 0; g < 4 * DG; ++g) o[i][g] *= alpha;
+                }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const float2 f = unpack2(acc[i][u]);
-                    s[i][u] = (f.x + f.y) * scale;
-                    if (!whole) {
-                        const bool keep = tx + 16 * u <= lim[i];
-                        s[i][u] = keep ? s[i][u] : -INFINITY;
-                        dots += keep;
+                    if (!EDGE || tx + 16 * u <= lim[i]) {
+                        const float e = expf(s[i][u] - sub);
+                        l[i] += e;
+                        Pw[(ty + 2 * i) * C::PP + tx + 16 * u] = e;
                     }
                 }
-        }
-        // ---- phase 2 (Eq. 2): running row maximum and sum; the sum stays per lane until the end
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float mx = s[i][0];
-#pragma unroll
-            for (int u = 1; u < U; ++u) mx = fmaxf(mx, s[i][u]);
-#pragma unroll
-            for (int off = 8; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            mx = fmaxf(mx, m[i]);
-            const float sub = mx == -INFINITY ? 0.f : mx;               // (no finite score yet: every weight is 0)
-            if (mx != m[i]) {
-                const float alpha = expf(m[i] - mx);
-                m[i] = mx;
-                l[i] *= alpha;
-                const unsigned long long a2 = dup2(alpha);
-#pragma unroll
-                for (int g = 0; g < 2 * DG; ++g) asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(o[i][g]) : "l"(a2));
+                if (EDGE && tx == 0) wts += min(max(lim[i] + 1, 0), C::KW);
             }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (whole || tx + 16 * u <= lim[i]) {
-                    const float e = expf(s[i][u] - sub);
-                    l[i] += e;
-                    Pw[fa_poff<DG, KS>(ty + 2 * i, (tx >> 2) + 4 * u) + (tx & 3)] = e;
-                }
-            }
-            if (tx == 0) wts += min(max(lim[i] + 1, 0), C::KW);
-        }
+            if (!EDGE && tx == 0) wts += 8 * C::KW;
+        };
+        const bool whole = minlim >= C::KW - 1;
+        if (whole) block(std::false_type{});
+        else block(std::true_type{});
         cp_async_wait_all();
         __syncthreads();            // V_j has landed, P is written; every warp is done with K_j
-        if (MODE != 2 && jb + 1 < nblk) fa_load<DG>(Ks, K + base, (jb + 1) * FA_BC, FA_BC, n, ld, d4);
+        if (MODE != 2 && jb + 1 < nblk) fa_load<DG, FA_BC, C::KP, false>(Ks, K + base, (jb + 1) * FA_BC, n, ld, d4);
         cp_async_commit();
         // ---- phase 3 (Eq. 3): keys in order, the warp's columns of V against its weights
         if (act0) {
             const int jfull = whole ? C::KW : (minlim + 1 > 0 ? (minlim + 1) & ~3 : 0);
-            const float* vb = Vs + kw * 64 * DG;                        // (kw is a multiple of 16: rows keep their phase)
-            for (int j = 0; j < jfull; j += 4) {
+            const float* pj = Pr;
+            const float* vj = vb;
+#pragma unroll 1
+            for (int j = 0; j < jfull; j += 4, pj += 4, vj += 4 * C::DP) {
                 float4 p[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) p[i] = *reinterpret_cast<const float4*>(Pw + fa_poff<DG, KS>(ty + 2 * i, j >> 2));
+                for (int i = 0; i < 8; ++i) p[i] = *reinterpret_cast<const float4*>(pj + 2 * i * C::PP);
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj) {
-                    ulonglong2 v[DG];
-                    v[0] = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j + jj, tx));
-                    if (DG == 2 && act1) v[DG - 1] = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j + jj, 16 + tx));
+                    const float4 v0 = *reinterpret_cast<const float4*>(vj + jj * C::DP);
+                    float4 v1 = v0;
+                    if (DG == 2 && act1) v1 = *reinterpret_cast<const float4*>(vj + jj * C::DP + 64);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        const unsigned long long w = dup2(jj == 0 ? p[i].x : jj == 1 ? p[i].y : jj == 2 ? p[i].z : p[i].w);
-                        fma2(o[i][0], w, v[0].x);
-                        fma2(o[i][1], w, v[0].y);
+                        const float w = jj == 0 ? p[i].x : jj == 1 ? p[i].y : jj == 2 ? p[i].z : p[i].w;
+                        o[i][0] = fmaf(w, v0.x, o[i][0]); o[i][1] = fmaf(w, v0.y, o[i][1]);
+                        o[i][2] = fmaf(w, v0.z, o[i][2]); o[i][3] = fmaf(w, v0.w, o[i][3]);
                         if (DG == 2 && act1) {
-                            fma2(o[i][2 * DG - 2], w, v[DG - 1].x);
-                            fma2(o[i][2 * DG - 1], w, v[DG - 1].y);
+                            o[i][4 * DG - 4] = fmaf(w, v1.x, o[i][4 * DG - 4]); o[i][4 * DG - 3] = fmaf(w, v1.y, o[i][4 * DG - 3]);
+                            o[i][4 * DG - 2] = fmaf(w, v1.z, o[i][4 * DG - 2]); o[i][4 * DG - 1] = fmaf(w, v1.w, o[i][4 * DG - 1]);
                         }
                     }
                 }
             }
             if (!whole) {
                 const int jend = min(maxlim + 1, C::KW);
+                int lim[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) lim[i] = row + 2 * i >= n ? -1 : min(masked ? row + 2 * i : n - 1, n - 1) - k0;
 #pragma unroll 1
-                for (int j = jfull; j < jend; ++j) {
-                    const ulonglong2 v0 = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j, tx));
-                    ulonglong2 v1 = v0;
-                    if (DG == 2 && act1) v1 = *reinterpret_cast<const ulonglong2*>(vb + fa_off<DG>(j, 16 + tx));
+                for (int j = jfull; j < jend; ++j, ++pj, vj += C::DP) {
+                    const float4 v0 = *reinterpret_cast<const float4*>(vj);
+                    float4 v1 = v0;
+                    if (DG == 2 && act1) v1 = *reinterpret_cast<const float4*>(vj + 64);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         if (j > lim[i]) continue;
-                        const unsigned long long w = dup2(Pw[fa_poff<DG, KS>(ty + 2 * i, j >> 2) + (j & 3)]);
-                        fma2(o[i][0], w, v0.x);
-                        fma2(o[i][1], w, v0.y);
-                        if (DG == 2 && act1) { fma2(o[i][2 * DG - 2], w, v1.x); fma2(o[i][2 * DG - 1], w, v1.y); }
+                        const float w = pj[2 * i * C::PP];
+                        o[i][0] = fmaf(w, v0.x, o[i][0]); o[i][1] = fmaf(w, v0.y, o[i][1]);
+                        o[i][2] = fmaf(w, v0.z, o[i][2]); o[i][3] = fmaf(w, v0.w, o[i][3]);
+                        if (DG == 2 && act1) {
+                            o[i][4 * DG - 4] = fmaf(w, v1.x, o[i][4 * DG - 4]); o[i][4 * DG - 3] = fmaf(w, v1.y, o[i][4 * DG - 3]);
+                            o[i][4 * DG - 2] = fmaf(w, v1.z, o[i][4 * DG - 2]); o[i][4 * DG - 1] = fmaf(w, v1.w, o[i][4 * DG - 1]);
+                        }
                     }
                 }
             }
@@ -391,26 +422,22 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
             const float inv = 1.f / l[i];
             float* dst = out + base + (size_t)(row + 2 * i) * ld + 4 * tx;
 #pragma unroll
-            for (int g = 0; g < DG; ++g) {
-                if (!(g == 0 ? act0 : act1)) continue;
-                const float2 lo = unpack2(o[i][2 * g]), hi = unpack2(o[i][2 * g + 1]);
-                *reinterpret_cast<float4*>(dst + 64 * g) = make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv);
-            }
+            for (int g = 0; g < DG; ++g)
+                if (g == 0 ? act0 : act1)
+                    *reinterpret_cast<float4*>(dst + 64 * g) = make_float4(o[i][4 * g] * inv, o[i][4 * g + 1] * inv, o[i][4 * g + 2] * inv, o[i][4 * g + 3] * inv);
         }
     } else {
         // the KS partial results of a row, brought to their common maximum and added up
         __syncthreads();            // every warp is done with V and P
-        float* part = Ks;           // [KS][BR][64 DG], over the K tile
+        float* part = Ks;           // [KS][BR][DP], over the K tile
         float* ml = Ps;             // [KS][BR] maxima, then [KS][BR] sums
         const int ks = warp % KS;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int r = qrow + 2 * i;
 #pragma unroll
-            for (int g = 0; g < DG; ++g) {
-                const float2 lo = unpack2(o[i][2 * g]), hi = unpack2(o[i][2 * g + 1]);
-                *reinterpret_cast<float4*>(part + (size_t)(ks * C::BR + r) * 64 * DG + 64 * g + 4 * tx) = make_float4(lo.x, lo.y, hi.x, hi.y);
-            }
+            for (int g = 0; g < DG; ++g)
+                *reinterpret_cast<float4*>(part + (size_t)(ks * C::BR + r) * C::DP + 64 * g + 4 * tx) = make_float4(o[i][4 * g], o[i][4 * g + 1], o[i][4 * g + 2], o[i][4 * g + 3]);
             if (tx == 0) { ml[ks * C::BR + r] = m[i]; ml[KS * C::BR + ks * C::BR + r] = l[i]; }
         }
         __syncthreads();
@@ -427,7 +454,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
                 const float mk = ml[k * C::BR + r];
                 if (mk == -INFINITY && ml[KS * C::BR + k * C::BR + r] == 0.f) continue;      // no key of this share counts
                 const float w = mk == mx ? 1.f : expf(mk - mx);
-                const float4 f = *reinterpret_cast<const float4*>(part + (size_t)(k * C::BR + r) * 64 * DG + 4 * c);
+                const float4 f = *reinterpret_cast<const float4*>(part + (size_t)(k * C::BR + r) * C::DP + 4 * c);
                 sum = fmaf(w, ml[KS * C::BR + k * C::BR + r], sum);
                 y.x = fmaf(w, f.x, y.x); y.y = fmaf(w, f.y, y.y); y.z = fmaf(w, f.z, y.z); y.w = fmaf(w, f.w, y.w);
             }
@@ -441,8 +468,8 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
         wts += __shfl_xor_sync(0xffffffffu, wts, off);
     }
     if (lane == 0) {
-        if (MODE != 2 && dots) atomicAdd(&dc->qk_macs, dots * (unsigned long long)d);
-        if (wts) { atomicAdd(&dc->pv_macs, wts * (unsigned long long)d); atomicAdd(&dc->exps, wts); }
+        if (MODE != 2 && dots) atomicAdd(&dc->qk_macs, (unsigned long long)dots * d);
+        if (wts) { atomicAdd(&dc->pv_macs, (unsigned long long)wts * d); atomicAdd(&dc->exps, (unsigned long long)wts); }
     }
 }
 
@@ -451,17 +478,18 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 template <int DG>
 __global__ void __launch_bounds__(FA_THREADS)
 f32_sym_scores_kernel(const float* __restrict__ X, float* __restrict__ S, int n, int H, int d, float scale, DeviceCounters* dc) {
+    using C = FACfg<DG, 1>;
     extern __shared__ float4 fa_smem4[];
     float* Qs = reinterpret_cast<float*>(fa_smem4);
-    float* Ks = Qs + 64 * 64 * DG;
+    float* Ks = Qs + C::Q_FLOATS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
     const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
     int I = 0, t = blockIdx.y;
     while (t > I) { t -= I + 1; ++I; }
     const int r0 = 64 * I, c0 = 64 * t;
     const size_t ld = (size_t)H * d, base = ((size_t)b * n) * ld + (size_t)h * d;
-    fa_load<DG>(Qs, X + base, r0, 64, n, ld, d >> 2);
-    fa_load<DG>(Ks, X + base, c0, 64, n, ld, d >> 2);
+    fa_load<DG, 64, C::DP, true>(Qs, X + base, r0, n, ld, d >> 2);
+    fa_load<DG, 64, C::KP, false>(Ks, X + base, c0, n, ld, d >> 2);
     cp_async_wait_all();
     __syncthreads();
     const int qrow = 16 * warp + ty, row = r0 + qrow, wr0 = r0 + 16 * warp;
@@ -470,8 +498,8 @@ f32_sym_scores_kernel(const float* __restrict__ X, float* __restrict__ S, int n,
     for (int i = 0; i < 8; ++i) lim[i] = row + 2 * i >= n ? -1 : row + 2 * i - c0;
     const int maxlim = wr0 >= n ? -1 : min(wr0 + 15, n - 1) - c0, minlim = wr0 + 15 >= n ? -1 : wr0 - c0;
     unsigned long long acc[8][4] = {}, dots = 0;
-    if (minlim >= 63) fa_scores<DG, 4, false>(acc, Qs, Ks, qrow, tx, d >> 2, lim, tx, minlim, maxlim);
-    else if (maxlim >= 0) fa_scores<DG, 4, true>(acc, Qs, Ks, qrow, tx, d >> 2, lim, tx, minlim, maxlim);
+    if (minlim >= 63) fa_scores<DG, 4, false>(acc, Qs + qrow * C::DP, Ks + tx * C::KP, d >> 2, tx, ty, lim, minlim, maxlim);
+    else if (maxlim >= 0) fa_scores<DG, 4, true>(acc, Qs + qrow * C::DP, Ks + tx * C::KP, d >> 2, tx, ty, lim, minlim, maxlim);
     __syncthreads();                // the operand tiles become the block's staging buffer, [64][65]
     float* Sh = S + (size_t)bh * n * n;
 #pragma unroll
@@ -1111,8 +1139,8 @@ cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, f
     if (sms <= 0) return cudaErrorUnknown;
     auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
     // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs:
-    // measured, two resident CTAs per SM are where the line lies (us for KS = 1 / 2 / 4).  80 tiles of 64 rows: 208 / 144 /
-    // 112; 256 tiles, masked, d = 128: 268 / 216 / 252; 384 tiles: 137 / 155 / 180.
+    // measured, two resident CTAs per SM are where the line lies (us for KS = 1 / 2 / 4, with the first form of the kernel).  80
+    // tiles of 64 rows: 208 / 144 / 112; 256 tiles, masked, d = 128: 268 / 216 / 252; 384 tiles: 137 / 155 / 180.
     if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
     if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
     return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
@@ -1122,7 +1150,7 @@ cudaError_t tiled_attention(const float* Q, const float* K, const float* V, floa
                             float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
     if (scheme != PSA_SYMMETRIC)
         return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, stream);
-    constexpr int SMEM = 2 * 64 * 64 * DG * (int)sizeof(float);
+    constexpr int SMEM = (FACfg<DG, 1>::Q_FLOATS + FACfg<DG, 1>::K_FLOATS) * (int)sizeof(float);
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
             return cudaFuncSetAttribute(f32_sym_scores_kernel<DG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
