@@ -66,45 +66,41 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Projection, tiled: BM x BN outputs per CTA, TM x TN per thread (rows strided by BM / TM, columns in groups of four),
-// operands staged GP_STAGES deep with asynchronous copies.  Every output is the same chain of fmaf over k = 0, 1, ...
-// as in f32_project_kernel, so the results are bitwise the same.  Needs D and N to be multiples of 4.
-constexpr int GP_BK = 32, GP_LDA = GP_BK + 4, GP_STAGES = 3;
-template <int BM, int BN, int TM, int TN>
-struct GPCfg {
-    static constexpr int TX = BN / TN, TY = BM / TM, THREADS = TX * TY;
-    static constexpr int A_FLOATS = BM * GP_LDA, B_FLOATS = GP_BK * BN, STAGE = A_FLOATS + B_FLOATS;
-    static constexpr int SMEM = GP_STAGES * STAGE * (int)sizeof(float);
-};
-template <int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__(GPCfg<BM, BN, TM, TN>::THREADS, 2)
+// Projection of small calls on CUDA cores: 32 x 32 outputs per CTA of 128 threads, two rows 16 apart by four columns per
+// thread, operands staged GP_STAGES deep with asynchronous copies.  Every output is the same chain of fmaf over k = 0, 1, ...
+// as in f32_project_kernel, so the results are bitwise the same.  Needs D and N to be multiples of 4.  Bound by the latency of
+// its k-steps: 768 deep, 16 ... 256 rows take 23-30 us.
+constexpr int GP_BM = 32, GP_BN = 32, GP_TM = 2, GP_BK = 32, GP_LDA = GP_BK + 4, GP_STAGES = 3;
+constexpr int GP_TX = GP_BN / 4, GP_TY = GP_BM / GP_TM, GP_THREADS = GP_TX * GP_TY;
+constexpr int GP_A_FLOATS = GP_BM * GP_LDA, GP_STAGE = GP_A_FLOATS + GP_BK * GP_BN;
+constexpr int GP_SMEM = GP_STAGES * GP_STAGE * (int)sizeof(float);
+
+__global__ void __launch_bounds__(GP_THREADS)
 f32_project_tiled_kernel(const float* __restrict__ X, const float* W0, const float* W1, const float* W2, float* O0,
                          float* O1, float* O2, int rows, int D, int N, const float* __restrict__ R, DeviceCounters* dc) {
-    using C = GPCfg<BM, BN, TM, TN>;
-    static_assert(C::TX % 8 == 0 && C::TY % 4 == 0 && TN % 4 == 0, "a warp is 4 x 8 threads");
     extern __shared__ float4 gp_smem4[];
     float* sm = reinterpret_cast<float*>(gp_smem4);
     const float* W = blockIdx.z == 0 ? W0 : (blockIdx.z == 1 ? W1 : W2);
     float* O = blockIdx.z == 0 ? O0 : (blockIdx.z == 1 ? O1 : O2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tx = (warp % (C::TX / 8)) * 8 + (lane & 7), ty = (warp / (C::TX / 8)) * 4 + (lane >> 3);
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int tx = lane & 7, ty = warp * 4 + (lane >> 3);
+    const int m0 = blockIdx.y * GP_BM, n0 = blockIdx.x * GP_BN;
     const int nk = (D + GP_BK - 1) / GP_BK;
 
     auto load = [&](int kt) {       // k-step kt: rows beyond the matrix are clamped, columns of k beyond D skipped
-        float* a = sm + (kt % GP_STAGES) * C::STAGE;
-        float* b = a + C::A_FLOATS;
+        float* a = sm + (kt % GP_STAGES) * GP_STAGE;
+        float* b = a + GP_A_FLOATS;
         const int k0 = kt * GP_BK;
-        for (int t = tid; t < BM * (GP_BK / 4); t += C::THREADS) {
+        for (int t = tid; t < GP_BM * (GP_BK / 4); t += GP_THREADS) {
             const int r = t / (GP_BK / 4), c = (t % (GP_BK / 4)) * 4;
             if (k0 + c < D) cp_async16(a + r * GP_LDA + c, X + (size_t)min(m0 + r, rows - 1) * D + k0 + c);
         }
-        for (int t = tid; t < GP_BK * (BN / 4); t += C::THREADS) {
-            const int k = t / (BN / 4), c = (t % (BN / 4)) * 4;
-            if (k0 + k < D) cp_async16(b + k * BN + c, W + (size_t)(k0 + k) * N + min(n0 + c, N - 4));
+        for (int t = tid; t < GP_BK * (GP_BN / 4); t += GP_THREADS) {
+            const int k = t / (GP_BN / 4), c = (t % (GP_BN / 4)) * 4;
+            if (k0 + k < D) cp_async16(b + k * GP_BN + c, W + (size_t)(k0 + k) * N + min(n0 + c, N - 4));
         }
     };
-    unsigned long long acc[TM][TN / 2] = {};
+    unsigned long long acc[GP_TM][2] = {};
 #pragma unroll
     for (int s = 0; s < GP_STAGES - 1; ++s) {
         if (s < nk) load(s);
@@ -115,47 +111,42 @@ f32_project_tiled_kernel(const float* __restrict__ X, const float* W0, const flo
         __syncthreads();            // step kt has landed, and step kt - 1's buffer is free
         if (kt + GP_STAGES - 1 < nk) load(kt + GP_STAGES - 1);
         cp_async_commit();
-        const float* a = sm + (kt % GP_STAGES) * C::STAGE + ty * GP_LDA;
-        const float* b = sm + (kt % GP_STAGES) * C::STAGE + C::A_FLOATS + 4 * tx;
+        const float* a = sm + (kt % GP_STAGES) * GP_STAGE + ty * GP_LDA;
+        const float* b = sm + (kt % GP_STAGES) * GP_STAGE + GP_A_FLOATS + 4 * tx;
         const int kn = min(GP_BK, D - kt * GP_BK);
 #pragma unroll 2
         for (int k = 0; k < kn; k += 4) {
-            float4 av[TM];
+            float4 av[GP_TM];
 #pragma unroll
-            for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a + i * C::TY * GP_LDA + k);
+            for (int i = 0; i < GP_TM; ++i) av[i] = *reinterpret_cast<const float4*>(a + i * GP_TY * GP_LDA + k);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                ulonglong2 bv[TN / 4];
+                const ulonglong2 bv = *reinterpret_cast<const ulonglong2*>(b + (k + kk) * GP_BN);
 #pragma unroll
-                for (int g = 0; g < TN / 4; ++g) bv[g] = *reinterpret_cast<const ulonglong2*>(b + (k + kk) * BN + g * 4 * C::TX);
-#pragma unroll
-                for (int i = 0; i < TM; ++i) {
+                for (int i = 0; i < GP_TM; ++i) {
                     const unsigned long long x = dup2(kk == 0 ? av[i].x : kk == 1 ? av[i].y : kk == 2 ? av[i].z : av[i].w);
-#pragma unroll
-                    for (int g = 0; g < TN / 4; ++g) { fma2(acc[i][2 * g], x, bv[g].x); fma2(acc[i][2 * g + 1], x, bv[g].y); }
+                    fma2(acc[i][0], x, bv.x);
+                    fma2(acc[i][1], x, bv.y);
                 }
             }
         }
     }
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int r = m0 + ty + i * C::TY;
+    for (int i = 0; i < GP_TM; ++i) {
+        const int r = m0 + ty + i * GP_TY;
         if (r >= rows) continue;
-#pragma unroll
-        for (int g = 0; g < TN / 4; ++g) {
-            const int c = n0 + 4 * tx + g * 4 * C::TX;
-            if (c >= N) continue;
-            const float2 lo = unpack2(acc[i][2 * g]), hi = unpack2(acc[i][2 * g + 1]);
-            float4 o = make_float4(lo.x, lo.y, hi.x, hi.y);
-            if (R) {
-                const float4 x = *reinterpret_cast<const float4*>(R + (size_t)r * N + c);
-                o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
-            }
-            *reinterpret_cast<float4*>(O + (size_t)r * N + c) = o;
+        const int c = n0 + 4 * tx;
+        if (c >= N) continue;
+        const float2 lo = unpack2(acc[i][0]), hi = unpack2(acc[i][1]);
+        float4 o = make_float4(lo.x, lo.y, hi.x, hi.y);
+        if (R) {
+            const float4 x = *reinterpret_cast<const float4*>(R + (size_t)r * N + c);
+            o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
         }
+        *reinterpret_cast<float4*>(O + (size_t)r * N + c) = o;
     }
     if (tid == 0)
-        atomicAdd(&dc->proj_macs, (unsigned long long)min(BM, rows - m0) * min(BN, N - n0) * D);
+        atomicAdd(&dc->proj_macs, (unsigned long long)min(GP_BM, rows - m0) * min(GP_BN, N - n0) * D);
 }
 
 // Attention, tiled: a CTA of four warps works on BR = 64 / KS query rows of one (batch, head) and walks the keys in
@@ -1028,15 +1019,6 @@ size_t attn_smem_bytes(int n, int d) {
 namespace {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-template <int BM, int BN, int TM, int TN>
-cudaError_t launch_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
-                           const float* residual, DeviceCounters* dc, cudaStream_t stream) {
-    using C = GPCfg<BM, BN, TM, TN>;
-    const dim3 grid((N + BN - 1) / BN, (rows + BM - 1) / BM, nW);
-    f32_project_tiled_kernel<BM, BN, TM, TN><<<grid, C::THREADS, C::SMEM, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2],
-                                                                                    rows, D, N, residual, dc);
-    return cudaGetLastError();
-}
 }  // namespace
 
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
@@ -1046,19 +1028,17 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
     // (grid.y holds 65535 row tiles)
     if (tiled && (rows + 31) / 32 <= 65535) {
         static DeviceSetup setup;
-        const int sms = device_setup(&setup, [] {
-            cudaError_t e = cudaFuncSetAttribute(f32_project_tiled_kernel<128, 128, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 GPCfg<128, 128, 8, 8>::SMEM);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(f32_project_tiled_kernel<64, 64, 4, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         GPCfg<64, 64, 4, 8>::SMEM);
-            return e;
-        }, "fp32 projection set-up");
+        const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 projection set-up");
         if (sms <= 0) return cudaErrorUnknown;
-        auto tiles = [&](int t) { return (long long)((rows + t - 1) / t) * ((N + t - 1) / t) * nW; };
-        if (tiles(128) >= sms) return launch_project<128, 128, 8, 8>(X, W, out, nW, rows, D, N, residual, dc, stream);
-        if (tiles(64) >= sms) return launch_project<64, 64, 4, 8>(X, W, out, nW, rows, D, N, residual, dc, stream);
-        return launch_project<32, 32, 2, 4>(X, W, out, nW, rows, D, N, residual, dc, stream);
+        // The tensor cores from two 32 x 32 tiles per SM on, by measurement (us, 32 x 32 tiles on CUDA cores / tensor cores):
+        // 64 x 768 x 3 x 64 23.5 / 32.3, 128 x 768 x 3 x 768 (288 tiles) 29.6 / 33.6, 2048 x 768 x 3 x 64 (384) 37.5 / 33.4,
+        // 600 x 320 x 3 x 320 (570) 27.3 / 21.3, 64 x 2048 x 3 x 2048 (384) 89 / 72; larger ones, against 128 x 128 tiles on CUDA
+        // cores, 2048 x 768 x 3 x 768 171 / 70.
+        const long long tiles = (long long)((rows + 31) / 32) * ((N + 31) / 32) * nW;
+        if (tiles > 2 * sms) return f32_project_tensor(X, W, out, nW, rows, D, N, residual, dc, stream);
+        const dim3 grid((N + GP_BN - 1) / GP_BN, (rows + GP_BM - 1) / GP_BM, nW);
+        f32_project_tiled_kernel<<<grid, GP_THREADS, GP_SMEM, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);
+        return cudaGetLastError();
     }
     dim3 block(PROJ_TILE, PROJ_TILE), grid((N + PROJ_TILE - 1) / PROJ_TILE, (rows + PROJ_TILE - 1) / PROJ_TILE, nW);
     f32_project_kernel<<<grid, block, 0, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);

@@ -26,6 +26,9 @@ struct DeviceCounters {
 // `residual` ([rows, N], may be null) is added to every output.
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
                         int N, const float* residual, DeviceCounters* dc, cudaStream_t stream);
+// The same on the tensor cores, to the same accuracy (psa_f32_tensor.cu); f32_project chooses.  Rows of 16 bytes, as there.
+cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
+                               const float* residual, DeviceCounters* dc, cudaStream_t stream);
 // Q, K, V, out: [B, n, H, d] fp32.  S: scratch [B*H, n, n] fp32, used by PSA_SYMMETRIC only.
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H,
                           int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream);

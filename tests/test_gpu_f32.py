@@ -137,17 +137,56 @@ def test_core_with_infinite_scores(n, H):
     assert np.isnan(masked[:130]).all() and np.isfinite(masked[130:]).all()
 
 
-# Tile sizes of the projection (128, 64 and 32, by how many tiles the call has) and the general kernel where a row is not a
-# multiple of 16 bytes: ragged rows, columns and k.
-@pytest.mark.parametrize("rows,D,H,d", [(1, 4, 1, 4), (33, 36, 3, 20), (300, 100, 9, 68), (1100, 68, 12, 100), (1100, 66, 12, 100)])
-def test_projection_tiles(rows, D, H, d):
+# The projection has three forms: 32 x 32 tiles on CUDA cores for small calls, the tensor cores (numbers split into three bf16
+# parts) from two such tiles per SM on, and the general kernel where a row is not a multiple of 16 bytes.  Sequences of one
+# vector make the layer the projection itself (y = v), and y is what the block's output projection starts from.  The shapes
+# put rows, columns and k (= H d in the output projection) at the edges of tiles, of 32-deep steps, of 64-deep operand
+# buffers and of the 128-deep accumulator passes, with one and several tiles per CTA.
+@pytest.mark.parametrize("rows,D,H,d", [(1, 4, 1, 4), (33, 36, 3, 20), (300, 100, 9, 68), (1100, 300, 1, 4), (1100, 300, 3, 20),
+                                        (1153, 260, 1, 64), (1025, 292, 1, 68), (1024, 768, 11, 12), (2000, 260, 5, 52),
+                                        (4100, 388, 3, 128), (1100, 66, 12, 100)])
+def test_projection_forms(rows, D, H, d):
     rng = np.random.default_rng(rows + d)
-    X = (rng.standard_normal((1, 1, D)) * 0.5).astype(np.float32).repeat(rows, 0)       # rows sequences of one vector:
-    X *= np.linspace(0.5, 1.5, rows, dtype=np.float32)[:, None, None]                   # y = v, the projection itself
+    X = rng.standard_normal((rows, 1, D)).astype(np.float32)
     W = (rng.standard_normal((D, H * d)) / np.sqrt(D)).astype(np.float32)
     Wo = (rng.standard_normal((H * d, D)) / np.sqrt(H * d)).astype(np.float32)
-    out = binding.psa_attention_block(_dev(X), _dev(W), _dev(W), _dev(W), _dev(Wo), H, binding.FULL, residual=_dev(X * 2))
-    ref = X.astype(np.float64) @ W.astype(np.float64) @ Wo.astype(np.float64) + 2.0 * X
-    assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= TOL_F32
+    y = binding.psa_attention_f32(_dev(X), _dev(W), _dev(W), _dev(W), H, binding.FULL).cpu().numpy().reshape(rows, H * d)
+    z = binding.psa_attention_block(_dev(X), _dev(W), _dev(W), _dev(W), _dev(Wo), H, binding.FULL, residual=_dev(2 * X))
     st, got = binding.psa_last_issued()
     assert st == binding.OK and got["proj_macs"] == 4 * rows * D * H * d
+    for a, b, out, add in ((X.reshape(rows, D), W, y, None), (y, Wo, z.cpu().numpy().reshape(rows, D), 2.0 * X.reshape(rows, D))):
+        ref = a.astype(np.float64) @ b.astype(np.float64)
+        size = np.abs(a).astype(np.float64) @ np.abs(b).astype(np.float64)
+        # a chain of K fp32 additions: each off by at most half a unit of a partial sum of at most `size`; the tensor-core
+        # form makes 8 of a whole unit per 128 k and fewer additions than K in all, so that the same bound covers it (K >= 16)
+        bound = 2.0 ** -24 * max(a.shape[1], 16) * size
+        if add is not None:
+            ref, bound = ref + add, bound + 2.0 ** -24 * (np.abs(ref) + np.abs(add))
+        assert (np.abs(out - ref) <= bound).all()
+
+
+# Inputs that have no bf16 parts (infinite, NaN, beyond the largest bf16) and sums that overflow come out of the tensor-core
+# form as the plain chain has them, and leave every other output alone.  The layer's y reaches infinity and NaN through a
+# column of value weights around 1e37; the output matrix brings its own.
+def test_projection_of_numbers_without_parts():
+    rows, D, d = 1100, 300, 64
+    rng = np.random.default_rng(1)
+    X = rng.standard_normal((rows, 1, D)).astype(np.float32)
+    Wq, Wk, Wv = ((rng.standard_normal((D, d)) / np.sqrt(D)).astype(np.float32) for _ in range(3))
+    Wv[:, 3] = rng.standard_normal(D) * 2e37
+    Wo = (rng.uniform(0.01, 0.1, (d, D)) * rng.choice([-1, 1], (d, D))).astype(np.float32)
+    Wo[9, 17], Wo[10, 290], Wo[5, 33], Wo[3, 40] = np.inf, np.nan, 3.4e38, 1e-38
+    y = binding.psa_attention_f32(_dev(X), _dev(Wq), _dev(Wk), _dev(Wv), 1, binding.FULL).cpu().numpy().reshape(rows, d)
+    assert (~np.isfinite(y)).sum() > 20 and (np.abs(y[np.isfinite(y)]) > 1e38).sum() > 20
+    z = binding.psa_attention_block(_dev(X), _dev(Wq), _dev(Wk), _dev(Wv), _dev(Wo), 1, binding.FULL).cpu().numpy().reshape(rows, D)
+    with np.errstate(all="ignore"):
+        ref = y.astype(np.float64) @ Wo.astype(np.float64)
+        size = np.abs(y).astype(np.float64) @ np.abs(Wo).astype(np.float64)
+    near = np.isfinite(ref) & (size > 3e38)                      # overflow on the way depends on the order of the sum
+    with np.errstate(all="ignore"):
+        ref32 = np.where(np.abs(ref) > 3.4028235e38, np.sign(ref) * np.inf, ref)
+    assert np.array_equal(np.isnan(z)[~near], np.isnan(ref32)[~near]) and np.array_equal(np.isinf(z)[~near], np.isinf(ref32)[~near])
+    ok = np.isfinite(ref32) & ~near
+    # the column has a deviation of sqrt(300) 2e37 = 3.5e38, the largest fp32 number: some two thirds of the rows stay finite,
+    # fewer where single products overflow on the way; those rows have to be right in full
+    assert ok.sum() > 0.3 * ok.size and (np.abs(z - ref32)[ok] <= (2.0 ** -24 * d * size)[ok]).all()
