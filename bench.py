@@ -281,10 +281,10 @@ class Prepared:
                 self.step = lambda: psa.psa_attention_block(dev["X"], dev["Wq"], dev.get("Wk"), dev.get("Wv"), dev["Wo"], H, scheme, out=out)
             else:
                 self.step = lambda: layer(dev["X"], dev["Wq"], dev.get("Wk"), dev.get("Wv"), H, scheme, out=out)
-            self.kernels_per_step = 2 + (1 if self.sym else 0) + (1 if w.get("wo") else 0)
+            self.kernels_per_step = 2 + (1 if w.get("wo") else 0)
         else:
             self.step = lambda: psa.psa_attention_core(dev["Q"], dev.get("K"), dev.get("V"), scheme, out=out)
-            self.kernels_per_step = 2 if self.sym else 1
+            self.kernels_per_step = 1
         fl = useful_flops(w)
         self.flops = fl
         self.flops_step = fl["core"] + fl["proj"]
@@ -570,7 +570,7 @@ def main():
     sustained = total_s >= 0.5 and not prep.flush
     peak = peaks["bf16_tflops_sustained"] if sustained else peaks["bf16_tflops"]
     mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 1965.0
-    roofline = {"bound": "tensor", "kernel": ("sym_scores_kernel + sym_attn_kernel (symmetric scheme, all passes)" if sym else "attn_persist_kernel (fused scores-softmax-weighted sum)") if dominant == "attn" else "gemm_bf16_kernel (projections)",
+    roofline = {"bound": "tensor", "kernel": ("sym_attn_kernel (symmetric scheme, all passes)" if sym else "attn_persist_kernel (fused scores-softmax-weighted sum)") if dominant == "attn" else "gemm_bf16_kernel (projections)",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None,
                 "peak_source": peaks["source"] + (" sustained bf16 (timed region of %.2f s, steps back to back)" % total_s if sustained else " burst bf16"),
