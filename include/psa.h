@@ -101,7 +101,9 @@ int psa_attention_core(const void* Q, const void* K, const void* V, int batch, i
 /*
  * psa_attention / psa_attention_f32 with HOST buffers (pageable or pinned): copies X and the
  * projection matrices to the device, runs the layer, copies `out` back and waits for `stream`.
- * dtype selects bf16 or fp32 storage.  The staging buffers are part of the workspace.
+ * dtype selects bf16 or fp32 storage.  The staging buffers are part of the workspace.  A large batch is worked off in
+ * parts, the copies of one under the kernels of the others; out_host may overlap X_host all the same (the call then runs
+ * in one part: X is read in full before anything is written).
  */
 int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_host, const void* Wv_host,
                        int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out_host,

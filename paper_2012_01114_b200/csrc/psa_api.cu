@@ -49,8 +49,6 @@ Context* current_ctx() {
     return &g_ctxs[dev];
 }
 
-constexpr size_t HOST_CHUNK_BYTES = 3 << 20;    // see psa_attention_host
-constexpr int HOST_CHUNKS = 8;                  // most parts a batch on host buffers is worked off in
 struct HostPipe {
     cudaStream_t in = nullptr, out = nullptr;
     cudaEvent_t start = nullptr, weights = nullptr, loaded[HOST_CHUNKS] = {}, computed[HOST_CHUNKS] = {}, stored = nullptr;
@@ -355,9 +353,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     if (!ws) return PSA_ERR_WORKSPACE;
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
     const size_t xb = (size_t)n * d_model * es, wb = (size_t)d_model * heads * d_k * es, ob = (size_t)n * heads * d_k * es;   // per sequence; per matrix
-    // The batch is worked off in parts of at least HOST_CHUNK_BYTES in and out, so that the copies of one part run under the
-    // copies and kernels of the others (both directions of the link are busy at once).
-    const int parts = (int)std::max<size_t>(1, std::min<size_t>(std::min(batch, HOST_CHUNKS), batch * (xb + ob) / HOST_CHUNK_BYTES));
+    const int parts = host_parts(batch, xb, ob, X_host, out_host);
     // (a call that is being timed runs in one part, and so does one whose score scratch, sized for the batch's passes, is
     // smaller than a part's passes would have it)
     const bool scratch_fits = dtype != PSA_BF16 || scheme != PSA_SYMMETRIC ||

@@ -6,6 +6,7 @@
 // multiplied and never exponentiated (paper Sec. 4.1 for the symmetric scheme, Sec. 5.1 for the
 // masked one), as opposed to being computed and masked afterwards.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/psa.h"
@@ -178,5 +179,19 @@ PSA_HD void sym_pair(int t, int* I, int* J) {
     *J = t - i * (i + 1) / 2;
 }
 PSA_HD int sym_pairs(int T) { return T * (T + 1) / 2; }
+
+// Parts that a layer on host buffers works its batch off in: at least HOST_CHUNK_BYTES in and out each, so that the copies of
+// one part run under the copies and kernels of the others (both directions of the link are busy at once).  The output of a
+// part may arrive before the input of a later one has left, so buffers that overlap go in one part: all of X is copied in
+// before any of the output is copied out.
+constexpr size_t HOST_CHUNK_BYTES = 3 << 20;
+constexpr int HOST_CHUNKS = 8;
+inline int host_parts(int batch, size_t x_bytes, size_t out_bytes, const void* x, const void* out) {      // bytes per sequence
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(x), o0 = reinterpret_cast<uintptr_t>(out);
+    if (x0 < o0 + batch * out_bytes && o0 < x0 + batch * x_bytes) return 1;
+    const size_t parts = batch * (x_bytes + out_bytes) / HOST_CHUNK_BYTES;
+    const size_t most = batch < HOST_CHUNKS ? batch : HOST_CHUNKS;
+    return parts < 1 ? 1 : (int)(parts < most ? parts : most);
+}
 
 }  // namespace psa

@@ -241,3 +241,22 @@ def test_host_batch_in_parts(scheme, B, H, n, D, d, pinned):
         assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
         st, got = binding.psa_last_issued()
         assert st == binding.OK and got == binding.psa_skip_count(B, H, n, D, d, scheme, binding.BF16)
+
+
+# `out` may share storage with X: all of X is read before any of the output is written.  Outputs wider than inputs, X at the
+# front, in the middle and at the end of the output's storage: the output of one sequence covers the inputs of others.
+@pytest.mark.parametrize("at", [0.0, 0.37, 1.0])
+def test_host_output_over_the_input(at):
+    B, H, n, D, d = 8, 16, 512, 512, 64
+    g = torch.Generator().manual_seed(11)
+    X = torch.randn(B, n, D, generator=g).bfloat16()
+    W = [(torch.randn(D, H * d, generator=g) * D ** -0.5).bfloat16().pin_memory() for _ in range(3)]
+    want = torch.empty(B, n, H * d, dtype=torch.bfloat16).pin_memory()
+    binding.psa_attention_host(X.pin_memory(), *W, H, binding.FULL, want)
+    for call in range(3):
+        out = torch.empty(B, n, H * d, dtype=torch.bfloat16).pin_memory()
+        first = int(at * (out.numel() - X.numel())) // 8 * 8
+        shared = out.view(-1)[first:first + X.numel()].view(B, n, D)
+        shared.copy_(X)
+        binding.psa_attention_host(shared, *W, H, binding.FULL, out)
+        assert torch.equal(out.view(torch.int16), want.view(torch.int16))
