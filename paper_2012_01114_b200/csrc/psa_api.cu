@@ -354,12 +354,9 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
     const size_t xb = (size_t)n * d_model * es, wb = (size_t)d_model * heads * d_k * es, ob = (size_t)n * heads * d_k * es;   // per sequence; per matrix
     const int parts = host_parts(batch, xb, ob, X_host, out_host);
-    // (a call that is being timed runs in one part, and so does one whose score scratch, sized for the batch's passes, is
-    // smaller than a part's passes would have it)
-    const bool scratch_fits = dtype != PSA_BF16 || scheme != PSA_SYMMETRIC ||
-                              bf16_symmetric_scratch_bytes((batch + parts - 1) / parts, heads, n) <= L.s_bytes;
+    // (a call that is being timed runs in one part)
     HostPipe* pipe = nullptr;
-    if (parts > 1 && scratch_fits && cx.prof_calls >= cx.prof_max) {
+    if (parts > 1 && cx.prof_calls >= cx.prof_max) {
         pipe = acquire_pipe(cx);
         if (!pipe) return PSA_ERR_CUDA;
     }

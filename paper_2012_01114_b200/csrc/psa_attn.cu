@@ -37,7 +37,6 @@ namespace psa {
 
 namespace {
 
-constexpr int S_BLOCK_BYTES = 128 * 128 * 4;    // one 128 x 128 fp32 score block of the scratch: 64 KB
 constexpr int S_HALF_BYTES = S_BLOCK_BYTES / 2; // 64 of its rows = 64 key columns of the tile that reads it transposed
 constexpr int SYM_WARPS = SOFTMAX_WARPS_PER_TILE;                    // 8
 constexpr int SYM_PUBLISHER = CTRL_WARPS + SYM_WARPS;                // warp that announces finished blocks
@@ -521,20 +520,6 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// Heads per pass: as many as the scratch cap allows, in passes of equal size (the scratch is reused from pass
-// to pass).  Passes small enough to stay in L2 were measured slower: the kernels of a small pass do not fill the GPU.
-constexpr size_t SYM_SCRATCH_CAP = size_t(2) << 30;   // bytes of score scratch per pass
-
-int sym_heads_per_pass(int B, int H, int n) {
-    const size_t per_head = (size_t)sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
-    const size_t all = (size_t)B * H;
-    size_t hp = SYM_SCRATCH_CAP / per_head;
-    if (hp < 1) hp = 1;
-    if (hp > all) hp = all;
-    const size_t passes = (all + hp - 1) / hp;
-    return (int)((all + passes - 1) / passes);
-}
-
 // Heads per group of the item list: the tiles of one head are started a group apart.  A tile needs its first handed-on block
 // one step after its neighbour has computed it, so tiles that start together wait for one another; started 256 / T items
 // apart (two steps, on 148 CTAs) they do not, and a head's scratch still lives briefly enough to stay in L2.  Measured for
@@ -543,8 +528,9 @@ int sym_heads_per_pass(int B, int H, int n) {
 constexpr int SYM_GROUP_ITEMS = 256;
 
 // D: head size the kernel works with (64 or 128); d <= D: the tensors' head size (see the 4-D tensor maps).
+// s_bytes: size of the score scratch, which sets the heads per pass.
 template <int D>
-int launch_symmetric(const void* X, void* out, float* S, int B, int H, int n, int d, float scale, DeviceCounters* dc,
+int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, int B, int H, int n, int d, float scale, DeviceCounters* dc,
                      cudaStream_t stream) {
     using Cfg = SymCfg<D>;
     static DeviceSetup setup;
@@ -554,7 +540,7 @@ int launch_symmetric(const void* X, void* out, float* S, int B, int H, int n, in
     if (sm_count <= 0) return PSA_ERR_CUDA;
     const int T = row_tiles(n);
     const size_t head_bytes = (size_t)sym_pairs(T) * S_BLOCK_BYTES;
-    const int hp = sym_heads_per_pass(B, H, n);
+    const int hp = sym_heads_per_pass((size_t)B * H, n, s_bytes);
     SymMaps maps;
     if (!make_tensor_map_bf16_4d(&maps.x, X, B, n, H, d, 128) || !make_tensor_map_bf16_4d(&maps.o, out, B, n, H, d, 16))
         return PSA_ERR_CUDA;
@@ -577,7 +563,7 @@ int launch_symmetric(const void* X, void* out, float* S, int B, int H, int n, in
 }  // namespace
 
 size_t bf16_symmetric_scratch_bytes(int B, int H, int n) {
-    return (size_t)sym_heads_per_pass(B, H, n) * sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
+    return (size_t)sym_heads_per_pass((size_t)B * H, n, SYM_SCRATCH_CAP) * sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
 }
 
 int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, int B, int H,
@@ -585,11 +571,11 @@ int bf16_attention(const void* Q, const void* K, const void* V, void* out, float
                    cudaStream_t stream) {
     if (scheme != PSA_SYMMETRIC && d > 128) return bf16_attention_wide(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
     if (scheme != PSA_SYMMETRIC) return bf16_attention_persist(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
-    if (!S || s_bytes < bf16_symmetric_scratch_bytes(B, H, n)) return PSA_ERR_WORKSPACE;
+    if (!S || s_bytes < (size_t)sym_pairs(row_tiles(n)) * S_BLOCK_BYTES) return PSA_ERR_WORKSPACE;       // (one head)
     if ((reinterpret_cast<uintptr_t>(S) & 15u) != 0) return PSA_ERR_ALIGN;
     if (d < 8 || d > 128 || d % 8) return PSA_ERR_UNSUPPORTED;
-    if (d <= 64) return launch_symmetric<64>(Q, out, S, B, H, n, d, scale, dc, stream);
-    return launch_symmetric<128>(Q, out, S, B, H, n, d, scale, dc, stream);
+    if (d <= 64) return launch_symmetric<64>(Q, out, S, s_bytes, B, H, n, d, scale, dc, stream);
+    return launch_symmetric<128>(Q, out, S, s_bytes, B, H, n, d, scale, dc, stream);
 }
 
 }  // namespace psa

@@ -46,7 +46,8 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
 int bf16_project(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N,
                  const void* residual, DeviceCounters* dc, cudaStream_t stream);
 // Q, K, V, out: [B, n, H, d] bf16.  S: scratch for PSA_SYMMETRIC (bf16_symmetric_scratch_bytes:
-// one 64 KB fp32 image per score block at or below the block diagonal, for the heads of one pass).
+// one 64 KB fp32 image per score block at or below the block diagonal, for the heads of one pass; with less, down to
+// one head's worth, the call runs in more passes).
 // `dc_next`, if not null, is a second counter block that the call's attention kernel clears (FULL, MASKED only).
 // `cursor` is the work counter of the fused kernel (FULL, MASKED), zero when the call's kernels start.
 int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, int B,

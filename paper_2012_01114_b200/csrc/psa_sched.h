@@ -179,6 +179,20 @@ PSA_HD void sym_pair(int t, int* I, int* J) {
     *J = t - i * (i + 1) / 2;
 }
 PSA_HD int sym_pairs(int T) { return T * (T + 1) / 2; }
+// Heads per pass of the symmetric scheme's kernel: as many as a scratch of `scratch_bytes` holds, one block per pair of
+// tiles, in passes of equal size (the scratch is reused from pass to pass).  A call's own scratch is what its passes need
+// under the cap; a part of it (see host_parts) may hold fewer heads and yet fill its passes fuller -- the number of heads per
+// pass does not grow with the number of heads --, so a launch goes by the scratch that it is given.  Passes small enough to
+// stay in L2 were measured slower: the kernels of a small pass do not fill the GPU.
+constexpr size_t S_BLOCK_BYTES = 128 * 128 * 4;          // one 128 x 128 fp32 score block: 64 KB
+constexpr size_t SYM_SCRATCH_CAP = size_t(2) << 30;      // bytes of score scratch per pass
+inline int sym_heads_per_pass(size_t heads, int n, size_t scratch_bytes) {
+    size_t hp = scratch_bytes / ((size_t)sym_pairs(row_tiles(n)) * S_BLOCK_BYTES);
+    if (hp < 1) hp = 1;
+    if (hp > heads) hp = heads;
+    const size_t passes = (heads + hp - 1) / hp;
+    return (int)((heads + passes - 1) / passes);
+}
 
 // Parts that a layer on host buffers works its batch off in: at least HOST_CHUNK_BYTES in and out each, so that the copies of
 // one part run under the copies and kernels of the others (both directions of the link are busy at once).  The output of a

@@ -260,3 +260,18 @@ def test_host_output_over_the_input(at):
         shared.copy_(X)
         binding.psa_attention_host(shared, *W, H, binding.FULL, out)
         assert torch.equal(out.view(torch.int16), want.view(torch.int16))
+
+
+# Parts of uneven size whose scores do not fit the scratch in one pass: 40 heads of n = 7296 run in 3 passes of 14 under the
+# scratch limit of 2 GB, the part of 2 sequences has 16 heads, which alone would run in one.
+def test_symmetric_host_parts_at_the_scratch_limit():
+    B, H, n, D, d = 5, 8, 7296, 64, 8
+    g = torch.Generator().manual_seed(5)
+    X = torch.randn(B, n, D, generator=g).bfloat16().pin_memory()
+    W = (torch.randn(D, H * d, generator=g) * D ** -0.5).bfloat16().pin_memory()
+    out = torch.empty(B, n, H * d, dtype=torch.bfloat16).pin_memory()
+    binding.psa_attention_host(X, W, None, None, H, binding.SYMMETRIC, out)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got == binding.psa_skip_count(B, H, n, D, d, binding.SYMMETRIC, binding.BF16)
+    ref = binding.psa_attention(X.cuda(), W.cuda(), None, None, H, binding.SYMMETRIC).cpu()
+    assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
