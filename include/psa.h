@@ -29,6 +29,10 @@
  *   - Every function returns a psa_status (0 = PSA_OK) unless stated otherwise.
  *   - Calls that share a workspace must be ordered on one stream; the library is not re-entrant
  *     across streams.
+ *   - The entry points on device pointers may be captured into a CUDA graph once a call of that size has run (the first
+ *     one sets up kernels and may allocate the workspace); every replay is a whole call.  The graph keeps the workspace it
+ *     was captured with: register one (psa_set_workspace), or capture after the largest call, and replay only while that
+ *     workspace stands.  After a replay psa_last_issued reports on it as long as the captured call was the last one made.
  */
 #ifndef PSA_H_
 #define PSA_H_

@@ -25,9 +25,11 @@ struct Context {
     void* own_ws = nullptr;
     size_t own_bytes = 0;
     DeviceCounters* last_dc = nullptr;  // counters of the most recent call
-    // The workspace starts with two counter blocks.  The bf16 FULL / MASKED path uses them in turn: the attention
-    // kernel of a call clears the block of the next call, so that no clearing copy has to run ahead of the
-    // call's first kernel.  `clean_ws` is the workspace whose block `next_block` is known to be clear.
+    // The workspace starts with three counter blocks.  The bf16 FULL / MASKED path uses the first two in turn: the
+    // attention kernel of a call clears the block of the next call, so that no clearing copy has to run ahead of the
+    // call's first kernel.  `clean_ws` is the workspace whose block `next_block` is known to be clear.  A call that is being
+    // captured into a graph has the third to itself and clears it first: the graph may run any number of times, between
+    // any other calls.
     char* clean_ws = nullptr;
     int next_block = 0;
     // Streams and events of the entry points on host buffers, created by the first such call and kept.
@@ -54,11 +56,12 @@ struct HostPipe {
     cudaEvent_t start = nullptr, weights = nullptr, loaded[HOST_CHUNKS] = {}, computed[HOST_CHUNKS] = {}, stored = nullptr;
 };
 
-constexpr size_t COUNTER_BYTES = 256;          // two counter blocks
-constexpr size_t COUNTER_BLOCK_BYTES = 128;
-constexpr size_t CURSOR_OFFSET = 64;           // work counters of a call in several parts, behind the counters
-static_assert(sizeof(DeviceCounters) <= CURSOR_OFFSET, "counter block too small");
-static_assert(CURSOR_OFFSET + HOST_CHUNKS * sizeof(unsigned int) <= COUNTER_BLOCK_BYTES, "counter block too small");
+constexpr size_t COUNTER_BYTES = 256;          // counter blocks and cursors at the start of the workspace
+constexpr size_t COUNTER_BLOCK_BYTES = 64;
+constexpr int TURN_BLOCKS = 2, CAPTURE_BLOCK = 2;      // blocks used in turn; block of captured calls
+constexpr size_t CURSOR_OFFSET = 3 * COUNTER_BLOCK_BYTES;   // work counters of a call in several parts
+static_assert(sizeof(DeviceCounters) <= COUNTER_BLOCK_BYTES, "counter block too small");
+static_assert(CURSOR_OFFSET + HOST_CHUNKS * sizeof(unsigned int) <= COUNTER_BYTES, "no room for the cursors");
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -212,16 +215,23 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     // the paths whose last kernel clears the other counter block: the fused bf16 kernels and the one-launch fp32 layer
     const bool turns = (dtype == PSA_BF16 && scheme != PSA_SYMMETRIC) ||
                        (with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme));
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &capture);
+    if (e != cudaSuccess) { set_cuda_error(e, "cudaStreamIsCapturing"); return PSA_ERR_CUDA; }
+    const bool captured = capture != cudaStreamCaptureStatusNone;
     int block = 0;
-    if (turns && cx.clean_ws == ws) {
+    if (captured) {
+        block = CAPTURE_BLOCK;
+        e = cudaMemsetAsync(ws + CAPTURE_BLOCK * COUNTER_BLOCK_BYTES, 0, COUNTER_BLOCK_BYTES, stream);
+    } else if (turns && cx.clean_ws == ws) {
         block = cx.next_block;
     } else {
-        const cudaError_t e = cudaMemsetAsync(ws, 0, 2 * COUNTER_BLOCK_BYTES, stream);
-        if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync(counters)"); return PSA_ERR_CUDA; }
+        e = cudaMemsetAsync(ws, 0, TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
     }
-    cx.clean_ws = nullptr;           // until this call's kernels are known to be queued
+    if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync(counters)"); return PSA_ERR_CUDA; }
+    if (!captured) cx.clean_ws = nullptr;          // until this call's kernels are known to be queued
     DeviceCounters* dc = reinterpret_cast<DeviceCounters*>(ws + block * COUNTER_BLOCK_BYTES);
-    DeviceCounters* dc_next = turns ? reinterpret_cast<DeviceCounters*>(ws + (block ^ 1) * COUNTER_BLOCK_BYTES) : nullptr;
+    DeviceCounters* dc_next = turns && !captured ? reinterpret_cast<DeviceCounters*>(ws + (block ^ 1) * COUNTER_BLOCK_BYTES) : nullptr;
     cx.last_dc = dc;
     memset(&cx.last_useful, 0, sizeof(psa_counts));
     useful_counts(batch, heads, n, d_model, d_k, scheme, with_proj, &cx.last_useful);
@@ -236,7 +246,7 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     float* S = scheme == PSA_SYMMETRIC ? reinterpret_cast<float*>(ws + L.s) : nullptr;
     const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
                                  qkv, S, L.s_bytes, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
-    if (rc == PSA_OK && turns) {        // the other block will be clear once this call has run
+    if (rc == PSA_OK && turns && !captured) {        // the other block will be clear once this call has run
         cx.clean_ws = ws;
         cx.next_block = block ^ 1;
     }
@@ -378,13 +388,13 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         return PSA_OK;
     }
     // In parts: copies in on one stream, kernels on the caller's, copies out on another.  The counters of all parts go to one
-    // block; the work counter of each has a place of its own behind them.  All copies in are queued before the first copy
+    // block; the work counter of each has a place of its own behind the blocks.  All copies in are queued before the first copy
     // out: with pageable buffers a copy may hold the calling thread until it is done.
     const char* what = "ordering the streams of a host call";
     cudaError_t e = cudaEventRecord(pipe->start, stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->start, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->out, pipe->start, 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, 2 * COUNTER_BLOCK_BYTES, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, COUNTER_BYTES, stream);
     cx.clean_ws = nullptr;
     DeviceCounters* dc = reinterpret_cast<DeviceCounters*>(ws);
     cx.last_dc = dc;
@@ -645,7 +655,7 @@ int psa_selftest_wait_expiry(unsigned limit_us, void* stream_v) {
     char* ws = acquire_ws(cx, COUNTER_BYTES);
     if (!ws) return PSA_ERR_WORKSPACE;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
-    cudaError_t e = cudaMemsetAsync(ws, 0, 2 * COUNTER_BLOCK_BYTES, stream);
+    cudaError_t e = cudaMemsetAsync(ws, 0, COUNTER_BLOCK_BYTES, stream);
     if (e == cudaSuccess) e = launch_wait_expiry(reinterpret_cast<DeviceCounters*>(ws), limit_us, stream);
     if (e != cudaSuccess) { set_cuda_error(e, "psa_selftest_wait_expiry"); return PSA_ERR_CUDA; }
     cx.clean_ws = nullptr;
