@@ -1019,14 +1019,52 @@ size_t attn_smem_bytes(int n, int d) {
 namespace {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The general kernels count row tiles, or sequences, in a grid dimension that holds 65535: calls with more go in several launches.
+constexpr int GRID_MAX = 65535;
+
+cudaError_t project_general(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
+                            const float* residual, DeviceCounters* dc, cudaStream_t stream) {
+    constexpr int SLICE = GRID_MAX * PROJ_TILE;
+    for (int r0 = 0; r0 < rows; r0 += min(SLICE, rows - r0)) {
+        const int nr = min(SLICE, rows - r0);
+        const size_t o = (size_t)r0 * N;
+        const dim3 block(PROJ_TILE, PROJ_TILE), grid((N + PROJ_TILE - 1) / PROJ_TILE, (nr + PROJ_TILE - 1) / PROJ_TILE, nW);
+        f32_project_kernel<<<grid, block, 0, stream>>>(X + (size_t)r0 * D, W[0], W[1], W[2], out[0] + o, out[1] + o, out[2] + o, nr, D, N,
+                                                       residual ? residual + o : nullptr, dc);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t attention_general(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H, int n, int d,
+                              float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+    const size_t smem = attn_smem_bytes(n, d);
+    for (int b0 = 0; b0 < B; b0 += min(GRID_MAX, B - b0)) {
+        const int nb = min(GRID_MAX, B - b0);
+        const size_t o = (size_t)b0 * n * H * d;
+        const dim3 grid((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, H, nb), block(ROWS_PER_BLOCK * 32);
+        if (scheme == PSA_SYMMETRIC) {
+            float* s = S + (size_t)b0 * H * n * n;
+            f32_attn_kernel<1><<<grid, block, smem, stream>>>(Q + o, Q + o, Q + o, out + o, s, n, H, d, scale, 0, dc);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            f32_attn_kernel<2><<<grid, block, smem, stream>>>(Q + o, Q + o, Q + o, out + o, s, n, H, d, scale, 0, dc);
+        } else {
+            f32_attn_kernel<0><<<grid, block, smem, stream>>>(Q + o, K + o, V + o, out + o, nullptr, n, H, d, scale, scheme == PSA_MASKED ? 1 : 0, dc);
+        }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
 }  // namespace
 
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
                         int N, const float* residual, DeviceCounters* dc, cudaStream_t stream) {
     bool tiled = D % 4 == 0 && N % 4 == 0 && aligned16(X) && aligned16(residual);      // 16-byte rows
     for (int w = 0; w < nW; ++w) tiled = tiled && aligned16(W[w]) && aligned16(out[w]);
-    // (grid.y holds 65535 row tiles)
-    if (tiled && (rows + 31) / 32 <= 65535) {
+    if (tiled) {
         static DeviceSetup setup;
         const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 projection set-up");
         if (sms <= 0) return cudaErrorUnknown;
@@ -1040,9 +1078,7 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
         f32_project_tiled_kernel<<<grid, GP_THREADS, GP_SMEM, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);
         return cudaGetLastError();
     }
-    dim3 block(PROJ_TILE, PROJ_TILE), grid((N + PROJ_TILE - 1) / PROJ_TILE, (rows + PROJ_TILE - 1) / PROJ_TILE, nW);
-    f32_project_kernel<<<grid, block, 0, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);
-    return cudaGetLastError();
+    return project_general(X, W, out, nW, rows, D, N, residual, dc, stream);
 }
 
 bool f32_fused_fits(int n, int D, int d, int scheme) {
@@ -1149,18 +1185,7 @@ cudaError_t f32_attention(const float* Q, const float* K, const float* V, float*
     if (d % 4 == 0 && (long long)B * H <= 0x7fffffff && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(out))      // 16-byte rows
         return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream)
                        : tiled_attention<2>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
-    dim3 grid((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, H, B), block(ROWS_PER_BLOCK * 32);
-    const size_t smem = attn_smem_bytes(n, d);
-    if (scheme == PSA_SYMMETRIC) {
-        f32_attn_kernel<1><<<grid, block, smem, stream>>>(Q, Q, Q, out, S, n, H, d, scale, 0, dc);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        f32_attn_kernel<2><<<grid, block, smem, stream>>>(Q, Q, Q, out, S, n, H, d, scale, 0, dc);
-    } else {
-        f32_attn_kernel<0><<<grid, block, smem, stream>>>(Q, K, V, out, nullptr, n, H, d, scale,
-                                                          scheme == PSA_MASKED ? 1 : 0, dc);
-    }
-    return cudaGetLastError();
+    return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
 }
 
 }  // namespace psa

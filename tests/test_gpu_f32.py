@@ -190,3 +190,28 @@ def test_projection_of_numbers_without_parts():
     # the column has a deviation of sqrt(300) 2e37 = 3.5e38, the largest fp32 number: some two thirds of the rows stay finite,
     # fewer where single products overflow on the way; those rows have to be right in full
     assert ok.sum() > 0.3 * ok.size and (np.abs(z - ref32)[ok] <= (2.0 ** -24 * d * size)[ok]).all()
+
+
+# More row tiles or sequences than a grid dimension holds (65535): aligned rows on both sides of 65535 x 32, rows that are
+# not a multiple of 16 bytes on both sides of 65535 x 16, and more than 65535 sequences in the general attention kernel.  The
+# last rows, where a wrong offset or a missing launch shows, are compared in full, a stride of the others beside them.
+@pytest.mark.parametrize("B,n,D,d", [(65535, 32, 4, 4), (65536, 32, 4, 4), (2097153, 1, 4, 4), (32767, 32, 6, 6),
+                                     (32769, 32, 6, 6), (65537, 9, 6, 6)])
+@pytest.mark.parametrize("scheme", [oracle.MASKED, oracle.SYMMETRIC])
+def test_more_rows_than_a_grid_holds(B, n, D, d, scheme):
+    g = torch.Generator(device="cuda").manual_seed(B + d)
+    sym = scheme == oracle.SYMMETRIC
+    X = torch.randn(B, n, D, device="cuda", generator=g)
+    W = [torch.randn(D, d, device="cuda", generator=g) * D ** -0.5 for _ in range(1 if sym else 3)]
+    Wo = torch.randn(d, D, device="cuda", generator=g) * d ** -0.5
+    z = binding.psa_attention_block(X, *W, *([None, None] if sym else []), Wo, 1, scheme, residual=X)
+    st, got = binding.psa_last_issued()
+    tri = n * (n + 1) // 2
+    assert st == binding.OK and got["proj_macs"] == (2 if sym else 4) * B * n * D * d
+    assert got["qk_macs"] == B * d * tri and got["pv_macs"] == B * d * (n * n if sym else tri)
+    pick = torch.cat([torch.arange(0, B, max(1, B // 37)), torch.arange(max(0, B - 300), B)])
+    x = X[pick.cuda()].cpu().numpy().astype(np.float64)
+    ref = oracle.attention_block(x, *[w.cpu().numpy().astype(np.float64) for w in (W * 3 if sym else W)], Wo.cpu().numpy().astype(np.float64),
+                                 1, scheme, residual=x)
+    ref = ref[0] if isinstance(ref, tuple) else ref
+    assert np.abs(z[pick.cuda()].cpu().numpy() - ref).max() <= TOL_F32
