@@ -19,9 +19,16 @@
 // slots per scheduler beside them, and its stores share the shared-memory port with the MMAs' operands.  Measured 2300
 // cycles per step; 2048 x 768 x 3 x 768 171 us on CUDA cores (128 x 128 tiles), 70 us here.
 //
-// An output that is not finite (an input is infinite or NaN or rounds to infinity, or a sum overflows) is formed again by the
-// plain chain, so that it is what that chain gives; so are the outputs of a tile one of whose operands is nonzero but below
-// 2^-100, where the smaller parts leave the range of normal bf16 numbers.
+// What the parts cannot carry is formed again by the plain chain of fmaf, per output (ft_form_again):
+//   * an output that is not finite (an input is infinite or NaN or rounds to infinity, or a sum overflows);
+//   * an output of a tile with a nonzero operand below 2^-60, if it is small enough to have lost something: an operand below
+//     2^-100 has parts below the normal range of bf16 and loses up to 2^-125, and products below 2^-120 lose up to 2^-149 in
+//     each addition.  With the largest magnitudes of the output's row and column that bounds its error, K times over; it is
+//     formed again where that could be more than half a unit.
+// Such tiles are marked on the way and looked at when the CTA's other work is done, so that the main loop keeps its registers.
+// What it costs, in a layer of 4 x 512 vectors, d_model = 768, 12 heads, of whose 176 us the projection takes 60: one 1e-35 in
+// every vector, so that every tile is looked at, 208 us; nothing but numbers around 1e-33, so that every output is formed
+// again, 439; nothing but NaN 416 (as a loop of one thread per 32 outputs in global memory it was 3300 in all three).
 #include "psa_internal.h"
 #include "sm100.cuh"
 
@@ -37,7 +44,8 @@ constexpr int FT_SLOTS = 4;                              // steps in the ring (t
 constexpr int FT_CHUNK = 4;                              // steps whose leading products share an accumulator pass
 constexpr int FT_SMEM = FT_SLOTS / 2 * FT_BUF_BYTES + 1024;
 constexpr int FT_TMEM_MAIN = 0, FT_TMEM_CROSS = 256;     // leading products (two accumulators), smaller products
-constexpr uint32_t FT_TINY = 2u * (27u << 23);           // twice the bits of 2^-100
+constexpr uint32_t FT_SMALL = 2u * (67u << 23), FT_TINY = 2u * (27u << 23);      // twice the bits of 2^-60, 2^-100
+constexpr int FT_MARKS = 1024;                           // marks of a CTA's tiles
 constexpr int FT_PITCH = 36;                             // floats per row of a warp's 32 x 32 output staging
 
 __device__ __forceinline__ uint32_t ft_pack(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }    // upper halves
@@ -61,6 +69,121 @@ __device__ __forceinline__ void ft_split_store(uint8_t* dst, const float4& v, ui
         *reinterpret_cast<uint2*>(dst + k * FT_PLANE_BYTES) = make_uint2(ft_pack(p[k][0], p[k][1]), ft_pack(p[k][2], p[k][3]));
 }
 
+// Shared memory of ft_form_again, over the ring: 32 k of the operands as they are (X rows padded by 16 bytes), and twice the
+// bits of the smallest nonzero magnitude (less one) and of the largest, per row of X and column of W.
+struct FtAgain {
+    float x[FT_M * (FT_K + 4)], w[FT_K * FT_N];
+    uint32_t row_least[FT_M], row_most[FT_M], col_least[FT_N], col_most[FT_N];
+};
+static_assert(sizeof(FtAgain) <= FT_BUF_BYTES, "does not fit the ring");
+
+// Replaces those outputs of a finished tile that the parts cannot carry, by the plain chain: called by all FT_WORKERS warps.  A
+// thread has the eight rows row0 + 4 i and the four columns from col0 on.  Without a residual the outputs say whether there is
+// anything to replace; with one the tile is computed again in any case.
+__device__ __noinline__ void ft_form_again(const float* X, const float* W, float* O, const float* R, int m_first, int n_first, int M, int K,
+                                           int N, FtAgain* sm) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int row0 = 32 * (warp & 3) + (lane >> 3), col0 = 32 * (warp >> 2) + 4 * (lane & 7);
+    named_bar_sync(1, 32 * FT_WORKERS);       // (the tile before is done with the shared memory)
+    if (tid < FT_M) { sm->row_least[tid] = sm->col_least[tid] = 0xffffffffu; sm->row_most[tid] = sm->col_most[tid] = 0; }
+    named_bar_sync(1, 32 * FT_WORKERS);
+    for (int r = warp; r < FT_M && m_first + r < M; r += FT_WORKERS) {
+        uint32_t least = 0xffffffffu, most = 0;
+#pragma unroll 4
+        for (int k = 4 * lane; k < K; k += 128) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(X + (size_t)(m_first + r) * K + k));
+            const uint32_t t[4] = {2u * __float_as_uint(v.x), 2u * __float_as_uint(v.y), 2u * __float_as_uint(v.z), 2u * __float_as_uint(v.w)};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { least = min(least, t[e] - 1u); most = max(most, t[e]); }
+        }
+        least = __reduce_min_sync(0xffffffffu, least);
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (lane == 0) { sm->row_least[r] = least; sm->row_most[r] = most; }
+    }
+    if (n_first + 4 * lane < N) {
+        uint32_t least[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu}, most[4] = {0, 0, 0, 0};
+#pragma unroll 8
+        for (int k = warp; k < K; k += FT_WORKERS) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(W + (size_t)k * N + n_first + 4 * lane));
+            const uint32_t t[4] = {2u * __float_as_uint(v.x), 2u * __float_as_uint(v.y), 2u * __float_as_uint(v.z), 2u * __float_as_uint(v.w)};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { least[e] = min(least[e], t[e] - 1u); most[e] = max(most[e], t[e]); }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { atomicMin(&sm->col_least[4 * lane + e], least[e]); atomicMax(&sm->col_most[4 * lane + e], most[e]); }
+    }
+    named_bar_sync(1, 32 * FT_WORKERS);
+    const bool inside = n_first + col0 < N;                 // (N is a multiple of 4)
+    float* out = O + (size_t)(m_first + row0) * N + n_first + col0;
+    auto lost = [&](float v, int r, int c) {                // whether value v at (r, c) may have lost something
+        if (!(fabsf(v) < INFINITY)) return true;
+        if (sm->row_most[r] == 0 || sm->col_most[c] == 0) return false;       // a row or column of zeros gives exact zeros
+        float limit = 7.5231638e-37f;                                         // 2^-120
+        if (sm->row_least[r] < FT_TINY) limit += 7.8886091e-31f * __uint_as_float(sm->col_most[c] >> 1);       // 2^-100
+        if (sm->col_least[c] < FT_TINY) limit += 7.8886091e-31f * __uint_as_float(sm->row_most[r] >> 1);
+        return !(fabsf(v) >= limit * (float)K);
+    };
+    if (!R) {
+        bool any = false;
+        for (int i = 0; i < 8; ++i) {
+            if (!inside || m_first + row0 + 4 * i >= M) continue;
+            const float4 o = *reinterpret_cast<const float4*>(out + (size_t)(4 * i) * N);
+            any = any || lost(o.x, row0 + 4 * i, col0) || lost(o.y, row0 + 4 * i, col0 + 1) || lost(o.z, row0 + 4 * i, col0 + 2) ||
+                  lost(o.w, row0 + 4 * i, col0 + 3);
+        }
+        if (named_bar_all(!any, 1, 32 * FT_WORKERS)) return;
+    }
+    float acc[8][4] = {};
+#pragma unroll 1
+    for (int k0 = 0; k0 < K; k0 += FT_K) {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 xv[2], wv[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int t = tid + 32 * FT_WORKERS * u, m = m_first + (t >> 3), kx = k0 + 4 * (t & 7), kw = k0 + (t >> 5), n = n_first + 4 * (t & 31);
+            xv[u] = m < M && kx < K ? __ldg(reinterpret_cast<const float4*>(X + (size_t)m * K + kx)) : zero;
+            wv[u] = kw < K && n < N ? __ldg(reinterpret_cast<const float4*>(W + (size_t)kw * N + n)) : zero;
+        }
+        named_bar_sync(1, 32 * FT_WORKERS);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int t = tid + 32 * FT_WORKERS * u;
+            *reinterpret_cast<float4*>(sm->x + (t >> 3) * (FT_K + 4) + 4 * (t & 7)) = xv[u];
+            *reinterpret_cast<float4*>(sm->w + 4 * t) = wv[u];
+        }
+        named_bar_sync(1, 32 * FT_WORKERS);
+        const int kn = min(FT_K, K - k0);     // (a multiple of 4)
+#pragma unroll 1
+        for (int k = 0; k < kn; k += 4) {
+            float4 w[4];
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) w[kk] = *reinterpret_cast<const float4*>(sm->w + (k + kk) * FT_N + col0);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(sm->x + (row0 + 4 * i) * (FT_K + 4) + k);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const float f = kk == 0 ? x.x : kk == 1 ? x.y : kk == 2 ? x.z : x.w;
+                    acc[i][0] = fmaf(f, w[kk].x, acc[i][0]); acc[i][1] = fmaf(f, w[kk].y, acc[i][1]);
+                    acc[i][2] = fmaf(f, w[kk].z, acc[i][2]); acc[i][3] = fmaf(f, w[kk].w, acc[i][3]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = row0 + 4 * i;
+        if (!inside || m_first + r >= M) continue;
+        const size_t at = (size_t)(4 * i) * N;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float o = out[at + e];
+            if (!(fabsf(o) < INFINITY) || lost(R ? acc[i][e] : o, r, col0 + e))
+                out[at + e] = R ? acc[i][e] + R[(size_t)(m_first + r) * N + n_first + col0 + e] : acc[i][e];
+        }
+    }
+}
+
 __global__ void __launch_bounds__(FT_THREADS, 1)
 f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const float* W1, const float* W2, float* O0, float* O1,
                           float* O2, int M, int K, int N, int nW, const float* __restrict__ R, DeviceCounters* dc) {
@@ -69,7 +192,7 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
     __shared__ uint64_t full_bar[FT_SLOTS], empty_bar[FT_SLOTS], main_full[2], main_empty[2], cross_full, cross_empty;
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_flag;
-    __shared__ int tiny[2];              // a tile of even / odd number has an operand below 2^-100
+    __shared__ uint32_t marks[FT_MARKS / 32];      // tiles of this CTA to look at again: see mark_of
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mt = (M + FT_M - 1) / FT_M, nt = (N + FT_N - 1) / FT_N, ntiles = mt * nt * nW;
@@ -77,13 +200,13 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        tiny[0] = tiny[1] = 0;
         for (int s = 0; s < FT_SLOTS; ++s) { mbar_init(&full_bar[s], FT_WORKERS); mbar_init(&empty_bar[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&main_full[b], 1); mbar_init(&main_empty[b], FT_WORKERS); }
         mbar_init(&cross_full, 1);
         mbar_init(&cross_empty, FT_WORKERS);
         fence_mbar_init();
     }
+    for (int i = threadIdx.x; i < FT_MARKS / 32; i += FT_THREADS) marks[i] = 0;
     if (warp == FT_WORKERS) { tmem_alloc(&tmem_base_s, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
@@ -147,6 +270,10 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
         const uint32_t lanes = (q * 32) << 16;
         uint32_t g = 0, gc = 0, i = 0;
         bool ok = true;
+        auto mark_of = [&](uint32_t tile) {             // (a mark stands for one tile but in very large calls)
+            return tile / (((ntiles + gridDim.x - 1) / gridDim.x + FT_MARKS - 1) / FT_MARKS);
+        };
+        auto mark = [&]() { atomicOr(&marks[mark_of(i) / 32], 1u << (mark_of(i) % 32)); };
         // the stream of loads, two steps ahead of the splitting: tile, step, and where this thread stands in X and W
         float4 xv[2][2], wv[2][2];
         int lt = blockIdx.x, lk = 0;
@@ -211,7 +338,7 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
                     ft_split_store(buf + 3 * FT_PLANE_BYTES + (lane >> 4) * (FT_PLANE_BYTES / 2) +
                                        swz128_offset((slot & 1) * 32 + warp + 16 * u, (lane & 15) >> 1) + 8 * (lane & 1), w[u], least);
                 }
-                if (least < FT_TINY) tiny[i & 1] = 1;
+                if (least < FT_SMALL) mark();
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&full_bar[slot]);
@@ -229,35 +356,28 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
                 tc_fence_after();
                 drain(tmem + FT_TMEM_CROSS);
                 if (lane == 0) mbar_arrive(&cross_empty);
+                bool finite = true;
+#pragma unroll
+                for (int e = 0; e < 32; ++e) finite = finite && fabsf(acc[e]) < INFINITY;
+                if (!finite) mark();
             }
-            // (makes the marks complete; the warps leave together if one of them gave up a wait)
+            // (the warps leave together if one of them gave up a wait)
             ok = named_bar_all(ok, 1, 32 * FT_WORKERS);
             if (!ok) break;
             // every MMA of the tile is complete: the ring's first buffer stages the outputs, a warp's 32 rows x 32 columns on
             // their own, so that a row leaves as 128 consecutive bytes
             const int r = t / nt, m0 = (r % mt) * FT_M + 32 * q, n0 = (t % nt) * FT_N + col0, w = r / mt;
-            const float* W = w == 0 ? W0 : (w == 1 ? W1 : W2);
             float* O = w == 0 ? O0 : (w == 1 ? O1 : O2);
             float* stage = reinterpret_cast<float*>(smem) + warp * 32 * FT_PITCH;
 #pragma unroll
             for (int e = 0; e < 32; e += 4)
                 *reinterpret_cast<float4*>(stage + lane * FT_PITCH + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
             __syncwarp();
-            const bool again = tiny[i & 1] != 0;
 #pragma unroll 2
             for (int rr = lane >> 3; rr < 32; rr += 4) {
                 const int m = m0 + rr, n = n0 + 4 * (lane & 7);
                 if (m >= M || n >= N) continue;
-                float o[4];
-                *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(stage + rr * FT_PITCH + 4 * (lane & 7));
-                if (again || !(fabsf(o[0]) < INFINITY && fabsf(o[1]) < INFINITY && fabsf(o[2]) < INFINITY && fabsf(o[3]) < INFINITY)) {
-                    for (int e = 0; e < 4; ++e) {
-                        float sum = 0.f;
-                        for (int k = 0; k < K; ++k) sum = fmaf(X[(size_t)m * K + k], W[(size_t)k * N + n + e], sum);
-                        if (again || !(fabsf(o[e]) < INFINITY)) o[e] = sum;
-                    }
-                }
-                float4 y = make_float4(o[0], o[1], o[2], o[3]);
+                float4 y = *reinterpret_cast<const float4*>(stage + rr * FT_PITCH + 4 * (lane & 7));
                 if (R) {
                     const float4 x = __ldg(reinterpret_cast<const float4*>(R + (size_t)m * N + n));
                     y.x += x.x; y.y += x.y; y.z += x.z; y.w += x.w;
@@ -265,7 +385,15 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
                 *reinterpret_cast<float4*>(O + (size_t)m * N + n) = y;
             }
             named_bar_sync(1, 32 * FT_WORKERS);          // the staging area is an operand buffer again
-            if (threadIdx.x == 0) tiny[i & 1] = 0;       // (next marked in the tile after the next, behind the next one's barriers)
+        }
+        // ---- tiles that were marked (outputs and marks of all warps are complete behind the last barrier)
+        if (ok) {
+            for (uint32_t j = 0; j < i; ++j) {
+                if (!(marks[mark_of(j) / 32] >> (mark_of(j) % 32) & 1u)) continue;
+                const int t = blockIdx.x + j * gridDim.x, r = t / nt, w = r / mt;
+                ft_form_again(X, w == 0 ? W0 : (w == 1 ? W1 : W2), w == 0 ? O0 : (w == 1 ? O1 : O2), R, (r % mt) * FT_M, (t % nt) * FT_N, M, K,
+                              N, reinterpret_cast<FtAgain*>(smem));
+            }
         }
     }
     tc_fence_before();

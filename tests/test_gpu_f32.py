@@ -215,3 +215,89 @@ def test_more_rows_than_a_grid_holds(B, n, D, d, scheme):
                                  1, scheme, residual=x)
     ref = ref[0] if isinstance(ref, tuple) else ref
     assert np.abs(z[pick.cuda()].cpu().numpy() - ref).max() <= TOL_F32
+
+
+def _signed(rng, shape, exponent):
+    return (rng.choice([-1.0, 1.0], shape) * rng.uniform(1, 2, shape) * 2.0 ** exponent).astype(np.float32)
+
+
+# Operands and products near and below the smallest normal numbers: the outputs are then those of the plain chain of fmaf, bit
+# for bit (small calls run that chain), also where the call is large enough for the tensor cores.
+@pytest.mark.parametrize("ex,ew", [(-70, -65), (-99, -30), (-99, -40), (-110, 0), (-20, -110), (-130, 0), (-145, 3), (-65, -75)])
+def test_projection_of_tiny_numbers(ex, ew):
+    rows, D, d = 1100, 300, 64
+    rng = np.random.default_rng(5)
+    X, W = _signed(rng, (rows, 1, D), ex), _signed(rng, (D, d), ew)
+    y = binding.psa_attention_f32(_dev(X), _dev(W), _dev(W), _dev(W), 1, binding.FULL).cpu().numpy()
+    for at in (0, 113, rows - 33):
+        few = binding.psa_attention_f32(_dev(X[at:at + 33]), _dev(W), _dev(W), _dev(W), 1, binding.FULL).cpu().numpy()
+        assert np.array_equal(few.view(np.int32), y[at:at + 33].view(np.int32))
+
+
+# Single tiny numbers among ordinary ones, as the tail of an exponential leaves them, rows of zeros beside them, and a row that
+# holds nothing but tiny numbers: the ordinary outputs keep their accuracy, zeros are exact, the tiny row is the plain chain's.
+@pytest.mark.parametrize("rows,D,d", [(1100, 300, 64), (1025, 1000, 68)])
+def test_projection_of_ordinary_rows_with_tiny_numbers(rows, D, d):
+    rng = np.random.default_rng(6)
+    X = rng.standard_normal((rows, 1, D)).astype(np.float32)
+    W = (rng.standard_normal((D, d)) / np.sqrt(D)).astype(np.float32)
+    X[:, 0, 5], X[::7], X[10, 0, :] = 1e-35, 0.0, 3e-34
+    W[9, 3], W[:, 11] = 1e-38, 0.0
+    y = binding.psa_attention_f32(_dev(X), _dev(W), _dev(W), _dev(W), 1, binding.FULL).cpu().numpy().reshape(rows, d)
+    a, b = X.reshape(rows, D).astype(np.float64), W.astype(np.float64)
+    assert (np.abs(y - a @ b) <= 2.0 ** -24 * D * (np.abs(a) @ np.abs(b)) + 2.0 ** -149).all()      # (bound: test_projection_forms)
+    assert (y[::7] == 0).all() and (y[:, 11] == 0).all()
+    few = binding.psa_attention_f32(_dev(X[:33]), _dev(W), _dev(W), _dev(W), 1, binding.FULL).cpu().numpy().reshape(33, d)
+    assert np.array_equal(few[10].view(np.int32), y[10].view(np.int32))
+
+
+# Numbers that the parts cannot carry must not decide what a call costs.  Tile by tile on one thread per 32 outputs, they made
+# the projection of this layer 20 to 40 times as long; computed again from shared memory it is two to four times.
+@pytest.mark.parametrize("what", ["one per row", "all tiny", "all NaN", "one row NaN"])
+def test_projection_time_with_tiny_numbers(what):
+    rows, D, d = 4096, 768, 64
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.randn(64, rows // 64, D, device="cuda", generator=g)
+    W = [torch.randn(D, 12 * d, device="cuda", generator=g) * D ** -0.5 for _ in range(3)]
+    Y = X.clone()
+    if what == "one per row":
+        Y[:, :, 5] = 1e-35
+    elif what == "all tiny":
+        Y *= 1e-33
+    elif what == "all NaN":
+        Y[:] = float("nan")
+    else:
+        Y[0, 3] = float("nan")
+    out = torch.empty(64, rows // 64, 12 * d, device="cuda")
+
+    def us(x):
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                binding.psa_attention_f32(x, *W, 12, binding.MASKED, out=out)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[3]
+    us(X)
+    assert us(Y) <= 6 * us(X)
+
+
+# A CTA marks its tiles one by one up to 1024 of them, in groups beyond (here 1035 per CTA on 148 SMs): sequences of tiny numbers
+# in marked tiles at both ends and in the middle of the call come out as in a small call, their neighbours stay accurate.
+def test_projection_of_tiny_numbers_in_a_very_large_call():
+    B, n, D = 1225000, 16, 4
+    g = torch.Generator(device="cuda").manual_seed(2)
+    X = torch.randn(B, n, D, device="cuda", generator=g)
+    W = [torch.randn(D, D, device="cuda", generator=g) for _ in range(3)]
+    at = [0, 5, 777777, B - 9, B - 1]
+    X[at] *= 1e-34
+    Wo = torch.randn(D, D, device="cuda", generator=g)
+    z = binding.psa_attention_block(X, *W, Wo, 1, binding.FULL)
+    few = binding.psa_attention_block(X[at].repeat(8, 1, 1).contiguous(), *W, Wo, 1, binding.FULL)       # 40 heads
+    assert torch.equal(z[at].view(torch.int32), few[:len(at)].view(torch.int32))
+    near = [1, 4, 6, 777776, 777778, B - 10, B - 2]
+    ref, _, _ = oracle.attention_block(X[near].cpu().numpy(), *[w.cpu().numpy() for w in W], Wo.cpu().numpy(), 1, oracle.FULL)
+    assert np.abs(z[near].cpu().numpy() - ref).max() <= TOL_F32
