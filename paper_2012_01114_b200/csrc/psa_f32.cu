@@ -87,17 +87,17 @@ f32_project_tiled_kernel(const float* __restrict__ X, const float* W0, const flo
     const int m0 = blockIdx.y * GP_BM, n0 = blockIdx.x * GP_BN;
     const int nk = (D + GP_BK - 1) / GP_BK;
 
-    auto load = [&](int kt) {       // k-step kt: rows beyond the matrix are clamped, columns of k beyond D skipped
+    auto load = [&](int kt) {       // k-step kt; what lies outside the matrices is not loaded, and nothing that is stored reads it
         float* a = sm + (kt % GP_STAGES) * GP_STAGE;
         float* b = a + GP_A_FLOATS;
         const int k0 = kt * GP_BK;
         for (int t = tid; t < GP_BM * (GP_BK / 4); t += GP_THREADS) {
             const int r = t / (GP_BK / 4), c = (t % (GP_BK / 4)) * 4;
-            if (k0 + c < D) cp_async16(a + r * GP_LDA + c, X + (size_t)min(m0 + r, rows - 1) * D + k0 + c);
+            if (m0 + r < rows && k0 + c < D) cp_async16(a + r * GP_LDA + c, X + (size_t)(m0 + r) * D + k0 + c);
         }
         for (int t = tid; t < GP_BK * (GP_BN / 4); t += GP_THREADS) {
             const int k = t / (GP_BN / 4), c = (t % (GP_BN / 4)) * 4;
-            if (k0 + k < D) cp_async16(b + k * GP_BN + c, W + (size_t)(k0 + k) * N + min(n0 + c, N - 4));
+            if (n0 + c < N && k0 + k < D) cp_async16(b + k * GP_BN + c, W + (size_t)(k0 + k) * N + n0 + c);
         }
     };
     unsigned long long acc[GP_TM][2] = {};
@@ -1068,6 +1068,12 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
         static DeviceSetup setup;
         const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 projection set-up");
         if (sms <= 0) return cudaErrorUnknown;
+        // Bound by the latency of their k-steps, the smallest calls run best on the 16 x 16 tiles of the general kernel, as long
+        // as these are not more than the SMs (by the library's events, us, 16 x 16 / 32 x 32: 96 x 768 x 3 x 64, 72 tiles, 22.8 /
+        // 24.7; 16 x 768 x 3 x 768, 144 tiles, 22.9 / 24.9; 200 x 768 x 3 x 64, 156 tiles, 25.5 / 24.8; 128 x 2048 x 64, 32 tiles,
+        // 51.2 / 55.0), for calls of one row of tiles up to three times that (16 x 1024 x 3 x 2048, 384 tiles, 43.2 / 46.6).
+        const long long tiles16 = (long long)((rows + 15) / 16) * ((N + 15) / 16) * nW;
+        if (tiles16 <= (rows <= 16 ? 3 * sms : sms)) return project_general(X, W, out, nW, rows, D, N, residual, dc, stream);
         // The tensor cores from two 32 x 32 tiles per SM on, by measurement (us, 32 x 32 tiles on CUDA cores / tensor cores):
         // 64 x 768 x 3 x 64 23.5 / 32.3, 128 x 768 x 3 x 768 (288 tiles) 29.6 / 33.6, 2048 x 768 x 3 x 64 (384) 37.5 / 33.4,
         // 600 x 320 x 3 x 320 (570) 27.3 / 21.3, 64 x 2048 x 3 x 2048 (384) 89 / 72; larger ones, against 128 x 128 tiles on CUDA

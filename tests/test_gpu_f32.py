@@ -301,3 +301,11 @@ def test_projection_of_tiny_numbers_in_a_very_large_call():
     near = [1, 4, 6, 777776, 777778, B - 10, B - 2]
     ref, _, _ = oracle.attention_block(X[near].cpu().numpy(), *[w.cpu().numpy() for w in W], Wo.cpu().numpy(), 1, oracle.FULL)
     assert np.abs(z[near].cpu().numpy() - ref).max() <= TOL_F32
+
+
+# The lines between the 16 x 16 and the 32 x 32 tiles of small projections (148 SMs: 144, 156 and 204 tiles of 16 x 16; one row of
+# tiles with 384 and 480), rows and columns beside the edges of both.
+@pytest.mark.parametrize("rows,D,H,d", [(192, 300, 1, 64), (197, 300, 1, 64), (260, 300, 1, 64), (257, 308, 1, 68), (16, 300, 32, 64),
+                                        (16, 300, 40, 64), (1, 300, 40, 64), (31, 300, 13, 20), (33, 332, 10, 36)])
+def test_projection_forms_of_small_calls(rows, D, H, d):
+    test_projection_forms(rows, D, H, d)
