@@ -1152,13 +1152,10 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
 }
 template <int DG, int MODE>
 cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n,
-                               int d, float scale, int masked, DeviceCounters* dc, cudaStream_t stream) {
+                               int d, float scale, int masked, DeviceCounters* dc, int sms, cudaStream_t stream) {
 #ifdef PSA_FA_KS
     return launch_flash<DG, PSA_FA_KS, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
 #endif
-    static DeviceSetup setup;
-    const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
-    if (sms <= 0) return cudaErrorUnknown;
     auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
     // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs:
     // measured, two resident CTAs per SM are where the line lies (us for KS = 1 / 2 / 4, with the first form of the kernel).  80
@@ -1169,9 +1166,9 @@ cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, f
 }
 template <int DG>
 cudaError_t tiled_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H, int n, int d,
-                            float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+                            float scale, int scheme, DeviceCounters* dc, int sms, cudaStream_t stream) {
     if (scheme != PSA_SYMMETRIC)
-        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, stream);
+        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, sms, stream);
     constexpr int SMEM = (FACfg<DG, 1>::Q_FLOATS + FACfg<DG, 1>::K_FLOATS) * (int)sizeof(float);
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
@@ -1182,15 +1179,37 @@ cudaError_t tiled_attention(const float* Q, const float* K, const float* V, floa
     f32_sym_scores_kernel<DG><<<dim3(B * H, T * (T + 1) / 2), FA_THREADS, SMEM, stream>>>(Q, S, n, H, d, scale, dc);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, stream);
+    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, sms, stream);
+}
+}  // namespace
+
+namespace {
+// Whether the general kernel, a warp per row and many small CTAs per SM, is the faster one: heads of few vectors.  The tiled
+// one has two or three CTAs per SM, in each of which one warp of four has work then, and the symmetric scheme's takes 64 x 64
+// blocks whatever the length.  Measured on 148 SMs (us, general / tiled; FULL, MASKED is alike): 1024 heads of n = 8, d = 16 22.7 /
+// 26.5, n = 12 30.9 / 27.4; d = 64, n = 8 26.8 / 41.0, n = 12 36.0 / 42.5, n = 16 46.2 / 42.3; d = 128, n = 16 53.6 / 78.0, n = 28
+// 103 / 115, n = 32 123 / 94; 4096 heads of d = 128, n = 16 253 / 269, n = 20 360 / 330; up to a head per SM no difference (148
+// heads of n = 12, d = 128: 16.6 / 14.5).  Symmetric: a head of n = 8, d = 16 14.3 / 14.5, d = 64 14.2 / 18.6, d = 128 14.4 / 28.8;
+// 1024 heads of n = 12, d = 16 35.1 / 32.9, d = 64 39.9 / 47.3, n = 16 51.8 / 47.3, d = 128, n = 20 84 / 92, n = 24 99 / 100; 64 heads
+// of n = 28, d = 32 16.6 / 16.6, n = 32, d = 64 18.6 / 19.1, n = 40, d = 128 33.0 / 32.9, 16 heads 27.3 / 30.9.
+bool short_heads(long long heads, int n, int d, bool sym, int sms) {
+    if (sym) return n <= (d <= 16 ? 8 : d <= 64 ? 12 : 20) || (2 * heads <= sms && d > 16 && n <= (d <= 64 ? 32 : 40));
+    if (heads <= sms) return false;
+    if (n <= (d <= 16 ? 8 : d <= 48 ? 10 : 12)) return true;
+    return d > 64 && heads > (d <= 96 ? 4 : 3) * sms && n <= (heads <= 8 * sms ? 28 : 16);
 }
 }  // namespace
 
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H,
                           int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+    static DeviceSetup setup;
+    const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
+    if (sms <= 0) return cudaErrorUnknown;
+    if (H <= GRID_MAX && short_heads((long long)B * H, n, d, scheme == PSA_SYMMETRIC, sms))
+        return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
     if (d % 4 == 0 && (long long)B * H <= 0x7fffffff && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(out))      // 16-byte rows
-        return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream)
-                       : tiled_attention<2>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
+        return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, sms, stream)
+                       : tiled_attention<2>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, sms, stream);
     return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
 }
 

@@ -309,3 +309,13 @@ def test_projection_of_tiny_numbers_in_a_very_large_call():
                                         (16, 300, 40, 64), (1, 300, 40, 64), (31, 300, 13, 20), (33, 332, 10, 36)])
 def test_projection_forms_of_small_calls(rows, D, H, d):
     test_projection_forms(rows, D, H, d)
+
+
+# Heads of few vectors run on the general kernel; the line depends on the number of heads, their size and the scheme (148 SMs).
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.SYMMETRIC, oracle.MASKED])
+@pytest.mark.parametrize("B,H,n,d", [(150, 1, 8, 16), (40, 4, 9, 16), (75, 2, 10, 48), (75, 2, 11, 48), (10, 15, 12, 64), (10, 15, 13, 64),
+                                     (300, 2, 16, 128), (300, 2, 28, 68), (300, 2, 29, 128), (1200, 1, 16, 100), (1200, 1, 17, 100),
+                                     (1, 1, 1, 8), (1, 3, 32, 64), (37, 2, 33, 64), (1, 74, 40, 68), (5, 15, 20, 128), (5, 15, 21, 128),
+                                     (1, 75, 40, 68)])
+def test_core_of_short_heads(scheme, B, H, n, d):
+    test_core_at_tile_edges(scheme, B, H, n, d)
