@@ -117,6 +117,14 @@ WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme
     return L;
 }
 
+// Whether copies from or to this host memory run beside the calling thread (memory that CUDA knows of).
+bool pinned(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type != cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    return false;
+}
+
 HostPipe* acquire_pipe(Context& cx) {
     if (cx.pipe) return cx.pipe;
     HostPipe* p = new (std::nothrow) HostPipe;
@@ -364,9 +372,11 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
     const size_t xb = (size_t)n * d_model * es, wb = (size_t)d_model * heads * d_k * es, ob = (size_t)n * heads * d_k * es;   // per sequence; per matrix
     const int parts = host_parts(batch, xb, ob, X_host, out_host);
-    // (a call that is being timed runs in one part)
+    // One part if the call is being timed, and for bf16 in pageable buffers: copies from and to these hold the calling
+    // thread, so that little overlaps, and every further copy costs (16 x 512 x 768, 12 heads: 1560 us in one part, 1790 in
+    // eight; in fp32, whose kernels take longer, 4140 and 3310).
     HostPipe* pipe = nullptr;
-    if (parts > 1 && cx.prof_calls >= cx.prof_max) {
+    if (parts > 1 && cx.prof_calls >= cx.prof_max && (dtype == PSA_F32 || (pinned(X_host) && pinned(out_host)))) {
         pipe = acquire_pipe(cx);
         if (!pipe) return PSA_ERR_CUDA;
     }
@@ -389,7 +399,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     }
     // In parts: copies in on one stream, kernels on the caller's, copies out on another.  The counters of all parts go to one
     // block; the work counter of each has a place of its own behind the blocks.  All copies in are queued before the first copy
-    // out: with pageable buffers a copy may hold the calling thread until it is done.
+    // out: one from pageable memory (a matrix) holds the calling thread until it is done.
     const char* what = "ordering the streams of a host call";
     cudaError_t e = cudaEventRecord(pipe->start, stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->start, 0);
