@@ -94,15 +94,15 @@ WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme
     WsLayout L;
     memset(&L, 0, sizeof(L));
     size_t off = COUNTER_BYTES;
+    if (scheme == PSA_SYMMETRIC) {       // (right behind the counters: one clear serves both, see run_layer)
+        L.s_bytes = dtype == PSA_BF16 ? bf16_symmetric_scratch_bytes(batch, heads, n)
+                                      : align_up((size_t)batch * heads * n * n * sizeof(float), 256);
+        L.s = off; off += L.s_bytes;
+    }
     if (with_proj) {
         L.q = off; off += qkv;
         if (scheme == PSA_SYMMETRIC) { L.k = L.q; L.v = L.q; }
         else { L.k = off; off += qkv; L.v = off; off += qkv; }
-    }
-    if (scheme == PSA_SYMMETRIC) {
-        L.s_bytes = dtype == PSA_BF16 ? bf16_symmetric_scratch_bytes(batch, heads, n)
-                                      : align_up((size_t)batch * heads * n * n * sizeof(float), 256);
-        L.s = off; off += L.s_bytes;
     }
     if (staging) {
         const size_t xb = align_up((size_t)batch * n * d_model * es, 256);
@@ -180,7 +180,7 @@ void useful_counts(int batch, int heads, int n, int d_model, int d_k, int scheme
 // Context (may be null).  `between`, if given, is recorded between projections and attention.
 int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K, const void* V,
                   int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out, cudaStream_t stream,
-                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, DeviceCounters* dc, unsigned int* cursor,
+                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, bool s_clear, DeviceCounters* dc, unsigned int* cursor,
                   DeviceCounters* dc_next, cudaEvent_t between) {
     const float scale = 1.0f / sqrtf((float)d_k);
     const int nW = scheme == PSA_SYMMETRIC ? 1 : 3;
@@ -214,7 +214,7 @@ int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv,
         if (e != cudaSuccess) { set_cuda_error(e, "f32_attention"); return PSA_ERR_CUDA; }
         return PSA_OK;
     }
-    return bf16_attention(Q, K, V, out, S, s_bytes, batch, heads, n, d_k, scale, scheme, dc, cursor, dc_next, stream);
+    return bf16_attention(Q, K, V, out, S, s_bytes, s_clear, batch, heads, n, d_k, scale, scheme, dc, cursor, dc_next, stream);
 }
 
 int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K,
@@ -227,10 +227,14 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     cudaError_t e = cudaStreamIsCapturing(stream, &capture);
     if (e != cudaSuccess) { set_cuda_error(e, "cudaStreamIsCapturing"); return PSA_ERR_CUDA; }
     const bool captured = capture != cudaStreamCaptureStatusNone;
+    float* S = scheme == PSA_SYMMETRIC ? reinterpret_cast<float*>(ws + L.s) : nullptr;
+    const bool s_clear = !captured && S && dtype == PSA_BF16;      // counters and flags of the symmetric kernel cleared in one go
     int block = 0;
     if (captured) {
         block = CAPTURE_BLOCK;
         e = cudaMemsetAsync(ws + CAPTURE_BLOCK * COUNTER_BLOCK_BYTES, 0, COUNTER_BLOCK_BYTES, stream);
+    } else if (s_clear) {
+        e = bf16_symmetric_clear(S, L.s_bytes, batch, heads, n, L.s, stream);
     } else if (turns && cx.clean_ws == ws) {
         block = cx.next_block;
     } else {
@@ -251,9 +255,8 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     } tail{pev, stream};
     if (pev) cudaEventRecord(pev[0], stream);
     void* const qkv[3] = {ws + L.q, ws + L.k, ws + L.v};
-    float* S = scheme == PSA_SYMMETRIC ? reinterpret_cast<float*>(ws + L.s) : nullptr;
     const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
-                                 qkv, S, L.s_bytes, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
+                                 qkv, S, L.s_bytes, s_clear, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
     if (rc == PSA_OK && turns && !captured) {        // the other block will be clear once this call has run
         cx.clean_ws = ws;
         cx.next_block = block ^ 1;
@@ -430,7 +433,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
         rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
                            d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,
-                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, dc,
+                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, dc,
                            reinterpret_cast<unsigned int*>(ws + CURSOR_OFFSET) + c, nullptr, nullptr);
         if (rc != PSA_OK) break;
         e = cudaEventRecord(pipe->computed[c], stream);

@@ -153,6 +153,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
     volatile int* abortp = &abort_flag;
+    grid_dependency_wait();      // (programmatic dependent launch, as in attn_persist_kernel)
 
     if (warp == 0) {
         if (lane == 0) {
@@ -512,12 +513,22 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
             }
             tc_fence_before();
         }
+        if (wq == 0 && lane == 0) grid_launch_dependents();
         if (lane == 0) tma_store_wait_read();   // shared memory may be released; the writes complete on their own
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) atomicExch(&dc->status, (int)PSA_ERR_TIMEOUT);
     if (warp == 1) tmem_dealloc(tmem, 512);
+}
+
+// The flags of `heads` heads and the work counter of a launch (the diagonal block whose place they take has room for 16384),
+// cleared together with `before` bytes ahead of each of these places: for the first head, what lies ahead of the scratch;
+// for the others the end of a diagonal block, which nothing uses.
+cudaError_t sym_clear(float* S, int heads, int T, size_t before, cudaStream_t stream) {
+    char* p = reinterpret_cast<char*>(S) - before;
+    const size_t bytes = before + (size_t)(T + 1) * sizeof(int);
+    return heads == 1 ? cudaMemsetAsync(p, 0, bytes, stream) : cudaMemset2DAsync(p, (size_t)sym_pairs(T) * S_BLOCK_BYTES, 0, bytes, heads, stream);
 }
 
 // Heads per group of the item list: the tiles of one head are started a group apart.  A tile needs its first handed-on block
@@ -528,9 +539,9 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, in
 constexpr int SYM_GROUP_ITEMS = 256;
 
 // D: head size the kernel works with (64 or 128); d <= D: the tensors' head size (see the 4-D tensor maps).
-// s_bytes: size of the score scratch, which sets the heads per pass.
+// s_bytes: size of the score scratch, which sets the heads per pass; s_clear: the first pass finds its flags clear.
 template <int D>
-int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, int B, int H, int n, int d, float scale, DeviceCounters* dc,
+int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, bool s_clear, int B, int H, int n, int d, float scale, DeviceCounters* dc,
                      cudaStream_t stream) {
     using Cfg = SymCfg<D>;
     static DeviceSetup setup;
@@ -539,7 +550,6 @@ int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, int B, 
     }, "cudaFuncSetAttribute(symmetric attention)");
     if (sm_count <= 0) return PSA_ERR_CUDA;
     const int T = row_tiles(n);
-    const size_t head_bytes = (size_t)sym_pairs(T) * S_BLOCK_BYTES;
     const int hp = sym_heads_per_pass((size_t)B * H, n, s_bytes);
     SymMaps maps;
     if (!make_tensor_map_bf16_4d(&maps.x, X, B, n, H, d, 128) || !make_tensor_map_bf16_4d(&maps.o, out, B, n, H, d, 16))
@@ -548,13 +558,19 @@ int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, int B, 
         const int heads = min(hp, B * H - bh0);
         if ((long long)heads * T > 0x7fffffffLL - 2 * sm_count) return PSA_ERR_SHAPE;      // (the work counter runs past the list)
         const int nitems = heads * T;
-        // flags of every head and the work counter (the diagonal block whose place they take has room for 16384)
-        const size_t flag_bytes = (size_t)(T + 1) * sizeof(int);
-        cudaError_t e = heads == 1 ? cudaMemsetAsync(S, 0, flag_bytes, stream)
-                                   : cudaMemset2DAsync(S, head_bytes, 0, flag_bytes, heads, stream);
+        cudaError_t e = bh0 == 0 && s_clear ? cudaSuccess : sym_clear(S, heads, T, 0, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "symmetric scheme: clearing the flags"); return PSA_ERR_CUDA; }
-        sym_attn_kernel<D><<<min(nitems, sm_count), SYM_THREADS, Cfg::SMEM, stream>>>(maps, S, n, H, bh0, heads, min(heads, max(1, SYM_GROUP_ITEMS / T)), scale * LOG2E, dc);
-        e = cudaGetLastError();
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(min(nitems, sm_count));
+        cfg.blockDim = dim3(SYM_THREADS);
+        cfg.dynamicSmemBytes = Cfg::SMEM;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, sym_attn_kernel<D>, maps, S, n, H, bh0, heads, min(heads, max(1, SYM_GROUP_ITEMS / T)), scale * LOG2E, dc);
         if (e != cudaSuccess) { set_cuda_error(e, "sym_attn_kernel launch"); return PSA_ERR_CUDA; }
     }
     return PSA_OK;
@@ -566,7 +582,11 @@ size_t bf16_symmetric_scratch_bytes(int B, int H, int n) {
     return (size_t)sym_heads_per_pass((size_t)B * H, n, SYM_SCRATCH_CAP) * sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
 }
 
-int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, int B, int H,
+cudaError_t bf16_symmetric_clear(float* S, size_t s_bytes, int B, int H, int n, size_t before, cudaStream_t stream) {
+    return sym_clear(S, sym_heads_per_pass((size_t)B * H, n, s_bytes), row_tiles(n), before, stream);
+}
+
+int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, bool s_clear, int B, int H,
                    int n, int d, float scale, int scheme, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next,
                    cudaStream_t stream) {
     if (scheme != PSA_SYMMETRIC && d > 128) return bf16_attention_wide(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
@@ -574,8 +594,8 @@ int bf16_attention(const void* Q, const void* K, const void* V, void* out, float
     if (!S || s_bytes < (size_t)sym_pairs(row_tiles(n)) * S_BLOCK_BYTES) return PSA_ERR_WORKSPACE;       // (one head)
     if ((reinterpret_cast<uintptr_t>(S) & 15u) != 0) return PSA_ERR_ALIGN;
     if (d < 8 || d > 128 || d % 8) return PSA_ERR_UNSUPPORTED;
-    if (d <= 64) return launch_symmetric<64>(Q, out, S, s_bytes, B, H, n, d, scale, dc, stream);
-    return launch_symmetric<128>(Q, out, S, s_bytes, B, H, n, d, scale, dc, stream);
+    if (d <= 64) return launch_symmetric<64>(Q, out, S, s_bytes, s_clear, B, H, n, d, scale, dc, stream);
+    return launch_symmetric<128>(Q, out, S, s_bytes, s_clear, B, H, n, d, scale, dc, stream);
 }
 
 }  // namespace psa

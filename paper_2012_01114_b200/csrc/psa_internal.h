@@ -50,10 +50,13 @@ int bf16_project(const void* A, const void* const Bw[3], void* const C[3], int n
 // one head's worth, the call runs in more passes).
 // `dc_next`, if not null, is a second counter block that the call's attention kernel clears (FULL, MASKED only).
 // `cursor` is the work counter of the fused kernel (FULL, MASKED), zero when the call's kernels start.
-int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, int B,
+// `s_clear`: bf16_symmetric_clear has been queued ahead of the call's kernels.
+int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, bool s_clear, int B,
                    int H, int n, int d, float scale, int scheme, DeviceCounters* dc, unsigned int* cursor,
                    DeviceCounters* dc_next, cudaStream_t stream);
 size_t bf16_symmetric_scratch_bytes(int B, int H, int n);
+// Clears what the first pass of the symmetric kernel needs clear in its scratch, and `before` bytes ahead of the scratch.
+cudaError_t bf16_symmetric_clear(float* S, size_t s_bytes, int B, int H, int n, size_t before, cudaStream_t stream);
 // PSA_FULL and PSA_MASKED for 128 < d <= 256 (psa_attn_wide.cu).
 int bf16_attention_wide(const void* Q, const void* K, const void* V, void* out, int B, int H, int n, int d, float scale,
                         int scheme, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next, cudaStream_t stream);
