@@ -374,12 +374,9 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     if (!ws) return PSA_ERR_WORKSPACE;
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
     const size_t xb = (size_t)n * d_model * es, wb = (size_t)d_model * heads * d_k * es, ob = (size_t)n * heads * d_k * es;   // per sequence; per matrix
-    const int parts = host_parts(batch, xb, ob, X_host, out_host);
-    // One part if the call is being timed, and for bf16 in pageable buffers: copies from and to these hold the calling
-    // thread, so that little overlaps, and every further copy costs (16 x 512 x 768, 12 heads: 1560 us in one part, 1790 in
-    // eight; in fp32, whose kernels take longer, 4140 and 3310).
+    int parts = host_parts(batch, xb, ob, X_host, out_host);
     HostPipe* pipe = nullptr;
-    if (parts > 1 && cx.prof_calls >= cx.prof_max && (dtype == PSA_F32 || (pinned(X_host) && pinned(out_host)))) {
+    if (parts > 1 && cx.prof_calls >= cx.prof_max) {         // (a call that is being timed runs in one part, on one stream)
         pipe = acquire_pipe(cx);
         if (!pipe) return PSA_ERR_CUDA;
     }
@@ -419,6 +416,10 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         if (e == cudaSuccess && !sym) e = cudaMemcpyAsync(ws + L.wk, Wk_host, wb, cudaMemcpyHostToDevice, pipe->in);
         if (e == cudaSuccess && !sym) e = cudaMemcpyAsync(ws + L.wv, Wv_host, wb, cudaMemcpyHostToDevice, pipe->in);
     }
+    // One part for bf16 in pageable buffers: copies from and to these hold the calling thread, so that little overlaps, and every
+    // further copy costs (16 x 512 x 768, 12 heads: 1560 us in one part, 1790 in eight; in fp32, whose kernels take longer, 4140
+    // and 3310).  Asked here, under the copies of the matrices: the answer takes a few microseconds per buffer.
+    if (dtype == PSA_BF16 && !(pinned(X_host) && pinned(out_host))) parts = 1;
     auto first = [&](int c) { return (int)((long long)batch * c / parts); };      // first sequence of part c
     for (int c = 0; c < parts && e == cudaSuccess; ++c) {
         const size_t b0 = first(c), nb = first(c + 1) - b0;
