@@ -69,6 +69,8 @@ typedef enum {
  *                   FULL d*n^2 each; MASKED d*n(n+1)/2 each; SYMMETRIC d*n(n+1)/2 and d*n^2
  * The bf16 path issues whole 128x128 blocks of the weight matrix, so issued >= useful there (a
  * block on the diagonal, or a ragged last block, is issued in full); the fp32 path skips element by element, issued = useful.
+ * proj_macs counts the multiply-accumulates of the plain product on every path (the fp32 projections of large calls form six
+ * bf16 products for each, on padded tiles).
  */
 typedef struct {
     uint64_t proj_macs, qk_macs, pv_macs, exps, useful_qk_macs, useful_pv_macs;
@@ -86,8 +88,10 @@ typedef struct {
 int psa_attention(const void* X, const void* Wq, const void* Wk, const void* Wv, int batch, int heads, int n,
                   int d_model, int d_k, int scheme, void* out, void* stream);
 
-/* Same computation in fp32 storage and fp32 arithmetic on CUDA cores, element-exact skipping
- * (issued = useful).  Supported: n <= 1024, d_k <= 128 (any d_model). */
+/* Same computation in fp32 storage, to fp32 accuracy.  The three phases run in fp32 arithmetic on CUDA cores with element-
+ * exact skipping (issued = useful), and so do the projections of small calls; those of large calls run on the tensor cores,
+ * every number split into three bf16 parts, with an error below that of a chain of fp32 additions (outputs too small for that,
+ * or not finite, are formed by such a chain).  Supported: n <= 1024, d_k <= 128 (any d_model). */
 int psa_attention_f32(const void* X, const void* Wq, const void* Wk, const void* Wv, int batch, int heads, int n,
                       int d_model, int d_k, int scheme, void* out, void* stream);
 
@@ -175,7 +179,8 @@ int psa_last_issued(void* stream, psa_counts* counts);
  * output and partial row sum by exp(old maximum - new maximum).  The kernels raise the maximum only
  * when it has grown by more than 2^8, so on inputs whose scores stay within a few units of each other
  * the count is zero; it is nonzero when later keys carry much larger scores than earlier ones.
- * The fp32 path finds each row's maximum before its first exponential and always reports zero.
+ * The fp32 path does not count such events (its online softmax rescales whenever a block of keys raises a row's maximum)
+ * and always reports zero.
  */
 int psa_last_rescales(void* stream, uint64_t* rescales);
 

@@ -53,7 +53,7 @@ Context* current_ctx() {
 
 struct HostPipe {
     cudaStream_t in = nullptr, out = nullptr;
-    cudaEvent_t start = nullptr, weights = nullptr, loaded[HOST_CHUNKS] = {}, computed[HOST_CHUNKS] = {}, stored = nullptr;
+    cudaEvent_t start = nullptr, loaded[HOST_CHUNKS] = {}, computed[HOST_CHUNKS] = {}, stored = nullptr;
 };
 
 constexpr size_t COUNTER_BYTES = 256;          // counter blocks and cursors at the start of the workspace
@@ -132,13 +132,13 @@ HostPipe* acquire_pipe(Context& cx) {
     cudaError_t e = cudaStreamCreateWithFlags(&p->in, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->out, cudaStreamNonBlocking);
     auto event = [&](cudaEvent_t* ev) { if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming); };
-    event(&p->start); event(&p->weights); event(&p->stored);
+    event(&p->start); event(&p->stored);
     for (int c = 0; c < HOST_CHUNKS; ++c) { event(&p->loaded[c]); event(&p->computed[c]); }
     if (e == cudaSuccess) return cx.pipe = p;
     set_cuda_error(e, "streams of the host entry points");
     if (p->in) cudaStreamDestroy(p->in);
     if (p->out) cudaStreamDestroy(p->out);
-    for (cudaEvent_t ev : {p->start, p->weights, p->stored}) if (ev) cudaEventDestroy(ev);
+    for (cudaEvent_t ev : {p->start, p->stored}) if (ev) cudaEventDestroy(ev);
     for (int c = 0; c < HOST_CHUNKS; ++c) {
         if (p->loaded[c]) cudaEventDestroy(p->loaded[c]);
         if (p->computed[c]) cudaEventDestroy(p->computed[c]);
@@ -417,7 +417,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         if (e == cudaSuccess && !sym) e = cudaMemcpyAsync(ws + L.wv, Wv_host, wb, cudaMemcpyHostToDevice, pipe->in);
     }
     // One part for bf16 in pageable buffers: copies from and to these hold the calling thread, so that little overlaps, and every
-    // further copy costs (16 x 512 x 768, 12 heads: 1560 us in one part, 1790 in eight; in fp32, whose kernels take longer, 4140
+    // further copy costs (16 x 512 x 768, 12 heads: 1597 us in one part, 1812 in eight; in fp32, whose kernels take longer, 4140
     // and 3310).  Asked here, under the copies of the matrices: the answer takes a few microseconds per buffer.
     if (dtype == PSA_BF16 && !(pinned(X_host) && pinned(out_host))) parts = 1;
     auto first = [&](int c) { return (int)((long long)batch * c / parts); };      // first sequence of part c

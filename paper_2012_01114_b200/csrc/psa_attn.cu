@@ -22,8 +22,8 @@
 //
 // What bounds it: softmax (1024 cycles of exponentials per block) and, in step with it, the operands of one row
 // tile per SM: 32 KB of X per block, 64 KB of scores stored or loaded for all but the diagonal one.  Measured
-// (L2 flushed, B = 64, H = 16, n = 1024, d_k = 128): 1430 us as two kernels through 36 blocks written and 64 read
-// per head, 955 us as one with 28 and 28.  An SM spends 4000 cycles per block; clock stamps of a softmax warp put
+// (L2 flushed, B = 64, H = 16, n = 1024, d_k = 128): 1505 us as two kernels through 36 blocks written and 64 read
+// per head, 917 us as one with 28 and 28.  An SM spends 4000 cycles per block; clock stamps of a softmax warp put
 // 950 of them in the exponentials, 550 in the stores of computed blocks, 1000 in waits for handed-on ones.
 //
 // The fused persistent kernel of the FULL and MASKED schemes is in psa_attn_persist.cu.

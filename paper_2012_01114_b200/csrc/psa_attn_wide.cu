@@ -13,7 +13,7 @@
 //
 // What bounds it: 16 MMAs at 92 cycles and 8 at 129 are 2500 cycles per block, 128 KB of operands at an SM's 64 bytes per
 // cycle from L2 2050; measured 3300 on long sequences (16 heads of n = 8192, d_k = 192, masked: 559 us as one CTA per
-// tile with one K and one V stage, 379 now; 32 heads of n = 2048, d_k = 256, masked: 104 and 73).
+// tile with one K and one V stage, 379 now; 32 heads of n = 2048, d_k = 256, masked: 103 and 80).
 //
 // CTA layout (320 threads): warp 0 = work list and TMA producer, warp 1 = MMA issuer, warps 2-9 = softmax and epilogue
 // (a warp owns 16 rows, read in the quad layout of sm100.cuh).  The tensors' head size may be any multiple of 8 in (128,

@@ -1,7 +1,6 @@
-// fp32 storage, fp32 arithmetic path on CUDA cores with element-exact skipping: a weight that the
-// scheme does not need is never computed (paper Sec. 4.1, 5.1), so issued MACs equal the paper's
-// element counts (Sec. 3.2, 4.2, 5.2).  Meant for small problems and as the full-precision path;
-// the throughput path is the bf16 tensor-core one.
+// The full-precision path: fp32 storage, and fp32 arithmetic on CUDA cores but for the projections of large calls, which are
+// in psa_f32_tensor.cu.  Skipping is element-exact: a weight that the scheme does not need is never computed (paper Sec. 4.1,
+// 5.1), so issued MACs equal the paper's element counts (Sec. 3.2, 4.2, 5.2).  The throughput path is the bf16 one.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -163,6 +162,7 @@ f32_project_tiled_kernel(const float* __restrict__ X, const float* W0, const flo
 // it, instruction issue: phase 1 pairs components in two-wide fma, which leaves issue slots to its loads; phase 3 would have to
 // double every weight into a pair and runs on plain fma.  Measured (us, one warp per row before): 48 heads of n = 512, d = 64,
 // full 1554 -> 117; 16 heads of n = 1024, d = 128, masked 2003 -> 172; in a large call 61 multiply-accumulates per clock and SM.
+// (DG = 1 is compiled for three CTAs per SM, 168 registers; with KS = 1 it spills 128 bytes there.)
 //
 // Shared memory, so that no address needs arithmetic in the inner loops: K rows are padded by 16 bytes (16 rows are read at
 // once), Q rows keep 16-byte chunk c at c ^ (row & 1) (rows of both half-warps are read at once), V rows are plain.
@@ -1153,13 +1153,12 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
 template <int DG, int MODE>
 cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n,
                                int d, float scale, int masked, DeviceCounters* dc, int sms, cudaStream_t stream) {
-#ifdef PSA_FA_KS
-    return launch_flash<DG, PSA_FA_KS, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
-#endif
     auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
-    // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs:
-    // measured, two resident CTAs per SM are where the line lies (us for KS = 1 / 2 / 4, with the first form of the kernel).  80
-    // tiles of 64 rows: 208 / 144 / 112; 256 tiles, masked, d = 128: 268 / 216 / 252; 384 tiles: 137 / 155 / 180.
+    // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs: the
+    // line lies at two CTAs per SM (us for KS = 1 / 2 / 4).  16 heads of n = 300, d = 64, 80 tiles of 64 rows: 70 / 44 / 35; 16 of
+    // n = 1024, d = 128, masked, 256 tiles: 210 / 166 / 216; 74 of n = 256, d = 64, 296 tiles: 46 / 54 / 70; 48 of n = 512, d = 64, 384
+    // tiles: 110 / 124 / 159.  It is not exact: 16 heads of n = 1024, FULL, d = 64 161 / 179 / 208; 64 of n = 300, 320 tiles with a
+    // nearly empty last one, 101 / 82 / 87.
     if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
     if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
     return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);

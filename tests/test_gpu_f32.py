@@ -319,3 +319,22 @@ def test_projection_forms_of_small_calls(rows, D, H, d):
                                      (1, 75, 40, 68)])
 def test_core_of_short_heads(scheme, B, H, n, d):
     test_core_at_tile_edges(scheme, B, H, n, d)
+
+
+# Host buffers of some size are worked off in parts of the batch; a part's projections may take another form than the whole
+# call's, so that results agree with the oracle rather than bit for bit with the device entry point.
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("scheme,B,H,n,D,d", [(oracle.FULL, 5, 4, 300, 768, 64), (oracle.MASKED, 9, 3, 257, 320, 20), (oracle.SYMMETRIC, 3, 8, 512, 512, 64),
+                                              (oracle.MASKED, 11, 2, 130, 1026, 50), (oracle.FULL, 130, 1, 64, 192, 32)])
+def test_host_batch_in_parts(scheme, B, H, n, D, d, pinned):
+    rng = np.random.default_rng(B + n)
+    sym = scheme == oracle.SYMMETRIC
+    X = rng.standard_normal((B, n, D)).astype(np.float32)
+    W = [(rng.standard_normal((D, H * d)) / np.sqrt(D)).astype(np.float32) for _ in range(1 if sym else 3)]
+    host = [torch.from_numpy(a).pin_memory() if pinned else torch.from_numpy(a) for a in [X] + W] + ([None, None] if sym else [])
+    out = torch.full((B, n, H * d), float("nan"))
+    out = out.pin_memory() if pinned else out
+    binding.psa_attention_host(*host, H, scheme, out)
+    ref, cnt = oracle.attention_layer(X, *(W * 3 if sym else W), H, scheme)
+    _check_counts(cnt, (1 if sym else 3) * B * n * D * H * d)
+    assert np.abs(out.numpy().astype(np.float64) - ref).max() <= TOL_F32
