@@ -1185,17 +1185,29 @@ cudaError_t tiled_attention(const float* Q, const float* K, const float* V, floa
 namespace {
 // Whether the general kernel, a warp per row and many small CTAs per SM, is the faster one: heads of few vectors.  The tiled
 // one has two or three CTAs per SM, in each of which one warp of four has work then, and the symmetric scheme's takes 64 x 64
-// blocks whatever the length.  Measured on 148 SMs (us, general / tiled; FULL, MASKED is alike): 1024 heads of n = 8, d = 16 22.7 /
-// 26.5, n = 12 30.9 / 27.4; d = 64, n = 8 26.8 / 41.0, n = 12 36.0 / 42.5, n = 16 46.2 / 42.3; d = 128, n = 16 53.6 / 78.0, n = 28
-// 103 / 115, n = 32 123 / 94; 4096 heads of d = 128, n = 16 253 / 269, n = 20 360 / 330; up to a head per SM no difference (148
-// heads of n = 12, d = 128: 16.6 / 14.5).  Symmetric: a head of n = 8, d = 16 14.3 / 14.5, d = 64 14.2 / 18.6, d = 128 14.4 / 28.8;
-// 1024 heads of n = 12, d = 16 35.1 / 32.9, d = 64 39.9 / 47.3, n = 16 51.8 / 47.3, d = 128, n = 20 84 / 92, n = 24 99 / 100; 64 heads
-// of n = 28, d = 32 16.6 / 16.6, n = 32, d = 64 18.6 / 19.1, n = 40, d = 128 33.0 / 32.9, 16 heads 27.3 / 30.9.
-bool short_heads(long long heads, int n, int d, bool sym, int sms) {
-    if (sym) return n <= (d <= 16 ? 8 : d <= 64 ? 12 : 20) || (2 * heads <= sms && d > 16 && n <= (d <= 64 ? 32 : 40));
-    if (heads <= sms) return false;
+// blocks whatever the length.  Measured on 148 SMs (us, general / tiled).  FULL; MASKED is alike up to d = 64: 1024 heads of n = 8,
+// d = 16 22.7 / 26.5, n = 12 30.9 / 27.4; d = 64, n = 8 26.8 / 41.0, n = 12 36.0 / 42.5, n = 16 46.2 / 42.3; up to a head per SM no
+// difference (148 heads of n = 12, d = 128: 16.6 / 14.5).  d > 64: 230 heads of n = 10, d = 128 16.6 / 12.6.  d = 68: 296 heads of n = 18
+// 22.7 / 20.7, 400 heads 28.9 / 35.0, 1500 heads of n = 24 88 / 112; 512 heads, which fill two rounds of the tiled kernel better,
+// of n = 16 30.9 / 29.0, of n = 28 47.7 / 45.6.  d = 128: 400 heads of n = 28
+// 48.8 / 57.5, 1024 heads 103 / 115, 1180 heads 127 / 116, of n = 24 94 / 104, 1500 heads 129 / 154; 4096 heads of n = 16 253 / 269,
+// n = 20 360 / 330.  MASKED, where the general kernel skips more: 4096 heads of n = 20, d = 68 196 / 234, d = 128 301 / 330, of n = 24
+// 267 / 253, 398 / 350.  Symmetric: a head of n = 8, d = 16 14.3 / 14.5, d = 64 14.2 / 18.6, d = 128 14.4 / 28.8; 1024 heads of d = 16,
+// n = 9 28.8 / 32.9, n = 12 35.1 / 32.9, 400 heads of n = 10 18.6 / 16.6; d = 64, n = 12 39.9 / 47.3, n = 16 51.8 / 47.3; d = 128, n = 20 84 / 92, n = 24 99 / 100, 400 heads
+// of n = 14 33.5 / 39.1, n = 16 35.9 / 33.0, 150 heads of n = 28 30.5 / 37.4; 64 heads of n = 28, d = 32 16.6 / 16.6, n = 32, d = 64 18.6 / 19.1, n = 40, d = 128 33.0 / 32.9.
+bool short_heads(long long heads, int n, int d, int scheme, int sms) {
+    const bool masked = scheme == PSA_MASKED;
+    if (scheme == PSA_SYMMETRIC) {
+        if (n <= (d <= 16 ? (heads > 3 * sms ? 9 : 8) : 12)) return true;
+        if (2 * heads <= sms) return d > 16 && n <= (d <= 64 ? 32 : 40);
+        if (d <= 64 || n > (2 * heads <= 3 * sms ? 28 : 20)) return false;
+        return n < 16 || heads > 3 * sms || (n == 16 ? 2 * heads <= 3 * sms : heads < 2 * sms);
+    }
+    if (heads <= sms || (d > 64 && heads < 2 * sms)) return false;
     if (n <= (d <= 16 ? 8 : d <= 48 ? 10 : 12)) return true;
-    return d > 64 && heads > (d <= 96 ? 4 : 3) * sms && n <= (heads <= 8 * sms ? 28 : 16);
+    if (d <= 64 || heads <= 2 * sms) return false;
+    if (d <= 80 && heads > 3 * sms && heads <= 4 * sms && (n > 20 || (n == 16 && !masked))) return false;
+    return n <= (heads <= 7 * sms ? 28 : heads <= 11 * sms ? 24 : masked ? 20 : 16);
 }
 }  // namespace
 
@@ -1204,7 +1216,7 @@ cudaError_t f32_attention(const float* Q, const float* K, const float* V, float*
     static DeviceSetup setup;
     const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
     if (sms <= 0) return cudaErrorUnknown;
-    if (H <= GRID_MAX && short_heads((long long)B * H, n, d, scheme == PSA_SYMMETRIC, sms))
+    if (H <= GRID_MAX && short_heads((long long)B * H, n, d, scheme, sms))
         return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
     if (d % 4 == 0 && (long long)B * H <= 0x7fffffff && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(out))      // 16-byte rows
         return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, sms, stream)

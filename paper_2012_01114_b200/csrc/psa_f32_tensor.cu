@@ -16,8 +16,9 @@
 // issues 12 MMAs of 128 x 128 x 16 per step; warps 0-15 also drain the accumulators, 32 rows by 32 columns each.
 //
 // What bounds it: 12 MMAs per step at 92 cycles (N = 128) are 1104 cycles for 32 k; splitting a step takes about 600 issue
-// slots per scheduler beside them, and its stores share the shared-memory port with the MMAs' operands.  Measured 2300
-// cycles per step; 2048 x 768 x 3 x 768 171 us on CUDA cores (128 x 128 tiles), 70 us here.
+// slots per scheduler beside them, and its stores share the shared-memory port with the MMAs' operands (at the 96 registers
+// that 17 warps leave, 92 bytes are spilled, most of them around the call of ft_form_again).  Measured 2300 cycles per step;
+// 2048 x 768 x 3 x 768 171 us on CUDA cores (128 x 128 tiles), 70 us here.
 //
 // What the parts cannot carry is formed again by the plain chain of fmaf, per output (ft_form_again):
 //   * an output that is not finite (an input is infinite or NaN or rounds to infinity, or a sum overflows);

@@ -316,7 +316,9 @@ def test_projection_forms_of_small_calls(rows, D, H, d):
 @pytest.mark.parametrize("B,H,n,d", [(150, 1, 8, 16), (40, 4, 9, 16), (75, 2, 10, 48), (75, 2, 11, 48), (10, 15, 12, 64), (10, 15, 13, 64),
                                      (300, 2, 16, 128), (300, 2, 28, 68), (300, 2, 29, 128), (1200, 1, 16, 100), (1200, 1, 17, 100),
                                      (1, 1, 1, 8), (1, 3, 32, 64), (37, 2, 33, 64), (1, 74, 40, 68), (5, 15, 20, 128), (5, 15, 21, 128),
-                                     (1, 75, 40, 68)])
+                                     (1, 75, 40, 68), (10, 50, 16, 68), (10, 50, 28, 68), (10, 50, 29, 68), (300, 4, 24, 72), (300, 4, 25, 72),
+                                     (425, 4, 20, 72), (425, 4, 21, 72), (20, 15, 20, 100), (20, 14, 20, 100), (37, 4, 20, 100), (50, 4, 20, 100), (37, 6, 12, 72), (223, 1, 12, 72), (223, 1, 16, 72),
+                                     (222, 1, 28, 72), (295, 1, 12, 72), (296, 1, 12, 72), (295, 1, 20, 72), (445, 1, 9, 16), (444, 1, 9, 16)])
 def test_core_of_short_heads(scheme, B, H, n, d):
     test_core_at_tile_edges(scheme, B, H, n, d)
 
