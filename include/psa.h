@@ -70,8 +70,8 @@ typedef enum {
  *                   FULL d*n^2 each; MASKED d*n(n+1)/2 each; SYMMETRIC d*n(n+1)/2 and d*n^2
  * The bf16 path issues whole 128x128 blocks of the weight matrix, so issued >= useful there (a
  * block on the diagonal, or a ragged last block, is issued in full); the fp32 path skips element by element, issued = useful.
- * proj_macs counts the multiply-accumulates of the plain product on every path (the fp32 projections of large calls form six
- * bf16 products for each, on padded tiles).
+ * On the fp32 path every number is one multiply-accumulate of the plain product (in large calls six bf16 products are formed for
+ * each, on tiles padded with zeros); so is proj_macs on either path.
  */
 typedef struct {
     uint64_t proj_macs, qk_macs, pv_macs, exps, useful_qk_macs, useful_pv_macs;
@@ -89,10 +89,11 @@ typedef struct {
 int psa_attention(const void* X, const void* Wq, const void* Wk, const void* Wv, int batch, int heads, int n,
                   int d_model, int d_k, int scheme, void* out, void* stream);
 
-/* Same computation in fp32 storage, to fp32 accuracy.  The three phases run in fp32 arithmetic on CUDA cores with element-
- * exact skipping (issued = useful), and so do the projections of small calls; those of large calls run on the tensor cores,
- * every number split into three bf16 parts, with an error below that of a chain of fp32 additions (outputs too small for that,
- * or not finite, are formed by such a chain).  Supported: n <= 1024, d_k <= 128 (any d_model). */
+/* Same computation in fp32 storage, to fp32 accuracy.  Small calls run in fp32 arithmetic on CUDA cores; large ones (projections; the
+ * full and masked schemes with d_k a multiple of 8) on the tensor cores, every number split into three bf16 parts, with an error
+ * below that of a chain of fp32 additions (projections too small for that, or not finite, and heads with numbers beyond 2^50, not
+ * finite or, in V, below 2^-60, are worked off on CUDA cores).  Skipping is element-exact either way (issued = useful): the
+ * diagonal tiles of the masked scheme stay on CUDA cores.  Supported: n <= 1024, d_k <= 128 (any d_model). */
 int psa_attention_f32(const void* X, const void* Wq, const void* Wk, const void* Wv, int batch, int heads, int n,
                       int d_model, int d_k, int scheme, void* out, void* stream);
 

@@ -84,7 +84,7 @@ int check_shape(int batch, int heads, int n, int d_model, int d_k, int scheme, i
 }
 
 struct WsLayout {
-    size_t q, k, v, s, s_bytes, xs, wq, wk, wv, outs, total;
+    size_t q, k, v, s, s_bytes, bad, bad_bytes, ml, parts, xs, wq, wk, wv, outs, total;
 };
 
 WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, bool with_proj,
@@ -98,6 +98,13 @@ WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme
         L.s_bytes = dtype == PSA_BF16 ? bf16_symmetric_scratch_bytes(batch, heads, n)
                                       : align_up((size_t)batch * heads * n * n * sizeof(float), 256);
         L.s = off; off += L.s_bytes;
+    }
+    if (dtype == PSA_F32 && f32_tensor_attention_fits(batch, heads, n, d_k, scheme)) {
+        const size_t bh = (size_t)batch * heads;
+        L.bad_bytes = align_up(bh * sizeof(int), 256);      // (right behind the counters, as above)
+        L.bad = off; off += L.bad_bytes;
+        L.ml = off; off += align_up(2 * bh * n * sizeof(float), 256);
+        L.parts = off; off += align_up(12 * bh * n * d_k, 256);
     }
     if (with_proj) {
         L.q = off; off += qkv;
@@ -115,6 +122,10 @@ WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme
     }
     L.total = off;
     return L;
+}
+
+F32Scratch f32_scratch(char* ws, const WsLayout& L, size_t first_head) {
+    return F32Scratch{reinterpret_cast<int*>(ws + L.bad) + first_head, reinterpret_cast<float*>(ws + L.ml), ws + L.parts};
 }
 
 // Whether copies from or to this host memory run beside the calling thread (memory that CUDA knows of).
@@ -180,7 +191,7 @@ void useful_counts(int batch, int heads, int n, int d_model, int d_k, int scheme
 // Context (may be null).  `between`, if given, is recorded between projections and attention.
 int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K, const void* V,
                   int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out, cudaStream_t stream,
-                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, bool s_clear, DeviceCounters* dc, unsigned int* cursor,
+                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, bool s_clear, const F32Scratch* fs, DeviceCounters* dc, unsigned int* cursor,
                   DeviceCounters* dc_next, cudaEvent_t between) {
     const float scale = 1.0f / sqrtf((float)d_k);
     const int nW = scheme == PSA_SYMMETRIC ? 1 : 3;
@@ -210,7 +221,7 @@ int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv,
     if (between) cudaEventRecord(between, stream);
     if (dtype == PSA_F32) {
         e = f32_attention(static_cast<const float*>(Q), static_cast<const float*>(K), static_cast<const float*>(V),
-                          static_cast<float*>(out), S, batch, heads, n, d_k, scale, scheme, dc, stream);
+                          static_cast<float*>(out), S, fs, batch, heads, n, d_k, scale, scheme, dc, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "f32_attention"); return PSA_ERR_CUDA; }
         return PSA_OK;
     }
@@ -233,12 +244,13 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     if (captured) {
         block = CAPTURE_BLOCK;
         e = cudaMemsetAsync(ws + CAPTURE_BLOCK * COUNTER_BLOCK_BYTES, 0, COUNTER_BLOCK_BYTES, stream);
+        if (e == cudaSuccess && L.bad_bytes) e = cudaMemsetAsync(ws + L.bad, 0, L.bad_bytes, stream);
     } else if (s_clear) {
         e = bf16_symmetric_clear(S, L.s_bytes, batch, heads, n, L.s, stream);
     } else if (turns && cx.clean_ws == ws) {
         block = cx.next_block;
     } else {
-        e = cudaMemsetAsync(ws, 0, TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
+        e = cudaMemsetAsync(ws, 0, L.bad_bytes ? L.bad + L.bad_bytes : TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
     }
     if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync(counters)"); return PSA_ERR_CUDA; }
     if (!captured) cx.clean_ws = nullptr;          // until this call's kernels are known to be queued
@@ -255,8 +267,9 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     } tail{pev, stream};
     if (pev) cudaEventRecord(pev[0], stream);
     void* const qkv[3] = {ws + L.q, ws + L.k, ws + L.v};
+    const F32Scratch fs = f32_scratch(ws, L, 0);
     const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
-                                 qkv, S, L.s_bytes, s_clear, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
+                                 qkv, S, L.s_bytes, s_clear, L.bad_bytes ? &fs : nullptr, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
     if (rc == PSA_OK && turns && !captured) {        // the other block will be clear once this call has run
         cx.clean_ws = ws;
         cx.next_block = block ^ 1;
@@ -404,7 +417,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     cudaError_t e = cudaEventRecord(pipe->start, stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->start, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->out, pipe->start, 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, COUNTER_BYTES, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, L.bad_bytes ? L.bad + L.bad_bytes : COUNTER_BYTES, stream);
     cx.clean_ws = nullptr;
     DeviceCounters* dc = reinterpret_cast<DeviceCounters*>(ws);
     cx.last_dc = dc;
@@ -432,9 +445,10 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         e = cudaStreamWaitEvent(stream, pipe->loaded[c], 0);
         if (e != cudaSuccess) break;
         void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
+        const F32Scratch fs = f32_scratch(ws, L, b0 * heads);       // (a part has marks of its own; the rest is used by one after another)
         rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
                            d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,
-                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, dc,
+                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, L.bad_bytes ? &fs : nullptr, dc,
                            reinterpret_cast<unsigned int*>(ws + CURSOR_OFFSET) + c, nullptr, nullptr);
         if (rc != PSA_OK) break;
         e = cudaEventRecord(pipe->computed[c], stream);

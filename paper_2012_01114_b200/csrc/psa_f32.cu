@@ -1,11 +1,12 @@
-// The full-precision path: fp32 storage, and fp32 arithmetic on CUDA cores but for the projections of large calls, which are
-// in psa_f32_tensor.cu.  Skipping is element-exact: a weight that the scheme does not need is never computed (paper Sec. 4.1,
+// The full-precision path: fp32 storage, and fp32 arithmetic on CUDA cores but for large calls, whose projections are in
+// psa_f32_tensor.cu and whose attention (FULL, MASKED) is in psa_f32_attn_tensor.cu.  Skipping is element-exact: a weight that the scheme does not need is never computed (paper Sec. 4.1,
 // 5.1), so issued MACs equal the paper's element counts (Sec. 3.2, 4.2, 5.2).  The throughput path is the bf16 one.
 #include <cooperative_groups.h>
 
 #include <type_traits>
 
 #include "psa_internal.h"
+#include "sm100.cuh"
 
 namespace psa {
 
@@ -226,12 +227,15 @@ __device__ __forceinline__ void fa_scores(unsigned long long (&acc)[8][U], const
     if (c < d4) step(qe + 4 * c, k + 4 * c);
 }
 
-// MODE 0: the three phases for FULL / MASKED.  MODE 2: phases 2 and 3 of the symmetric scheme, scores read from S.
+// MODE 0: the three phases for FULL / MASKED.  MODE 2: phases 2 and 3 of the symmetric scheme, scores read from S.  MODE 3: the
+// masked scheme's weights inside the 128-row tiles of f32_attn_tensor_kernel; the first tile of a head is done then, rows of the
+// others leave their maximum and sum in `ml` (B H n numbers each) and their output undivided.
+// `bad` (may be null): MODE 0 works on the heads marked there only, MODE 3 on the others.
 template <int DG, int KS, int MODE>
 __global__ void __launch_bounds__(FA_THREADS, DG == 1 ? 3 : 2)
 f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                  float* __restrict__ out, const float* __restrict__ S, int n, int H, int d, float scale, int masked,
-                 DeviceCounters* dc) {
+                 DeviceCounters* dc, const int* __restrict__ bad, float* __restrict__ ml) {
     using C = FACfg<DG, KS>;
     constexpr int U = C::U;
     extern __shared__ float4 fa_smem4[];
@@ -241,6 +245,10 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     float* Ps = Vs + C::V_FLOATS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
     const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
+    if (MODE == 0 || MODE == 3) {
+        grid_dependency_wait();
+        if (bad && (bad[bh] != 0) != (MODE == 0)) return;
+    }
     const int rb = masked ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // the longest rows first
     const int r0 = rb * C::BR;
     const int rg = warp / KS, kw = (warp % KS) * C::KW;                 // the warp's row group and first key of a block
@@ -250,7 +258,8 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     const size_t base = ((size_t)b * n) * ld + (size_t)h * d;
     const int d4 = d >> 2;
     const int kend = masked ? min(r0 + C::BR, n) : n;                   // keys that some row of the CTA keeps
-    const int nblk = (kend + FA_BC - 1) / FA_BC;
+    const int nblk = (kend + FA_BC - 1) / FA_BC, jfirst = MODE == 3 ? r0 / 128 * (128 / FA_BC) : 0;
+    const bool undivided = MODE == 3 && r0 >= 128;
     const float* Sh = MODE == 2 ? S + (size_t)bh * n * n : nullptr;
     float* Pw = Ps + warp * 16 * C::PP;
     const float* Pr = Pw + ty * C::PP;                                  // row i of the lane: + 2 i PP
@@ -259,7 +268,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 
     if (MODE != 2) {
         fa_load<DG, C::BR, C::DP, true>(Qs, Q + base, r0, n, ld, d4);
-        fa_load<DG, FA_BC, C::KP, false>(Ks, K + base, 0, n, ld, d4);
+        fa_load<DG, FA_BC, C::KP, false>(Ks, K + base, jfirst * FA_BC, n, ld, d4);
     }
     cp_async_commit();
 
@@ -272,7 +281,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     }
     unsigned int dots = 0, wts = 0;                                     // weights of this lane; of its rows in phase 3
 
-    for (int jb = 0; jb < nblk; ++jb) {
+    for (int jb = jfirst; jb < nblk; ++jb) {
         const int k0 = jb * FA_BC + kw;                                 // first key of the warp's share
         const int last = min(wr0 + 15, n - 1);                          // last row of the warp that exists
         const int maxlim = wr0 >= n ? -1 : (masked ? last : n - 1) - k0;
@@ -410,7 +419,11 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if (row + 2 * i >= n) continue;
-            const float inv = 1.f / l[i];
+            const float inv = undivided ? 1.f : 1.f / l[i];
+            if (undivided && tx == 0) {
+                ml[(size_t)bh * n + row + 2 * i] = m[i];
+                ml[((size_t)gridDim.x + bh) * n + row + 2 * i] = l[i];
+            }
             float* dst = out + base + (size_t)(row + 2 * i) * ld + 4 * tx;
 #pragma unroll
             for (int g = 0; g < DG; ++g)
@@ -421,7 +434,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
         // the KS partial results of a row, brought to their common maximum and added up
         __syncthreads();            // every warp is done with V and P
         float* part = Ks;           // [KS][BR][DP], over the K tile
-        float* ml = Ps;             // [KS][BR] maxima, then [KS][BR] sums
+        float* part_ml = Ps;        // [KS][BR] maxima, then [KS][BR] sums
         const int ks = warp % KS;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -429,7 +442,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 #pragma unroll
             for (int g = 0; g < DG; ++g)
                 *reinterpret_cast<float4*>(part + (size_t)(ks * C::BR + r) * C::DP + 64 * g + 4 * tx) = make_float4(o[i][4 * g], o[i][4 * g + 1], o[i][4 * g + 2], o[i][4 * g + 3]);
-            if (tx == 0) { ml[ks * C::BR + r] = m[i]; ml[KS * C::BR + ks * C::BR + r] = l[i]; }
+            if (tx == 0) { part_ml[ks * C::BR + r] = m[i]; part_ml[KS * C::BR + ks * C::BR + r] = l[i]; }
         }
         __syncthreads();
         for (int t = tid; t < C::BR * d4; t += FA_THREADS) {
@@ -437,19 +450,23 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
             if (r0 + r >= n) continue;
             float mx = -INFINITY;
 #pragma unroll
-            for (int k = 0; k < KS; ++k) mx = fmaxf(mx, ml[k * C::BR + r]);
+            for (int k = 0; k < KS; ++k) mx = fmaxf(mx, part_ml[k * C::BR + r]);
             float sum = 0.f;
             float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < KS; ++k) {
-                const float mk = ml[k * C::BR + r];
-                if (mk == -INFINITY && ml[KS * C::BR + k * C::BR + r] == 0.f) continue;      // no key of this share counts
+                const float mk = part_ml[k * C::BR + r];
+                if (mk == -INFINITY && part_ml[KS * C::BR + k * C::BR + r] == 0.f) continue;      // no key of this share counts
                 const float w = mk == mx ? 1.f : expf(mk - mx);
                 const float4 f = *reinterpret_cast<const float4*>(part + (size_t)(k * C::BR + r) * C::DP + 4 * c);
-                sum = fmaf(w, ml[KS * C::BR + k * C::BR + r], sum);
+                sum = fmaf(w, part_ml[KS * C::BR + k * C::BR + r], sum);
                 y.x = fmaf(w, f.x, y.x); y.y = fmaf(w, f.y, y.y); y.z = fmaf(w, f.z, y.z); y.w = fmaf(w, f.w, y.w);
             }
-            const float inv = 1.f / sum;
+            const float inv = undivided ? 1.f : 1.f / sum;
+            if (undivided && c == 0) {
+                ml[(size_t)bh * n + r0 + r] = mx;
+                ml[((size_t)gridDim.x + bh) * n + r0 + r] = sum;
+            }
             *reinterpret_cast<float4*>(out + base + (size_t)(r0 + r) * ld + 4 * c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
         }
     }
@@ -1139,7 +1156,7 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
 namespace {
 template <int DG, int KS, int MODE>
 cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n, int d,
-                         float scale, int masked, DeviceCounters* dc, cudaStream_t stream) {
+                         float scale, int masked, DeviceCounters* dc, const F32Scratch* fs, cudaStream_t stream) {
     using C = FACfg<DG, KS>;
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
@@ -1147,27 +1164,40 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
         }, "fp32 attention set-up") <= 0)
         return cudaErrorUnknown;
     const dim3 grid(B * H, (n + C::BR - 1) / C::BR);
-    f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc);
-    return cudaGetLastError();
+    if (!fs) {
+        f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc, nullptr, nullptr);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(FA_THREADS);
+    cfg.dynamicSmemBytes = C::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (waits for its predecessor itself)
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f32_flash_kernel<DG, KS, MODE>, Q, K, V, out, S, n, H, d, scale, masked, dc, static_cast<const int*>(fs->bad), fs->ml);
 }
 template <int DG, int MODE>
 cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n,
-                               int d, float scale, int masked, DeviceCounters* dc, int sms, cudaStream_t stream) {
+                               int d, float scale, int masked, DeviceCounters* dc, const F32Scratch* fs, int sms, cudaStream_t stream) {
     auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
     // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs: the
     // line lies at two CTAs per SM (us for KS = 1 / 2 / 4).  16 heads of n = 300, d = 64, 80 tiles of 64 rows: 70 / 44 / 35; 16 of
     // n = 1024, d = 128, masked, 256 tiles: 210 / 166 / 216; 74 of n = 256, d = 64, 296 tiles: 46 / 54 / 70; 48 of n = 512, d = 64, 384
     // tiles: 110 / 124 / 159.  It is not exact: 16 heads of n = 1024, FULL, d = 64 161 / 179 / 208; 64 of n = 300, 320 tiles with a
     // nearly empty last one, 101 / 82 / 87.
-    if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
-    if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
-    return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, stream);
+    if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, fs, stream);
+    if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, fs, stream);
+    return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, fs, stream);
 }
 template <int DG>
 cudaError_t tiled_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H, int n, int d,
                             float scale, int scheme, DeviceCounters* dc, int sms, cudaStream_t stream) {
     if (scheme != PSA_SYMMETRIC)
-        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, sms, stream);
+        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, nullptr, sms, stream);
     constexpr int SMEM = (FACfg<DG, 1>::Q_FLOATS + FACfg<DG, 1>::K_FLOATS) * (int)sizeof(float);
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
@@ -1178,7 +1208,17 @@ cudaError_t tiled_attention(const float* Q, const float* K, const float* V, floa
     f32_sym_scores_kernel<DG><<<dim3(B * H, T * (T + 1) / 2), FA_THREADS, SMEM, stream>>>(Q, S, n, H, d, scale, dc);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, sms, stream);
+    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, nullptr, sms, stream);
+}
+// The call on the tensor cores (psa_f32_attn_tensor.cu), with the weights on the diagonal tiles and the heads that path cannot take here.
+template <int DG>
+cudaError_t tensor_attention(const float* Q, const float* K, const float* V, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale,
+                             int masked, DeviceCounters* dc, int sms, cudaStream_t stream) {
+    cudaError_t e = f32_attention_split(Q, K, V, fs, B, H, n, d, stream);
+    if (e == cudaSuccess && masked) e = launch_flash_split<DG, 3>(Q, K, V, out, nullptr, B, H, n, d, scale, 1, dc, &fs, sms, stream);
+    if (e == cudaSuccess) e = f32_attention_tensor(Q, out, fs, B, H, n, d, scale, masked, dc, stream);
+    if (e == cudaSuccess) e = launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, masked, dc, &fs, sms, stream);
+    return e;
 }
 }  // namespace
 
@@ -1211,11 +1251,24 @@ bool short_heads(long long heads, int n, int d, int scheme, int sms) {
 }
 }  // namespace
 
-cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H,
+// Whether a call is better off on the tensor cores: four launches instead of one, and under the masked scheme the diagonal tiles stay on
+// CUDA cores.  Measured (us, CUDA cores / tensor cores): FULL 16 heads of n = 160, d = 16 15.4 / 16.8, of n = 192, d = 64 17.4 / 17.4, of n = 1024, d =
+// 128 166 / 54; 48 of n = 512, d = 64 114 / 42; MASKED 16 heads of n = 384, d = 128 48 / 56, 16 of n = 512, d = 16 31.8 / 33.3, of n = 700, d = 64
+// 48 / 45, of n = 1024, d = 128 166 / 102; 256 of n = 256, d = 128 204 / 218.
+bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme) {
+    const long long T = (n + 127) / 128, blocks = (long long)B * H * T * T;
+    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || blocks < 64 || (long long)B * H * n * d >= (1LL << 31)) return false;
+    return scheme == PSA_MASKED ? n > 512 : n > 128 && (n >= 256 || d >= 64);
+}
+
+cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, const F32Scratch* fs, int B, int H,
                           int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
     static DeviceSetup setup;
     const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
     if (sms <= 0) return cudaErrorUnknown;
+    if (fs && f32_tensor_attention_fits(B, H, n, d, scheme))
+        return d <= 64 ? tensor_attention<1>(Q, K, V, out, *fs, B, H, n, d, scale, scheme == PSA_MASKED, dc, sms, stream)
+                       : tensor_attention<2>(Q, K, V, out, *fs, B, H, n, d, scale, scheme == PSA_MASKED, dc, sms, stream);
     if (H <= GRID_MAX && short_heads((long long)B * H, n, d, scheme, sms))
         return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
     if (d % 4 == 0 && (long long)B * H <= 0x7fffffff && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(out))      // 16-byte rows

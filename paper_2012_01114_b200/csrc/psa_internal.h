@@ -29,8 +29,21 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
 // The same on the tensor cores, to the same accuracy (psa_f32_tensor.cu); f32_project chooses.  Rows of 16 bytes, as there.
 cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
                                const float* residual, DeviceCounters* dc, cudaStream_t stream);
-// Q, K, V, out: [B, n, H, d] fp32.  S: scratch [B*H, n, n] fp32, used by PSA_SYMMETRIC only.
-cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H,
+// Scratch of the tensor-core attention: marks of the heads it cannot take (B H ints, clear when the call's kernels start), maxima
+// and sums of the rows on the diagonal tiles (2 B H n numbers), bf16 parts of K and V (6 B n H d each numbers of 16 bits, together).
+struct F32Scratch {
+    int* bad;
+    float* ml;
+    void* parts;
+};
+// Whether attention of this shape runs on the tensor cores, given that scratch and rows of 16 bytes (psa_f32_attn_tensor.cu).
+bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme);
+// Its two kernels.
+cudaError_t f32_attention_split(const float* Q, const float* K, const float* V, const F32Scratch& fs, int B, int H, int n, int d, cudaStream_t stream);
+cudaError_t f32_attention_tensor(const float* Q, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale, int masked, DeviceCounters* dc,
+                                 cudaStream_t stream);
+// Q, K, V, out: [B, n, H, d] fp32.  S: scratch [B*H, n, n] fp32, used by PSA_SYMMETRIC only.  fs: may be null.
+cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, const F32Scratch* fs, int B, int H,
                           int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream);
 
 // Small layers in one launch (projections and the three phases of a (batch, head) per CTA, all in shared memory):

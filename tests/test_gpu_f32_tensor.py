@@ -1,0 +1,63 @@
+"""fp32 attention on the tensor cores (FULL from 128 vectors per head on, MASKED from 512): block and tile edges, head sizes that are not a
+multiple of the tile, rows on and off the diagonal tiles, and heads whose numbers its bf16 parts cannot carry.  Reference: the fp64
+oracle.  Bounds: an fp32 softmax over scores of size s is off by about 2^-24 (s + 1) per weight and the weighted sum by as much
+again; 4e-6 of the output's root mean square, the accuracy that the CUDA-core path shows on these inputs, four times over."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2012_01114_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(B, H, n, d, scheme, change=None):
+    t = [inputs.tensor(11 * n + d, 4 + i, (B, n, H, d), 1.0, "f32")[1] for i in range(3)]
+    if change:
+        change(t)
+    out = binding.psa_attention_core(*[torch.from_numpy(x).cuda() for x in t], scheme)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got == binding.psa_skip_count(B, H, n, 0, d, scheme, binding.F32)
+    ref, _ = oracle.attention_core(*[x.astype(np.float64) for x in t], scheme)
+    return out.cpu().numpy().astype(np.float64), ref
+
+
+def _close(got, ref, rel=4e-6):
+    assert np.isfinite(got).all()
+    assert np.linalg.norm(got - ref) <= rel * np.linalg.norm(ref)
+    assert np.abs(got - ref).max() <= 10 * rel * max(np.sqrt((ref ** 2).mean()), np.abs(ref).max() / 10)
+
+
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("B,H,n,d", [(2, 10, 129, 64), (4, 8, 192, 8), (2, 10, 193, 128), (2, 8, 256, 72), (1, 9, 449, 40), (1, 4, 1024, 120), (1, 2, 1000, 16), (1, 4, 513, 64), (1, 3, 705, 128)])
+def test_edges(scheme, B, H, n, d):
+    _close(*_run(B, H, n, d, scheme))
+
+
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+def test_rising_keys(scheme):
+    # every block raises the running maxima (a factor per key: scores of up to about 60)
+    n = 640
+
+    def grow(t):
+        t[1] *= (1.0 + 2.0 * np.arange(n, dtype=np.float32) / 128)[None, :, None, None]
+    got, ref = _run(1, 4, n, 64, scheme, grow)
+    _close(got, ref, 2e-5)           # (scores of 60: 2^-24 * 61 = 3.6e-6 per weight, five times over)
+
+
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+def test_heads_with_numbers_without_parts(scheme):
+    # head 1: one infinite key, head 2: values around 1e-30, head 3: one value of 1e25; heads 0 and 4 must not notice
+    B, H, n, d = 2, 5, 600, 64
+
+    def spoil(t):
+        t[1][1, 590, 1, 3] = np.inf
+        t[2][:, :, 2] *= np.float32(1e-30)
+        t[2][0, 7, 3, 5] = np.float32(1e25)
+    got, ref = _run(B, H, n, d, scheme, spoil)
+    got, ref = got.reshape(B, n, H, d), ref.reshape(B, n, H, d)
+    for h in (0, 2, 4):
+        _close(got[:, :, h], ref[:, :, h])
+    _close(got[0, :, 1], ref[0, :, 1])
+    _close(got[:, :, 3][:, :, :5], ref[:, :, 3][:, :, :5])
