@@ -84,7 +84,8 @@ int check_shape(int batch, int heads, int n, int d_model, int d_k, int scheme, i
 }
 
 struct WsLayout {
-    size_t q, k, v, s, s_bytes, bad, bad_bytes, ml, parts, xs, wq, wk, wv, outs, total;
+    size_t q, k, v, s, s_bytes, clear, clear_bytes, bad, marks_in, marks_out, ml, parts, xs, wq, wk, wv, outs, total;
+    bool attn_tensor, proj_pairs;      // fp32: whether bad / ml / parts and marks_* / parts are there
 };
 
 WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, bool with_proj,
@@ -94,17 +95,25 @@ WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme
     WsLayout L;
     memset(&L, 0, sizeof(L));
     size_t off = COUNTER_BYTES;
-    if (scheme == PSA_SYMMETRIC) {       // (right behind the counters: one clear serves both, see run_layer)
+    if (dtype == PSA_F32) {      // marks right behind the counters: one clear serves both, see run_layer
+        const bool one_launch = with_proj && f32_fused_fits(n, d_model, d_k, scheme);       // (needs none of this, but for an output projection)
+        const size_t bh = (size_t)batch * heads, in = with_proj && !one_launch ? f32_project_parts_bytes(batch * n, d_model, heads * d_k, scheme == PSA_SYMMETRIC ? 1 : 3) : 0,
+                     outp = with_proj ? f32_project_parts_bytes(batch * n, heads * d_k, d_model, 1) : 0;
+        L.attn_tensor = !one_launch && f32_tensor_attention_fits(batch, heads, n, d_k, scheme);
+        L.proj_pairs = in || outp;
+        L.clear = off;
+        if (L.attn_tensor) { L.bad = off; off += align_up(bh * sizeof(int), 256); }
+        if (in) { L.marks_in = off; off += align_up(f32_project_marks(batch * n, heads * d_k, 3) * sizeof(int), 256); }
+        if (outp) { L.marks_out = off; off += align_up(f32_project_marks(batch * n, d_model, 1) * sizeof(int), 256); }
+        L.clear_bytes = one_launch ? 0 : off - L.clear;
+        if (L.attn_tensor) { L.ml = off; off += align_up(2 * bh * n * sizeof(float), 256); }
+        L.parts = off;           // (used by one kernel after another)
+        off += align_up(std::max(std::max(in, outp), L.attn_tensor ? 12 * bh * n * d_k : (size_t)0), 256);
+    }
+    if (scheme == PSA_SYMMETRIC) {       // (bf16: right behind the counters, as above)
         L.s_bytes = dtype == PSA_BF16 ? bf16_symmetric_scratch_bytes(batch, heads, n)
                                       : align_up((size_t)batch * heads * n * n * sizeof(float), 256);
         L.s = off; off += L.s_bytes;
-    }
-    if (dtype == PSA_F32 && f32_tensor_attention_fits(batch, heads, n, d_k, scheme)) {
-        const size_t bh = (size_t)batch * heads;
-        L.bad_bytes = align_up(bh * sizeof(int), 256);      // (right behind the counters, as above)
-        L.bad = off; off += L.bad_bytes;
-        L.ml = off; off += align_up(2 * bh * n * sizeof(float), 256);
-        L.parts = off; off += align_up(12 * bh * n * d_k, 256);
     }
     if (with_proj) {
         L.q = off; off += qkv;
@@ -191,7 +200,8 @@ void useful_counts(int batch, int heads, int n, int d_model, int d_k, int scheme
 // Context (may be null).  `between`, if given, is recorded between projections and attention.
 int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K, const void* V,
                   int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out, cudaStream_t stream,
-                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, bool s_clear, const F32Scratch* fs, DeviceCounters* dc, unsigned int* cursor,
+                  bool with_proj, void* const qkv[3], float* S, size_t s_bytes, bool s_clear, const F32Scratch* fs, const F32ProjectScratch* ps,
+                  DeviceCounters* dc, unsigned int* cursor,
                   DeviceCounters* dc_next, cudaEvent_t between) {
     const float scale = 1.0f / sqrtf((float)d_k);
     const int nW = scheme == PSA_SYMMETRIC ? 1 : 3;
@@ -210,7 +220,7 @@ int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv,
         if (dtype == PSA_F32) {
             float* const outs[3] = {static_cast<float*>(qkv[0]), static_cast<float*>(qkv[1]), static_cast<float*>(qkv[2])};
             e = f32_project(static_cast<const float*>(X), reinterpret_cast<const float* const*>(Ws), outs, nW, batch * n, d_model,
-                            heads * d_k, nullptr, dc, stream);
+                            heads * d_k, nullptr, ps, dc, stream);
             if (e != cudaSuccess) { set_cuda_error(e, "f32_project"); return PSA_ERR_CUDA; }
         } else {
             int rc = bf16_project(X, Ws, qkv, nW, batch * n, d_model, heads * d_k, nullptr, dc, stream);
@@ -244,13 +254,13 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     if (captured) {
         block = CAPTURE_BLOCK;
         e = cudaMemsetAsync(ws + CAPTURE_BLOCK * COUNTER_BLOCK_BYTES, 0, COUNTER_BLOCK_BYTES, stream);
-        if (e == cudaSuccess && L.bad_bytes) e = cudaMemsetAsync(ws + L.bad, 0, L.bad_bytes, stream);
+        if (e == cudaSuccess && L.clear_bytes) e = cudaMemsetAsync(ws + L.clear, 0, L.clear_bytes, stream);
     } else if (s_clear) {
         e = bf16_symmetric_clear(S, L.s_bytes, batch, heads, n, L.s, stream);
     } else if (turns && cx.clean_ws == ws) {
         block = cx.next_block;
     } else {
-        e = cudaMemsetAsync(ws, 0, L.bad_bytes ? L.bad + L.bad_bytes : TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
+        e = cudaMemsetAsync(ws, 0, L.clear_bytes ? L.clear + L.clear_bytes : TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
     }
     if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync(counters)"); return PSA_ERR_CUDA; }
     if (!captured) cx.clean_ws = nullptr;          // until this call's kernels are known to be queued
@@ -268,8 +278,9 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     if (pev) cudaEventRecord(pev[0], stream);
     void* const qkv[3] = {ws + L.q, ws + L.k, ws + L.v};
     const F32Scratch fs = f32_scratch(ws, L, 0);
+    const F32ProjectScratch ps = {ws + L.parts, reinterpret_cast<int*>(ws + L.marks_in)};
     const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
-                                 qkv, S, L.s_bytes, s_clear, L.bad_bytes ? &fs : nullptr, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
+                                 qkv, S, L.s_bytes, s_clear, L.attn_tensor ? &fs : nullptr, L.proj_pairs ? &ps : nullptr, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
     if (rc == PSA_OK && turns && !captured) {        // the other block will be clear once this call has run
         cx.clean_ws = ws;
         cx.next_block = block ^ 1;
@@ -417,7 +428,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     cudaError_t e = cudaEventRecord(pipe->start, stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->start, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->out, pipe->start, 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, L.bad_bytes ? L.bad + L.bad_bytes : COUNTER_BYTES, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, L.clear_bytes ? L.clear + L.clear_bytes : COUNTER_BYTES, stream);
     cx.clean_ws = nullptr;
     DeviceCounters* dc = reinterpret_cast<DeviceCounters*>(ws);
     cx.last_dc = dc;
@@ -445,10 +456,11 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         e = cudaStreamWaitEvent(stream, pipe->loaded[c], 0);
         if (e != cudaSuccess) break;
         void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
+        const F32ProjectScratch ps = {ws + L.parts, reinterpret_cast<int*>(ws + L.marks_in)};
         const F32Scratch fs = f32_scratch(ws, L, b0 * heads);       // (a part has marks of its own; the rest is used by one after another)
         rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
                            d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,
-                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, L.bad_bytes ? &fs : nullptr, dc,
+                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, L.attn_tensor ? &fs : nullptr, L.proj_pairs ? &ps : nullptr, dc,
                            reinterpret_cast<unsigned int*>(ws + CURSOR_OFFSET) + c, nullptr, nullptr);
         if (rc != PSA_OK) break;
         e = cudaEventRecord(pipe->computed[c], stream);
@@ -554,9 +566,12 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
     const void* Ws[3] = {Wo, Wo, Wo};
     void* outs[3] = {out, out, out};
     if (dtype == PSA_F32) {
-        cudaError_t e = f32_project(static_cast<const float*>(y), reinterpret_cast<const float* const*>(Ws),
+        const F32ProjectScratch ps = {ws + L.parts, reinterpret_cast<int*>(ws + L.marks_out)};
+        cudaError_t e = cudaSuccess;
+        if (L.marks_out && !L.clear_bytes) e = cudaMemsetAsync(ps.marks, 0, f32_project_marks(batch * n, d_model, 1) * sizeof(int), stream);
+        if (e == cudaSuccess) e = f32_project(static_cast<const float*>(y), reinterpret_cast<const float* const*>(Ws),
                                     reinterpret_cast<float* const*>(outs), 1, batch * n, heads * d_k, d_model,
-                                    static_cast<const float*>(R), cx.last_dc, stream);
+                                    static_cast<const float*>(R), L.proj_pairs ? &ps : nullptr, cx.last_dc, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "f32_project(Wo)"); return PSA_ERR_CUDA; }
         return PSA_OK;
     }

@@ -1078,7 +1078,7 @@ cudaError_t attention_general(const float* Q, const float* K, const float* V, fl
 }  // namespace
 
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
-                        int N, const float* residual, DeviceCounters* dc, cudaStream_t stream) {
+                        int N, const float* residual, const F32ProjectScratch* ps, DeviceCounters* dc, cudaStream_t stream) {
     bool tiled = D % 4 == 0 && N % 4 == 0 && aligned16(X) && aligned16(residual);      // 16-byte rows
     for (int w = 0; w < nW; ++w) tiled = tiled && aligned16(W[w]) && aligned16(out[w]);
     if (tiled) {
@@ -1096,6 +1096,8 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
         // 600 x 320 x 3 x 320 (570) 27.3 / 21.3, 64 x 2048 x 3 x 2048 (384) 89 / 72; larger ones, against 128 x 128 tiles on CUDA
         // cores, 2048 x 768 x 3 x 768 171 / 70.
         const long long tiles = (long long)((rows + 31) / 32) * ((N + 31) / 32) * nW;
+        if (ps && f32_project_parts_bytes(rows, D, N, nW) && f32_project_pairs_pay(rows, D, N, nW, sms))
+            return f32_project_pairs(X, W, out, nW, rows, D, N, residual, ps->parts, ps->marks, dc, stream);
         if (tiles > 2 * sms) return f32_project_tensor(X, W, out, nW, rows, D, N, residual, dc, stream);
         const dim3 grid((N + GP_BN - 1) / GP_BN, (rows + GP_BM - 1) / GP_BM, nW);
         f32_project_tiled_kernel<<<grid, GP_THREADS, GP_SMEM, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);

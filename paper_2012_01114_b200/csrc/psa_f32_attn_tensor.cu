@@ -69,6 +69,7 @@ f32_split_kernel(const float4* __restrict__ Q, const float4* __restrict__ K, con
     const int which = blockIdx.y;
     const float4* src = which == 0 ? K : (which == 1 ? V : Q);
     uint2* dst = parts + (size_t)which * 3 * count4;
+    grid_dependency_wait();
     for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < count4; i += gridDim.x * 256u) {
         const float4 x = __ldg(src + i);
         const uint32_t most = max(max(__float_as_uint(x.x) & 0x7fffffffu, __float_as_uint(x.y) & 0x7fffffffu),
@@ -411,9 +412,17 @@ cudaError_t launch_main(const float* Q, float* out, const F32Scratch& fs, int B,
 cudaError_t f32_attention_split(const float* Q, const float* K, const float* V, const F32Scratch& fs, int B, int H, int n, int d, cudaStream_t stream) {
     const uint32_t count4 = (uint32_t)((size_t)B * n * H * d / 4);
     const uint32_t blocks = (count4 + 1023) / 1024;
-    f32_split_kernel<<<dim3(blocks < 1024 ? blocks : 1024, 3), 256, 0, stream>>>(reinterpret_cast<const float4*>(Q), reinterpret_cast<const float4*>(K),
-                                                                               reinterpret_cast<const float4*>(V), static_cast<uint2*>(fs.parts), count4, d, H, n, fs.bad);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks < 1024 ? blocks : 1024, 3);
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f32_split_kernel, reinterpret_cast<const float4*>(Q), reinterpret_cast<const float4*>(K), reinterpret_cast<const float4*>(V),
+                              static_cast<uint2*>(fs.parts), count4, d, H, n, fs.bad);
 }
 cudaError_t f32_attention_tensor(const float* Q, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale, int masked, DeviceCounters* dc,
                                  cudaStream_t stream) {

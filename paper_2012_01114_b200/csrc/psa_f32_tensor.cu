@@ -11,7 +11,7 @@
 // chain of fmaf has 3.2e-7 / 5.0e-7 / 8.1e-7; positive inputs, K = 768, 1.4e-7 (of which 1.3e-7 is the accumulators' rounding
 // towards zero) against 4.3e-7.
 //
-// A CTA takes tiles of 128 x 128.  Warps 0-15 read X and W (two steps of 32 k ahead, in registers), split them into parts
+// f32_project_tensor_kernel: a CTA takes tiles of 128 x 128.  Warps 0-15 read X and W (two steps of 32 k ahead, in registers), split them into parts
 // and write these as operand tiles in the 128-byte swizzle (X K-major, W MN-major) into a ring of four steps; warp 16
 // issues 12 MMAs of 128 x 128 x 16 per step; warps 0-15 also drain the accumulators, 32 rows by 32 columns each.
 //
@@ -27,10 +27,11 @@
 //     each addition.  With the largest magnitudes of the output's row and column that bounds its error, K times over; it is
 //     formed again where that could be more than half a unit.
 // Such tiles are marked on the way and looked at when the CTA's other work is done, so that the main loop keeps its registers.
-// What it costs, in a layer of 4 x 512 vectors, d_model = 768, 12 heads, of whose 176 us the projection takes 60: one 1e-35 in
+// What it cost, in a layer of 4 x 512 vectors, d_model = 768, 12 heads, of whose 176 us the projection took 60: one 1e-35 in
 // every vector, so that every tile is looked at, 208 us; nothing but numbers around 1e-33, so that every output is formed
 // again, 439; nothing but NaN 416 (as a loop of one thread per 32 outputs in global memory it was 3300 in all three).
 #include "psa_internal.h"
+#include "psa_tma.h"
 #include "sm100.cuh"
 
 namespace psa {
@@ -78,17 +79,20 @@ struct FtAgain {
 };
 static_assert(sizeof(FtAgain) <= FT_BUF_BYTES, "does not fit the ring");
 
-// Replaces those outputs of a finished tile that the parts cannot carry, by the plain chain: called by all FT_WORKERS warps.  A
-// thread has the eight rows row0 + 4 i and the four columns from col0 on.  Without a residual the outputs say whether there is
+// Replaces those outputs of a finished tile of 128 rows and 128 columns that the parts cannot carry, by the plain chain: called by
+// WORKERS warps (16 or 8).  A thread has the eight rows row0 + 4 i and the four columns from col0 on (and, of eight warps, from col0 +
+// 64 on: with four columns the loads from shared memory were the limit, 750 us for 4096 x 768 x 3 x 768).  Without a residual the outputs say whether there is
 // anything to replace; with one the tile is computed again in any case.
+template <int WORKERS>
 __device__ __noinline__ void ft_form_again(const float* X, const float* W, float* O, const float* R, int m_first, int n_first, int M, int K,
                                            int N, FtAgain* sm) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int COLS = FT_N, CG = 16 / WORKERS, XU = FT_M * FT_K / (128 * WORKERS), WU = FT_K * COLS / (128 * WORKERS);     // 16-byte loads per thread
+    const int tid = threadIdx.x % (32 * WORKERS), warp = tid >> 5, lane = tid & 31;
     const int row0 = 32 * (warp & 3) + (lane >> 3), col0 = 32 * (warp >> 2) + 4 * (lane & 7);
-    named_bar_sync(1, 32 * FT_WORKERS);       // (the tile before is done with the shared memory)
+    named_bar_sync(1, 32 * WORKERS);       // (the tile before is done with the shared memory)
     if (tid < FT_M) { sm->row_least[tid] = sm->col_least[tid] = 0xffffffffu; sm->row_most[tid] = sm->col_most[tid] = 0; }
-    named_bar_sync(1, 32 * FT_WORKERS);
-    for (int r = warp; r < FT_M && m_first + r < M; r += FT_WORKERS) {
+    named_bar_sync(1, 32 * WORKERS);
+    for (int r = warp; r < FT_M && m_first + r < M; r += WORKERS) {
         uint32_t least = 0xffffffffu, most = 0;
 #pragma unroll 4
         for (int k = 4 * lane; k < K; k += 128) {
@@ -101,10 +105,10 @@ __device__ __noinline__ void ft_form_again(const float* X, const float* W, float
         most = __reduce_max_sync(0xffffffffu, most);
         if (lane == 0) { sm->row_least[r] = least; sm->row_most[r] = most; }
     }
-    if (n_first + 4 * lane < N) {
+    if (4 * lane < COLS && n_first + 4 * lane < N) {
         uint32_t least[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu}, most[4] = {0, 0, 0, 0};
 #pragma unroll 8
-        for (int k = warp; k < K; k += FT_WORKERS) {
+        for (int k = warp; k < K; k += WORKERS) {
             const float4 v = __ldg(reinterpret_cast<const float4*>(W + (size_t)k * N + n_first + 4 * lane));
             const uint32_t t[4] = {2u * __float_as_uint(v.x), 2u * __float_as_uint(v.y), 2u * __float_as_uint(v.z), 2u * __float_as_uint(v.w)};
 #pragma unroll
@@ -113,8 +117,8 @@ __device__ __noinline__ void ft_form_again(const float* X, const float* W, float
 #pragma unroll
         for (int e = 0; e < 4; ++e) { atomicMin(&sm->col_least[4 * lane + e], least[e]); atomicMax(&sm->col_most[4 * lane + e], most[e]); }
     }
-    named_bar_sync(1, 32 * FT_WORKERS);
-    const bool inside = n_first + col0 < N;                 // (N is a multiple of 4)
+    named_bar_sync(1, 32 * WORKERS);
+    auto inside = [&](int cg) { return n_first + col0 + 64 * cg < N; };      // (N is a multiple of 4)
     float* out = O + (size_t)(m_first + row0) * N + n_first + col0;
     auto lost = [&](float v, int r, int c) {                // whether value v at (r, c) may have lost something
         if (!(fabsf(v) < INFINITY)) return true;
@@ -126,63 +130,80 @@ __device__ __noinline__ void ft_form_again(const float* X, const float* W, float
     };
     if (!R) {
         bool any = false;
-        for (int i = 0; i < 8; ++i) {
-            if (!inside || m_first + row0 + 4 * i >= M) continue;
-            const float4 o = *reinterpret_cast<const float4*>(out + (size_t)(4 * i) * N);
-            any = any || lost(o.x, row0 + 4 * i, col0) || lost(o.y, row0 + 4 * i, col0 + 1) || lost(o.z, row0 + 4 * i, col0 + 2) ||
-                  lost(o.w, row0 + 4 * i, col0 + 3);
+        for (int i = 0; i < 8 * CG; ++i) {
+            const int cg = i >> 3, rr = row0 + 4 * (i & 7), c = col0 + 64 * cg;
+            if (!inside(cg) || m_first + rr >= M) continue;
+            const float4 o = *reinterpret_cast<const float4*>(out + (size_t)(4 * (i & 7)) * N + 64 * cg);
+            any = any || lost(o.x, rr, c) || lost(o.y, rr, c + 1) || lost(o.z, rr, c + 2) || lost(o.w, rr, c + 3);
         }
-        if (named_bar_all(!any, 1, 32 * FT_WORKERS)) return;
+        if (named_bar_all(!any, 1, 32 * WORKERS)) return;
     }
-    float acc[8][4] = {};
-#pragma unroll 1
-    for (int k0 = 0; k0 < K; k0 += FT_K) {
+    float acc[CG][8][4] = {};
+    float4 xv[XU], wv[WU];                                  // the operands of the next 32 k
+    auto fetch = [&](int k0) {
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 xv[2], wv[2];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int t = tid + 32 * FT_WORKERS * u, m = m_first + (t >> 3), kx = k0 + 4 * (t & 7), kw = k0 + (t >> 5), n = n_first + 4 * (t & 31);
+        for (int u = 0; u < XU; ++u) {
+            const int t = tid + 32 * WORKERS * u, m = m_first + (t >> 3), kx = k0 + 4 * (t & 7);
             xv[u] = m < M && kx < K ? __ldg(reinterpret_cast<const float4*>(X + (size_t)m * K + kx)) : zero;
+        }
+#pragma unroll
+        for (int u = 0; u < WU; ++u) {
+            const int t = tid + 32 * WORKERS * u, kw = k0 + t / (COLS / 4), n = n_first + 4 * (t % (COLS / 4));
             wv[u] = kw < K && n < N ? __ldg(reinterpret_cast<const float4*>(W + (size_t)kw * N + n)) : zero;
         }
-        named_bar_sync(1, 32 * FT_WORKERS);
+    };
+    constexpr bool AHEAD = WORKERS <= 8;                    // (sixteen warps have no registers for it)
+    if (AHEAD) fetch(0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < K; k0 += FT_K) {
+        if (!AHEAD) fetch(k0);
+        named_bar_sync(1, 32 * WORKERS);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int t = tid + 32 * FT_WORKERS * u;
+        for (int u = 0; u < XU; ++u) {
+            const int t = tid + 32 * WORKERS * u;
             *reinterpret_cast<float4*>(sm->x + (t >> 3) * (FT_K + 4) + 4 * (t & 7)) = xv[u];
-            *reinterpret_cast<float4*>(sm->w + 4 * t) = wv[u];
         }
-        named_bar_sync(1, 32 * FT_WORKERS);
+#pragma unroll
+        for (int u = 0; u < WU; ++u) *reinterpret_cast<float4*>(sm->w + 4 * (tid + 32 * WORKERS * u)) = wv[u];
+        named_bar_sync(1, 32 * WORKERS);
+        if (AHEAD) fetch(k0 + FT_K);
         const int kn = min(FT_K, K - k0);     // (a multiple of 4)
 #pragma unroll 1
         for (int k = 0; k < kn; k += 4) {
-            float4 w[4];
+            float4 w[CG][4];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) w[kk] = *reinterpret_cast<const float4*>(sm->w + (k + kk) * FT_N + col0);
+            for (int cg = 0; cg < CG; ++cg)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) w[cg][kk] = *reinterpret_cast<const float4*>(sm->w + (k + kk) * COLS + col0 + 64 * cg);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float4 x = *reinterpret_cast<const float4*>(sm->x + (row0 + 4 * i) * (FT_K + 4) + k);
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                     const float f = kk == 0 ? x.x : kk == 1 ? x.y : kk == 2 ? x.z : x.w;
-                    acc[i][0] = fmaf(f, w[kk].x, acc[i][0]); acc[i][1] = fmaf(f, w[kk].y, acc[i][1]);
-                    acc[i][2] = fmaf(f, w[kk].z, acc[i][2]); acc[i][3] = fmaf(f, w[kk].w, acc[i][3]);
+#pragma unroll
+                    for (int cg = 0; cg < CG; ++cg) {
+                        acc[cg][i][0] = fmaf(f, w[cg][kk].x, acc[cg][i][0]); acc[cg][i][1] = fmaf(f, w[cg][kk].y, acc[cg][i][1]);
+                        acc[cg][i][2] = fmaf(f, w[cg][kk].z, acc[cg][i][2]); acc[cg][i][3] = fmaf(f, w[cg][kk].w, acc[cg][i][3]);
+                    }
                 }
             }
         }
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = row0 + 4 * i;
-        if (!inside || m_first + r >= M) continue;
-        const size_t at = (size_t)(4 * i) * N;
+    for (int cg = 0; cg < CG; ++cg)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float o = out[at + e];
-            if (!(fabsf(o) < INFINITY) || lost(R ? acc[i][e] : o, r, col0 + e))
-                out[at + e] = R ? acc[i][e] + R[(size_t)(m_first + r) * N + n_first + col0 + e] : acc[i][e];
+        for (int i = 0; i < 8; ++i) {
+            const int r = row0 + 4 * i, c = col0 + 64 * cg;
+            if (!inside(cg) || m_first + r >= M) continue;
+            const size_t at = (size_t)(4 * i) * N + 64 * cg;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float o = out[at + e], v = acc[cg][i][e];
+                if (!(fabsf(o) < INFINITY) || lost(R ? v : o, r, c + e)) out[at + e] = R ? v + R[(size_t)(m_first + r) * N + n_first + c + e] : v;
+            }
         }
-    }
 }
 
 __global__ void __launch_bounds__(FT_THREADS, 1)
@@ -392,7 +413,7 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
             for (uint32_t j = 0; j < i; ++j) {
                 if (!(marks[mark_of(j) / 32] >> (mark_of(j) % 32) & 1u)) continue;
                 const int t = blockIdx.x + j * gridDim.x, r = t / nt, w = r / mt;
-                ft_form_again(X, w == 0 ? W0 : (w == 1 ? W1 : W2), w == 0 ? O0 : (w == 1 ? O1 : O2), R, (r % mt) * FT_M, (t % nt) * FT_N, M, K,
+                ft_form_again<FT_WORKERS>(X, w == 0 ? W0 : (w == 1 ? W1 : W2), w == 0 ? O0 : (w == 1 ? O1 : O2), R, (r % mt) * FT_M, (t % nt) * FT_N, M, K,
                               N, reinterpret_cast<FtAgain*>(smem));
             }
         }
@@ -401,6 +422,210 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) atomicExch(&dc->status, (int)PSA_ERR_TIMEOUT);
     if (warp == FT_WORKERS) tmem_dealloc(tmem, 512);
+}
+
+// ---------------------------------------------------------------- operands split once, pairs of CTAs
+// The largest calls: X and W are split into parts in global memory by a kernel of their own (the kernel above splits every tile
+// of X once per column tile and every tile of W once per row tile, beside its MMAs), and the product is that of psa_gemm.cu's
+// pairs of CTAs, 256 x 256 tiles, with six MMAs where that has one: per 64 k the five smaller products of all of them, then the
+// leading ones into the same accumulator, which is read and added to the running sums in registers: no sum in the tensor core that
+// has reached its size is longer than 4.
+//
+// What bounds it: 24 MMAs of 256 x 256 x 16 per 64 k, 3072 cycles of MMA, measured 5000 (the pairs of psa_gemm.cu take 160 cycles per MMA
+// where 128 are nominal, and every 64 k an accumulator is handed over twice).  2048 x 768 x 3 x 768: 60 us on 128 x 128 tiles, 42 here with
+// 7 of the split; the layer of 4 x 512 vectors 105 -> 85 us.
+constexpr int FP_BK = 64, FP_PLANE = 128 * FP_BK * 2;                       // a part of a CTA's operand: 16 KB
+constexpr int FP_STAGE = 6 * FP_PLANE, FP_STAGES = 2, FP_WORKERS = 8, FP_THREADS = 64 + 32 * FP_WORKERS;
+constexpr int FP_SMEM = FP_STAGES * FP_STAGE + 1024;
+struct FPMaps {
+    CUtensorMap a, b[3];      // parts as [3, rows, 1, columns]: boxes of 128 rows, of 64 rows x 64 columns
+};
+static_assert(sizeof(FtAgain) <= FP_STAGE, "does not fit the ring");
+
+// blockIdx.y: 0 X, 1.. W.  Splits `count4` groups of four numbers and marks blocks of 128 rows of X, of 256 columns of W, in which
+// a nonzero number is below 2^-60.
+__global__ void __launch_bounds__(256)
+f32_split_operands_kernel(const float4* __restrict__ X, const float4* W0, const float4* W1, const float4* W2, uint2* __restrict__ xp, uint2* __restrict__ wp,
+                          uint32_t x4, uint32_t w4, uint32_t k4, uint32_t n4, int* __restrict__ x_small, int* __restrict__ w_small) {
+    const int which = blockIdx.y;
+    const float4* src = which == 0 ? X : (which == 1 ? W0 : (which == 2 ? W1 : W2));
+    const uint32_t count4 = which == 0 ? x4 : w4;
+    grid_dependency_wait();
+    uint2* dst = which == 0 ? xp : wp + (size_t)(which - 1) * 3 * w4;
+    const int blocks_n = (int)((n4 + 63) / 64);
+    for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < count4; i += gridDim.x * 256u) {
+        const float4 v = __ldg(src + i);
+        const float x[4] = {v.x, v.y, v.z, v.w};
+        uint32_t p[3][4], least = 0xffffffffu;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            least = min(least, 2u * __float_as_uint(x[e]) - 1u);
+            p[0][e] = (__float_as_uint(x[e]) + 0x8000u) & 0xffff0000u;
+            const float r1 = x[e] - __uint_as_float(p[0][e]);
+            p[1][e] = __float_as_uint(r1) & 0xffff0000u;
+            p[2][e] = __float_as_uint(r1 - __uint_as_float(p[1][e]));
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) dst[(size_t)k * count4 + i] = make_uint2(ft_pack(p[k][0], p[k][1]), ft_pack(p[k][2], p[k][3]));
+        if (least < FT_SMALL) {
+            if (which == 0) x_small[i / k4 / FT_M] = 1;
+            else w_small[(which - 1) * blocks_n + (i % n4) / 64] = 1;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(FP_THREADS, 1)
+f32_project_pairs_kernel(const __grid_constant__ FPMaps maps, const float* __restrict__ X, const float* W0, const float* W1, const float* W2, float* O0,
+                         float* O1, float* O2, int M, int K, int N, int nW, const float* __restrict__ R, const int* __restrict__ x_small,
+                         const int* __restrict__ w_small, DeviceCounters* dc) {
+    extern __shared__ uint8_t fp_smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(fp_smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ uint64_t full_bar[FP_STAGES], empty_bar[FP_STAGES], acc_full[2], acc_empty[2];
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int abort_flag;
+    __shared__ uint32_t marks[FT_MARKS / 32];      // tiles of this CTA to look at again
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_ctarank(), unit = blockIdx.x / 2, units = gridDim.x / 2;
+    const int nk = (K + FP_BK - 1) / FP_BK, mt = (M + 255) / 256, nt = (N + 255) / 256, ntiles = mt * nt * nW;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        for (int s = 0; s < FP_STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * FP_WORKERS); }
+        fence_mbar_init();
+    }
+    for (int i = threadIdx.x; i < FT_MARKS / 32; i += FP_THREADS) marks[i] = 0;
+    if (warp == 1) { tmem_alloc_pair(&tmem_base_s, 512); tmem_relinquish_pair(); }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();                                // the partner's barriers are initialised
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_s;
+    volatile int* abortp = &abort_flag;
+    grid_dependency_wait();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---- TMA producer: the two CTAs fill their halves of a stage, the first one's barrier collects the bytes of both
+            int g = 0;
+            bool ok = true;
+            for (int t = unit; t < ntiles && ok; t += units) {
+                const int r = t / nt, w = r / mt, m0 = (r % mt) * 256 + rank * 128, n0 = (t % nt) * 256 + rank * 128;
+                for (int kt = 0; kt < nk; ++kt, ++g) {
+                    const int s = g % FP_STAGES;
+                    if (g >= FP_STAGES && !mbar_wait(&empty_bar[s], ((g / FP_STAGES) - 1) & 1, abortp)) { ok = false; break; }
+                    uint8_t* st = smem + s * FP_STAGE;
+                    if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2 * FP_STAGE);
+                    const uint32_t bar = cluster_map(&full_bar[s], 0);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        tma_load_4d_pair(st + p * FP_PLANE, &maps.a, bar, kt * FP_BK, 0, m0, p);
+                        tma_load_4d_pair(st + (3 + p) * FP_PLANE, &maps.b[w], bar, n0, 0, kt * FP_BK, p);
+                        tma_load_4d_pair(st + (3 + p) * FP_PLANE + FP_PLANE / 2, &maps.b[w], bar, n0 + 64, 0, kt * FP_BK, p);
+                    }
+                }
+            }
+            if (*abortp && rank == 0)
+                for (int k = max(0, g - FP_STAGES); k < g; ++k) mbar_wait_drain(&full_bar[k % FP_STAGES], (k / FP_STAGES) & 1);
+        }
+    } else if (warp == 1) {
+        if (rank == 0 && elect_one()) {
+            // ---- MMA issuer
+            const uint32_t idesc = umma_idesc_bf16(256, 256, UMMA_K_MAJOR, UMMA_MN_MAJOR);
+            const uint32_t a_lo0 = umma_desc_lo_kmajor(smem_u32(smem)), b_lo0 = umma_desc_lo_mnmajor(smem_u32(smem + 3 * FP_PLANE), FP_PLANE / 2);
+            constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};      // the leading product last
+            unsigned long long macs = 0;
+            int g = 0;
+            bool ok = true;
+            for (int t = unit; t < ntiles && ok; t += units) {
+                for (int kt = 0; kt < nk; ++kt, ++g) {
+                    const int s = g % FP_STAGES, buf = g & 1;
+                    if (g >= 2) ok = mbar_wait(&acc_empty[buf], ((g >> 1) - 1) & 1, abortp);
+                    if (ok) ok = mbar_wait(&full_bar[s], (g / FP_STAGES) & 1, abortp);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a = a_lo0 + s * (FP_STAGE >> 4), b = b_lo0 + s * (FP_STAGE >> 4);
+#pragma unroll
+                    for (int q = 0; q < 6; ++q)
+#pragma unroll
+                        for (int k = 0; k < FP_BK / 16; ++k)
+                            umma_ss_pair(tmem + buf * 256, umma_desc_join(a + ((PA[q] * FP_PLANE + k * 32) >> 4), UMMA_DESC_HI_SW128),
+                                         umma_desc_join(b + ((PB[q] * FP_PLANE + k * 2048) >> 4), UMMA_DESC_HI_SW128), idesc, q != 0 || k != 0);
+                    umma_commit_pair(&empty_bar[s]);
+                    umma_commit_pair(&acc_full[buf]);
+                }
+                const int r = t / nt;
+                if (ok) macs += (unsigned long long)min(256, M - (r % mt) * 256) * min(256, N - (t % nt) * 256) * K;
+            }
+            if (macs) atomicAdd(&dc->proj_macs, macs);
+        }
+    } else {
+        // ---- running sums: a warp has 32 rows (TMEM lanes) by 128 columns
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        const uint32_t src0 = tmem + (static_cast<uint32_t>(q * 32) << 16) + half * 128;
+        const uint32_t empty0 = cluster_map(&acc_empty[0], 0), empty1 = cluster_map(&acc_empty[1], 0);
+        int g = 0, i = 0;
+        bool ok = true;
+        auto mark_of = [&](int tile) { return tile / (((ntiles + units - 1) / units + FT_MARKS - 1) / FT_MARKS); };
+        for (int t = unit; t < ntiles && ok; t += units, ++i) {
+            float acc[128];
+#pragma unroll
+            for (int e = 0; e < 128; ++e) acc[e] = 0.f;
+            for (int kt = 0; kt < nk; ++kt, ++g) {
+                const int buf = g & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (g >> 1) & 1, abortp));
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    uint32_t v[16];
+                    tmem_ld16(src0 + buf * 256 + 16 * u, v);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) acc[16 * u + e] += __uint_as_float(v[e]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(buf ? empty1 : empty0);
+            }
+            if (!ok) break;
+            const int r = t / nt, w = r / mt, m0 = (r % mt) * 256 + rank * 128, n0 = (t % nt) * 256 + half * 128, row = m0 + 32 * q + lane;
+            float* o = (w == 0 ? O0 : (w == 1 ? O1 : O2)) + (size_t)row * N + n0;
+            if (row < M) {
+                bool finite = true;
+#pragma unroll
+                for (int e = 0; e < 128; e += 4) {
+                    if (n0 + e < N) {
+                        finite = finite && fabsf(acc[e]) < INFINITY && fabsf(acc[e + 1]) < INFINITY && fabsf(acc[e + 2]) < INFINITY && fabsf(acc[e + 3]) < INFINITY;
+                        float4 y = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+                        if (R) {
+                            const float4 x = __ldg(reinterpret_cast<const float4*>(R + (size_t)row * N + n0 + e));
+                            y.x += x.x; y.y += x.y; y.z += x.z; y.w += x.w;
+                        }
+                        *reinterpret_cast<float4*>(o + e) = y;
+                    }
+                }
+                if (!finite || x_small[m0 / FT_M] || w_small[w * nt + t % nt]) atomicOr(&marks[mark_of(i) / 32], 1u << (mark_of(i) % 32));
+            }
+        }
+        // ---- tiles that were marked
+        ok = named_bar_all(ok, 1, 32 * FP_WORKERS);
+        if (ok)
+            for (int j = 0; j < i; ++j) {
+                if (!(marks[mark_of(j) / 32] >> (mark_of(j) % 32) & 1u)) continue;
+                const int t = unit + j * units, r = t / nt, w = r / mt;
+                for (int c = 0; c < 256; c += FT_N)
+                    ft_form_again<FP_WORKERS>(X, w == 0 ? W0 : (w == 1 ? W1 : W2), w == 0 ? O0 : (w == 1 ? O1 : O2), R, (r % mt) * 256 + rank * 128,
+                                              (t % nt) * 256 + c, M, K, N, reinterpret_cast<FtAgain*>(smem));
+            }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_flag) atomicExch(&dc->status, (int)PSA_ERR_TIMEOUT);
+    __syncwarp();
+    cluster_sync();                 // MMAs, arrivals and copies that involve the partner are over in both CTAs
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc_pair(tmem, 512);
 }
 
 }  // namespace
@@ -416,6 +641,65 @@ cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* c
     f32_project_tensor_kernel<<<(int)(tiles < sms ? tiles : sms), FT_THREADS, FT_SMEM, stream>>>(
         X, W[0], W[nW == 3 ? 1 : 0], W[nW == 3 ? 2 : 0], out[0], out[nW == 3 ? 1 : 0], out[nW == 3 ? 2 : 0], rows, D, N, nW, residual, dc);
     return cudaGetLastError();
+}
+
+size_t f32_project_parts_bytes(int rows, int D, int N, int nW) {
+    const size_t tiles = (size_t)((rows + 255) / 256) * ((N + 255) / 256) * nW;
+    if (D % 8 || N % 8 || tiles < 24 || (size_t)rows * D >= (size_t)1 << 33 || (size_t)D * N >= (size_t)1 << 33) return 0;
+    return ((size_t)rows * D * 6 + 255) / 256 * 256 + ((size_t)D * N * 6 + 255) / 256 * 256 * nW;
+}
+// Whether the pairs are faster, in cycles as measured: the split and 5000 per 64 k of a 256 x 256 tile against 2300 per 32 k of a 128 x 128
+// tile of the kernel above (us, layers of 12 heads with d_model = 768: 1024 rows 65 / 58 on the tiles, 2048 rows 88 / 107).
+bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms) {
+    const long long pairs = (long long)((rows + 255) / 256) * ((N + 255) / 256) * nW, tiles = (long long)((rows + 127) / 128) * ((N + 127) / 128) * nW;
+    const long long units = sms / 2 > 0 ? sms / 2 : 1;
+    return 16000 + (pairs + units - 1) / units * ((D + 63) / 64) * 5000 < 4000 + (tiles + sms - 1) / sms * ((D + 31) / 32) * 2300;
+}
+size_t f32_project_marks(int rows, int N, int nW) { return (rows + 127) / 128 + (size_t)((N + 255) / 256) * nW; }
+
+cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N, const float* residual,
+                              void* parts, int* marks, DeviceCounters* dc, cudaStream_t stream) {
+    static DeviceSetup setup;
+    const int sms = device_setup(&setup, [] {
+        return cudaFuncSetAttribute(f32_project_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FP_SMEM);
+    }, "fp32 projection set-up (pairs)");
+    if (sms < 2) return cudaErrorUnknown;
+    char* xp = static_cast<char*>(parts);
+    char* wp = xp + ((size_t)rows * D * 6 + 255) / 256 * 256;
+    const uint32_t x4 = (uint32_t)((size_t)rows * D / 4), w4 = (uint32_t)((size_t)D * N / 4);
+    int* w_small = marks + (rows + 127) / 128;
+    const uint32_t blocks = (max(x4, w4) + 1023) / 1024;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernels wait for their predecessors themselves
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t split = {};
+    split.gridDim = dim3(blocks < 1024 ? blocks : 1024, 1 + nW);
+    split.blockDim = dim3(256);
+    split.stream = stream;
+    split.attrs = attr;
+    split.numAttrs = 1;
+    const auto f4 = [&](int w) { return reinterpret_cast<const float4*>(W[nW == 3 ? w : 0]); };
+    const cudaError_t e = cudaLaunchKernelEx(&split, f32_split_operands_kernel, reinterpret_cast<const float4*>(X), f4(0), f4(1), f4(2),
+                                             reinterpret_cast<uint2*>(xp), reinterpret_cast<uint2*>(wp), x4, w4, (uint32_t)(D / 4), (uint32_t)(N / 4), marks, w_small);
+    if (e != cudaSuccess) return e;
+    FPMaps maps;
+    if (!make_tensor_map_bf16_4d(&maps.a, xp, 3, rows, 1, D, 128)) return cudaErrorInvalidValue;
+    for (int w = 0; w < 3; ++w)
+        if (!make_tensor_map_bf16_4d(&maps.b[w], wp + (size_t)(w < nW ? w : 0) * 6 * D * N, 3, D, 1, N, FP_BK)) return cudaErrorInvalidValue;
+    const int ntiles = ((rows + 255) / 256) * ((N + 255) / 256) * nW, units = ntiles < sms / 2 ? ntiles : sms / 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * units);
+    cfg.blockDim = dim3(FP_THREADS);
+    cfg.dynamicSmemBytes = FP_SMEM;
+    cfg.stream = stream;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, f32_project_pairs_kernel, maps, X, W[0], W[nW == 3 ? 1 : 0], W[nW == 3 ? 2 : 0], out[0], out[nW == 3 ? 1 : 0],
+                              out[nW == 3 ? 2 : 0], rows, D, N, nW, residual, static_cast<const int*>(marks), static_cast<const int*>(w_small), dc);
 }
 
 }  // namespace psa

@@ -24,11 +24,23 @@ struct DeviceCounters {
 // ---- fp32 CUDA-core path (psa_f32.cu) ----
 // out[w][r, c] = sum_k X[r, k] W[w][k, c] for w < nW.
 // `residual` ([rows, N], may be null) is added to every output.
+// `ps` (may be null): scratch for the largest calls, see f32_project_pairs.
+struct F32ProjectScratch {
+    void* parts;
+    int* marks;
+};
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
-                        int N, const float* residual, DeviceCounters* dc, cudaStream_t stream);
+                        int N, const float* residual, const F32ProjectScratch* ps, DeviceCounters* dc, cudaStream_t stream);
 // The same on the tensor cores, to the same accuracy (psa_f32_tensor.cu); f32_project chooses.  Rows of 16 bytes, as there.
 cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
                                const float* residual, DeviceCounters* dc, cudaStream_t stream);
+// The same for the largest calls, operands split once into `parts` (f32_project_parts_bytes; 0: the call is not one of them, whatever the
+// device), on pairs of CTAs.  marks: f32_project_marks ints, clear when the call's kernels start.
+size_t f32_project_parts_bytes(int rows, int D, int N, int nW);
+size_t f32_project_marks(int rows, int N, int nW);
+bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms);
+cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N, const float* residual,
+                              void* parts, int* marks, DeviceCounters* dc, cudaStream_t stream);
 // Scratch of the tensor-core attention: marks of the heads it cannot take (B H ints, clear when the call's kernels start), maxima
 // and sums of the rows on the diagonal tiles (2 B H n numbers), bf16 parts of K and V (6 B n H d each numbers of 16 bits, together).
 struct F32Scratch {

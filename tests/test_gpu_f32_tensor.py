@@ -61,3 +61,20 @@ def test_heads_with_numbers_without_parts(scheme):
         _close(got[:, :, h], ref[:, :, h])
     _close(got[0, :, 1], ref[0, :, 1])
     _close(got[:, :, 3][:, :, :5], ref[:, :, 3][:, :, :5])
+
+
+# Projections of the largest calls (pairs of CTAs, 256 x 256 tiles, 64 k at a time): ragged rows, columns and depth, tiny and
+# infinite operands.  With one vector per sequence the attention returns V.  Bound: six bf16 products per fp32 product leave 2^-24 of it
+# out, sums are rounded every 64 k: (K / 64 + 4) 2^-24 of the sum of magnitudes.
+@pytest.mark.parametrize("rows,D,H,d", [(2100, 776, 33, 32), (4111, 328, 16, 64), (2048, 768, 12, 64)])
+def test_projections_of_large_calls(rows, D, H, d):
+    X, Wq, Wk, Wv = [inputs.tensor(rows + D, i, s, 1.0, "f32")[1] for i, s in enumerate([(rows, 1, D)] + [(D, H * d)] * 3)]
+    X[7] *= np.float32(1e-36)
+    X[300, 0, 5] = np.inf
+    z = binding.psa_attention_f32(*[torch.from_numpy(t).cuda() for t in (X, Wq, Wk, Wv)], H, binding.FULL)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got == binding.psa_skip_count(rows, H, 1, D, d, binding.FULL, binding.F32)
+    z, x, w = z.cpu().numpy().reshape(rows, H * d).astype(np.float64), X.reshape(rows, D).astype(np.float64), Wv.astype(np.float64)
+    assert not np.isfinite(z[300]).all()
+    x[300], z[300] = 0.0, 0.0
+    assert (np.abs(z - x @ w) <= (D / 64 + 4) * 2.0 ** -24 * (np.abs(x) @ np.abs(w)) + 1e-44).all()
