@@ -227,15 +227,13 @@ __device__ __forceinline__ void fa_scores(unsigned long long (&acc)[8][U], const
     if (c < d4) step(qe + 4 * c, k + 4 * c);
 }
 
-// MODE 0: the three phases for FULL / MASKED.  MODE 2: phases 2 and 3 of the symmetric scheme, scores read from S.  MODE 3: the
-// masked scheme's weights inside the 128-row tiles of f32_attn_tensor_kernel; the first tile of a head is done then, rows of the
-// others leave their maximum and sum in `ml` (B H n numbers each) and their output undivided.
-// `bad` (may be null): MODE 0 works on the heads marked there only, MODE 3 on the others.
+// MODE 0: the three phases for FULL / MASKED.  MODE 2: phases 2 and 3 of the symmetric scheme, scores read from S.
+// `bad` (may be null): MODE 0 works on the heads marked there only.
 template <int DG, int KS, int MODE>
 __global__ void __launch_bounds__(FA_THREADS, DG == 1 ? 3 : 2)
 f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                  float* __restrict__ out, const float* __restrict__ S, int n, int H, int d, float scale, int masked,
-                 DeviceCounters* dc, const int* __restrict__ bad, float* __restrict__ ml) {
+                 DeviceCounters* dc, const int* __restrict__ bad) {
     using C = FACfg<DG, KS>;
     constexpr int U = C::U;
     extern __shared__ float4 fa_smem4[];
@@ -245,9 +243,9 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     float* Ps = Vs + C::V_FLOATS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
     const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
-    if (MODE == 0 || MODE == 3) {
+    if (MODE == 0) {
         grid_dependency_wait();
-        if (bad && (bad[bh] != 0) != (MODE == 0)) return;
+        if (bad && !bad[bh]) return;
     }
     const int rb = masked ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // the longest rows first
     const int r0 = rb * C::BR;
@@ -258,8 +256,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     const size_t base = ((size_t)b * n) * ld + (size_t)h * d;
     const int d4 = d >> 2;
     const int kend = masked ? min(r0 + C::BR, n) : n;                   // keys that some row of the CTA keeps
-    const int nblk = (kend + FA_BC - 1) / FA_BC, jfirst = MODE == 3 ? r0 / 128 * (128 / FA_BC) : 0;
-    const bool undivided = MODE == 3 && r0 >= 128;
+    const int nblk = (kend + FA_BC - 1) / FA_BC;
     const float* Sh = MODE == 2 ? S + (size_t)bh * n * n : nullptr;
     float* Pw = Ps + warp * 16 * C::PP;
     const float* Pr = Pw + ty * C::PP;                                  // row i of the lane: + 2 i PP
@@ -268,7 +265,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 
     if (MODE != 2) {
         fa_load<DG, C::BR, C::DP, true>(Qs, Q + base, r0, n, ld, d4);
-        fa_load<DG, FA_BC, C::KP, false>(Ks, K + base, jfirst * FA_BC, n, ld, d4);
+        fa_load<DG, FA_BC, C::KP, false>(Ks, K + base, 0, n, ld, d4);
     }
     cp_async_commit();
 
@@ -281,7 +278,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     }
     unsigned int dots = 0, wts = 0;                                     // weights of this lane; of its rows in phase 3
 
-    for (int jb = jfirst; jb < nblk; ++jb) {
+    for (int jb = 0; jb < nblk; ++jb) {
         const int k0 = jb * FA_BC + kw;                                 // first key of the warp's share
         const int last = min(wr0 + 15, n - 1);                          // last row of the warp that exists
         const int maxlim = wr0 >= n ? -1 : (masked ? last : n - 1) - k0;
@@ -419,11 +416,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if (row + 2 * i >= n) continue;
-            const float inv = undivided ? 1.f : 1.f / l[i];
-            if (undivided && tx == 0) {
-                ml[(size_t)bh * n + row + 2 * i] = m[i];
-                ml[((size_t)gridDim.x + bh) * n + row + 2 * i] = l[i];
-            }
+            const float inv = 1.f / l[i];
             float* dst = out + base + (size_t)(row + 2 * i) * ld + 4 * tx;
 #pragma unroll
             for (int g = 0; g < DG; ++g)
@@ -462,11 +455,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
                 sum = fmaf(w, part_ml[KS * C::BR + k * C::BR + r], sum);
                 y.x = fmaf(w, f.x, y.x); y.y = fmaf(w, f.y, y.y); y.z = fmaf(w, f.z, y.z); y.w = fmaf(w, f.w, y.w);
             }
-            const float inv = undivided ? 1.f : 1.f / sum;
-            if (undivided && c == 0) {
-                ml[(size_t)bh * n + r0 + r] = mx;
-                ml[((size_t)gridDim.x + bh) * n + r0 + r] = sum;
-            }
+            const float inv = 1.f / sum;
             *reinterpret_cast<float4*>(out + base + (size_t)(r0 + r) * ld + 4 * c) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
         }
     }
@@ -478,6 +467,215 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     if (lane == 0) {
         if (MODE != 2 && dots) atomicAdd(&dc->qk_macs, (unsigned long long)dots * d);
         if (wts) { atomicAdd(&dc->pv_macs, (unsigned long long)wts * d); atomicAdd(&dc->exps, (unsigned long long)wts); }
+    }
+}
+
+// ---------------------------------------------------------------- diagonal tiles of the masked scheme
+// The weights inside a 128-row tile, j <= i, for the calls whose other blocks are on the tensor cores (f32_attn_tensor_kernel): maximum,
+// sum and undivided output of every row, or the output itself where the tile is the head's first and so has nothing else.  A CTA per
+// tile, all of it in shared memory.
+//
+// Phase 1 gives a thread 8 rows by 4 keys: 240 such pieces lie below the diagonal, one per thread of warps 0-7, and the 32 on it are
+// warp 8's, which alone tests weight by weight.  Phase 3 gives a warp two groups of 8 rows, r and 15 - r, which together have 17 groups of
+// 8 keys; the last group's triangle is unrolled.  Bound by the port of shared memory (12 loads of 16 bytes for 128 multiply-accumulates).
+// Rows of Q and K are stored so that rows read at the same time are neighbours, 4 banks apart.
+// Measured: the 128 tiles of 16 heads of n = 1024, d = 128 54 us as blocks of f32_flash_kernel, 30 here.
+constexpr int FD_THREADS = 288;
+template <int DG>
+struct FDCfg {
+    static constexpr int P = 64 * DG + 4, PP = 132;                      // row pitches of Q and K, of the weights, in floats
+    static constexpr int QK = 128 * P, W = 128 * PP, V = 128 * 64 * DG;
+    static constexpr int FRONT = 2 * QK > W ? 2 * QK : W;                // Q and K, then the weights over them
+    static constexpr int SMEM = (FRONT + V + 256) * (int)sizeof(float);
+};
+
+template <int DG>
+__global__ void __launch_bounds__(FD_THREADS, 3 - DG)
+f32_diagonal_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V, float* __restrict__ out, float* __restrict__ ml,
+                    const int* __restrict__ bad, int heads, int n, int H, int d, float scale, DeviceCounters* dc) {
+    using C = FDCfg<DG>;
+    extern __shared__ float4 fd_smem4[];
+    float* Qs = reinterpret_cast<float*>(fd_smem4);
+    float* Ks = Qs + C::QK;
+    float* Ws = Qs;
+    float* Vs = Qs + C::FRONT;
+    float* row_m = Vs + C::V;
+    float* row_l = row_m + 128;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int bh = blockIdx.x % heads, tile = blockIdx.x / heads, b = bh / H, h = bh - b * H;
+    grid_dependency_wait();
+    if (bad[bh]) return;
+    const size_t ld = (size_t)H * d, base = ((size_t)b * n + tile * 128) * ld + (size_t)h * d;
+    const int rows = min(128, n - tile * 128), d4 = d >> 2;
+    for (int t = tid; t < 128 * d4; t += FD_THREADS) {
+        const int r = t / d4, c = t - r * d4;
+        if (r >= rows) continue;
+        cp_async16(Qs + ((r & 7) * 16 + (r >> 3)) * C::P + 4 * c, Q + base + r * ld + 4 * c);       // row 8 r + i at 16 i + r
+        cp_async16(Ks + ((r & 3) * 32 + (r >> 2)) * C::P + 4 * c, K + base + r * ld + 4 * c);       // row 4 c + u at 32 u + c
+    }
+    cp_async_commit();
+    for (int t = tid; t < 128 * d4; t += FD_THREADS) {
+        const int r = t / d4, c = t - r * d4;
+        if (r < rows) cp_async16(Vs + r * 64 * DG + 4 * c, V + base + r * ld + 4 * c);
+    }
+    cp_async_commit();
+    // zeros below the last row: nothing that is not a number may come in there
+    for (int t = tid; t < (128 - rows) * d4; t += FD_THREADS) {
+        const int r = rows + t / d4, c = t % d4;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(Qs + ((r & 7) * 16 + (r >> 3)) * C::P + 4 * c) = zero;
+        *reinterpret_cast<float4*>(Ks + ((r & 3) * 32 + (r >> 2)) * C::P + 4 * c) = zero;
+        *reinterpret_cast<float4*>(Vs + r * 64 * DG + 4 * c) = zero;
+    }
+    cp_async_wait_group<1>();
+    __syncthreads();
+    // ---- phase 1 (Eq. 1): piece (r, c) = rows 8 r .. 8 r + 7, keys 4 c .. 4 c + 3
+    int r, c;
+    if (warp < 8) {
+        r = (int)((1.f + sqrtf(1.f + 4.f * tid)) * 0.5f);               // r (r - 1) <= tid < r (r + 1)
+        if (r * (r - 1) > tid) --r;
+        if (r * (r + 1) <= tid) ++r;
+        c = tid - r * (r - 1);
+    } else {
+        r = lane >> 1;
+        c = 2 * r + (lane & 1);
+    }
+    const bool have = warp == 8 || tid < 240;
+    unsigned long long acc[8][4] = {};
+    if (have) {
+        const float* q = Qs + r * C::P;
+        const float* k = Ks + c * C::P;
+        auto step = [&](int x, auto edge_tag) {
+            constexpr bool EDGE = decltype(edge_tag)::value;
+            ulonglong2 kv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) kv[u] = *reinterpret_cast<const ulonglong2*>(k + 32 * u * C::P + 4 * x);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(q + 16 * i * C::P + 4 * x);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (!EDGE || 4 * (lane & 1) + u <= i) { fma2(acc[i][u], qv.x, kv[u].x); fma2(acc[i][u], qv.y, kv[u].y); }
+            }
+        };
+        if (warp < 8) {
+#pragma unroll 2
+            for (int x = 0; x < d4; ++x) step(x, std::false_type{});
+        } else {
+#pragma unroll 1
+            for (int x = 0; x < d4; ++x) step(x, std::true_type{});
+        }
+    }
+    __syncthreads();                // every thread is done with Q and K
+    if (have) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float s[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float2 f = unpack2(acc[i][u]);
+                s[u] = (f.x + f.y) * scale;
+            }
+            *reinterpret_cast<float4*>(Ws + (8 * r + i) * C::PP + 4 * c) = make_float4(s[0], s[1], s[2], s[3]);
+        }
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    // ---- phase 2 (Eq. 2): two threads a row, alternating groups of four keys
+    if (tid < 256) {
+        const int row = tid >> 1, part = tid & 1;
+        float* w = Ws + row * C::PP;
+        float m = -INFINITY;
+        for (int j = 4 * part; j <= row; j += 8) {
+            const float4 f = *reinterpret_cast<const float4*>(w + j);
+            m = fmaxf(m, f.x);
+            if (j + 1 <= row) m = fmaxf(m, f.y);
+            if (j + 2 <= row) m = fmaxf(m, f.z);
+            if (j + 3 <= row) m = fmaxf(m, f.w);
+        }
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        float l = 0.f;
+        for (int j = 4 * part; j <= row; j += 8) {
+            float4 f = *reinterpret_cast<const float4*>(w + j);
+            f.x = expf(f.x - m); l += f.x;
+            if (j + 1 <= row) { f.y = expf(f.y - m); l += f.y; }
+            if (j + 2 <= row) { f.z = expf(f.z - m); l += f.z; }
+            if (j + 3 <= row) { f.w = expf(f.w - m); l += f.w; }
+            *reinterpret_cast<float4*>(w + j) = f;
+        }
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        if (part == 0) {
+            row_m[row] = m;
+            row_l[row] = l;
+            if (tile > 0 && row < rows) {
+                ml[(size_t)bh * n + tile * 128 + row] = m;
+                ml[((size_t)heads + bh) * n + tile * 128 + row] = l;
+            }
+        }
+    }
+    __syncthreads();
+    // ---- phase 3 (Eq. 3): a lane has 2 DG columns of 8 rows
+    constexpr int CW = 2 * DG;
+    if (warp < 8 && CW * lane < d) {
+        const float* v = Vs + CW * lane;
+        auto value = [&](int j, float (&f)[CW]) {
+            if constexpr (CW == 4) {
+                const float4 t = *reinterpret_cast<const float4*>(v + j * 64 * DG);
+                f[0] = t.x; f[1] = t.y; f[2] = t.z; f[3] = t.w;
+            } else {
+                const float2 t = *reinterpret_cast<const float2*>(v + j * 64 * DG);
+                f[0] = t.x; f[1] = t.y;
+            }
+        };
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            const int g = side ? 15 - warp : warp;
+            float o[8][CW] = {};
+            const float* w = Ws + 8 * g * C::PP;
+#pragma unroll 1
+            for (int j = 0; j < 8 * g; j += 4) {
+                float4 p[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) p[i] = *reinterpret_cast<const float4*>(w + i * C::PP + j);
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    float f[CW];
+                    value(j + jj, f);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float x = jj == 0 ? p[i].x : jj == 1 ? p[i].y : jj == 2 ? p[i].z : p[i].w;
+#pragma unroll
+                        for (int e = 0; e < CW; ++e) o[i][e] = fmaf(x, f[e], o[i][e]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {                    // the diagonal: rows from jj on
+                float f[CW];
+                value(8 * g + jj, f);
+#pragma unroll
+                for (int i = jj; i < 8; ++i) {
+                    const float x = w[i * C::PP + 8 * g + jj];
+#pragma unroll
+                    for (int e = 0; e < CW; ++e) o[i][e] = fmaf(x, f[e], o[i][e]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int row = 8 * g + i;
+                if (row >= rows) continue;
+                const float f = tile > 0 ? 1.f : 1.f / row_l[row];
+                float* y = out + base + (size_t)row * ld + CW * lane;
+                if constexpr (CW == 4) *reinterpret_cast<float4*>(y) = make_float4(o[i][0] * f, o[i][1] * f, o[i][2] * f, o[i][3] * f);
+                else *reinterpret_cast<float2*>(y) = make_float2(o[i][0] * f, o[i][1] * f);
+            }
+        }
+    }
+    if (tid == 0) {
+        const unsigned long long pairs = (unsigned long long)rows * (rows + 1) / 2;
+        atomicAdd(&dc->qk_macs, pairs * d);
+        atomicAdd(&dc->pv_macs, pairs * d);
+        atomicAdd(&dc->exps, pairs);
     }
 }
 
@@ -1167,7 +1365,7 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
         return cudaErrorUnknown;
     const dim3 grid(B * H, (n + C::BR - 1) / C::BR);
     if (!fs) {
-        f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc, nullptr, nullptr);
+        f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc, nullptr);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
@@ -1180,7 +1378,7 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f32_flash_kernel<DG, KS, MODE>, Q, K, V, out, S, n, H, d, scale, masked, dc, static_cast<const int*>(fs->bad), fs->ml);
+    return cudaLaunchKernelEx(&cfg, f32_flash_kernel<DG, KS, MODE>, Q, K, V, out, S, n, H, d, scale, masked, dc, static_cast<const int*>(fs->bad));
 }
 template <int DG, int MODE>
 cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n,
@@ -1217,7 +1415,24 @@ template <int DG>
 cudaError_t tensor_attention(const float* Q, const float* K, const float* V, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale,
                              int masked, DeviceCounters* dc, int sms, cudaStream_t stream) {
     cudaError_t e = f32_attention_split(Q, K, V, fs, B, H, n, d, stream);
-    if (e == cudaSuccess && masked) e = launch_flash_split<DG, 3>(Q, K, V, out, nullptr, B, H, n, d, scale, 1, dc, &fs, sms, stream);
+    if (e == cudaSuccess && masked) {
+        static DeviceSetup setup;
+        if (device_setup(&setup, [] {
+                return cudaFuncSetAttribute(f32_diagonal_kernel<DG>, cudaFuncAttributeMaxDynamicSharedMemorySize, FDCfg<DG>::SMEM);
+            }, "fp32 diagonal tiles set-up") <= 0)
+            return cudaErrorUnknown;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(B * H * ((n + 127) / 128));
+        cfg.blockDim = dim3(FD_THREADS);
+        cfg.dynamicSmemBytes = FDCfg<DG>::SMEM;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (waits for its predecessor itself)
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, f32_diagonal_kernel<DG>, Q, K, V, out, fs.ml, static_cast<const int*>(fs.bad), B * H, n, H, d, scale, dc);
+    }
     if (e == cudaSuccess) e = f32_attention_tensor(Q, out, fs, B, H, n, d, scale, masked, dc, stream);
     if (e == cudaSuccess) e = launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, masked, dc, &fs, sms, stream);
     return e;
@@ -1253,14 +1468,16 @@ bool short_heads(long long heads, int n, int d, int scheme, int sms) {
 }
 }  // namespace
 
-// Whether a call is better off on the tensor cores: four launches instead of one, and under the masked scheme the diagonal tiles stay on
-// CUDA cores.  Measured (us, CUDA cores / tensor cores): FULL 16 heads of n = 160, d = 16 15.4 / 16.8, of n = 192, d = 64 17.4 / 17.4, of n = 1024, d =
-// 128 166 / 54; 48 of n = 512, d = 64 114 / 42; MASKED 16 heads of n = 384, d = 128 48 / 56, 16 of n = 512, d = 16 31.8 / 33.3, of n = 700, d = 64
-// 48 / 45, of n = 1024, d = 128 166 / 102; 256 of n = 256, d = 128 204 / 218.
+// Whether a call is better off on the tensor cores: three launches instead of one, and under the masked scheme a fourth for the diagonal
+// tiles, which takes 20 to 30 us however few they are.  Measured (us, CUDA cores / tensor cores): FULL 16 heads of n = 129, d = 64 17 / 19, of n =
+// 160, d = 16 15.4 / 16.8, of n = 192, d = 64 17.4 / 17.4, of n = 1024, d = 128 308 / 54; 48 of n = 512, d = 64 111 / 42.  MASKED 64 heads of n = 256, d = 64
+// 35.9 / 36.4; 16 of n = 384, d = 128 48 / 52, of n = 512, d = 16 31.8 / 34.1, of n = 1024, d = 128 166 / 76; 8 of n = 512, d = 64 36 / 40; 4 of n = 640, d =
+// 64 38 / 42; 48 of n = 512, d = 64 93 / 52.
 bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme) {
     const long long T = (n + 127) / 128, blocks = (long long)B * H * T * T;
-    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || blocks < 64 || (long long)B * H * n * d >= (1LL << 31)) return false;
-    return scheme == PSA_MASKED ? n > 512 : n > 128 && (n >= 256 || d >= 64);
+    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || (long long)B * H * n * d >= (1LL << 31)) return false;
+    if (scheme == PSA_MASKED) return n > 256 && blocks >= (d >= 64 ? 256 : 320);
+    return n >= 160 && (n >= 256 || d >= 64) && blocks >= 64;
 }
 
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, const F32Scratch* fs, int B, int H,

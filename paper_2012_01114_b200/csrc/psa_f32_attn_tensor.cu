@@ -10,7 +10,7 @@
 // Q once per row tile by the warps that need it.
 //
 // Skipping stays element-exact: under the masked scheme only blocks of keys before the row tile come here; the weights inside the
-// tile (128 x 128, on the diagonal) are computed one by one by f32_flash_kernel (psa_f32.cu) ahead of this kernel, which
+// tile (128 x 128, on the diagonal) are computed one by one by f32_diagonal_kernel (psa_f32.cu) ahead of this kernel, which
 // continues from their maximum, sum and partial output.
 //
 // What the parts cannot carry: f32_split_kernel marks heads with an operand that is not finite or beyond 2^50, or a nonzero value
@@ -18,9 +18,9 @@
 // can hold has parts in the normal range.
 //
 // What bounds it: per block of 64 keys 72 MMAs, 3072 cycles at d = 128 and 1536 at d = 64, beside about 1500 issue slots per scheduler of
-// softmax and splitting; the masked scheme also its longest row tiles and the diagonal tiles ahead of them (54 of its 100 us at 16
+// softmax and splitting; the masked scheme also its longest row tiles and the diagonal tiles ahead of them (30 of its 76 us at 16
 // heads of n = 1024, d = 128).  Measured (us, CUDA cores before / whole call now): 16 heads of n = 1024, d = 128 FULL 308 / 54, MASKED
-// 166 / 100; 48 of n = 512, d = 64, FULL 111 / 42.  Error against 64 bits 1.6e-7 .. 3.1e-7, on CUDA cores 1.6e-7 .. 4.8e-7.
+// 166 / 76; 48 of n = 512, d = 64, FULL 111 / 42.  Error against 64 bits 1.6e-7 .. 3.1e-7, on CUDA cores 1.6e-7 .. 4.8e-7.
 //
 // Roles (320 threads): warp 0 = TMA producer, warp 1 = MMA issuer, warps 2-9 = softmax, running output (a warp owns 16 rows, quad
 // layout of sm100.cuh).  S of the next block is computed during the softmax of a block, its PV during the softmax of the next.
