@@ -864,6 +864,8 @@ f32_fused_layer_kernel(const float* __restrict__ X, const float* __restrict__ Wq
                        int scheme, DeviceCounters* dc, DeviceCounters* dc_next) {
     extern __shared__ float4 fs_smem4[];
     float* sm = reinterpret_cast<float*>(fs_smem4);
+    grid_launch_dependents();     // (the next kernel may come in at once: its launch is hidden behind this one, its work is not)
+    grid_dependency_wait();
     // the counter block of the NEXT call on this workspace is cleared here, off that call's critical path
     if (blockIdx.x == 0 && threadIdx.x == 0 && dc_next) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};
     const int nW = scheme == PSA_SYMMETRIC ? 1 : 3;
@@ -1081,6 +1083,9 @@ f32_fused_cluster_kernel(const float* __restrict__ X, const float* __restrict__ 
     const int own_rows = own_tiles * 4;                                // (the last tile's rows beyond n are skipped)
     auto own_row = [&](int lr) { return 4 * (rank + (lr >> 2) * C) + (lr & 3); };     // local row -> row of the head
     unsigned long long qk = 0, pv = 0, ex = 0, pj = 0;
+    // The next kernel may come in at once: a call of one head takes 8 SMs, and the launch of the next one is hidden behind it.
+    grid_launch_dependents();
+    grid_dependency_wait();
     if (blockIdx.x == 0 && tid == 0 && dc_next) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};
 
     // ---- stage this CTA's rows of X[b] and the head's columns of the three projection matrices: asynchronous copies
@@ -1337,13 +1342,15 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
         cfg.blockDim = dim3(FS_THREADS);
         cfg.dynamicSmemBytes = fused_layout(n, D, d, 3).total * sizeof(float);
         cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = C;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         return cudaLaunchKernelEx(&cfg, f32_fused_cluster_kernel, X, Wq, Wk, Wv, out, n, H, D, d, scale, scheme, dc, dc_next);
     }
     const size_t smem = fused_layout(n, D, d, scheme == PSA_SYMMETRIC ? 1 : 3).total * sizeof(float);
