@@ -11,9 +11,10 @@
 // Operands: Q 64 KB, and K and V through one ring of four 32 KB slots in the order the MMAs use them -- a K tile as two
 // halves of the head's columns, a V tile as two halves of its keys -- so that a slot is free again after 8 or 4 MMAs.
 //
-// What bounds it: 16 MMAs at 92 cycles and 8 at 129 are 2500 cycles per block, 128 KB of operands at an SM's 64 bytes per
-// cycle from L2 2050; measured 3300 on long sequences (16 heads of n = 8192, d_k = 192, masked: 559 us as one CTA per
-// tile with one K and one V stage, 379 now; 32 heads of n = 2048, d_k = 256, masked: 103 and 80).
+// What bounds it: 16 MMAs of 64 cycles and 8 of 128 are 2048 cycles per block, 128 KB of operands at an SM's 64 bytes per
+// cycle from L2 as many; the issuing thread spends 100-130 more on each of six barriers and five commits (with slots of 16 KB, nine of
+// them, it was slower: 76 -> 89 us); measured 3000 on long sequences (16 heads of n = 8192, d_k = 192, masked: 559 us as one CTA per
+// tile with one K and one V stage, 379 now; 32 heads of n = 2048, d_k = 256, masked: 103, then 80 and 70).
 //
 // CTA layout (320 threads): warp 0 = work list and TMA producer, warp 1 = MMA issuer, warps 2-9 = softmax and epilogue
 // (a warp owns 16 rows, read in the quad layout of sm100.cuh).  The tensors' head size may be any multiple of 8 in (128,
@@ -162,8 +163,10 @@ attn_wide_kernel(const __grid_constant__ WMaps maps, int n, int d, int H, int nb
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ------------------------------------------------------------ MMA issuer
+            // (`lane == 0` instead of an elected lane: 76 and 70 us at 32 heads of n = 2048, d_k = 256, masked, 213 and 193 at 64 heads of n =
+            // 2048, d_k = 192, full.)
             // Order of an item: S_0, S_1, PV_0, S_2, PV_1, ...  S_{j+1} overwrites S_{j-1} and P_{j-1}, which PV_{j-1}, issued
             // before it, has read: the tensor pipe runs this thread's MMAs in order.
             const uint32_t idescS = umma_idesc_bf16(128, 128, UMMA_K_MAJOR, UMMA_K_MAJOR);

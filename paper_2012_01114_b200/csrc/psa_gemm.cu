@@ -199,7 +199,7 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
         if (*abortp && rank == 0) {
             for (int k = max(0, g - STAGES); k < g; ++k) mbar_wait_drain(&full_bar[k % STAGES], (k / STAGES) & 1);
         }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
+    } else if (warp == 1 && rank == 0 && elect_one()) {
         // ---- MMA issuer
         const uint32_t idesc = umma_idesc_bf16(CTAS * BM, BN, UMMA_K_MAJOR, UMMA_MN_MAJOR);
         // descriptor low words of stage 0; a stage or k-step is a constant added to them (sm100.cuh)
