@@ -45,11 +45,11 @@ L2_FLUSH_BYTES = 256 << 20
 # kernel it was measured on; once one of them changes the roofline reports traffic = null.
 NCU_TRAFFIC = {
     "sources": {
-        "psa_attn_persist.cu": "ccfc97f7fceedb017fa46810e0f8d58df93cab8616bc7145783c106f72051cd5",
+        "psa_attn_persist.cu": "c809ad7eef03f4331762b2e69228796567f04af1479ba862a128cb0eafdc1b8b",
         "psa_softmax.cuh": "f7c2c8092d61159a139d9f5938bbf907bbe8a8d77e4a239ee94079816cb5aaa7",
         "psa_sched.h": "5db1035f5bc41698396fed66ead14f0b4a9ef0408738ccb324301a4ae99be214",
-        "psa_gemm.cu": "725040bfa8318d703c4ea4b6436bf132f22b3d00a174f60bbb59858b6eab0ca4",
-        "sm100.cuh": "e5bfdd9871fd45a54cc813fdaf0e5023eada764282d163263a9b3efd12234532"
+        "psa_gemm.cu": "6259df700b4ff7b71e80dff7fccf14358b7ef73294b01235e530e013c3f57bae",
+        "sm100.cuh": "e84f5c826a88c4c0c2171f4ba6c4c1ff9f0ddb02e90d5fcefe41dd47048b181d"
     },
     "kernel_sources": {
         "attn": ["psa_attn_persist.cu", "psa_softmax.cuh", "psa_sched.h", "sm100.cuh"],
@@ -57,21 +57,21 @@ NCU_TRAFFIC = {
     },
     "traffic_bytes": {
         "c4": {
-            "attn": 596048384
+            "attn": 593439744
         },
         "c3": {
-            "attn": 37832704,
-            "proj": 16183808
+            "attn": 37815808,
+            "proj": 16184576
         },
         "c2": {
-            "attn": 18934528,
-            "proj": 9859840
+            "attn": 18928640,
+            "proj": 9852416
         },
         "c5-n256-full": {
-            "attn": 1046624000
+            "attn": 1046671360
         },
         "c5-n256-masked": {
-            "attn": 1048085248
+            "attn": 1048395776
         }
     }
 }

@@ -15,7 +15,7 @@
 // and write these as operand tiles in the 128-byte swizzle (X K-major, W MN-major) into a ring of four steps; warp 16
 // issues 12 MMAs of 128 x 128 x 16 per step; warps 0-15 also drain the accumulators, 32 rows by 32 columns each.
 //
-// What bounds it: 12 MMAs per step at 92 cycles (N = 128) are 1104 cycles for 32 k; splitting a step takes about 600 issue
+// What bounds it: 12 MMAs per step at 64 cycles (N = 128) are 768 cycles for 32 k; splitting a step takes about 600 issue
 // slots per scheduler beside them, and its stores share the shared-memory port with the MMAs' operands (at the 96 registers
 // that 17 warps leave, 92 bytes are spilled, most of them around the call of ft_form_again).  Measured 2300 cycles per step;
 // 2048 x 768 x 3 x 768 171 us on CUDA cores (128 x 128 tiles), 70 us here.
