@@ -57,21 +57,21 @@ NCU_TRAFFIC = {
     },
     "traffic_bytes": {
         "c4": {
-            "attn": 593439744
+            "attn": 593319168
         },
         "c3": {
-            "attn": 37815808,
-            "proj": 16184576
+            "attn": 37804544,
+            "proj": 16297728
         },
         "c2": {
-            "attn": 18928640,
-            "proj": 9852416
+            "attn": 18928896,
+            "proj": 9852672
         },
         "c5-n256-full": {
-            "attn": 1046671360
+            "attn": 1046480128
         },
         "c5-n256-masked": {
-            "attn": 1048395776
+            "attn": 1048277760
         }
     }
 }
