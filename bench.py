@@ -570,7 +570,7 @@ def main():
     sustained = total_s >= 0.5 and not prep.flush
     peak = peaks["bf16_tflops_sustained"] if sustained else peaks["bf16_tflops"]
     mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 1965.0
-    roofline = {"bound": "tensor", "kernel": ("sym_shared_kernel, and sym_attn_kernel for the heads it gives up (symmetric scheme)" if sym else "attn_persist_kernel (fused scores-softmax-weighted sum)") if dominant == "attn" else "gemm_bf16_kernel (projections)",
+    roofline = {"bound": "tensor", "kernel": ("sym_attn_kernel (symmetric scheme, all passes)" if sym else "attn_persist_kernel (fused scores-softmax-weighted sum)") if dominant == "attn" else "gemm_bf16_kernel (projections)",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None,
                 "peak_source": peaks["source"] + (" sustained bf16 (timed region of %.2f s, steps back to back)" % total_s if sustained else " burst bf16"),

@@ -64,8 +64,7 @@ typedef enum {
  * Multiply-accumulate census of one call (summed over batch and heads).
  *   proj_macs       projection MACs (paper Sec. 3.1; not part of the paper's own count)
  *   qk_macs         phase-1 MACs issued      pv_macs   phase-3 MACs issued
- *   exps            phase-2 weights of issued blocks (one exponential each; under the symmetric scheme in bf16 an exponential
- *                   may serve both members of a pair)
+ *   exps            phase-2 exponentials evaluated
  *   useful_*        the paper's element-level counts for the scheme (Sec. 3.2, 4.2, 5.2):
  *                   FULL d*n^2 each; MASKED d*n(n+1)/2 each; SYMMETRIC d*n(n+1)/2 and d*n^2
  * The bf16 path issues whole 128x128 blocks of the weight matrix, so issued >= useful there (a

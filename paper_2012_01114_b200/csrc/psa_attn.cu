@@ -1,5 +1,4 @@
-// Attention core of the bf16 path: dispatch, and the kernel of the symmetric scheme (paper Sec. 4) that takes any input.  Calls of
-// many heads go to sym_shared_kernel (psa_attn_sym.cu) first, and this one works off the heads that it gives up.
+// Attention core of the bf16 path: dispatch, and the kernel of the symmetric scheme (paper Sec. 4).
 //
 // With query = key = value = X the weight matrix before the softmax is symmetric, w'_ij = w'_ji (paper
 // Eq. 4), and the paper computes one member of each pair and reuses it.  On this machine the reuse goes
@@ -31,7 +30,6 @@
 #include "psa_internal.h"
 #include "psa_sched.h"
 #include "psa_softmax.cuh"
-#include "psa_sym.h"
 #include "psa_tma.h"
 #include "sm100.cuh"
 
@@ -68,10 +66,41 @@ struct SymBars {
     uint64_t s_full[2], s_free[2], p_ready[2], o_done[2];
 };
 
+// The scratch of a head is one 64 KB block per tile pair (I, J), J <= I, numbered I (I + 1) / 2 + J.  Diagonal blocks are
+// never handed on; the place of block (0, 0) holds the head's flags instead: flag I = blocks that tile I has handed on.  The
+// first head's place also holds, behind its T flags, the work counter of the launch.
+__device__ __forceinline__ float* sym_head(float* Sg, int hl, int np) { return Sg + (size_t)hl * np * (S_BLOCK_BYTES / 4); }
+
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(int* p, int v) { asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ int ld_acquire_cta(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_cta(int* p, int v) { asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory"); }
+
+// Bounded wait until read() >= target.
+template <class Read>
+__device__ __forceinline__ bool wait_at_least(Read read, int target, volatile int* abort_flag) {
+    if (read() >= target) return true;
+    const uint64_t t0 = globaltimer_ns();
+    while (read() < target) {
+        if (*abort_flag) return false;
+        if (globaltimer_ns() - t0 > PSA_WAIT_LIMIT_NS) { *abort_flag = 1; return false; }
+        __nanosleep(64);
+    }
+    return true;
+}
+
 template <int D>
 __global__ void __launch_bounds__(SYM_THREADS, 1)
-sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int header_heads, int first_entry, int most_heads, int from_list,
-                int launch, int n, int H, int bh0, int most_group, float sl2, DeviceCounters* dc) {
+sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ Sg, int n, int H, int bh0, int heads, int group, float sl2,
+                DeviceCounters* dc) {
     using Cfg = SymCfg<D>;
     constexpr int XST = Cfg::XST, MST = Cfg::MST;
     extern __shared__ uint8_t smem_raw[];
@@ -88,11 +117,10 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int T = row_tiles(n);
-    const SymHeader hd = sym_header(S, header_heads, T);
-    float* blocks = S + sym_header_bytes(header_heads, T) / 4;                  // one per tile pair (I, J), J < I
-    int heads = 0, group = 1, nitems = 0;                                       // set below, behind the kernel before this one
-    int* work_counter = hd.general_work + launch;
-    // item -> head of this launch and row tile: groups of heads, in a group the last tiles of all heads first
+    const int np = sym_pairs(T);
+    const int nitems = heads * T;
+    int* work_counter = reinterpret_cast<int*>(Sg) + T;
+    // item -> head inside this pass and row tile: groups of heads, in a group the last tiles of all heads first
     auto item_work = [&](int idx, int& hl, int& It) {
         const int g = idx / (group * T), first = g * group, size = min(group, heads - first);
         const int off = idx - first * T, r = off / size;
@@ -126,27 +154,13 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
     const uint32_t tmem = tmem_base_s;
     volatile int* abortp = &abort_flag;
     grid_dependency_wait();      // (programmatic dependent launch, as in attn_persist_kernel)
-    heads = from_list ? min(max(*hd.given_up - first_entry, 0), most_heads) : most_heads;
-    group = max(1, min(heads, most_group));
-    nitems = heads * T;
-    auto head_of = [&](int hl) { return bh0 + (from_list ? hd.list[first_entry + hl] : first_entry + hl); };
-    auto head_blocks = [&](int hl) { return blocks + (size_t)hl * sym_lower_blocks(T) * (S_BLOCK_BYTES / 4); };
-    // the census of the heads that sym_shared_kernel has finished (what it issued for the others counts for nothing)
-    if (from_list && first_entry == 0 && blockIdx.x == 0) {
-        unsigned long long qk = 0, pv = 0;
-        for (int i = threadIdx.x; i < header_heads; i += SYM_THREADS)
-            if (!hd.bad[i]) { qk += hd.qk_blocks[i]; pv += hd.pv_blocks[i]; }
-        const unsigned long long block_macs = (unsigned long long)TILE * TILE * D;
-        if (qk) atomicAdd(&dc->qk_macs, qk * block_macs);
-        if (pv) { atomicAdd(&dc->pv_macs, pv * block_macs); atomicAdd(&dc->exps, pv * (unsigned long long)(TILE * TILE)); }
-    }
 
     if (warp == 0) {
         if (lane == 0) {
             // ------------------------------------------------------------ work items, X tiles, handed-on score blocks
             uint32_t xc = 0, mc = 0, qc = 0;         // X tiles, half blocks and row tiles requested so far
             bool ok = true;
-            int idx = nitems > 0 ? atomicAdd(work_counter, 1) : 0;
+            int idx = atomicAdd(work_counter, 1);
             for (uint32_t it = 0; ok; ++it) {
                 const int slot = it & 1;
                 if (it >= 2) ok = mbar_wait(&bars.item_empty[slot], ((it >> 1) - 1) & 1, abortp);
@@ -156,9 +170,9 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
                 if (idx >= nitems) break;
                 int hl, It;
                 item_work(idx, hl, It);
-                const int bh = head_of(hl), b = bh / H, h = bh - b * H;
-                const float* head = head_blocks(hl);
-                const int* flags = hd.general_flags + (size_t)(first_entry + hl) * sym_flag_pitch(T);
+                const int bh = bh0 + hl, b = bh / H, h = bh - b * H;
+                float* head = sym_head(Sg, hl, np);
+                const int* flags = reinterpret_cast<const int*>(head);
                 int next = 0;
                 for (int j = 0; j < T && ok; ++j) {
                     const int s = xc % XST;
@@ -183,7 +197,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
                     ok = wait_at_least([&] { return ld_acquire(flags + j); }, It + 1, abortp);
                     if (!ok) break;
                     asm volatile("fence.proxy.async;" ::: "memory");
-                    const float* src = head + sym_block_index(j, It) * (S_BLOCK_BYTES / 4);
+                    const float* src = head + (size_t)(j * (j + 1) / 2 + It) * (S_BLOCK_BYTES / 4);
                     for (int half = 0; half < 2 && ok; ++half) {
                         const int ms = mc % MST;
                         if (mc >= (uint32_t)MST) ok = mbar_wait(&bars.m_empty[ms], ((mc / MST) - 1) & 1, abortp);
@@ -290,7 +304,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
             if (idx < 0) break;
             int hl, It;
                 item_work(idx, hl, It);
-            int* flag = hd.general_flags + (size_t)(first_entry + hl) * sym_flag_pitch(T) + It;
+            int* flag = reinterpret_cast<int*>(sym_head(Sg, hl, np)) + It;
             int sent = 0;
             bool ok = true;
             while (sent < It) {
@@ -355,7 +369,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
             if (idx < 0) break;
             int hl, It;
                 item_work(idx, hl, It);
-            float* own = head_blocks(hl) + (It ? sym_block_index(It, 0) : 0) * (S_BLOCK_BYTES / 4) + kw * 2048;
+            float* own = sym_head(Sg, hl, np) + (size_t)(It * (It + 1) / 2) * (S_BLOCK_BYTES / 4) + kw * 2048;
             float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;       // running maxima (log2 units) and row sums
             for (int j = 0; j < T; ++j, ++blk) {
                 uint32_t s0[32], s1[32];
@@ -471,7 +485,7 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
             // ---- epilogue: y = O / l (the division of Eq. 2, applied once per output row), bf16, 64 columns at a time.  (The
             // next write to O, PV_0 of the next item, waits for that item's first P from every warp.)
             tc_fence_after();
-            const int bh = head_of(hl), b = bh / H, h = bh - b * H;
+            const int bh = bh0 + hl, b = bh / H, h = bh - b * H;
             const float invA = 1.f / quad_sum(lA), invB = 1.f / quad_sum(lB);
 #pragma unroll
             for (int u = 0; u < Cfg::SUB; ++u) {
@@ -508,6 +522,15 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
+// The flags of `heads` heads and the work counter of a launch (the diagonal block whose place they take has room for 16384),
+// cleared together with `before` bytes ahead of each of these places: for the first head, what lies ahead of the scratch;
+// for the others the end of a diagonal block, which nothing uses.
+cudaError_t sym_clear(float* S, int heads, int T, size_t before, cudaStream_t stream) {
+    char* p = reinterpret_cast<char*>(S) - before;
+    const size_t bytes = before + (size_t)(T + 1) * sizeof(int);
+    return heads == 1 ? cudaMemsetAsync(p, 0, bytes, stream) : cudaMemset2DAsync(p, (size_t)sym_pairs(T) * S_BLOCK_BYTES, 0, bytes, heads, stream);
+}
+
 // Heads per group of the item list: the tiles of one head are started a group apart.  A tile needs its first handed-on block
 // one step after its neighbour has computed it, so tiles that start together wait for one another; started 256 / T items
 // apart (two steps, on 148 CTAs) they do not, and a head's scratch still lives briefly enough to stay in L2.  Measured for
@@ -516,9 +539,10 @@ sym_attn_kernel(const __grid_constant__ SymMaps maps, float* __restrict__ S, int
 constexpr int SYM_GROUP_ITEMS = 256;
 
 // D: head size the kernel works with (64 or 128); d <= D: the tensors' head size (see the 4-D tensor maps).
+// s_bytes: size of the score scratch, which sets the heads per pass; s_clear: the first pass finds its flags clear.
 template <int D>
-int launch_general(const void* X, void* out, float* S, int header_heads, int first, int heads, bool from_list, int launch, int bh0, int B, int H, int n,
-                   int d, float scale, DeviceCounters* dc, cudaStream_t stream) {
+int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, bool s_clear, int B, int H, int n, int d, float scale, DeviceCounters* dc,
+                     cudaStream_t stream) {
     using Cfg = SymCfg<D>;
     static DeviceSetup setup;
     const int sm_count = device_setup(&setup, [] {
@@ -526,43 +550,28 @@ int launch_general(const void* X, void* out, float* S, int header_heads, int fir
     }, "cudaFuncSetAttribute(symmetric attention)");
     if (sm_count <= 0) return PSA_ERR_CUDA;
     const int T = row_tiles(n);
+    const int hp = sym_heads_per_pass((size_t)B * H, n, s_bytes);
     SymMaps maps;
     if (!make_tensor_map_bf16_4d(&maps.x, X, B, n, H, d, 128) || !make_tensor_map_bf16_4d(&maps.o, out, B, n, H, d, 16))
         return PSA_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(min(heads * T, sm_count));
-    cfg.blockDim = dim3(SYM_THREADS);
-    cfg.dynamicSmemBytes = Cfg::SMEM;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, sym_attn_kernel<D>, maps, S, header_heads, first, heads, from_list ? 1 : 0, launch, n, H, bh0,
-                                             max(1, SYM_GROUP_ITEMS / T), scale * LOG2E, dc);
-    if (e != cudaSuccess) { set_cuda_error(e, "sym_attn_kernel launch"); return PSA_ERR_CUDA; }
-    return PSA_OK;
-}
-
-// s_bytes: size of the score scratch, which sets the heads per pass; s_clear: the first header is clear.
-int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, bool s_clear, int B, int H, int n, int d, float scale, DeviceCounters* dc,
-                     cudaStream_t stream) {
-    const int T = row_tiles(n), all = B * H, per_header = sym_heads_per_header(all, n, s_bytes), hp = sym_heads_per_pass(all, n, s_bytes);
-    if ((long long)per_header * T > 0x7fffffffLL - 2 * 1024) return PSA_ERR_SHAPE;      // (the work counters run past the list)
-    static DeviceSetup setup;
-    const int sms = device_setup(&setup, [] { return cudaSuccess; }, "symmetric attention set-up");
-    if (sms <= 0) return PSA_ERR_CUDA;
-    for (int bh0 = 0; bh0 < all; bh0 += per_header) {
-        const int heads = min(per_header, all - bh0);
-        const cudaError_t e = bh0 == 0 && s_clear ? cudaSuccess : cudaMemsetAsync(S, 0, sym_header_bytes(heads, T), stream);
+    for (int bh0 = 0; bh0 < B * H; bh0 += hp) {
+        const int heads = min(hp, B * H - bh0);
+        if ((long long)heads * T > 0x7fffffffLL - 2 * sm_count) return PSA_ERR_SHAPE;      // (the work counter runs past the list)
+        const int nitems = heads * T;
+        cudaError_t e = bh0 == 0 && s_clear ? cudaSuccess : sym_clear(S, heads, T, 0, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "symmetric scheme: clearing the flags"); return PSA_ERR_CUDA; }
-        const bool shared = sym_shared_pays(heads, T, s_bytes, sms);
-        int rc = PSA_OK;
-        if (shared) rc = launch_sym_shared(X, out, S, s_bytes, heads, bh0, B, H, n, d, scale, dc, stream);
-        for (int first = 0, launch = 0; first < heads && rc == PSA_OK; first += hp, ++launch)
-            rc = launch_sym_general(X, out, S, heads, first, min(hp, heads - first), shared, launch, bh0, B, H, n, d, scale, dc, stream);
-        if (rc != PSA_OK) return rc;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(min(nitems, sm_count));
+        cfg.blockDim = dim3(SYM_THREADS);
+        cfg.dynamicSmemBytes = Cfg::SMEM;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel waits for its predecessor itself
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, sym_attn_kernel<D>, maps, S, n, H, bh0, heads, min(heads, max(1, SYM_GROUP_ITEMS / T)), scale * LOG2E, dc);
+        if (e != cudaSuccess) { set_cuda_error(e, "sym_attn_kernel launch"); return PSA_ERR_CUDA; }
     }
     return PSA_OK;
 }
@@ -573,18 +582,8 @@ size_t bf16_symmetric_scratch_bytes(int B, int H, int n) {
     return (size_t)sym_heads_per_pass((size_t)B * H, n, SYM_SCRATCH_CAP) * sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
 }
 
-// At least 16 KB are cleared (the scratch has 64 KB or more): a clear of a few KB takes 1.3 us less by itself, but the kernel behind it
-// then starts later.  Calls back to back, header alone / 16 KB, us: 4 heads of n = 420, d = 32 18.4 / 16.5; 2 of n = 1024, d = 64
-// 24.6 / 22.8; 2 of n = 256, d = 32 14.4 / 12.4 (a lone call waited for takes 1 us more: 27.1 / 28.4 at 2 heads of n = 420).
 cudaError_t bf16_symmetric_clear(float* S, size_t s_bytes, int B, int H, int n, size_t before, cudaStream_t stream) {
-    const size_t bytes = before + sym_header_bytes(sym_heads_per_header((size_t)B * H, n, s_bytes), row_tiles(n));
-    return cudaMemsetAsync(reinterpret_cast<char*>(S) - before, 0, s_bytes >= 16384 && bytes < 16384 ? 16384 : bytes, stream);
-}
-
-int launch_sym_general(const void* X, void* out, float* S, int header_heads, int first, int heads, bool from_list, int launch, int bh0, int B, int H,
-                       int n, int d, float scale, DeviceCounters* dc, cudaStream_t stream) {
-    if (d <= 64) return launch_general<64>(X, out, S, header_heads, first, heads, from_list, launch, bh0, B, H, n, d, scale, dc, stream);
-    return launch_general<128>(X, out, S, header_heads, first, heads, from_list, launch, bh0, B, H, n, d, scale, dc, stream);
+    return sym_clear(S, sym_heads_per_pass((size_t)B * H, n, s_bytes), row_tiles(n), before, stream);
 }
 
 int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, bool s_clear, int B, int H,
@@ -595,7 +594,8 @@ int bf16_attention(const void* Q, const void* K, const void* V, void* out, float
     if (!S || s_bytes < (size_t)sym_pairs(row_tiles(n)) * S_BLOCK_BYTES) return PSA_ERR_WORKSPACE;       // (one head)
     if ((reinterpret_cast<uintptr_t>(S) & 15u) != 0) return PSA_ERR_ALIGN;
     if (d < 8 || d > 128 || d % 8) return PSA_ERR_UNSUPPORTED;
-    return launch_symmetric(Q, out, S, s_bytes, s_clear, B, H, n, d, scale, dc, stream);
+    if (d <= 64) return launch_symmetric<64>(Q, out, S, s_bytes, s_clear, B, H, n, d, scale, dc, stream);
+    return launch_symmetric<128>(Q, out, S, s_bytes, s_clear, B, H, n, d, scale, dc, stream);
 }
 
 }  // namespace psa

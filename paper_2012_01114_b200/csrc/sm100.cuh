@@ -238,12 +238,6 @@ __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.b
 // ... all but the most recent group
 __device__ __forceinline__ void tma_store_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 
-// 32 bytes to global memory (32-byte aligned): a whole sector per thread.
-__device__ __forceinline__ void st_global_32(void* p, const uint32_t* v) {
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
-                 "r"(v[6]), "r"(v[7]) : "memory");
-}
-
 // ---------------------------------------------------------------- TMEM
 // Warp-collective.  ncols: power of two in [32, 512].  The base address lands in *smem_dst.
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
