@@ -91,7 +91,7 @@ int psa_attention(const void* X, const void* Wq, const void* Wk, const void* Wv,
 /* Same computation in fp32 storage, to fp32 accuracy.  Small calls run in fp32 arithmetic on CUDA cores; large ones (projections; the
  * full and masked schemes with d_k a multiple of 8) on the tensor cores, every number split into three bf16 parts, with an error
  * below that of a chain of fp32 additions (projections too small for that, or not finite, and heads with numbers beyond 2^50, not
- * finite or, in V, below 2^-60, are worked off on CUDA cores).  Skipping is element-exact either way (issued = useful): the
+ * finite or, in V, beyond 2^46 or below 2^-60, are worked off on CUDA cores).  Skipping is element-exact either way (issued = useful): the
  * diagonal tiles of the masked scheme stay on CUDA cores.  Supported: n <= 1024, d_k <= 128 (any d_model). */
 int psa_attention_f32(const void* X, const void* Wq, const void* Wk, const void* Wv, int batch, int heads, int n,
                       int d_model, int d_k, int scheme, void* out, void* stream);

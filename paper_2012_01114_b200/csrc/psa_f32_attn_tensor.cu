@@ -13,9 +13,10 @@
 // tile (128 x 128, on the diagonal) are computed one by one by f32_diagonal_kernel (psa_f32.cu) ahead of this kernel, which
 // continues from their maximum, sum and partial output.
 //
-// What the parts cannot carry: f32_split_kernel marks heads with an operand that is not finite or beyond 2^50, or a nonzero value
-// (V) below 2^-60; these are left to f32_flash_kernel altogether.  Weights are scaled by 2^64, so that every one that fp32
-// can hold has parts in the normal range.
+// What the parts cannot carry: f32_split_kernel marks heads with an operand that is not finite, a number of Q or K beyond 2^50, a
+// value (V) beyond 2^46 or a nonzero one below 2^-60; these are left to f32_flash_kernel altogether.  Weights are scaled by 2^64, so that
+// every one that fp32 can hold has parts in the normal range.  With a maximum that may lag by FM_RAISE a weight is at most 2^64 e^4, and
+// 1024 of them times 2^46 are below 2^126: the running output stays finite.  (Scores of 128 products of 2^100 are below 2^108.)
 //
 // What bounds it: per block of 64 keys 72 MMAs, 3072 cycles at d = 128 and 1536 at d = 64, beside about 1500 issue slots per scheduler of
 // softmax and splitting; the masked scheme also its longest row tiles and the diagonal tiles ahead of them (30 of its 76 us at 16
@@ -39,6 +40,8 @@ constexpr int FM_WARPS = 8, FM_THREADS = 32 * (2 + FM_WARPS);
 constexpr int FM_TMEM_Q = 0, FM_TMEM_S = 192, FM_TMEM_P = 256, FM_TMEM_O = 384;
 constexpr float FM_UP = 1.8446744e19f;                   // 2^64
 constexpr float FM_RAISE = 4.f;                          // the running maximum follows when a row's grew by more (natural units)
+// Bits of 2^50, 2^46 and 2^-60: what the parts can carry, see above.
+constexpr uint32_t FM_MOST = (127u + 50u) << 23, FM_VALUE_MOST = (127u + 46u) << 23, FM_VALUE_LEAST = (127u - 60u) << 23;
 
 template <int D>
 struct FMCfg {
@@ -76,7 +79,7 @@ f32_split_kernel(const float4* __restrict__ Q, const float4* __restrict__ K, con
                                   max(__float_as_uint(x.z) & 0x7fffffffu, __float_as_uint(x.w) & 0x7fffffffu));
         // (twice the bits less one: zero becomes the largest)
         const uint32_t least = min(min(2u * __float_as_uint(x.x) - 1u, 2u * __float_as_uint(x.y) - 1u), min(2u * __float_as_uint(x.z) - 1u, 2u * __float_as_uint(x.w) - 1u));
-        if (most > (177u << 23) || (which == 1 && least < 2u * (67u << 23) - 1u)) {      // 2^50, 2^-60
+        if (most > (which == 1 ? FM_VALUE_MOST : FM_MOST) || (which == 1 && least < 2u * FM_VALUE_LEAST - 1u)) {
             const uint32_t row = i / (uint32_t)(d >> 2);
             bad[(row / ((uint32_t)n * H)) * H + row % (uint32_t)H] = 1;
         }

@@ -64,6 +64,23 @@ def test_heads_with_numbers_without_parts(scheme):
     _close(got[:, :, 3][:, :, :5], ref[:, :, 3][:, :, :5])
 
 
+# Values up to and beyond the largest that the parts carry (2^46), all of one sign, under weights of up to e^3.9 relative to the running maximum, which
+# follows only a growth by more than 4: FULL through its first 64 keys, MASKED through the diagonal tile of the last 128 rows.  The
+# running sum of 832 such values was infinite from 2^48.6 on.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("power", [45, 46, 47, 49, 50, 60])
+def test_large_values_under_a_lagging_maximum(scheme, power):
+    B, H, n, d = 1, 16, 1024, 64
+
+    def set_up(t):
+        t[0][:], t[1][:] = 0.0, 0.0
+        t[0][..., 0] = 8.0                       # 1 / sqrt(d) = 1/8: a key's score is its first number
+        t[1][:, 64:n - 128, :, 0] = 3.9
+        t[2][:] = np.float32(2.0 ** power) * (1.0 - 0.5 * np.abs(t[2]) / np.abs(t[2]).max())
+    got, ref = _run(B, H, n, d, scheme, set_up)
+    _close(got / 2.0 ** power, ref / 2.0 ** power)
+
+
 # Projections of the largest calls (pairs of CTAs, 256 x 256 tiles, 64 k at a time): ragged rows, columns and depth, tiny and
 # infinite operands.  With one vector per sequence the attention returns V.  Bound: six bf16 products per fp32 product leave 2^-24 of it
 # out, sums are rounded every 64 k: (K / 64 + 4) 2^-24 of the sum of magnitudes.
