@@ -11,6 +11,7 @@
 
 #include "psa_internal.h"
 #include "psa_sched.h"
+#include "psa_ws.h"
 
 namespace psa {
 
@@ -56,13 +57,11 @@ struct HostPipe {
     cudaEvent_t start = nullptr, loaded[HOST_CHUNKS] = {}, computed[HOST_CHUNKS] = {}, stored = nullptr;
 };
 
-constexpr size_t COUNTER_BYTES = 256;          // counter blocks and cursors at the start of the workspace
 constexpr size_t COUNTER_BLOCK_BYTES = 64;
 constexpr int TURN_BLOCKS = 2, CAPTURE_BLOCK = 2;      // blocks used in turn; block of captured calls
 constexpr size_t CURSOR_OFFSET = 3 * COUNTER_BLOCK_BYTES;   // work counters of a call in several parts
 static_assert(sizeof(DeviceCounters) <= COUNTER_BLOCK_BYTES, "counter block too small");
 static_assert(CURSOR_OFFSET + HOST_CHUNKS * sizeof(unsigned int) <= COUNTER_BYTES, "no room for the cursors");
-size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -83,54 +82,9 @@ int check_shape(int batch, int heads, int n, int d_model, int d_k, int scheme, i
     return PSA_OK;
 }
 
-struct WsLayout {
-    size_t q, k, v, s, s_bytes, clear, clear_bytes, bad, marks_in, marks_out, ml, parts, xs, wq, wk, wv, outs, total;
-    bool attn_tensor, proj_pairs;      // fp32: whether bad / ml / parts and marks_* / parts are there
-};
-
-WsLayout ws_layout(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, bool with_proj,
-                   bool staging) {
-    const size_t es = dtype == PSA_BF16 ? 2 : 4;
-    const size_t qkv = align_up((size_t)batch * n * heads * d_k * es, 256);
-    WsLayout L;
-    memset(&L, 0, sizeof(L));
-    size_t off = COUNTER_BYTES;
-    if (dtype == PSA_F32) {      // marks right behind the counters: one clear serves both, see run_layer
-        const bool one_launch = with_proj && f32_fused_fits(n, d_model, d_k, scheme);       // (needs none of this, but for an output projection)
-        const size_t bh = (size_t)batch * heads, in = with_proj && !one_launch ? f32_project_parts_bytes(batch * n, d_model, heads * d_k, scheme == PSA_SYMMETRIC ? 1 : 3) : 0,
-                     outp = with_proj ? f32_project_parts_bytes(batch * n, heads * d_k, d_model, 1) : 0;
-        L.attn_tensor = !one_launch && f32_tensor_attention_fits(batch, heads, n, d_k, scheme);
-        L.proj_pairs = in || outp;
-        L.clear = off;
-        if (L.attn_tensor) { L.bad = off; off += align_up(bh * sizeof(int), 256); }
-        if (in) { L.marks_in = off; off += align_up(f32_project_marks(batch * n, heads * d_k, 3) * sizeof(int), 256); }
-        if (outp) { L.marks_out = off; off += align_up(f32_project_marks(batch * n, d_model, 1) * sizeof(int), 256); }
-        L.clear_bytes = one_launch ? 0 : off - L.clear;
-        if (L.attn_tensor) { L.ml = off; off += align_up(2 * bh * n * sizeof(float), 256); }
-        L.parts = off;           // (used by one kernel after another)
-        off += align_up(std::max(std::max(in, outp), L.attn_tensor ? 12 * bh * n * d_k : (size_t)0), 256);
-    }
-    if (scheme == PSA_SYMMETRIC) {       // (bf16: right behind the counters, as above)
-        L.s_bytes = dtype == PSA_BF16 ? bf16_symmetric_scratch_bytes(batch, heads, n)
-                                      : align_up((size_t)batch * heads * n * n * sizeof(float), 256);
-        L.s = off; off += L.s_bytes;
-    }
-    if (with_proj) {
-        L.q = off; off += qkv;
-        if (scheme == PSA_SYMMETRIC) { L.k = L.q; L.v = L.q; }
-        else { L.k = off; off += qkv; L.v = off; off += qkv; }
-    }
-    if (staging) {
-        const size_t xb = align_up((size_t)batch * n * d_model * es, 256);
-        const size_t wb = align_up((size_t)d_model * heads * d_k * es, 256);
-        L.xs = off; off += xb;
-        L.wq = off; off += wb;
-        if (scheme == PSA_SYMMETRIC) { L.wk = L.wq; L.wv = L.wq; }
-        else { L.wk = off; off += wb; L.wv = off; off += wb; }
-        L.outs = off; off += qkv;
-    }
-    L.total = off;
-    return L;
+WsLayout call_layout(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, bool with_proj, bool staging) {
+    return ws_layout(WsShape{batch, heads, n, d_model, d_k, scheme, dtype, with_proj, staging,
+                             with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme)});
 }
 
 F32Scratch f32_scratch(char* ws, const WsLayout& L, size_t first_head) {
@@ -278,9 +232,9 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     if (pev) cudaEventRecord(pev[0], stream);
     void* const qkv[3] = {ws + L.q, ws + L.k, ws + L.v};
     const F32Scratch fs = f32_scratch(ws, L, 0);
-    const F32ProjectScratch ps = {ws + L.parts, reinterpret_cast<int*>(ws + L.marks_in)};
+    const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in)};
     const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
-                                 qkv, S, L.s_bytes, s_clear, L.attn_tensor ? &fs : nullptr, L.proj_pairs ? &ps : nullptr, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
+                                 qkv, S, L.s_bytes, s_clear, L.attn_tensor ? &fs : nullptr, L.in_bytes ? &ps : nullptr, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
     if (rc == PSA_OK && turns && !captured) {        // the other block will be clear once this call has run
         cx.clean_ws = ws;
         cx.next_block = block ^ 1;
@@ -305,7 +259,7 @@ int layer_entry(const void* X, const void* Wq, const void* Wk, const void* Wv, i
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = ws_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
+    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
     char* ws = acquire_ws(cx, L.total);
     if (!ws) return PSA_ERR_WORKSPACE;
     return run_layer(cx, X, Wq, Wk, Wv, nullptr, nullptr, nullptr, batch, heads, n, d_model, d_k, scheme, dtype, out,
@@ -368,7 +322,7 @@ int psa_attention_core(const void* Q, const void* K, const void* V, int batch, i
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = ws_layout(batch, heads, n, 0, d_k, scheme, dtype, false, false);
+    const WsLayout L = call_layout(batch, heads, n, 0, d_k, scheme, dtype, false, false);
     char* ws = acquire_ws(cx, L.total);
     if (!ws) return PSA_ERR_WORKSPACE;
     return run_layer(cx, nullptr, nullptr, nullptr, nullptr, Q, K, V, batch, heads, n, 0, d_k, scheme, dtype, out,
@@ -393,7 +347,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = ws_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, true);
+    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, true);
     char* ws = acquire_ws(cx, L.total);
     if (!ws) return PSA_ERR_WORKSPACE;
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
@@ -456,11 +410,11 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         e = cudaStreamWaitEvent(stream, pipe->loaded[c], 0);
         if (e != cudaSuccess) break;
         void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
-        const F32ProjectScratch ps = {ws + L.parts, reinterpret_cast<int*>(ws + L.marks_in)};
+        const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in)};
         const F32Scratch fs = f32_scratch(ws, L, b0 * heads);       // (a part has marks of its own; the rest is used by one after another)
         rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
                            d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,
-                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, L.attn_tensor ? &fs : nullptr, L.proj_pairs ? &ps : nullptr, dc,
+                           sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, L.attn_tensor ? &fs : nullptr, L.in_bytes ? &ps : nullptr, dc,
                            reinterpret_cast<unsigned int*>(ws + CURSOR_OFFSET) + c, nullptr, nullptr);
         if (rc != PSA_OK) break;
         e = cudaEventRecord(pipe->computed[c], stream);
@@ -503,7 +457,7 @@ int psa_attention_core_host(const void* Q_host, const void* K_host, const void* 
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = ws_layout(batch, heads, n, 0, d_k, scheme, dtype, false, false);
+    const WsLayout L = call_layout(batch, heads, n, 0, d_k, scheme, dtype, false, false);
     const size_t tb = (size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4), tba = align_up(tb, 256);
     const size_t q_off = align_up(L.total, 256), k_off = q_off + tba, v_off = k_off + tba;
     const size_t o_off = sym ? k_off : v_off + tba;          // the symmetric scheme stages one input tensor
@@ -553,7 +507,7 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = ws_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
+    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
     const size_t y_off = align_up(L.total, 256);
     const size_t y_bytes = (size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4);
     char* ws = acquire_ws(cx, y_off + align_up(y_bytes, 256));
@@ -566,12 +520,12 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
     const void* Ws[3] = {Wo, Wo, Wo};
     void* outs[3] = {out, out, out};
     if (dtype == PSA_F32) {
-        const F32ProjectScratch ps = {ws + L.parts, reinterpret_cast<int*>(ws + L.marks_out)};
+        const F32ProjectScratch ps = {ws + L.parts, L.out_bytes, reinterpret_cast<int*>(ws + L.marks_out)};
         cudaError_t e = cudaSuccess;
-        if (L.marks_out && !L.clear_bytes) e = cudaMemsetAsync(ps.marks, 0, f32_project_marks(batch * n, d_model, 1) * sizeof(int), stream);
+        if (L.out_bytes && !L.clear_bytes) e = cudaMemsetAsync(ps.marks, 0, f32_project_marks(batch * n, d_model, 1) * sizeof(int), stream);
         if (e == cudaSuccess) e = f32_project(static_cast<const float*>(y), reinterpret_cast<const float* const*>(Ws),
                                     reinterpret_cast<float* const*>(outs), 1, batch * n, heads * d_k, d_model,
-                                    static_cast<const float*>(R), L.proj_pairs ? &ps : nullptr, cx.last_dc, stream);
+                                    static_cast<const float*>(R), L.out_bytes ? &ps : nullptr, cx.last_dc, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "f32_project(Wo)"); return PSA_ERR_CUDA; }
         return PSA_OK;
     }
@@ -580,7 +534,7 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
 
 size_t psa_block_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype) {
     if (d_model <= 0 || check_shape(batch, heads, n, d_model, d_k, scheme, dtype, true) != PSA_OK) return 0;
-    const WsLayout L = ws_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
+    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
     return align_up(L.total, 256) + align_up((size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4), 256);
 }
 
@@ -726,7 +680,7 @@ size_t psa_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, in
                            int with_host_staging) {
     const bool with_proj = d_model > 0;
     if (check_shape(batch, heads, n, d_model, d_k, scheme, dtype, with_proj) != PSA_OK) return 0;
-    return ws_layout(batch, heads, n, d_model, d_k, scheme, dtype, with_proj, with_host_staging != 0 && with_proj).total;
+    return call_layout(batch, heads, n, d_model, d_k, scheme, dtype, with_proj, with_host_staging != 0 && with_proj).total;
 }
 
 int psa_set_workspace(void* dev_ptr, size_t bytes) {

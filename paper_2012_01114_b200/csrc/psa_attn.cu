@@ -578,10 +578,6 @@ int launch_symmetric(const void* X, void* out, float* S, size_t s_bytes, bool s_
 
 }  // namespace
 
-size_t bf16_symmetric_scratch_bytes(int B, int H, int n) {
-    return (size_t)sym_heads_per_pass((size_t)B * H, n, SYM_SCRATCH_CAP) * sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
-}
-
 cudaError_t bf16_symmetric_clear(float* S, size_t s_bytes, int B, int H, int n, size_t before, cudaStream_t stream) {
     return sym_clear(S, sym_heads_per_pass((size_t)B * H, n, s_bytes), row_tiles(n), before, stream);
 }

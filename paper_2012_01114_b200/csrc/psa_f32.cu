@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "psa_internal.h"
+#include "psa_ws.h"
 #include "sm100.cuh"
 
 namespace psa {
@@ -1299,7 +1300,7 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
         // 600 x 320 x 3 x 320 (570) 27.3 / 21.3, 64 x 2048 x 3 x 2048 (384) 89 / 72; larger ones, against 128 x 128 tiles on CUDA
         // cores, 2048 x 768 x 3 x 768 171 / 70.
         const long long tiles = (long long)((rows + 31) / 32) * ((N + 31) / 32) * nW;
-        if (ps && f32_project_parts_bytes(rows, D, N, nW) && f32_project_pairs_pay(rows, D, N, nW, sms))
+        if (ps && f32_project_pairs_fit(rows, D, N, nW, ps->bytes) && f32_project_pairs_pay(rows, D, N, nW, sms))
             return f32_project_pairs(X, W, out, nW, rows, D, N, residual, ps->parts, ps->marks, dc, stream);
         if (tiles > 2 * sms) return f32_project_tensor(X, W, out, nW, rows, D, N, residual, dc, stream);
         const dim3 grid((N + GP_BN - 1) / GP_BN, (rows + GP_BM - 1) / GP_BM, nW);
@@ -1474,18 +1475,6 @@ bool short_heads(long long heads, int n, int d, int scheme, int sms) {
     return n <= (heads <= 7 * sms ? 28 : heads <= 11 * sms ? 24 : masked ? 20 : 16);
 }
 }  // namespace
-
-// Whether a call is better off on the tensor cores: three launches instead of one, and under the masked scheme a fourth for the diagonal
-// tiles, which takes 20 to 30 us however few they are.  Measured (us, CUDA cores / tensor cores): FULL 16 heads of n = 129, d = 64 17 / 19, of n =
-// 160, d = 16 15.4 / 16.8, of n = 192, d = 64 17.4 / 17.4, of n = 1024, d = 128 308 / 54; 48 of n = 512, d = 64 111 / 42.  MASKED 64 heads of n = 256, d = 64
-// 35.9 / 36.4; 16 of n = 384, d = 128 48 / 52, of n = 512, d = 16 31.8 / 34.1, of n = 1024, d = 128 166 / 76; 8 of n = 512, d = 64 36 / 40; 4 of n = 640, d =
-// 64 38 / 42; 48 of n = 512, d = 64 93 / 52.
-bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme) {
-    const long long T = (n + 127) / 128, blocks = (long long)B * H * T * T;
-    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || (long long)B * H * n * d >= (1LL << 31)) return false;
-    if (scheme == PSA_MASKED) return n > 256 && blocks >= (d >= 64 ? 256 : 320);
-    return n >= 160 && (n >= 256 || d >= 64) && blocks >= 64;
-}
 
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, const F32Scratch* fs, int B, int H,
                           int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {

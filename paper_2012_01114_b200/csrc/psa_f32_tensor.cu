@@ -643,11 +643,6 @@ cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* c
     return cudaGetLastError();
 }
 
-size_t f32_project_parts_bytes(int rows, int D, int N, int nW) {
-    const size_t tiles = (size_t)((rows + 255) / 256) * ((N + 255) / 256) * nW;
-    if (D % 8 || N % 8 || tiles < 24 || (size_t)rows * D >= (size_t)1 << 33 || (size_t)D * N >= (size_t)1 << 33) return 0;
-    return ((size_t)rows * D * 6 + 255) / 256 * 256 + ((size_t)D * N * 6 + 255) / 256 * 256 * nW;
-}
 // Whether the pairs are faster, in cycles as measured: the split and 5000 per 64 k of a 256 x 256 tile against 2300 per 32 k of a 128 x 128
 // tile of the kernel above (us, layers of 12 heads with d_model = 768: 1024 rows 65 / 58 on the tiles, 2048 rows 88 / 107).
 bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms) {
@@ -655,7 +650,6 @@ bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms) {
     const long long units = sms / 2 > 0 ? sms / 2 : 1;
     return 16000 + (pairs + units - 1) / units * ((D + 63) / 64) * 5000 < 4000 + (tiles + sms - 1) / sms * ((D + 31) / 32) * 2300;
 }
-size_t f32_project_marks(int rows, int N, int nW) { return (rows + 127) / 128 + (size_t)((N + 255) / 256) * nW; }
 
 cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N, const float* residual,
                               void* parts, int* marks, DeviceCounters* dc, cudaStream_t stream) {

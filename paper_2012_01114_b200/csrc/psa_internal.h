@@ -24,9 +24,10 @@ struct DeviceCounters {
 // ---- fp32 CUDA-core path (psa_f32.cu) ----
 // out[w][r, c] = sum_k X[r, k] W[w][k, c] for w < nW.
 // `residual` ([rows, N], may be null) is added to every output.
-// `ps` (may be null): scratch for the largest calls, see f32_project_pairs.
+// `ps` (may be null): scratch for the largest calls, see f32_project_pairs; `bytes`: room for the parts.
 struct F32ProjectScratch {
     void* parts;
+    size_t bytes;
     int* marks;
 };
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
@@ -34,10 +35,8 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
 // The same on the tensor cores, to the same accuracy (psa_f32_tensor.cu); f32_project chooses.  Rows of 16 bytes, as there.
 cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
                                const float* residual, DeviceCounters* dc, cudaStream_t stream);
-// The same for the largest calls, operands split once into `parts` (f32_project_parts_bytes; 0: the call is not one of them, whatever the
-// device), on pairs of CTAs.  marks: f32_project_marks ints, clear when the call's kernels start.
-size_t f32_project_parts_bytes(int rows, int D, int N, int nW);
-size_t f32_project_marks(int rows, int N, int nW);
+// The same for the largest calls, operands split once into `parts` (f32_project_parts_bytes, psa_ws.h), on pairs of CTAs.  marks:
+// f32_project_marks ints, clear when the call's kernels start.
 bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms);
 cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N, const float* residual,
                               void* parts, int* marks, DeviceCounters* dc, cudaStream_t stream);
@@ -48,9 +47,7 @@ struct F32Scratch {
     float* ml;
     void* parts;
 };
-// Whether attention of this shape runs on the tensor cores, given that scratch and rows of 16 bytes (psa_f32_attn_tensor.cu).
-bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme);
-// Its two kernels.
+// The two kernels of attention on the tensor cores (psa_f32_attn_tensor.cu), for shapes that f32_tensor_attention_fits (psa_ws.h) and rows of 16 bytes.
 cudaError_t f32_attention_split(const float* Q, const float* K, const float* V, const F32Scratch& fs, int B, int H, int n, int d, cudaStream_t stream);
 cudaError_t f32_attention_tensor(const float* Q, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale, int masked, DeviceCounters* dc,
                                  cudaStream_t stream);
@@ -70,7 +67,7 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
 // Returns a psa_status.
 int bf16_project(const void* A, const void* const Bw[3], void* const C[3], int nW, int M, int K, int N,
                  const void* residual, DeviceCounters* dc, cudaStream_t stream);
-// Q, K, V, out: [B, n, H, d] bf16.  S: scratch for PSA_SYMMETRIC (bf16_symmetric_scratch_bytes:
+// Q, K, V, out: [B, n, H, d] bf16.  S: scratch for PSA_SYMMETRIC (sym_scratch_bytes:
 // one 64 KB fp32 image per score block at or below the block diagonal, for the heads of one pass; with less, down to
 // one head's worth, the call runs in more passes).
 // `dc_next`, if not null, is a second counter block that the call's attention kernel clears (FULL, MASKED only).
@@ -79,7 +76,6 @@ int bf16_project(const void* A, const void* const Bw[3], void* const C[3], int n
 int bf16_attention(const void* Q, const void* K, const void* V, void* out, float* S, size_t s_bytes, bool s_clear, int B,
                    int H, int n, int d, float scale, int scheme, DeviceCounters* dc, unsigned int* cursor,
                    DeviceCounters* dc_next, cudaStream_t stream);
-size_t bf16_symmetric_scratch_bytes(int B, int H, int n);
 // Clears what the first pass of the symmetric kernel needs clear in its scratch, and `before` bytes ahead of the scratch.
 cudaError_t bf16_symmetric_clear(float* S, size_t s_bytes, int B, int H, int n, size_t before, cudaStream_t stream);
 // PSA_FULL and PSA_MASKED for 128 < d <= 256 (psa_attn_wide.cu).

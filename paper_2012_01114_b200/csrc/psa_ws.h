@@ -1,0 +1,102 @@
+// What lies where in the workspace of a call.  Host only, without CUDA, so that the layout can be checked on its own.
+#pragma once
+#include <stddef.h>
+#include <string.h>
+
+#include <algorithm>
+
+#include "psa_sched.h"
+
+namespace psa {
+
+constexpr size_t COUNTER_BYTES = 256;          // counter blocks and cursors at the start of the workspace
+
+inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// ---- which fp32 calls have scratch for the tensor cores
+// Projection of [rows, D] by nW matrices [D, N], f32_project_pairs: bytes of bf16 parts of the operands (0: the call is not one of the
+// largest ones, whatever the device), and number of marks.
+inline size_t f32_project_parts_bytes(int rows, int D, int N, int nW) {
+    const size_t tiles = (size_t)((rows + 255) / 256) * ((N + 255) / 256) * nW;
+    if (D % 8 || N % 8 || tiles < 24 || (size_t)rows * D >= (size_t)1 << 33 || (size_t)D * N >= (size_t)1 << 33) return 0;
+    return align_up((size_t)rows * D * 6, 256) + align_up((size_t)D * N * 6, 256) * nW;
+}
+inline size_t f32_project_marks(int rows, int N, int nW) { return (rows + 127) / 128 + (size_t)((N + 255) / 256) * nW; }
+// Whether a projection may run there with `bytes` of room for its parts.  (A part of a call may ask for more than the call as a
+// whole has: one with 2^33 numbers in X has no room for parts at all, a batch item of it would.)
+inline bool f32_project_pairs_fit(int rows, int D, int N, int nW, size_t bytes) {
+    const size_t need = f32_project_parts_bytes(rows, D, N, nW);
+    return need != 0 && need <= bytes;
+}
+
+// Whether a call is better off on the tensor cores: three launches instead of one, and under the masked scheme a fourth for the diagonal
+// tiles, which takes 20 to 30 us however few they are.  Measured (us, CUDA cores / tensor cores): FULL 16 heads of n = 129, d = 64 17 / 19, of n =
+// 160, d = 16 15.4 / 16.8, of n = 192, d = 64 17.4 / 17.4, of n = 1024, d = 128 308 / 54; 48 of n = 512, d = 64 111 / 42.  MASKED 64 heads of n = 256, d = 64
+// 35.9 / 36.4; 16 of n = 384, d = 128 48 / 52, of n = 512, d = 16 31.8 / 34.1, of n = 1024, d = 128 166 / 76; 8 of n = 512, d = 64 36 / 40; 4 of n = 640, d =
+// 64 38 / 42; 48 of n = 512, d = 64 93 / 52.
+inline bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme) {
+    const long long T = (n + 127) / 128, blocks = (long long)B * H * T * T;
+    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || (long long)B * H * n * d >= (1LL << 31)) return false;
+    if (scheme == PSA_MASKED) return n > 256 && blocks >= (d >= 64 ? 256 : 320);
+    return n >= 160 && (n >= 256 || d >= 64) && blocks >= 64;
+}
+
+// ---- the layout
+// Scratch of the symmetric scheme in bf16: its heads in passes, see sym_heads_per_pass.
+inline size_t sym_scratch_bytes(size_t heads, int n) {
+    return (size_t)sym_heads_per_pass(heads, n, SYM_SCRATCH_CAP) * sym_pairs(row_tiles(n)) * S_BLOCK_BYTES;
+}
+struct WsShape {
+    int batch, heads, n, d_model, d_k, scheme, dtype;
+    bool with_proj, staging;       // projections ahead of the core; buffers of the host entry point
+    bool one_launch;               // f32_fused_fits: a small fp32 layer, which needs no scratch but for an output projection
+};
+struct WsLayout {
+    size_t q, k, v, s, s_bytes, clear, clear_bytes, bad, marks_in, marks_out, ml, parts, in_bytes, out_bytes, xs, wq, wk, wv, outs, total;
+    bool attn_tensor;      // fp32: whether bad / ml / parts are there; in_bytes, out_bytes: room for the input and output projections' parts
+};
+
+inline WsLayout ws_layout(const WsShape& c) {
+    const size_t es = c.dtype == PSA_BF16 ? 2 : 4;
+    const size_t qkv = align_up((size_t)c.batch * c.n * c.heads * c.d_k * es, 256);
+    const int rows = c.batch * c.n, hd = c.heads * c.d_k;
+    WsLayout L;
+    memset(&L, 0, sizeof(L));
+    size_t off = COUNTER_BYTES;
+    if (c.dtype == PSA_F32) {      // marks right behind the counters: one clear serves both
+        const size_t bh = (size_t)c.batch * c.heads;
+        L.attn_tensor = !c.one_launch && f32_tensor_attention_fits(c.batch, c.heads, c.n, c.d_k, c.scheme);
+        L.in_bytes = c.with_proj && !c.one_launch ? f32_project_parts_bytes(rows, c.d_model, hd, c.scheme == PSA_SYMMETRIC ? 1 : 3) : 0;
+        L.out_bytes = c.with_proj ? f32_project_parts_bytes(rows, hd, c.d_model, 1) : 0;
+        L.clear = off;
+        if (L.attn_tensor) { L.bad = off; off += align_up(bh * sizeof(int), 256); }
+        if (L.in_bytes) { L.marks_in = off; off += align_up(f32_project_marks(rows, hd, 3) * sizeof(int), 256); }
+        if (L.out_bytes) { L.marks_out = off; off += align_up(f32_project_marks(rows, c.d_model, 1) * sizeof(int), 256); }
+        L.clear_bytes = c.one_launch ? 0 : off - L.clear;
+        if (L.attn_tensor) { L.ml = off; off += align_up(2 * bh * c.n * sizeof(float), 256); }
+        L.parts = off;           // (used by one kernel after another)
+        off += align_up(std::max(std::max(L.in_bytes, L.out_bytes), L.attn_tensor ? 12 * bh * c.n * c.d_k : (size_t)0), 256);
+    }
+    if (c.scheme == PSA_SYMMETRIC) {       // (bf16: right behind the counters, as above)
+        L.s_bytes = c.dtype == PSA_BF16 ? sym_scratch_bytes((size_t)c.batch * c.heads, c.n) : align_up((size_t)c.batch * c.heads * c.n * c.n * sizeof(float), 256);
+        L.s = off; off += L.s_bytes;
+    }
+    if (c.with_proj) {
+        L.q = off; off += qkv;
+        if (c.scheme == PSA_SYMMETRIC) { L.k = L.q; L.v = L.q; }
+        else { L.k = off; off += qkv; L.v = off; off += qkv; }
+    }
+    if (c.staging) {
+        const size_t xb = align_up((size_t)c.batch * c.n * c.d_model * es, 256);
+        const size_t wb = align_up((size_t)c.d_model * c.heads * c.d_k * es, 256);
+        L.xs = off; off += xb;
+        L.wq = off; off += wb;
+        if (c.scheme == PSA_SYMMETRIC) { L.wk = L.wq; L.wv = L.wq; }
+        else { L.wk = off; off += wb; L.wv = off; off += wb; }
+        L.outs = off; off += qkv;
+    }
+    L.total = off;
+    return L;
+}
+
+}  // namespace psa

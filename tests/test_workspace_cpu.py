@@ -1,0 +1,89 @@
+"""Host-side check of the workspace's layout (psa_ws.h compiled with g++): nothing overlaps, and what a part of a host call takes for its projections
+lies in the room that the layout of the whole call has for it."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <utility>
+#include <vector>
+#include "paper_2012_01114_b200/csrc/psa_ws.h"
+using namespace psa;
+typedef std::pair<size_t, size_t> Range;       // first byte, bytes
+
+static std::vector<Range> ranges(const WsShape& c, const WsLayout& L) {
+    const size_t es = c.dtype == PSA_BF16 ? 2 : 4, rows = (size_t)c.batch * c.n, hd = (size_t)c.heads * c.d_k, bh = (size_t)c.batch * c.heads;
+    const size_t in = rows * c.d_model * es, w = (size_t)c.d_model * hd * es, qkv = rows * hd * es;
+    std::vector<Range> r{{0, COUNTER_BYTES}};
+    size_t parts = L.in_bytes > L.out_bytes ? L.in_bytes : L.out_bytes;
+    if (L.attn_tensor) {
+        r.push_back({L.bad, bh * 4});
+        r.push_back({L.ml, 2 * bh * c.n * 4});
+        if (parts < 12 * rows * hd) parts = 12 * rows * hd;
+    }
+    if (L.in_bytes) r.push_back({L.marks_in, f32_project_marks((int)rows, (int)hd, 3) * 4});
+    if (L.out_bytes) r.push_back({L.marks_out, f32_project_marks((int)rows, c.d_model, 1) * 4});
+    if (parts) r.push_back({L.parts, parts});
+    const bool sym = c.scheme == PSA_SYMMETRIC;
+    if (sym) r.push_back({L.s, L.s_bytes});
+    if (c.with_proj) { r.push_back({L.q, qkv}); if (!sym) { r.push_back({L.k, qkv}); r.push_back({L.v, qkv}); } }
+    if (c.staging) {
+        r.push_back({L.xs, in}); r.push_back({L.wq, w}); r.push_back({L.outs, qkv});
+        if (!sym) { r.push_back({L.wk, w}); r.push_back({L.wv, w}); }
+    }
+    return r;
+}
+
+int main() {
+    // the last three: X of 2^33 numbers and more, with and without room for the parts of an output projection
+    const int shapes[][5] = {{1, 1, 64, 64, 64}, {4, 12, 512, 768, 64}, {9, 5, 300, 328, 40}, {64, 16, 1024, 128, 128}, {33, 1, 1023, 2048, 8}, {3, 7, 1, 24, 20},
+                             {2100, 33, 1, 776, 32}, {1024, 4, 1024, 8192, 64}, {1030, 1, 1024, 8192, 8}, {1100, 16, 1024, 8192, 128}};
+    long long used = 0, refused = 0;
+    for (const auto& s : shapes)
+        for (int scheme : {PSA_FULL, PSA_SYMMETRIC, PSA_MASKED})
+            for (int dtype : {PSA_F32, PSA_BF16})
+                for (int kind = 0; kind < 4; ++kind) {
+                    const WsShape c{s[0], s[1], s[2], kind ? s[3] : 0, s[4], scheme, dtype, kind > 0, kind > 1, kind == 3};
+                    const WsLayout L = ws_layout(c);
+                    const std::vector<Range> r = ranges(c, L);
+                    for (size_t i = 0; i < r.size(); ++i) {
+                        if (r[i].first % 256 || r[i].first + r[i].second > L.total) return 2;
+                        for (size_t j = 0; j < i; ++j)
+                            if (r[i].first < r[j].first + r[j].second && r[j].first < r[i].first + r[i].second) return 3;
+                    }
+                    if (dtype != PSA_F32 || kind != 2) continue;
+                    const int nW = scheme == PSA_SYMMETRIC ? 1 : 3, hd = c.heads * c.d_k;
+                    for (int parts = 1; parts <= HOST_CHUNKS && parts <= c.batch; ++parts)
+                        for (int k = 0; k < parts; ++k) {
+                            const int nb = (int)((long long)c.batch * (k + 1) / parts - (long long)c.batch * k / parts);
+                            const size_t need = f32_project_parts_bytes(nb * c.n, c.d_model, hd, nW);
+                            if (!need) continue;
+                            if (!f32_project_pairs_fit(nb * c.n, c.d_model, hd, nW, L.in_bytes)) { ++refused; continue; }
+                            ++used;
+                            if (need > L.in_bytes) return 4;
+                            if (f32_project_marks(nb * c.n, hd, nW) > f32_project_marks(c.batch * c.n, hd, 3)) return 5;
+                        }
+                }
+    printf("%lld %lld\n", used, refused);
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def layout(tmp_path_factory):
+    d = tmp_path_factory.mktemp("layout")
+    (d / "layout.cpp").write_text(SRC)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", ROOT, "-o", str(d / "layout"), str(d / "layout.cpp")])
+    return str(d / "layout")
+
+
+def test_nothing_overlaps_and_parts_stay_inside(layout):
+    run = subprocess.run([layout], capture_output=True, text=True)
+    assert run.returncode == 0, run.returncode
+    used, refused = (int(x) for x in run.stdout.split())
+    assert used > 20 and refused > 20        # parts of calls with and without room
