@@ -186,15 +186,18 @@ int psa_last_issued(void* stream, psa_counts* counts);
 int psa_last_rescales(void* stream, uint64_t* rescales);
 
 /* Bytes of scratch memory a call with these arguments needs (projected q, k, v; the symmetric
- * scheme's score matrix; counters).  with_host_staging != 0 adds psa_attention_host's buffers. */
+ * scheme's score matrix; counters; for large fp32 calls the bf16 parts of the operands, 12 bytes per number of Q for the attention
+ * and 6 per number of X and W for the projections, whichever is more, since one follows the other, with a few marks and sums).
+ * with_host_staging != 0 adds psa_attention_host's buffers.  An fp32 call does without the parts, on CUDA cores, where there is no
+ * memory for them: in a registered workspace that holds the rest, and when the private one cannot grow. */
 size_t psa_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype,
                            int with_host_staging);
 
 /*
  * Registers caller-owned device memory (256-byte aligned) as the workspace; it must stay valid
  * until replaced or until psa_set_workspace(NULL, 0).  Without a registered workspace, or when it
- * is too small, the library keeps a private one and grows it with cudaMalloc (synchronously, on
- * the first call that needs more).
+ * is too small (for an fp32 call: without the parts of psa_workspace_bytes), the library keeps a private one and grows it with
+ * cudaMalloc (synchronously, on the first call that needs more).
  */
 int psa_set_workspace(void* dev_ptr, size_t bytes);
 

@@ -82,9 +82,8 @@ int check_shape(int batch, int heads, int n, int d_model, int d_k, int scheme, i
     return PSA_OK;
 }
 
-WsLayout call_layout(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, bool with_proj, bool staging) {
-    return ws_layout(WsShape{batch, heads, n, d_model, d_k, scheme, dtype, with_proj, staging,
-                             with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme)});
+WsShape call_shape(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, bool with_proj, bool staging) {
+    return WsShape{batch, heads, n, d_model, d_k, scheme, dtype, with_proj, staging, with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme), false};
 }
 
 F32Scratch f32_scratch(char* ws, const WsLayout& L, size_t first_head) {
@@ -121,23 +120,62 @@ HostPipe* acquire_pipe(Context& cx) {
     return nullptr;
 }
 
-// Returns the base of a workspace of at least `bytes`, or nullptr (error text set).
-char* acquire_ws(Context& cx, size_t bytes) {
-    if (cx.user_ws && cx.user_bytes >= bytes) return static_cast<char*>(cx.user_ws);
-    if (cx.own_ws && cx.own_bytes >= bytes) return static_cast<char*>(cx.own_ws);
+// Replaces the library's own workspace.  nullptr (error text set) if there is no memory.
+char* grow_ws(Context& cx, size_t bytes) {
     if (cx.own_ws) {
         cudaDeviceSynchronize();
         cudaFree(cx.own_ws);
         cx.own_ws = nullptr;
         cx.own_bytes = 0;
+        cx.last_dc = nullptr;       // (may have been in it)
     }
     void* p = nullptr;
     const cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) { set_cuda_error(e, "cudaMalloc(workspace)"); return nullptr; }
+    if (e != cudaSuccess) {
+        set_cuda_error(e, "cudaMalloc(workspace)");
+        cudaGetLastError();         // (the next launch must not find it)
+        return nullptr;
+    }
     cx.own_ws = p;
     cx.clean_ws = nullptr;          // fresh memory: no counter block is known to be clear
     cx.own_bytes = bytes;
     return static_cast<char*>(p);
+}
+
+// Returns the base of a workspace of at least `bytes`, or nullptr (error text set).
+char* acquire_ws(Context& cx, size_t bytes) {
+    if (cx.user_ws && cx.user_bytes >= bytes) return static_cast<char*>(cx.user_ws);
+    if (cx.own_ws && cx.own_bytes >= bytes) return static_cast<char*>(cx.own_ws);
+    return grow_ws(cx, bytes);
+}
+
+// The workspace of a call and what lies where in it, `extra` bytes behind the layout (from L->total on) included; nullptr (error text set) if
+// there is none.  fp32 calls do with the lean layout where the whole one finds no memory.
+char* acquire_call_ws(Context& cx, WsShape c, size_t extra, cudaStream_t stream, WsLayout* L) {
+    *L = ws_layout(c);
+    const size_t whole = L->total + extra, user = cx.user_ws ? cx.user_bytes : 0, own = cx.own_ws ? cx.own_bytes : 0;
+    if (c.dtype != PSA_F32 || user >= whole || (!user && own >= whole)) return acquire_ws(cx, whole);
+    c.lean = true;
+    const WsLayout lean = ws_layout(c);
+    const size_t least = lean.total + extra;
+    const WsPlan plan = ws_plan(user, own, whole, least, [&] {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        size_t avail = 0, total = 0;
+        return cudaStreamIsCapturing(stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
+               cudaMemGetInfo(&avail, &total) == cudaSuccess && avail + own >= whole;
+    });
+    char* ws = static_cast<char*>(plan.from == WsFrom::USER ? cx.user_ws : cx.own_ws);
+    bool use_lean = !plan.whole;
+    if (plan.from == WsFrom::GROW) {
+        ws = grow_ws(cx, whole);
+        if (!ws && least < whole) {
+            ws = grow_ws(cx, least);
+            if (ws) g_err_text[0] = 0;
+            use_lean = true;
+        }
+    }
+    if (use_lean) *L = lean;
+    return ws;
 }
 
 void useful_counts(int batch, int heads, int n, int d_model, int d_k, int scheme, bool with_proj, psa_counts* c) {
@@ -259,8 +297,8 @@ int layer_entry(const void* X, const void* Wq, const void* Wk, const void* Wv, i
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
-    char* ws = acquire_ws(cx, L.total);
+    WsLayout L;
+    char* ws = acquire_call_ws(cx, call_shape(batch, heads, n, d_model, d_k, scheme, dtype, true, false), 0, static_cast<cudaStream_t>(stream), &L);
     if (!ws) return PSA_ERR_WORKSPACE;
     return run_layer(cx, X, Wq, Wk, Wv, nullptr, nullptr, nullptr, batch, heads, n, d_model, d_k, scheme, dtype, out,
                      static_cast<cudaStream_t>(stream), true, ws, L);
@@ -322,8 +360,8 @@ int psa_attention_core(const void* Q, const void* K, const void* V, int batch, i
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = call_layout(batch, heads, n, 0, d_k, scheme, dtype, false, false);
-    char* ws = acquire_ws(cx, L.total);
+    WsLayout L;
+    char* ws = acquire_call_ws(cx, call_shape(batch, heads, n, 0, d_k, scheme, dtype, false, false), 0, static_cast<cudaStream_t>(stream), &L);
     if (!ws) return PSA_ERR_WORKSPACE;
     return run_layer(cx, nullptr, nullptr, nullptr, nullptr, Q, K, V, batch, heads, n, 0, d_k, scheme, dtype, out,
                      static_cast<cudaStream_t>(stream), false, ws, L);
@@ -347,8 +385,8 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, true);
-    char* ws = acquire_ws(cx, L.total);
+    WsLayout L;
+    char* ws = acquire_call_ws(cx, call_shape(batch, heads, n, d_model, d_k, scheme, dtype, true, true), 0, stream, &L);
     if (!ws) return PSA_ERR_WORKSPACE;
     const size_t es = dtype == PSA_BF16 ? 2 : 4;
     const size_t xb = (size_t)n * d_model * es, wb = (size_t)d_model * heads * d_k * es, ob = (size_t)n * heads * d_k * es;   // per sequence; per matrix
@@ -457,12 +495,12 @@ int psa_attention_core_host(const void* Q_host, const void* K_host, const void* 
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = call_layout(batch, heads, n, 0, d_k, scheme, dtype, false, false);
     const size_t tb = (size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4), tba = align_up(tb, 256);
-    const size_t q_off = align_up(L.total, 256), k_off = q_off + tba, v_off = k_off + tba;
-    const size_t o_off = sym ? k_off : v_off + tba;          // the symmetric scheme stages one input tensor
-    char* ws = acquire_ws(cx, o_off + tba);
+    WsLayout L;
+    char* ws = acquire_call_ws(cx, call_shape(batch, heads, n, 0, d_k, scheme, dtype, false, false), (sym ? 2 : 4) * tba, stream, &L);
     if (!ws) return PSA_ERR_WORKSPACE;
+    const size_t q_off = L.total, k_off = q_off + tba, v_off = k_off + tba;
+    const size_t o_off = sym ? k_off : v_off + tba;          // the symmetric scheme stages one input tensor
     cudaError_t e = cudaMemcpyAsync(ws + q_off, Q_host, tb, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess && !sym) {
         e = cudaMemcpyAsync(ws + k_off, K_host, tb, cudaMemcpyHostToDevice, stream);
@@ -507,12 +545,11 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
     if (!cp) return PSA_ERR_CUDA;
     Context& cx = *cp;
     std::lock_guard<std::mutex> lock(cx.mu);
-    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
-    const size_t y_off = align_up(L.total, 256);
-    const size_t y_bytes = (size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4);
-    char* ws = acquire_ws(cx, y_off + align_up(y_bytes, 256));
+    WsLayout L;
+    char* ws = acquire_call_ws(cx, call_shape(batch, heads, n, d_model, d_k, scheme, dtype, true, false), align_up((size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4), 256),
+                               stream, &L);
     if (!ws) return PSA_ERR_WORKSPACE;
-    void* y = ws + y_off;
+    void* y = ws + L.total;
     rc = run_layer(cx, X, Wq, Wk, Wv, nullptr, nullptr, nullptr, batch, heads, n, d_model, d_k, scheme, dtype, y, stream,
                    true, ws, L);
     if (rc != PSA_OK) return rc;
@@ -534,8 +571,7 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
 
 size_t psa_block_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype) {
     if (d_model <= 0 || check_shape(batch, heads, n, d_model, d_k, scheme, dtype, true) != PSA_OK) return 0;
-    const WsLayout L = call_layout(batch, heads, n, d_model, d_k, scheme, dtype, true, false);
-    return align_up(L.total, 256) + align_up((size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4), 256);
+    return ws_layout(call_shape(batch, heads, n, d_model, d_k, scheme, dtype, true, false)).total + align_up((size_t)batch * n * heads * d_k * (dtype == PSA_BF16 ? 2 : 4), 256);
 }
 
 int psa_skip_count(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, psa_counts* c) {
@@ -680,7 +716,7 @@ size_t psa_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, in
                            int with_host_staging) {
     const bool with_proj = d_model > 0;
     if (check_shape(batch, heads, n, d_model, d_k, scheme, dtype, with_proj) != PSA_OK) return 0;
-    return call_layout(batch, heads, n, d_model, d_k, scheme, dtype, with_proj, with_host_staging != 0 && with_proj).total;
+    return ws_layout(call_shape(batch, heads, n, d_model, d_k, scheme, dtype, with_proj, with_host_staging != 0 && with_proj)).total;
 }
 
 int psa_set_workspace(void* dev_ptr, size_t bytes) {

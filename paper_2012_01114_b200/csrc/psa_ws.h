@@ -50,6 +50,7 @@ struct WsShape {
     int batch, heads, n, d_model, d_k, scheme, dtype;
     bool with_proj, staging;       // projections ahead of the core; buffers of the host entry point
     bool one_launch;               // f32_fused_fits: a small fp32 layer, which needs no scratch but for an output projection
+    bool lean;                     // without the scratch of the tensor cores: an fp32 call that has no memory for it runs on CUDA cores
 };
 struct WsLayout {
     size_t q, k, v, s, s_bytes, clear, clear_bytes, bad, marks_in, marks_out, ml, parts, in_bytes, out_bytes, xs, wq, wk, wv, outs, total;
@@ -63,7 +64,7 @@ inline WsLayout ws_layout(const WsShape& c) {
     WsLayout L;
     memset(&L, 0, sizeof(L));
     size_t off = COUNTER_BYTES;
-    if (c.dtype == PSA_F32) {      // marks right behind the counters: one clear serves both
+    if (c.dtype == PSA_F32 && !c.lean) {      // marks right behind the counters: one clear serves both
         const size_t bh = (size_t)c.batch * c.heads;
         L.attn_tensor = !c.one_launch && f32_tensor_attention_fits(c.batch, c.heads, c.n, c.d_k, c.scheme);
         L.in_bytes = c.with_proj && !c.one_launch ? f32_project_parts_bytes(rows, c.d_model, hd, c.scheme == PSA_SYMMETRIC ? 1 : 3) : 0;
@@ -97,6 +98,24 @@ inline WsLayout ws_layout(const WsShape& c) {
     }
     L.total = off;
     return L;
+}
+
+// ---- which memory a call runs in: the caller's workspace, the library's own, or a new one of its own; and whether with the whole layout or
+// the lean one.  A caller's workspace that holds the lean layout is used in any case: nothing is allocated behind the back of a
+// caller who has registered one, and a graph keeps the memory that it was captured with.  `may_grow` is asked only where there is
+// another way.
+enum class WsFrom { USER, OWN, GROW };
+struct WsPlan {
+    WsFrom from;
+    bool whole;
+};
+template <class MayGrow>
+WsPlan ws_plan(size_t user, size_t own, size_t whole, size_t least, MayGrow may_grow) {
+    if (user >= whole) return {WsFrom::USER, true};
+    if (user >= least) return {WsFrom::USER, false};
+    if (own >= whole) return {WsFrom::OWN, true};
+    if (own >= least && !may_grow()) return {WsFrom::OWN, false};
+    return {WsFrom::GROW, true};
 }
 
 }  // namespace psa

@@ -1,0 +1,86 @@
+"""fp32 calls in a registered workspace that holds everything but the operands of the tensor cores: nothing is allocated, the call runs on CUDA
+cores, and a captured graph stays in that workspace.  Reference: the same call in a workspace of psa_workspace_bytes, on the tensor cores; both
+are within 4e-6 of the exact result (tests/test_gpu_f32_tensor.py), so 8e-6 apart at most."""
+import pytest
+import torch
+
+from paper_2012_01114_b200 import binding
+
+pytestmark = pytest.mark.gpu
+COUNTERS = 256
+
+
+def _up(v):
+    return (v + 255) // 256 * 256
+
+
+def _inputs(shapes):
+    g = torch.Generator(device="cuda").manual_seed(5)
+    return [torch.empty(s, device="cuda").normal_(0.0, scale, generator=g) for s, scale in shapes]
+
+
+def _close(a, b):
+    assert torch.isfinite(a).all()
+    assert float((a.double() - b.double()).norm()) <= 8e-6 * float(b.double().norm())
+
+
+def _case(entry, scheme):
+    """The call, the bytes of its lean layout, the census it must show."""
+    if entry == "core":
+        B, H, n, d = 2, 20, 520, 64
+        t = _inputs([((B, n, H, d), 1.0)] * 3)
+        return lambda out: binding.psa_attention_core(*t, scheme, out=out), (B, n, H * d), COUNTERS, (B, H, n, 0, d)
+    B, H, n, d, D = 4, 12, 520, 64, 768
+    t = _inputs([((B, n, D), 1.0)] + [((D, H * d), D ** -0.5)] * 3 + [((H * d, D), (H * d) ** -0.5)])
+    lean = COUNTERS + 3 * _up(4 * B * n * H * d)
+    if entry == "layer":
+        return lambda out: binding.psa_attention_f32(*t[:4], H, scheme, out=out), (B, n, H * d), lean, (B, H, n, D, d)
+    return (lambda out: binding.psa_attention_block(*t, H, scheme, out=out, residual=t[0]), (B, n, D), lean + _up(4 * B * n * H * d), (B, H, n, D, d))
+
+
+@pytest.mark.parametrize("scheme", [binding.FULL, binding.MASKED])
+@pytest.mark.parametrize("entry", ["core", "layer", "block"])
+def test_small_registered_workspace(entry, scheme):
+    call, shape, lean, (B, H, n, D, d) = _case(entry, scheme)
+    whole = binding.psa_workspace_bytes(B, H, n, D, d, scheme, binding.F32) if entry != "block" else binding.psa_block_workspace_bytes(B, H, n, D, d, scheme, binding.F32)
+    assert lean < whole
+    outs = [torch.full(shape, float("nan"), device="cuda") for _ in range(3)]
+    big = torch.empty(whole, dtype=torch.uint8, device="cuda")
+    small = torch.full((lean + 4096,), 171, dtype=torch.uint8, device="cuda")
+    try:
+        binding.psa_set_workspace(big)
+        call(outs[0])
+        binding.psa_set_workspace(small[:lean])
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        call(outs[1])
+        st, got = binding.psa_last_issued()
+        # (a kernel's first launch may take a little memory; the whole layouts are 16 MB and more)
+        assert st == binding.OK and free - torch.cuda.mem_get_info()[0] < 8 << 20 and whole > 15 << 20
+        assert not (small[:COUNTERS] == 171).all() and (small[lean:] == 171).all()        # this memory was used, and nothing behind it
+        want = binding.psa_skip_count(B, H, n, D, d, scheme, binding.F32)
+        assert {k: v for k, v in got.items() if k != "proj_macs"} == {k: v for k, v in want.items() if k != "proj_macs"}
+        _close(outs[1], outs[0])
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            call(outs[2])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(outs[2], outs[1])
+    finally:
+        torch.cuda.synchronize()
+        binding.psa_set_workspace(None)
+
+
+def test_too_small_even_for_the_lean_layout():
+    call, shape, lean, _ = _case("layer", binding.FULL)
+    small = torch.empty(lean - 256, dtype=torch.uint8, device="cuda")
+    a, b = torch.empty(shape, device="cuda"), torch.empty(shape, device="cuda")
+    call(a)
+    try:
+        binding.psa_set_workspace(small)
+        call(b)                                              # in the library's own, on the tensor cores
+        torch.cuda.synchronize()
+    finally:
+        binding.psa_set_workspace(None)
+    assert torch.equal(a, b)

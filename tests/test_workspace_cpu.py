@@ -1,5 +1,5 @@
 """Host-side check of the workspace's layout (psa_ws.h compiled with g++): nothing overlaps, and what a part of a host call takes for its projections
-lies in the room that the layout of the whole call has for it."""
+lies in the room that the layout of the whole call has for it.  And which memory a call runs in, the lean layout of fp32 calls included."""
 import os
 import subprocess
 
@@ -47,8 +47,16 @@ int main() {
         for (int scheme : {PSA_FULL, PSA_SYMMETRIC, PSA_MASKED})
             for (int dtype : {PSA_F32, PSA_BF16})
                 for (int kind = 0; kind < 4; ++kind) {
-                    const WsShape c{s[0], s[1], s[2], kind ? s[3] : 0, s[4], scheme, dtype, kind > 0, kind > 1, kind == 3};
+                    const WsShape c{s[0], s[1], s[2], kind ? s[3] : 0, s[4], scheme, dtype, kind > 0, kind > 1, kind == 3, false};
                     const WsLayout L = ws_layout(c);
+                    WsShape lean = c;
+                    lean.lean = true;
+                    const WsLayout M = ws_layout(lean);
+                    // lean: counters, scores, q, k, v and staging only, all that the CUDA cores need
+                    size_t rest = COUNTER_BYTES;
+                    for (const Range& x : ranges(lean, M)) rest += x.first ? align_up(x.second, 256) : 0;
+                    if (M.total != rest || M.attn_tensor || M.in_bytes || M.out_bytes || M.clear_bytes) return 6;
+                    if (M.total > L.total || (dtype == PSA_BF16 && M.total != L.total)) return 7;
                     const std::vector<Range> r = ranges(c, L);
                     for (size_t i = 0; i < r.size(); ++i) {
                         if (r[i].first % 256 || r[i].first + r[i].second > L.total) return 2;
@@ -87,3 +95,34 @@ def test_nothing_overlaps_and_parts_stay_inside(layout):
     assert run.returncode == 0, run.returncode
     used, refused = (int(x) for x in run.stdout.split())
     assert used > 20 and refused > 20        # parts of calls with and without room
+
+
+PLAN = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "paper_2012_01114_b200/csrc/psa_ws.h"
+int main(int, char** a) {
+    bool asked = false;
+    const psa::WsPlan p = psa::ws_plan(atoi(a[1]), atoi(a[2]), atoi(a[3]), atoi(a[4]), [&] { asked = true; return atoi(a[5]) != 0; });
+    printf("%d %d %d\n", (int)p.from, (int)p.whole, (int)asked);
+    return 0;
+}
+"""
+USER, OWN, GROW = 0, 1, 2
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "plan.cpp").write_text(PLAN)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", ROOT, "-o", str(d / "plan"), str(d / "plan.cpp")])
+    return lambda *a: tuple(int(x) for x in subprocess.check_output([str(d / "plan")] + [str(x) for x in a]).split())
+
+
+# bytes registered, of the library's own workspace, of the whole layout, of the lean one; whether there is memory to grow into
+@pytest.mark.parametrize("user,own,whole,least,memory,want", [
+    (100, 0, 100, 40, 0, (USER, 1, 0)), (99, 100, 100, 40, 1, (USER, 0, 0)), (40, 0, 100, 40, 1, (USER, 0, 0)), (39, 100, 100, 40, 0, (OWN, 1, 0)),
+    (39, 99, 100, 40, 0, (OWN, 0, 1)), (0, 40, 100, 40, 0, (OWN, 0, 1)), (0, 40, 100, 40, 1, (GROW, 1, 1)), (0, 39, 100, 40, 0, (GROW, 1, 0)),
+    (0, 0, 100, 40, 0, (GROW, 1, 0)), (0, 99, 100, 100, 0, (GROW, 1, 0)), (99, 100, 100, 100, 0, (OWN, 1, 0))])
+def test_memory_of_a_call(plan, user, own, whole, least, memory, want):
+    assert plan(user, own, whole, least, memory) == want
