@@ -26,6 +26,7 @@
  *         W*   [d_model, heads*d_k]      head h owns columns h*d_k .. (h+1)*d_k-1
  *         Q,K,V[batch, n, heads, d_k]
  *         out  [batch, n, heads*d_k]
+ *     `out` must not overlap Q, K or V of the attention core, but in fp32 with the full and masked schemes, where it may be Q.
  *   - Every function returns a psa_status (0 = PSA_OK) unless stated otherwise.
  *   - Calls that share a workspace must be ordered on one stream; the library is not re-entrant
  *     across streams.

@@ -363,6 +363,10 @@ int psa_attention_core(const void* Q, const void* K, const void* V, int batch, i
     WsLayout L;
     char* ws = acquire_call_ws(cx, call_shape(batch, heads, n, 0, d_k, scheme, dtype, false, false), 0, static_cast<cudaStream_t>(stream), &L);
     if (!ws) return PSA_ERR_WORKSPACE;
+    // In place (fp32): the CUDA-core kernels read a row of Q before they write it, as the tensor-core one of the full scheme does; the masked
+    // one keeps partial outputs in `out` while Q is still to be read.
+    const uintptr_t q0 = reinterpret_cast<uintptr_t>(Q), o0 = reinterpret_cast<uintptr_t>(out), bytes = (uintptr_t)batch * n * heads * d_k * 4;
+    if (dtype == PSA_F32 && scheme == PSA_MASKED && q0 < o0 + bytes && o0 < q0 + bytes) L.attn_tensor = false;
     return run_layer(cx, nullptr, nullptr, nullptr, nullptr, Q, K, V, batch, heads, n, 0, d_k, scheme, dtype, out,
                      static_cast<cudaStream_t>(stream), false, ws, L);
 }

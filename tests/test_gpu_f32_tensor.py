@@ -96,3 +96,15 @@ def test_projections_of_large_calls(rows, D, H, d):
     assert not np.isfinite(z[300]).all()
     x[300], z[300] = 0.0, 0.0
     assert (np.abs(z - x @ w) <= (D / 64 + 4) * 2.0 ** -24 * (np.abs(x) @ np.abs(w)) + 1e-44).all()
+
+
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("B,H,n,d", [(1, 16, 1024, 64), (2, 10, 700, 128), (1, 4, 300, 64), (1, 3, 70, 20)])
+def test_output_over_q(scheme, B, H, n, d):
+    # in place, on the tensor cores or not: both results are within 4e-6 of the exact one
+    t = [torch.from_numpy(inputs.tensor(n + d, 4 + i, (B, n, H, d), 1.0, "f32")[1]).cuda() for i in range(3)]
+    want = binding.psa_attention_core(*t, scheme).double()
+    got = binding.psa_attention_core(*t, scheme, out=t[0].view(B, n, H * d)).double()
+    st, census = binding.psa_last_issued()
+    assert st == binding.OK and census == binding.psa_skip_count(B, H, n, 0, d, scheme, binding.F32)
+    assert float((got - want).norm()) <= 8e-6 * float(want.norm())
