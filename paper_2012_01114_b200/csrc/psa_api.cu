@@ -452,7 +452,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         e = cudaStreamWaitEvent(stream, pipe->loaded[c], 0);
         if (e != cudaSuccess) break;
         void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
-        const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in)};
+        const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in) + c * L.marks_pitch};
         const F32Scratch fs = f32_scratch(ws, L, b0 * heads);       // (a part has marks of its own; the rest is used by one after another)
         rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
                            d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,

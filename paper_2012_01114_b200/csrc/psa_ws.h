@@ -53,7 +53,7 @@ struct WsShape {
     bool lean;                     // without the scratch of the tensor cores: an fp32 call that has no memory for it runs on CUDA cores
 };
 struct WsLayout {
-    size_t q, k, v, s, s_bytes, clear, clear_bytes, bad, marks_in, marks_out, ml, parts, in_bytes, out_bytes, xs, wq, wk, wv, outs, total;
+    size_t q, k, v, s, s_bytes, clear, clear_bytes, bad, marks_in, marks_pitch, marks_out, ml, parts, in_bytes, out_bytes, xs, wq, wk, wv, outs, total;
     bool attn_tensor;      // fp32: whether bad / ml / parts are there; in_bytes, out_bytes: room for the input and output projections' parts
 };
 
@@ -71,7 +71,10 @@ inline WsLayout ws_layout(const WsShape& c) {
         L.out_bytes = c.with_proj ? f32_project_parts_bytes(rows, hd, c.d_model, 1) : 0;
         L.clear = off;
         if (L.attn_tensor) { L.bad = off; off += align_up(bh * sizeof(int), 256); }
-        if (L.in_bytes) { L.marks_in = off; off += align_up(f32_project_marks(rows, hd, 3) * sizeof(int), 256); }
+        if (L.in_bytes) {      // (a part of a host call has marks of its own)
+            L.marks_in = off; L.marks_pitch = f32_project_marks(rows, hd, 3);
+            off += align_up((c.staging ? HOST_CHUNKS : 1) * L.marks_pitch * sizeof(int), 256);
+        }
         if (L.out_bytes) { L.marks_out = off; off += align_up(f32_project_marks(rows, c.d_model, 1) * sizeof(int), 256); }
         L.clear_bytes = c.one_launch ? 0 : off - L.clear;
         if (L.attn_tensor) { L.ml = off; off += align_up(2 * bh * c.n * sizeof(float), 256); }

@@ -108,3 +108,17 @@ def test_output_over_q(scheme, B, H, n, d):
     st, census = binding.psa_last_issued()
     assert st == binding.OK and census == binding.psa_skip_count(B, H, n, 0, d, scheme, binding.F32)
     assert float((got - want).norm()) <= 8e-6 * float(want.norm())
+
+
+def test_projections_of_host_calls_in_parts():
+    # 8 parts of 2048 rows, on pairs of CTAs each; numbers without parts in the first and the last; bit by bit what the device call gives
+    rows, D, H, d = 16384, 768, 12, 64
+    X, Wq, Wk, Wv = [torch.from_numpy(inputs.tensor(3, i, s, 1.0, "f32")[1]).pin_memory() for i, s in enumerate([(rows, 1, D)] + [(D, H * d)] * 3)]
+    X[7] *= 1e-36
+    X[rows - 1, 0, :5] = 1e-33
+    out = torch.empty((rows, 1, H * d)).pin_memory()
+    binding.psa_attention_host(X, Wq, Wk, Wv, H, binding.FULL, out)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got == binding.psa_skip_count(rows, H, 1, D, d, binding.FULL, binding.F32)
+    want = binding.psa_attention_f32(X.cuda(), Wq.cuda(), Wk.cuda(), Wv.cuda(), H, binding.FULL)
+    assert torch.equal(out, want.cpu())

@@ -25,7 +25,7 @@ static std::vector<Range> ranges(const WsShape& c, const WsLayout& L) {
         r.push_back({L.ml, 2 * bh * c.n * 4});
         if (parts < 12 * rows * hd) parts = 12 * rows * hd;
     }
-    if (L.in_bytes) r.push_back({L.marks_in, f32_project_marks((int)rows, (int)hd, 3) * 4});
+    if (L.in_bytes) r.push_back({L.marks_in, f32_project_marks((int)rows, (int)hd, 3) * 4 * (c.staging ? HOST_CHUNKS : 1)});
     if (L.out_bytes) r.push_back({L.marks_out, f32_project_marks((int)rows, c.d_model, 1) * 4});
     if (parts) r.push_back({L.parts, parts});
     const bool sym = c.scheme == PSA_SYMMETRIC;
@@ -73,7 +73,10 @@ int main() {
                             if (!f32_project_pairs_fit(nb * c.n, c.d_model, hd, nW, L.in_bytes)) { ++refused; continue; }
                             ++used;
                             if (need > L.in_bytes) return 4;
-                            if (f32_project_marks(nb * c.n, hd, nW) > f32_project_marks(c.batch * c.n, hd, 3)) return 5;
+                            // marks of part k, cleared once ahead of all parts: behind those of the part before, before those of the next
+                            if (f32_project_marks(nb * c.n, hd, nW) > L.marks_pitch) return 5;
+                            const size_t last = L.marks_in + (k * L.marks_pitch + f32_project_marks(nb * c.n, hd, nW)) * 4;
+                            if (L.marks_in < L.clear || last > L.clear + L.clear_bytes || (L.marks_out && L.marks_in < L.marks_out && last > L.marks_out)) return 8;
                         }
                 }
     printf("%lld %lld\n", used, refused);
