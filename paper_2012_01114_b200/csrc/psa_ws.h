@@ -30,15 +30,29 @@ inline bool f32_project_pairs_fit(int rows, int D, int N, int nW, size_t bytes) 
 }
 
 // Whether a call is better off on the tensor cores: three launches instead of one, and under the masked scheme a fourth for the diagonal
-// tiles, which takes 20 to 30 us however few they are.  Measured (us, CUDA cores / tensor cores): FULL 16 heads of n = 129, d = 64 17 / 19, of n =
-// 160, d = 16 15.4 / 16.8, of n = 192, d = 64 17.4 / 17.4, of n = 1024, d = 128 308 / 54; 48 of n = 512, d = 64 111 / 42.  MASKED 64 heads of n = 256, d = 64
-// 35.9 / 36.4; 16 of n = 384, d = 128 48 / 52, of n = 512, d = 16 31.8 / 34.1, of n = 1024, d = 128 166 / 76; 8 of n = 512, d = 64 36 / 40; 4 of n = 640, d =
-// 64 38 / 42; 48 of n = 512, d = 64 93 / 52.
+// tiles, which takes 20 to 30 us however few they are.  Measured at 4000 sizes at the edges; the CUDA cores' kernel moves in steps, with
+// its rows per CTA (64, 32 or 16, by whether that makes two CTAs per SM) and slower where n is not a multiple of its 64 keys, and the diagonal
+// tiles in rounds of one per SM (two up to d = 64).  Figures: heads, time on the tensor cores over time on CUDA cores.
+// FULL: n = 129, d = 64 16 1.12; n = 160, d = 16 16 1.09, d = 64 16 0.89; n = 257, d = 16 8 1.08, 12 0.89; n = 256, d = 8 17 1.04, 20 0.88; n = 1024, d = 64 1 0.62.
+// MASKED, up to 320 keys, where a head has three diagonal tiles and one or two blocks off them: d = 64 n = 257 32 1.33, 40 0.93, 64 0.58, n = 300 29 1.16, 32 0.84, n = 320
+// 56 1.10, 79 0.82; d = 128 n = 257 29 1.04, 40 0.76, 53 1.12, 64 0.52; d = 32 n = 320 37 1.06, 63 0.78, n = 270 53 1.07; d = 8 n = 257 48 1.11, 64 0.80, 129 1.06,
+// n = 320 53 1.31, 66 0.90, 123 1.22.  Beyond: d = 64 n = 385 22 1.07, 24 0.77, n = 420 20 1.06; d = 32 n = 385 22 1.12, 24 0.85; d = 8 n = 513 17 1.06, 20 0.82, n = 385 40 1.02;
+// n = 640, d = 64 4 (100 blocks) 1.10, 12 0.86; n = 1024, d = 8 4 1.03, d = 64 4 0.80.
 inline bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme) {
-    const long long T = (n + 127) / 128, blocks = (long long)B * H * T * T;
-    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || (long long)B * H * n * d >= (1LL << 31)) return false;
-    if (scheme == PSA_MASKED) return n > 256 && blocks >= (d >= 64 ? 256 : 320);
-    return n >= 160 && (n >= 256 || d >= 64) && blocks >= 64;
+    constexpr int SMS = 148;
+    const long long heads = (long long)B * H, T = row_tiles(n), tiles = heads * T, blocks = tiles * T;
+    if (scheme == PSA_SYMMETRIC || d % 8 != 0 || heads * n * d >= (1LL << 31)) return false;
+    if (scheme == PSA_FULL)
+        return n >= (d >= 64 ? 160 : 256) && blocks >= (d < 16 && n <= 256 ? 80 : 64) && (d >= 32 || heads * n * n >= 34LL * TILE * TILE);
+    if (n <= 256 || blocks < (d >= 64 ? 256 : 320)) return false;
+    const bool rows64 = heads * ((n + 63) / 64) >= 2 * SMS, rows32 = heads * ((n + 31) / 32) >= 2 * SMS;
+    if (n <= 320) {
+        if (d > 64) return rows32 && (tiles <= SMS || rows64);
+        return d >= 32 ? rows64 || (n % 64 != 0 && rows32 && tiles <= SMS) : rows64 && tiles <= 2 * SMS;
+    }
+    if (d > 64) return true;
+    const long long off = heads * ((T - 1) * (T - 2) / 2 * TILE + (n - TILE * (T - 1)) * (T - 1));       // rows of 128 weights
+    return (n > 576 || rows32) && (d >= 32 || off >= 100 * TILE);
 }
 
 // ---- the layout

@@ -129,3 +129,30 @@ def plan(tmp_path_factory):
     (0, 0, 100, 40, 0, (GROW, 1, 0)), (0, 99, 100, 100, 0, (GROW, 1, 0)), (99, 100, 100, 100, 0, (OWN, 1, 0))])
 def test_memory_of_a_call(plan, user, own, whole, least, memory, want):
     assert plan(user, own, whole, least, memory) == want
+
+
+FITS = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "paper_2012_01114_b200/csrc/psa_ws.h"
+int main(int argc, char** a) {
+    for (int i = 1; i + 4 < argc; i += 5)
+        printf("%d ", (int)psa::f32_tensor_attention_fits(atoi(a[i]), atoi(a[i + 1]), atoi(a[i + 2]), atoi(a[i + 3]), atoi(a[i + 4])));
+    return 0;
+}
+"""
+FULL, MASKED = 0, 2
+
+
+def test_calls_with_little_off_the_diagonal_tiles_stay_on_cuda_cores(tmp_path):
+    # (batch, heads, n, d, scheme) measured faster on CUDA cores, and neighbours measured faster on the tensor cores
+    cuda = [(1, 29, 257, 64, MASKED), (2, 16, 257, 64, MASKED), (1, 29, 257, 128, MASKED), (1, 53, 257, 128, MASKED), (1, 48, 257, 16, MASKED), (1, 29, 300, 64, MASKED),
+            (4, 14, 320, 64, MASKED), (1, 53, 320, 8, MASKED), (1, 123, 320, 8, MASKED), (1, 16, 385, 64, MASKED), (4, 5, 385, 64, MASKED), (1, 22, 385, 32, MASKED),
+            (1, 20, 385, 8, MASKED), (1, 20, 420, 64, MASKED), (1, 17, 513, 8, MASKED), (1, 8, 257, 16, FULL), (1, 17, 256, 8, FULL)]
+    tensor = [(1, 64, 257, 64, MASKED), (1, 40, 257, 128, MASKED), (1, 64, 300, 64, MASKED), (1, 32, 300, 64, MASKED), (1, 79, 320, 64, MASKED), (1, 24, 385, 64, MASKED),
+              (4, 6, 385, 32, MASKED), (1, 20, 513, 8, MASKED), (1, 4, 1024, 64, MASKED), (2, 8, 1024, 128, MASKED), (1, 8, 257, 32, FULL), (1, 12, 257, 8, FULL),
+              (1, 20, 256, 8, FULL), (1, 1, 1024, 8, FULL), (4, 12, 512, 64, FULL)]
+    (tmp_path / "fits.cpp").write_text(FITS)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", ROOT, "-o", str(tmp_path / "fits"), str(tmp_path / "fits.cpp")])
+    got = subprocess.check_output([str(tmp_path / "fits")] + [str(x) for c in cuda + tensor for x in c]).split()
+    assert [int(x) for x in got] == [0] * len(cuda) + [1] * len(tensor)
