@@ -481,7 +481,7 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
 // 8 keys; the last group's triangle is unrolled.  Bound by the port of shared memory (12 loads of 16 bytes for 128 multiply-accumulates).
 // Rows of Q and K are stored so that rows read at the same time are neighbours, 4 banks apart.
 // Measured: the 128 tiles of 16 heads of n = 1024, d = 128 54 us as blocks of f32_flash_kernel, 30 here.
-constexpr int FD_THREADS = 288;
+constexpr int FD_THREADS = 288, FD_CHAIN = 16;
 template <int DG>
 struct FDCfg {
     static constexpr int P = 64 * DG + 4, PP = 132;                      // row pitches of Q and K, of the weights, in floats
@@ -595,15 +595,16 @@ f32_diagonal_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
             if (j + 3 <= row) m = fmaxf(m, f.w);
         }
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-        float l = 0.f;
+        float s[4] = {0.f, 0.f, 0.f, 0.f};                              // (chains of 16)
         for (int j = 4 * part; j <= row; j += 8) {
             float4 f = *reinterpret_cast<const float4*>(w + j);
-            f.x = expf(f.x - m); l += f.x;
-            if (j + 1 <= row) { f.y = expf(f.y - m); l += f.y; }
-            if (j + 2 <= row) { f.z = expf(f.z - m); l += f.z; }
-            if (j + 3 <= row) { f.w = expf(f.w - m); l += f.w; }
+            f.x = expf(f.x - m); s[0] += f.x;
+            if (j + 1 <= row) { f.y = expf(f.y - m); s[1] += f.y; }
+            if (j + 2 <= row) { f.z = expf(f.z - m); s[2] += f.z; }
+            if (j + 3 <= row) { f.w = expf(f.w - m); s[3] += f.w; }
             *reinterpret_cast<float4*>(w + j) = f;
         }
+        float l = (s[0] + s[1]) + (s[2] + s[3]);
         l += __shfl_xor_sync(0xffffffffu, l, 1);
         if (part == 0) {
             row_m[row] = m;
@@ -633,23 +634,34 @@ f32_diagonal_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
             const int g = side ? 15 - warp : warp;
             float o[8][CW] = {};
             const float* w = Ws + 8 * g * C::PP;
+            // 16 keys at a time, then added up: with a chain over all of them the call had more error than f32_flash_kernel, whose chains are
+            // split over warps (values of one sign, n = 385, d = 128 1.19e-7 and 0.89e-7 there, now 0.91e-7; 1-3 % of the call's time)
 #pragma unroll 1
-            for (int j = 0; j < 8 * g; j += 4) {
-                float4 p[8];
+            for (int j0 = 0; j0 < 8 * g; j0 += FD_CHAIN) {
+                float t[8][CW] = {};
+#pragma unroll 1
+                for (int j = j0; j < min(j0 + FD_CHAIN, 8 * g); j += 4) {
+                    float4 p[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) p[i] = *reinterpret_cast<const float4*>(w + i * C::PP + j);
+                    for (int i = 0; i < 8; ++i) p[i] = *reinterpret_cast<const float4*>(w + i * C::PP + j);
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) {
-                    float f[CW];
-                    value(j + jj, f);
+                    for (int jj = 0; jj < 4; ++jj) {
+                        float f[CW];
+                        value(j + jj, f);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float x = jj == 0 ? p[i].x : jj == 1 ? p[i].y : jj == 2 ? p[i].z : p[i].w;
+                        for (int i = 0; i < 8; ++i) {
+                            const float x = jj == 0 ? p[i].x : jj == 1 ? p[i].y : jj == 2 ? p[i].z : p[i].w;
 #pragma unroll
-                        for (int e = 0; e < CW; ++e) o[i][e] = fmaf(x, f[e], o[i][e]);
+                            for (int e = 0; e < CW; ++e) t[i][e] = fmaf(x, f[e], t[i][e]);
+                        }
                     }
                 }
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int e = 0; e < CW; ++e) o[i][e] += t[i][e];
             }
+            float t[8][CW] = {};
 #pragma unroll
             for (int jj = 0; jj < 8; ++jj) {                    // the diagonal: rows from jj on
                 float f[CW];
@@ -658,9 +670,13 @@ f32_diagonal_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
                 for (int i = jj; i < 8; ++i) {
                     const float x = w[i * C::PP + 8 * g + jj];
 #pragma unroll
-                    for (int e = 0; e < CW; ++e) o[i][e] = fmaf(x, f[e], o[i][e]);
+                    for (int e = 0; e < CW; ++e) t[i][e] = fmaf(x, f[e], t[i][e]);
                 }
             }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int e = 0; e < CW; ++e) o[i][e] += t[i][e];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int row = 8 * g + i;

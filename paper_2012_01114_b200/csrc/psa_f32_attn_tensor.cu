@@ -21,7 +21,10 @@
 // What bounds it: per block of 64 keys 72 MMAs, 3072 cycles at d = 128 and 1536 at d = 64, beside about 1500 issue slots per scheduler of
 // softmax and splitting; the masked scheme also its longest row tiles and the diagonal tiles ahead of them (30 of its 76 us at 16
 // heads of n = 1024, d = 128).  Measured (us, CUDA cores before / whole call now): 16 heads of n = 1024, d = 128 FULL 308 / 54, MASKED
-// 166 / 76; 48 of n = 512, d = 64, FULL 111 / 42.  Error against 64 bits 1.6e-7 .. 3.1e-7, on CUDA cores 1.6e-7 .. 4.8e-7.
+// 166 / 77; 48 of n = 512, d = 64, FULL 111 / 42.
+// Error against 64 bits (relative, 2-norm; here / on CUDA cores; normal q, k, v): FULL 1.5e-7 .. 3.1e-7 / 2.1e-7 .. 4.8e-7, MASKED 1.4e-7 .. 2.4e-7 / 1.6e-7 ..
+// 2.6e-7, nowhere larger.  Where all values have one sign the tensor core's rounding towards zero adds up, 1.0e-7 .. 1.2e-7, against 0.85e-7 .. 3.4e-7: more
+// than on CUDA cores (by up to a quarter) only for FULL calls of few heads of up to 513 keys, whose sums those split in four.
 //
 // Roles (320 threads): warp 0 = TMA producer, warp 1 = MMA issuer, warps 2-9 = softmax, running output (a warp owns 16 rows, quad
 // layout of sm100.cuh).  S of the next block is computed during the softmax of a block, its PV during the softmax of the next.

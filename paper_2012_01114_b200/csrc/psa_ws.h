@@ -38,14 +38,17 @@ inline bool f32_project_pairs_fit(int rows, int D, int N, int nW, size_t bytes) 
 // 56 1.10, 79 0.82; d = 128 n = 257 29 1.04, 40 0.76, 53 1.12, 64 0.52; d = 32 n = 320 37 1.06, 63 0.78, n = 270 53 1.07; d = 8 n = 257 48 1.11, 64 0.80, 129 1.06,
 // n = 320 53 1.31, 66 0.90, 123 1.22.  Beyond: d = 64 n = 385 22 1.07, 24 0.77, n = 420 20 1.06; d = 32 n = 385 22 1.12, 24 0.85; d = 8 n = 513 17 1.06, 20 0.82, n = 385 40 1.02;
 // n = 640, d = 64 4 (100 blocks) 1.10, 12 0.86; n = 1024, d = 8 4 1.03, d = 64 4 0.80.
+// Nor do calls come here whose error against 64 bits would be larger: with 16 rows per CTA the CUDA cores add up the keys in four chains, and for
+// d > 80 on few keys that has less error than the tensor core's scores (FULL n = 192, d = 128 2.72e-7 and 2.80e-7, MASKED n = 385 2.07e-7 and 2.08e-7).
 inline bool f32_tensor_attention_fits(int B, int H, int n, int d, int scheme) {
     constexpr int SMS = 148;
     const long long heads = (long long)B * H, T = row_tiles(n), tiles = heads * T, blocks = tiles * T;
     if (scheme == PSA_SYMMETRIC || d % 8 != 0 || heads * n * d >= (1LL << 31)) return false;
+    const bool rows64 = heads * ((n + 63) / 64) >= 2 * SMS, rows32 = heads * ((n + 31) / 32) >= 2 * SMS;
+    if (d > 80 && !rows32 && n <= (scheme == PSA_FULL ? 255 : 450)) return false;
     if (scheme == PSA_FULL)
         return n >= (d >= 64 ? 160 : 256) && blocks >= (d < 16 && n <= 256 ? 80 : 64) && (d >= 32 || heads * n * n >= 34LL * TILE * TILE);
     if (n <= 256 || blocks < (d >= 64 ? 256 : 320)) return false;
-    const bool rows64 = heads * ((n + 63) / 64) >= 2 * SMS, rows32 = heads * ((n + 31) / 32) >= 2 * SMS;
     if (n <= 320) {
         if (d > 64) return rows32 && (tiles <= SMS || rows64);
         return d >= 32 ? rows64 || (n % 64 != 0 && rows32 && tiles <= SMS) : rows64 && tiles <= 2 * SMS;

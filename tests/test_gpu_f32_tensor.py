@@ -81,6 +81,31 @@ def test_large_values_under_a_lagging_maximum(scheme, power):
     _close(got / 2.0 ** power, ref / 2.0 ** power)
 
 
+# The same calls on the tensor cores and, in a registered workspace without room for their operands, on CUDA cores: the error against 64 bits is not
+# larger (5 % for the draw).  Values of one sign show sums that are rounded in long chains.
+@pytest.mark.parametrize("positive", [False, True])
+@pytest.mark.parametrize("H,n,d,scheme", [(40, 257, 64, oracle.MASKED), (31, 300, 128, oracle.MASKED), (8, 768, 128, oracle.MASKED), (16, 1024, 128, oracle.MASKED),
+                                          (48, 512, 64, oracle.FULL), (60, 193, 128, oracle.FULL), (2, 1024, 64, oracle.FULL)])
+def test_error_is_not_above_that_on_cuda_cores(H, n, d, scheme, positive):
+    g = torch.Generator(device="cuda").manual_seed(n + d)
+    q, k, v = [torch.empty(1, n, H, d, device="cuda").normal_(generator=g) for _ in range(3)]
+    if positive:
+        v = v.abs()
+    s = torch.einsum("bihc,bjhc->bhij", q.double(), k.double()) / d ** 0.5
+    if scheme == oracle.MASKED:
+        s = s.masked_fill(~torch.ones(n, n, dtype=torch.bool, device="cuda").tril(), float("-inf"))
+    ref = torch.einsum("bhij,bjhc->bihc", torch.softmax(s, -1), v.double()).reshape(1, n, H * d)
+    assert binding.psa_workspace_bytes(1, H, n, 0, d, scheme, binding.F32) > 4096          # (a call of the tensor cores)
+    error = [float((binding.psa_attention_core(q, k, v, scheme).double() - ref).norm())]
+    try:
+        binding.psa_set_workspace(torch.empty(4096, dtype=torch.uint8, device="cuda"))
+        error.append(float((binding.psa_attention_core(q, k, v, scheme).double() - ref).norm()))
+        torch.cuda.synchronize()
+    finally:
+        binding.psa_set_workspace(None)
+    assert error[0] <= 1.05 * error[1], [e / float(ref.norm()) for e in error]
+
+
 # Projections of the largest calls (pairs of CTAs, 256 x 256 tiles, 64 k at a time): ragged rows, columns and depth, tiny and
 # infinite operands.  With one vector per sequence the attention returns V.  Bound: six bf16 products per fp32 product leave 2^-24 of it
 # out, sums are rounded every 64 k: (K / 64 + 4) 2^-24 of the sum of magnitudes.
