@@ -30,8 +30,8 @@ def _close(got, ref, rel=4e-6):
 
 
 @pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
-@pytest.mark.parametrize("B,H,n,d", [(2, 10, 161, 64), (4, 8, 256, 8), (2, 10, 193, 128), (2, 8, 257, 72), (4, 9, 300, 40), (1, 4, 1024, 120), (1, 6, 1000, 16), (3, 4, 513, 64), (1, 9, 705, 128),
-                                     (2, 20, 384, 8)])
+@pytest.mark.parametrize("B,H,n,d", [(2, 10, 161, 64), (4, 8, 256, 8), (2, 10, 193, 128), (2, 30, 193, 128), (2, 8, 257, 72), (4, 9, 300, 40), (1, 4, 1024, 120), (1, 6, 1000, 16), (3, 4, 513, 64), (1, 9, 705, 128),
+                                     (2, 20, 384, 8), (2, 32, 257, 64), (1, 41, 257, 128), (3, 13, 300, 48), (1, 24, 385, 32), (7, 3, 513, 8), (1, 16, 385, 64)])
 def test_edges(scheme, B, H, n, d):
     _close(*_run(B, H, n, d, scheme))
 
@@ -147,3 +147,46 @@ def test_projections_of_host_calls_in_parts():
     assert st == binding.OK and got == binding.psa_skip_count(rows, H, 1, D, d, binding.FULL, binding.F32)
     want = binding.psa_attention_f32(X.cuda(), Wq.cuda(), Wk.cuda(), Wv.cuda(), H, binding.FULL)
     assert torch.equal(out, want.cpu())
+
+
+@pytest.mark.parametrize("rows,D,H,d", [(2056, 768, 12, 64), (2100, 328, 16, 64), (1030, 776, 33, 32)])
+def test_all_three_projections_of_large_calls(rows, D, H, d):
+    # two vectors per sequence: the weights depend on q and k, so that a wrong tile of any of the three shows.  Scores of size 1 to 5:
+    # 2^-24 times that and the projections' error, 4e-6 as above
+    X, Wq, Wk, Wv = [inputs.tensor(rows + D, i, s, f, "f32")[1] for i, (s, f) in enumerate([((rows, 2, D), 1.0)] + [((D, H * d), D ** -0.5)] * 3)]
+    X[7] *= np.float32(1e-36)
+    Wq[3, :40] *= np.float32(1e-36)
+    Wk[5, -40:] *= np.float32(1e-36)
+    z = binding.psa_attention_f32(*[torch.from_numpy(t).cuda() for t in (X, Wq, Wk, Wv)], H, binding.FULL)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got == binding.psa_skip_count(rows, H, 2, D, d, binding.FULL, binding.F32)
+    q, k, v = [(X.astype(np.float64).reshape(2 * rows, D) @ W.astype(np.float64)).reshape(rows, 2, H, d) for W in (Wq, Wk, Wv)]
+    s = np.einsum("bihc,bjhc->bhij", q, k) / np.sqrt(d)
+    w = np.exp(s - s.max(-1, keepdims=True))
+    ref = np.einsum("bhij,bjhc->bihc", w / w.sum(-1, keepdims=True), v).reshape(rows, 2, H * d)
+    _close(z.cpu().numpy().astype(np.float64), ref)
+
+
+@pytest.mark.parametrize("residual", [False, True])
+@pytest.mark.parametrize("rows,D,H,d", [(4111, 768, 12, 64), (6500, 328, 9, 40)])
+def test_output_projection_of_large_blocks(rows, D, H, d, residual):
+    # one vector per sequence: y = X Wv.  Bound: that of the projections twice, the first one carried through |Wo|, and the rounding of z
+    X, Wq, Wk, Wv, Wo = [inputs.tensor(rows + D, i, s, f, "f32")[1] for i, (s, f) in
+                         enumerate([((rows, 1, D), 1.0)] + [((D, H * d), D ** -0.5)] * 3 + [((H * d, D), (H * d) ** -0.5)])]
+    X[7] *= np.float32(1e-36)
+    X[300, 0, 5] = np.inf
+    Wo[9, 20:60] *= np.float32(1e-36)
+    R = inputs.tensor(rows, 9, (rows, 1, D), 1.0, "f32")[1]
+    dev = [torch.from_numpy(t).cuda() for t in (X, Wq, Wk, Wv, Wo, R)]
+    z = binding.psa_attention_block(*dev[:5], H, binding.FULL, residual=dev[5] if residual else None)
+    st, _ = binding.psa_last_issued()
+    assert st == binding.OK
+    z = z.cpu().numpy().reshape(rows, D).astype(np.float64)
+    assert not np.isfinite(z[300]).any()
+    x, wv, wo, r = X.reshape(rows, D).astype(np.float64), Wv.astype(np.float64), Wo.astype(np.float64), R.reshape(rows, D).astype(np.float64) * residual
+    x[300], z[300], r[300] = 0.0, 0.0, 0.0
+    y = x @ wv
+    ey = (D / 64 + 4) * 2.0 ** -24 * (np.abs(x) @ np.abs(wv))
+    ref = y @ wo + r
+    bound = ey @ np.abs(wo) + (H * d / 64 + 4) * 2.0 ** -24 * ((np.abs(y) + ey) @ np.abs(wo)) + 2.0 ** -23 * np.abs(ref) + 1e-44
+    assert (np.abs(z - ref) <= bound).all()

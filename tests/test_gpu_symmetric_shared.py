@@ -64,7 +64,10 @@ def test_large_scores_in_some_heads(n, d):
     out = binding.psa_attention_core(x.repeat(B, 1, 1, 1), None, None, binding.SYMMETRIC)
     _census(B, H, n, d)
     ref, _ = oracle.attention_core(v, v, v, oracle.SYMMETRIC)
-    _check(out[:1], ref, TOL * 12.0)
+    # outputs of head 1 reach 12 times the size, of head 2 8 times; the others keep the plain bound
+    y, r = out[0].view(n, H, d), ref.reshape(n, H, d)
+    for h, size in enumerate((1.0, 12.0, 8.0, 1.0)):
+        _check(y[:, h], r[:, h], TOL * size)
     assert binding.psa_last_rescales() > 0 and (out == out[:1]).all()
 
 
