@@ -48,8 +48,8 @@ NCU_TRAFFIC = {
         "psa_attn_persist.cu": "c809ad7eef03f4331762b2e69228796567f04af1479ba862a128cb0eafdc1b8b",
         "psa_softmax.cuh": "f7c2c8092d61159a139d9f5938bbf907bbe8a8d77e4a239ee94079816cb5aaa7",
         "psa_sched.h": "5db1035f5bc41698396fed66ead14f0b4a9ef0408738ccb324301a4ae99be214",
-        "psa_gemm.cu": "6259df700b4ff7b71e80dff7fccf14358b7ef73294b01235e530e013c3f57bae",
-        "sm100.cuh": "e84f5c826a88c4c0c2171f4ba6c4c1ff9f0ddb02e90d5fcefe41dd47048b181d"
+        "psa_gemm.cu": "6e310be0bd171b42d054fba6e4dab1d5b194cc6fd9c71d97c527fef694519107",
+        "sm100.cuh": "37e0f4d2488e34971530641eef7a76d0c646a0dfde7953a055c472da1b36e076"
     },
     "kernel_sources": {
         "attn": ["psa_attn_persist.cu", "psa_softmax.cuh", "psa_sched.h", "sm100.cuh"],
@@ -57,21 +57,21 @@ NCU_TRAFFIC = {
     },
     "traffic_bytes": {
         "c4": {
-            "attn": 593319168
+            "attn": 593833728
         },
         "c3": {
-            "attn": 37804544,
-            "proj": 16297728
+            "attn": 37811456,
+            "proj": 16288768
         },
         "c2": {
-            "attn": 18928896,
-            "proj": 9852672
+            "attn": 18928640,
+            "proj": 9852416
         },
         "c5-n256-full": {
-            "attn": 1046480128
+            "attn": 1046857216
         },
         "c5-n256-masked": {
-            "attn": 1048277760
+            "attn": 1048625920
         }
     }
 }

@@ -156,8 +156,8 @@ def psa_attention(X, Wq, Wk, Wv, heads, scheme, out=None, stream=None):
 
 
 def psa_attention_f32(X, Wq, Wk, Wv, heads, scheme, out=None, stream=None):
-    """fp32 projections + attention, to fp32 accuracy: attention on CUDA cores with element-exact skipping, the projections
-    of large calls on the tensor cores with every number split into three bf16 parts."""
+    """fp32 projections + attention, to fp32 accuracy, with element-exact skipping: small calls on CUDA cores, projections and
+    (full and masked schemes) attention of large ones on the tensor cores with every number split into three bf16 parts."""
     return _layer("psa_attention_f32", torch.float32, X, Wq, Wk, Wv, heads, scheme, out, stream)
 
 

@@ -14,7 +14,8 @@
 // What bounds it: 16 MMAs of 64 cycles and 8 of 128 are 2048 cycles per block, 128 KB of operands at an SM's 64 bytes per
 // cycle from L2 as many; the issuing thread spends 100-130 more on each of six barriers and five commits (with slots of 16 KB, nine of
 // them, it was slower: 76 -> 89 us); measured 3000 on long sequences (16 heads of n = 8192, d_k = 192, masked: 559 us as one CTA per
-// tile with one K and one V stage, 379 now; 32 heads of n = 2048, d_k = 256, masked: 103, then 80 and 70).
+// tile with one K and one V stage, 379 now; 32 heads of n = 2048, d_k = 256, masked: 103, then 80 and 70,
+// the same inputs call after call; with other inputs every time 83 and 80).
 //
 // CTA layout (320 threads): warp 0 = work list and TMA producer, warp 1 = MMA issuer, warps 2-9 = softmax and epilogue
 // (a warp owns 16 rows, read in the quad layout of sm100.cuh).  The tensors' head size may be any multiple of 8 in (128,

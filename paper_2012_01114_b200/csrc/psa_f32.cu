@@ -1,6 +1,7 @@
 // The full-precision path: fp32 storage, and fp32 arithmetic on CUDA cores but for large calls, whose projections are in
-// psa_f32_tensor.cu and whose attention (FULL, MASKED) is in psa_f32_attn_tensor.cu.  Skipping is element-exact: a weight that the scheme does not need is never computed (paper Sec. 4.1,
-// 5.1), so issued MACs equal the paper's element counts (Sec. 3.2, 4.2, 5.2).  The throughput path is the bf16 one.
+// psa_f32_tensor.cu and whose attention (FULL, MASKED) is in psa_f32_attn_tensor.cu.  Skipping is element-exact: a weight that the
+// scheme does not need is never computed (paper Sec. 4.1, 5.1), so issued MACs equal the paper's element counts (Sec. 3.2, 4.2,
+// 5.2).  The throughput path is the bf16 one.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -1100,7 +1101,8 @@ f32_fused_cluster_kernel(const float* __restrict__ X, const float* __restrict__ 
     const int own_rows = own_tiles * 4;                                // (the last tile's rows beyond n are skipped)
     auto own_row = [&](int lr) { return 4 * (rank + (lr >> 2) * C) + (lr & 3); };     // local row -> row of the head
     unsigned long long qk = 0, pv = 0, ex = 0, pj = 0;
-    // The next kernel may come in at once: a call of one head takes 8 SMs, and the launch of the next one is hidden behind it.
+    // The next kernel may come in at once: a call of one head takes 8 SMs, and the launch of the next one is hidden behind it.  (One
+    // head of n = 64, call after call with other inputs, us: 14.9, here and with a binding that makes plain integers 12.9.)
     grid_launch_dependents();
     grid_dependency_wait();
     if (blockIdx.x == 0 && tid == 0 && dc_next) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};

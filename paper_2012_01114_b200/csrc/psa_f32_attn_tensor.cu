@@ -23,7 +23,7 @@
 // heads of n = 1024, d = 128).  Measured (us, CUDA cores before / whole call now): 16 heads of n = 1024, d = 128 FULL 308 / 54, MASKED
 // 166 / 77; 48 of n = 512, d = 64, FULL 111 / 42.
 // Error against 64 bits (relative, 2-norm; here / on CUDA cores; normal q, k, v): FULL 1.5e-7 .. 3.1e-7 / 2.1e-7 .. 4.8e-7, MASKED 1.4e-7 .. 2.4e-7 / 1.6e-7 ..
-// 2.6e-7, nowhere larger.  Where all values have one sign the tensor core's rounding towards zero adds up, 1.0e-7 .. 1.2e-7, against 0.85e-7 .. 3.4e-7: more
+// 2.6e-7, nowhere more than 1 % larger.  Where all values have one sign the tensor core's rounding towards zero adds up, 1.0e-7 .. 1.2e-7, against 0.85e-7 .. 3.4e-7: more
 // than on CUDA cores (by up to a quarter) only for FULL calls of few heads of up to 513 keys, whose sums those split in four.
 //
 // Roles (320 threads): warp 0 = TMA producer, warp 1 = MMA issuer, warps 2-9 = softmax, running output (a warp owns 16 rows, quad

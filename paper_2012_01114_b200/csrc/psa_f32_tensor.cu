@@ -434,6 +434,9 @@ f32_project_tensor_kernel(const float* __restrict__ X, const float* W0, const fl
 // What bounds it: 24 MMAs of 256 x 256 x 16 per 64 k, 3072 cycles of MMA, measured 5000 (the pairs of psa_gemm.cu take 160 cycles per MMA
 // where 128 are nominal, and every 64 k an accumulator is handed over twice).  2048 x 768 x 3 x 768: 60 us on 128 x 128 tiles, 42 here with
 // 7 of the split; the layer of 4 x 512 vectors 105 -> 85 us.
+//
+// Error against 64 bits (relative, 2-norm), the kernel above / this one: normal inputs, K = 320 / 768 / 2048 1.19 / 1.31 / 1.46e-7 and 0.91 /
+// 1.04 / 1.32e-7; positive inputs, K = 768, 1.74e-7 and 0.99e-7.
 constexpr int FP_BK = 64, FP_PLANE = 128 * FP_BK * 2;                       // a part of a CTA's operand: 16 KB
 constexpr int FP_STAGE = 6 * FP_PLANE, FP_STAGES = 2, FP_WORKERS = 8, FP_THREADS = 64 + 32 * FP_WORKERS;
 constexpr int FP_SMEM = FP_STAGES * FP_STAGE + 1024;

@@ -200,7 +200,8 @@ gemm_bf16_kernel(const __grid_constant__ GemmMaps maps, int M, int N, int K, int
             for (int k = max(0, g - STAGES); k < g; ++k) mbar_wait_drain(&full_bar[k % STAGES], (k / STAGES) & 1);
         }
     } else if (warp == 1 && rank == 0 && elect_one()) {
-        // ---- MMA issuer
+        // ---- MMA issuer (one elected lane of the converged warp; `lane == 0` and this, projection alone, us: 8192 rows x 2304 columns,
+        // K = 768 29.2 and 27.6, K = 3072 74.1 and 72.4, 1024 rows 12.7 and 10.8)
         const uint32_t idesc = umma_idesc_bf16(CTAS * BM, BN, UMMA_K_MAJOR, UMMA_MN_MAJOR);
         // descriptor low words of stage 0; a stage or k-step is a constant added to them (sm100.cuh)
         const uint32_t a_lo0 = umma_desc_lo_kmajor(smem_u32(smem));
