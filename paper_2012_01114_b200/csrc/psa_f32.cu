@@ -4,9 +4,11 @@
 // 5.2).  The throughput path is the bf16 one.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "psa_internal.h"
+#include "psa_sched.h"
 #include "psa_ws.h"
 #include "sm100.cuh"
 
@@ -1076,176 +1078,261 @@ f32_fused_layer_kernel(const float* __restrict__ X, const float* __restrict__ Wq
 }
 
 // The same layer spread over a cluster of C CTAs (FULL and MASKED): 4-row tiles are dealt to the CTAs in turn (tile ti
-// belongs to CTA ti % C, which balances the masked scheme's growing rows), each CTA projects q, k, v of its own rows,
-// the CTAs read one another's k and v through distributed shared memory, and each finishes phases 1-3 for its rows.
-// A layer of one head then occupies C SMs instead of one.  Tasks are one row by four columns, so that the few rows a
-// CTA owns still spread over its threads; the census is element-exact as above.
-__global__ void __launch_bounds__(FS_THREADS, 1)
+// belongs to CTA ti % C, which balances the masked scheme's growing rows), each CTA projects q, k, v of its own rows, writes k
+// and v into the shared memory of every CTA of the cluster, and finishes phases 1-3 for its rows.  A layer of one head then
+// occupies C SMs instead of one.  The census is element-exact as above.
+//
+// What bounds it: latency.  A call of one head of n = 64, d_model = d = 64 is eight phases of one or two thousand cycles between barriers
+// (clock stamps: first loads 2200, projections 2700, k and v to the other CTAs 1200 and their barrier 1200 .. 2700, phases 1-3 2200, 1100, 1300,
+// output 1100).  So a phase is spread over all warps, sums in parts, loops have several loads in flight and no branch inside (with one per
+// step the projections took 4100, phase 1 3500), and k and v rows are pushed (fetched by the CTAs that need them they took two barriers of the
+// cluster and a pass of 3100 .. 4600).  The layout comes from the host, indices are divided by multiplication.
+// Measured (us a call, among calls with other inputs; before / now): 1 head of n = 64, d = 64 masked 12.9 / 8.3, FULL 11.2 / 8.4; 12 heads FULL 11.8 / 8.6, 20 heads 22.6 / 10.9.
+struct ClusterLayout {
+    int ld, s_ld;                            // row pitches: q, k, v; weights, kept as [key][own row]
+    int tiles, group;                        // row tiles of a CTA (at most), rows that a task of the projections takes
+    int keys;                                // keys that a warp takes in phase 1
+    int splits, y_splits;                    // parts that a sum over components, over keys is taken in
+    int xs, ws, part, qs, ks, vs, sm, rinv, y;
+    size_t total;
+    FastDiv by_columns, by_columns4, by_d, by_d4, by_key_groups, by_blocks;    // 3 d, 3 d / 4, d, d / 4, groups of keys, 32-column blocks
+};
+constexpr int FC_SPLITS = 8;
+constexpr size_t FC_HALF_SM = 113 * 1024;     // shared memory of a CTA that leaves room for a second one
+inline ClusterLayout cluster_layout(int n, int D, int d, int C) {
+    ClusterLayout L;
+    L.tiles = ((n + 3) / 4 + C - 1) / C;
+    L.group = L.tiles == 1 ? 4 : 8;
+    L.ld = 4 * ((d / 4 + 1) | 1); L.s_ld = 4 * (L.tiles | 1);       // (odd numbers of 16 bytes: neighbouring rows lie in other banks)
+    const int groups = (L.tiles + 1) / 2, rows = L.group * groups, blocks = L.tiles * ((d + 31) / 32), cols = 3 * d;
+    L.keys = 8;                              // (four lanes to a key where one round of the warps does)
+    while (L.keys < 32 && L.tiles * ((n + L.keys - 1) / L.keys) > FS_THREADS / 32) L.keys *= 2;
+    L.y_splits = 1;
+    while (2 * L.y_splits <= FC_SPLITS && 2 * L.y_splits * blocks <= FS_THREADS / 32) L.y_splits *= 2;
+    L.xs = 0; L.ws = rows * D;
+    L.sm = 0; L.rinv = n * L.s_ld; L.y = L.rinv + 4 * L.tiles;      // (these and q over x and W, once the projections are done)
+    L.qs = L.y + L.y_splits * 4 * L.tiles * d;
+    const int inputs = L.ws + cols * D, later = L.qs + rows * L.ld;
+    L.ks = inputs > later ? inputs : later;
+    L.vs = L.ks + n * L.ld;
+    L.part = L.vs + n * L.ld;
+    L.splits = 1;                            // (8 components each at least)
+    while (2 * L.splits <= FC_SPLITS && 2 * L.splits * cols * groups <= FS_THREADS && 16 * L.splits <= D &&
+           L.part + 2 * L.splits * rows * cols <= FS_MAX_FLOATS)
+        L.splits *= 2;
+    L.total = (size_t)L.part + L.splits * rows * cols;
+    L.by_columns = fastdiv_make(cols); L.by_columns4 = fastdiv_make(cols / 4); L.by_d = fastdiv_make(d); L.by_d4 = fastdiv_make(d / 4);
+    L.by_key_groups = fastdiv_make((n + L.keys - 1) / L.keys); L.by_blocks = fastdiv_make((d + 31) / 32);
+    return L;
+}
+
+__global__ void __launch_bounds__(FS_THREADS, 2)
 f32_fused_cluster_kernel(const float* __restrict__ X, const float* __restrict__ Wq, const float* __restrict__ Wk,
                          const float* __restrict__ Wv, float* __restrict__ out, int n, int H, int D, int d, float scale,
-                         int scheme, DeviceCounters* dc, DeviceCounters* dc_next) {
+                         int scheme, DeviceCounters* dc, DeviceCounters* dc_next, const __grid_constant__ ClusterLayout L) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     extern __shared__ float4 fs_smem4[];
     float* sm = reinterpret_cast<float*>(fs_smem4);
-    const FusedLayout L = fused_layout(n, D, d, 3);
-    float* xs = sm + L.xs; float* ws = sm + L.ws; float* qt = sm + L.qt; float* kt = sm + L.kt; float* vs = sm + L.vs;
-    float* S = sm + L.sm; float* rinv = sm + L.rinv;
+    float* xs = sm + L.xs; float* ws = sm + L.ws; float* part = sm + L.part; float* qs = sm + L.qs; float* ks = sm + L.ks; float* vs = sm + L.vs;
+    float* S = sm + L.sm; float* rinv = sm + L.rinv; float* ypart = sm + L.y;
     const int head = blockIdx.x / C, b = head / H, h = head - b * H;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int WARPS = FS_THREADS / 32;
     const bool masked = scheme == PSA_MASKED;
     const size_t HD = (size_t)H * d;
-    const int tn = (n + 3) / 4, tc = d / 4;
+    const int tn = (n + 3) / 4;
     const int own_tiles = rank < tn ? (tn - rank + C - 1) / C : 0;     // tiles rank, rank + C, ...
-    const int own_rows = own_tiles * 4;                                // (the last tile's rows beyond n are skipped)
+    const int own_rows = 4 * own_tiles;                                // (rows beyond n, in the last tile only, are skipped)
     auto own_row = [&](int lr) { return 4 * (rank + (lr >> 2) * C) + (lr & 3); };     // local row -> row of the head
-    unsigned long long qk = 0, pv = 0, ex = 0, pj = 0;
-    // The next kernel may come in at once: a call of one head takes 8 SMs, and the launch of the next one is hidden behind it.  (One
-    // head of n = 64, call after call with other inputs, us: 14.9, here and with a binding that makes plain integers 12.9.)
+    const int valid_rows = own_tiles == 0 ? 0 : own_rows - max(0, own_row(own_rows - 1) + 1 - n);
+    // The next kernel may come in at once: a call of one head takes 8 SMs, and the launch of the next one is hidden behind it.
     grid_launch_dependents();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // (every CTA has started: waited for ahead of the first remote store)
     grid_dependency_wait();
     if (blockIdx.x == 0 && tid == 0 && dc_next) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};
 
-    // ---- stage this CTA's rows of X[b] and the head's columns of the three projection matrices: asynchronous copies
-    // straight into shared memory, all in flight at once (a layer this small lives on the latency of its first loads)
+    // ---- stage this CTA's rows of X[b], as [group of rows][component][row], and the head's columns of the three projection matrices:
+    // asynchronous copies, all in flight at once (a layer this small lives on the latency of its first loads)
+    const int d4 = d / 4, gr = L.group, groups = (own_tiles + 1) / 2;
     {
         const float* xb = X + (size_t)b * n * D;
-        for (int t = tid; t < own_rows * D; t += FS_THREADS) {
-            const int lr = t / D, k = t - lr * D, i = own_row(lr);
-            if (i < n) cp_async4(xs + i * L.xs_ld + k, xb + (size_t)i * D + k);
+        for (int lr = warp; lr < gr * groups; lr += WARPS) {
+            const int i = own_row(lr);
+            const bool have = lr < valid_rows;
+            float* dst = xs + (lr & -gr) * D + (lr & (gr - 1));
+            for (int k = lane; k < D; k += 32) {
+                if (have) cp_async4(dst + gr * k, xb + (size_t)i * D + k);
+                else dst[gr * k] = 0.f;
+            }
         }
-        const int d4 = d / 4;
-        for (int t = tid; t < 3 * D * d4; t += FS_THREADS) {
-            const int w = t / (D * d4), rem = t - w * D * d4, k = rem / d4, c4 = rem - k * d4;
-            const float* W = (w == 0 ? Wq : (w == 1 ? Wk : Wv)) + (size_t)h * d;
-            cp_async16(ws + (size_t)w * D * d + (size_t)k * d + 4 * c4, W + (size_t)k * HD + 4 * c4);
+        const int dk = fastdiv(FS_THREADS, L.by_d4), dc4 = FS_THREADS - dk * d4;
+        int k = fastdiv(tid, L.by_d4), c4 = tid - k * d4;
+        while (k < 3 * D) {
+            const float* W = k < D ? Wq : k < 2 * D ? Wk - (size_t)D * HD : Wv - (size_t)2 * D * HD;
+            cp_async16(ws + k * d + 4 * c4, W + (size_t)k * HD + (size_t)h * d + 4 * c4);
+            k += dk; c4 += dc4;
+            if (c4 >= d4) { c4 -= d4; ++k; }
         }
         cp_async_wait_all();
     }
     __syncthreads();
 
-    // ---- projections (Sec. 3.1) of the own rows: one row by four columns per task
-    for (int t = tid; t < 3 * own_rows * tc; t += FS_THREADS) {
-        const int w = t / (own_rows * tc), rem = t - w * own_rows * tc;
-        const int lr = rem / tc, c0 = (rem - lr * tc) * 4, i = own_row(lr);
-        if (i >= n) continue;
-        const float* wp = ws + (size_t)w * D * d + c0;
-        const float* xr = xs + (size_t)i * L.xs_ld;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    // ---- projections (Sec. 3.1) of the own rows.  A task is one column of q, k or v for a group of rows and a part of the D components.
+    const int splits = L.splits, step = (D + splits - 1) / splits, cols = 3 * d;
+    for (int t = tid; t < cols * groups * splits; t += FS_THREADS) {
+        const int rest = fastdiv(t, L.by_columns), col = t - rest * cols, g = rest >> __ffs(splits) - 1, p = rest & (splits - 1), which = fastdiv(col, L.by_d);
+        const int k0 = p * step, k1 = min(D, k0 + step);
+        const float* w = ws + (which * D + k0) * d + (col - which * d);
+        float* dst = part + (p * groups + g) * gr * cols + col;
+        auto rows = [&](auto rg_tag, const float* x) {
+            constexpr int RG = decltype(rg_tag)::value;
+            float acc[RG] = {};
 #pragma unroll 8
-        for (int k = 0; k < D; ++k) {
-            const float4 wv = *reinterpret_cast<const float4*>(wp + (size_t)k * d);
-            const float x = xr[k];
-            acc.x = fmaf(x, wv.x, acc.x); acc.y = fmaf(x, wv.y, acc.y); acc.z = fmaf(x, wv.z, acc.z); acc.w = fmaf(x, wv.w, acc.w);
-        }
-        if (w < 2) {
-            float* dst = (w == 0 ? qt : kt) + i;
-            dst[(size_t)(c0 + 0) * L.t_ld] = acc.x; dst[(size_t)(c0 + 1) * L.t_ld] = acc.y;
-            dst[(size_t)(c0 + 2) * L.t_ld] = acc.z; dst[(size_t)(c0 + 3) * L.t_ld] = acc.w;
-        } else {
-            *reinterpret_cast<float4*>(vs + (size_t)i * L.ds + c0) = acc;
-        }
-        pj += 4ull * D;
-    }
-    cluster.sync();           // every CTA's k and v rows are in its shared memory
-
-    // ---- k and v of the other CTAs' rows, one 4-row tile (16 bytes of a transposed k component; a row of v) at a time
-    for (int t = tid; t < d * tn; t += FS_THREADS) {
-        const int c = t / tn, ti = t - c * tn, owner = ti % C;
-        if (owner == rank) continue;
-        const float* src = cluster.map_shared_rank(kt, owner);
-        *reinterpret_cast<float4*>(kt + (size_t)c * L.t_ld + 4 * ti) = *reinterpret_cast<const float4*>(src + (size_t)c * L.t_ld + 4 * ti);
-    }
-    for (int t = tid; t < n * tc; t += FS_THREADS) {
-        const int i = t / tc, c0 = (t - i * tc) * 4, owner = (i >> 2) % C;
-        if (owner == rank) continue;
-        const float* src = cluster.map_shared_rank(vs, owner);
-        *reinterpret_cast<float4*>(vs + (size_t)i * L.ds + c0) = *reinterpret_cast<const float4*>(src + (size_t)i * L.ds + c0);
-    }
-    cluster.sync();           // no CTA reads another's shared memory from here on
-
-    // ---- phase 1 (Eq. 1) for the own rows: S_ij = scale q_i . k_j, one row by four keys per task; a key beyond the
-    // row's last kept one (masked: j > i; the edge: j >= n) is never computed
-    for (int t = tid; t < own_rows * tn; t += FS_THREADS) {
-        const int lr = t / tn, j0 = (t - lr * tn) * 4, i = own_row(lr);
-        if (i >= n) continue;
-        const int jlast = masked ? i : n - 1;
-        if (j0 > jlast) continue;
-        const int cnt = min(4, jlast - j0 + 1);                   // keys j0 .. j0 + cnt - 1 are kept
-        const float* qp = qt + i;
-        const float* kp = kt + j0;
-        float* row = S + (size_t)i * L.s_ld + j0;
-        if (cnt == 4) {
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-            for (int c = 0; c < d; ++c) {
-                const float q = qp[(size_t)c * L.t_ld];
-                const float4 k4 = *reinterpret_cast<const float4*>(kp + (size_t)c * L.t_ld);
-                acc.x = fmaf(q, k4.x, acc.x); acc.y = fmaf(q, k4.y, acc.y); acc.z = fmaf(q, k4.z, acc.z); acc.w = fmaf(q, k4.w, acc.w);
+            for (int k = k0; k < k1; ++k, w += d, x += RG) {
+                const float wk = *w;
+#pragma unroll
+                for (int r = 0; r < RG; r += 4) {
+                    const float4 f = *reinterpret_cast<const float4*>(x + r);
+                    acc[r] = fmaf(f.x, wk, acc[r]); acc[r + 1] = fmaf(f.y, wk, acc[r + 1]);
+                    acc[r + 2] = fmaf(f.z, wk, acc[r + 2]); acc[r + 3] = fmaf(f.w, wk, acc[r + 3]);
+                }
             }
-            row[0] = acc.x * scale; row[1] = acc.y * scale; row[2] = acc.z * scale; row[3] = acc.w * scale;
+#pragma unroll
+            for (int r = 0; r < RG; ++r) dst[r * cols] = acc[r];
+        };
+        if (gr == 4) rows(std::integral_constant<int, 4>{}, xs + 4 * (g * D + k0));
+        else rows(std::integral_constant<int, 8>{}, xs + 8 * (g * D + k0));
+    }
+    __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    // ---- the parts added up, four columns at a time: q stays here, k and v go to every CTA
+    const int c4 = cols / 4;
+    for (int t = tid; t < valid_rows * c4; t += FS_THREADS) {
+        const int lr = fastdiv(t, L.by_columns4), q4 = t - lr * c4, i = own_row(lr);
+        float4 s = *reinterpret_cast<const float4*>(part + lr * cols + 4 * q4);
+        for (int p = 1; p < splits; ++p) {
+            const float4 v = *reinterpret_cast<const float4*>(part + (p * groups * gr + lr) * cols + 4 * q4);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        const int which = fastdiv(q4, L.by_d4), c = 4 * (q4 - which * d4);
+        if (which == 0) {
+            *reinterpret_cast<float4*>(qs + lr * L.ld + c) = s;
         } else {
-            for (int u = 0; u < cnt; ++u) {
-                float acc = 0.f;
-                for (int c = 0; c < d; ++c) acc = fmaf(qp[(size_t)c * L.t_ld], kp[(size_t)c * L.t_ld + u], acc);
-                row[u] = acc * scale;
+            float* dst = (which == 1 ? ks : vs) + i * L.ld + c;
+            for (int r = 0; r < C; ++r) *reinterpret_cast<float4*>(cluster.map_shared_rank(dst, r)) = s;
+        }
+    }
+    cluster.sync();           // every k and v row is here; no CTA reaches into another's shared memory from here on
+
+    // ---- census of this CTA's rows: i + 1 (masked) or n weights each
+    if (warp == 0) {
+        unsigned pairs = 0;
+        for (int lr = lane; lr < valid_rows; lr += 32) pairs += masked ? own_row(lr) + 1 : n;
+        pairs = __reduce_add_sync(0xffffffffu, pairs);
+        if (lane == 0 && pairs) {
+            atomicAdd(&dc->qk_macs, (unsigned long long)pairs * d);
+            atomicAdd(&dc->pv_macs, (unsigned long long)pairs * d);
+            atomicAdd(&dc->exps, (unsigned long long)pairs);
+            atomicAdd(&dc->proj_macs, (unsigned long long)valid_rows * cols * D);
+        }
+    }
+    // ---- phase 1 (Eq. 1): S_ij = scale q_i . k_j.  A warp takes 32, 16 or 8 keys for the four rows of a tile; the lanes that share a key each
+    // have every so-manieth group of four components.  A weight beyond the row's last kept key (masked: j > i; the edge) is never computed.
+    const int keys = L.keys, lanes = 32 / keys, key_groups = (n + keys - 1) / keys;
+    for (int unit = warp; unit < own_tiles * key_groups; unit += WARPS) {
+        const int tile = fastdiv(unit, L.by_key_groups), j = keys * (unit - tile * key_groups) + (lane & (keys - 1)), p = lane / keys, i0 = own_row(4 * tile);
+        const int first = masked ? max(0, j - i0) : 0, last = j < n ? min(4, n - i0) : 0;     // rows first .. last - 1 of the tile keep key j
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        if (first < last) {
+            const float* k = ks + j * L.ld;
+            const float* q = qs + 4 * tile * L.ld;
+#pragma unroll 4
+            for (int c = 4 * p; c < d; c += 4 * lanes) {
+                const float4 kv = *reinterpret_cast<const float4*>(k + c);
+                float4 qv[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) qv[r] = *reinterpret_cast<const float4*>(q + r * L.ld + c);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (r >= first && r < last) {
+                        acc[r] = fmaf(qv[r].x, kv.x, acc[r]); acc[r] = fmaf(qv[r].y, kv.y, acc[r]);
+                        acc[r] = fmaf(qv[r].z, kv.z, acc[r]); acc[r] = fmaf(qv[r].w, kv.w, acc[r]);
+                    }
             }
         }
-        qk += (unsigned long long)cnt * d;
+        for (int off = keys; off < 32; off *= 2) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], off);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (r >= first && r < last && (r & (lanes - 1)) == p) S[j * L.s_ld + 4 * tile + r] = acc[r] * scale;
     }
     __syncthreads();
 
     // ---- phase 2 (Eq. 2): one warp per own row; the division is applied to the output row
-    for (int lr = warp; lr < own_rows; lr += FS_THREADS / 32) {
-        const int i = own_row(lr);
-        if (i >= n) continue;
-        const int jend = masked ? i + 1 : n;
-        float* row = S + (size_t)i * L.s_ld;
+    for (int lr = warp; lr < valid_rows; lr += WARPS) {
+        const int jend = masked ? own_row(lr) + 1 : n;
+        float* row = S + lr;
         float mx = -INFINITY;
-        for (int j = lane; j < jend; j += 32) mx = fmaxf(mx, row[j]);
+        for (int j = lane; j < jend; j += 32) mx = fmaxf(mx, row[j * L.s_ld]);
         for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
         float sum = 0.f;
         for (int j = lane; j < jend; j += 32) {
-            const float e = expf(row[j] - mx);
-            row[j] = e;
+            const float e = expf(row[j * L.s_ld] - mx);
+            row[j * L.s_ld] = e;
             sum += e;
         }
         for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-        if (lane == 0) { rinv[i] = 1.f / sum; ex += (unsigned long long)jend; }
+        if (lane == 0) rinv[lr] = 1.f / sum;
     }
     __syncthreads();
 
-    // ---- phase 3 (Eq. 3): y_i = sum_j w_ij v_j over the kept weights, four output components per task
-    for (int t = tid; t < own_rows * tc; t += FS_THREADS) {
-        const int lr = t / tc, c0 = (t - lr * tc) * 4, i = own_row(lr);
-        if (i >= n) continue;
-        const int jend = masked ? i + 1 : n;
-        const float* row = S + (size_t)i * L.s_ld;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-        for (int j = 0; j < jend; ++j) {
-            const float w = row[j];
-            const float4 v = *reinterpret_cast<const float4*>(vs + (size_t)j * L.ds + c0);
-            acc.x = fmaf(w, v.x, acc.x); acc.y = fmaf(w, v.y, acc.y); acc.z = fmaf(w, v.z, acc.z); acc.w = fmaf(w, v.w, acc.w);
+    // ---- phase 3 (Eq. 3): y_i = sum_j w_ij v_j over the kept weights.  A warp takes up to 32 columns of a tile's four rows; the keys are
+    // split among y_splits warps, and among a warp's lanes where there are less than 32 columns.
+    const int width = d <= 8 ? 8 : d <= 16 ? 16 : 32, blocks = (d + 31) / 32, ysplits = L.y_splits;
+    for (int unit = warp; unit < own_tiles * blocks * ysplits; unit += WARPS) {
+        const int rest = unit >> __ffs(ysplits) - 1, p = unit - rest * ysplits, tile = fastdiv(rest, L.by_blocks), c = 32 * (rest - tile * blocks) + (lane & (width - 1));
+        // keys that all four rows keep, that any row keeps (of rows beyond n nothing is read)
+        const int i0 = own_row(4 * tile), whole = masked ? i0 + 1 : n, jend = masked ? min(i0 + 4, n) : n, step = ysplits * (32 / width);
+        const float* w = S + 4 * tile;
+        const float* v = vs + min(c, d - 1);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        int j = p + ysplits * (lane / width);
+#pragma unroll 4
+        for (; j < whole; j += step) {
+            const float4 wj = *reinterpret_cast<const float4*>(w + j * L.s_ld);
+            const float x = v[j * L.ld];
+            acc[0] = fmaf(wj.x, x, acc[0]); acc[1] = fmaf(wj.y, x, acc[1]); acc[2] = fmaf(wj.z, x, acc[2]); acc[3] = fmaf(wj.w, x, acc[3]);
         }
-        const float r = rinv[i];
-        *reinterpret_cast<float4*>(out + ((size_t)b * n + i) * HD + (size_t)h * d + c0) = make_float4(acc.x * r, acc.y * r, acc.z * r, acc.w * r);
-        pv += 4ull * jend;
+#pragma unroll 1
+        for (; j < jend; j += step) {
+            const float x = v[j * L.ld];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (j <= i0 + r) acc[r] = fmaf(w[j * L.s_ld + r], x, acc[r]);
+        }
+        __syncwarp();
+        for (int off = width; off < 32; off *= 2) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], off);
+        }
+        if (lane < width && c < d) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) ypart[(p * own_rows + 4 * tile + r) * d + c] = acc[r];
+        }
     }
-
-    // ---- census
-    for (int off = 16; off; off >>= 1) {
-        qk += __shfl_xor_sync(0xffffffffu, qk, off);
-        pv += __shfl_xor_sync(0xffffffffu, pv, off);
-        ex += __shfl_xor_sync(0xffffffffu, ex, off);
-        pj += __shfl_xor_sync(0xffffffffu, pj, off);
-    }
-    if (lane == 0) {
-        if (qk) atomicAdd(&dc->qk_macs, qk);
-        if (pv) atomicAdd(&dc->pv_macs, pv);
-        if (ex) atomicAdd(&dc->exps, ex);
-        if (pj) atomicAdd(&dc->proj_macs, pj);
+    __syncthreads();
+    for (int lr = warp / 2; lr < valid_rows; lr += WARPS / 2) {        // two warps a row
+        float* y = out + ((size_t)b * n + own_row(lr)) * HD + (size_t)h * d;
+        const float f = rinv[lr];
+        for (int c = 32 * (warp & 1) + lane; c < d; c += 64) {
+            float s = ypart[lr * d + c];
+            for (int p = 1; p < ysplits; ++p) s += ypart[(p * own_rows + lr) * d + c];
+            y[c] = s * f;
+        }
     }
 }
 
@@ -1333,33 +1420,47 @@ bool f32_fused_fits(int n, int D, int d, int scheme) {
     return fused_layout(n, D, d, scheme == PSA_SYMMETRIC ? 1 : 3).total <= (size_t)FS_MAX_FLOATS;
 }
 
-// Heads few enough that one CTA each would leave most SMs idle are spread over clusters of up to 8 CTAs.
-int f32_fused_cluster_size(int B, int H, int n, int scheme) {
-    if (scheme == PSA_SYMMETRIC || B * H > 32) return 1;      // (the symmetric scheme's mirrored store crosses row owners)
+// Heads few enough that one CTA each would leave SMs idle are spread over clusters of up to 8 CTAs.  `*alone`: a CTA keeps others off its SM, by
+// the shared memory that it asks for.  Left to themselves the clusters of a call, and those of the next one that come in early, share SMs while
+// others are idle (12 heads of n = 64, d = 64: 13.0 us a call, 8.6 alone; a CTA per head 11.8).  The clusters that fit are fewer than the SMs divided by
+// their size, as a cluster stays inside a part of the GPU: 16 heads in clusters of 8 16.4 us alone and 12.2 sharing, in clusters of 4 10.8 alone.
+// Measured (us, a CTA per head / clusters of 2 / 4 / 8, sharing SMs; d_model = 64): 48 heads of n = 30, d = 32 16.4 11.1 9.1 16.1, of n = 64, d = 64 24.6
+// 20.9 19.4 25.9, of n = 100, d = 64 (too much shared memory for two on an SM) 47.1 40.9 52.5 59.4; 100 of n = 64, d = 64 26.7 41.3 29.7 45.6, of n = 64,
+// d = 16 14.4 16.8 18.0 29.8; 74 of n = 64, d = 8 12.3 14.2 14.2.  Many heads of up to 16 vectors gain nothing (48 of n = 16, d = 16 8.0 7.6 7.6).
+int f32_fused_cluster_size(int B, int H, int n, int D, int d, int scheme, int sms, bool* alone) {
+    const long long heads = (long long)B * H;
+    *alone = true;
+    if (scheme == PSA_SYMMETRIC || (heads > 32 && n <= 16)) return 1;      // (the symmetric scheme's mirrored store crosses row owners)
     const int tn = (n + 3) / 4;
-    int c = 1;
-    while (c < 8 && 2 * c <= tn) c *= 2;
-    return c;
+    auto floats = [&](int c) { return cluster_layout(n, D, d, c).total; };
+    auto fits = [&](int c) { return c <= tn && floats(c) <= (size_t)FS_MAX_FLOATS; };
+    if (fits(8) && 12 * heads <= sms) return 8;
+    if (fits(4) && 9 * heads <= 2 * sms) return 4;
+    *alone = false;
+    for (int c = 8; c > 2; c /= 2)
+        if (fits(c) && floats(c) * sizeof(float) <= FC_HALF_SM && 4 * heads * c <= 7 * sms) return c;
+    *alone = true;
+    return fits(2) && 2 * heads <= sms && (d >= 32 || heads <= 32) ? 2 : 1;
 }
 
 cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, const float* Wv, float* out, int B, int H,
                             int n, int D, int d, float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next,
                             cudaStream_t stream) {
     static DeviceSetup setup;
-    if (device_setup(&setup, [] {
-            cudaError_t e = cudaFuncSetAttribute(f32_fused_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 FS_MAX_FLOATS * (int)sizeof(float));
-            if (e != cudaSuccess) return e;
-            return cudaFuncSetAttribute(f32_fused_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        FS_MAX_FLOATS * (int)sizeof(float));
-        }, "fp32 fused layer set-up") <= 0)
-        return cudaErrorUnknown;
-    const int C = f32_fused_cluster_size(B, H, n, scheme);
+    const int sms = device_setup(&setup, [] {
+        constexpr int bytes = FS_MAX_FLOATS * (int)sizeof(float);
+        const cudaError_t e = cudaFuncSetAttribute(f32_fused_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(f32_fused_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    }, "fp32 fused layer set-up");
+    if (sms <= 0) return cudaErrorUnknown;
+    bool alone;
+    const int C = f32_fused_cluster_size(B, H, n, D, d, scheme, sms, &alone);
     if (C > 1) {
+        const ClusterLayout L = cluster_layout(n, D, d, C);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(B * H * C);
         cfg.blockDim = dim3(FS_THREADS);
-        cfg.dynamicSmemBytes = fused_layout(n, D, d, 3).total * sizeof(float);
+        cfg.dynamicSmemBytes = std::max(L.total * sizeof(float), alone ? FC_HALF_SM + 2048 : 0);
         cfg.stream = stream;
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1370,7 +1471,7 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        return cudaLaunchKernelEx(&cfg, f32_fused_cluster_kernel, X, Wq, Wk, Wv, out, n, H, D, d, scale, scheme, dc, dc_next);
+        return cudaLaunchKernelEx(&cfg, f32_fused_cluster_kernel, X, Wq, Wk, Wv, out, n, H, D, d, scale, scheme, dc, dc_next, L);
     }
     const size_t smem = fused_layout(n, D, d, scheme == PSA_SYMMETRIC ? 1 : 3).total * sizeof(float);
     f32_fused_layer_kernel<<<B * H, FS_THREADS, smem, stream>>>(X, Wq, scheme == PSA_SYMMETRIC ? Wq : Wk,

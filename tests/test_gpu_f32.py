@@ -51,9 +51,9 @@ def test_layer_shapes_and_schemes(scheme, B, H, n, D, d):
     _check_counts(cnt, (1 if sym else 3) * B * n * D * H * d)
 
 
-# Small layers run as one launch; with at most 32 heads the FULL and MASKED schemes spread a head over a cluster of
-# 1, 2, 4 or 8 CTAs (the largest power of two that leaves every CTA a 4-row tile).  The shapes walk those cluster sizes,
-# ragged last tiles, the switch back to one CTA per head at 33 heads, and d_k at both ends of the range.
+# Small layers run as one launch; the FULL and MASKED schemes spread a head over a cluster of
+# 1, 2, 4 or 8 CTAs (at most one per 4-row tile, and as many as fit the GPU at once).  The shapes walk those cluster sizes,
+# ragged last tiles, 32 and 33 heads, and d_k at both ends of the range.
 @pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
 @pytest.mark.parametrize("B,H,n,D,d", [(1, 1, 3, 16, 8), (1, 1, 8, 16, 8), (1, 2, 13, 24, 4), (2, 2, 17, 40, 12),
                                        (1, 1, 31, 64, 64), (1, 3, 33, 20, 128), (4, 8, 64, 64, 32), (3, 11, 45, 32, 16),
@@ -69,6 +69,15 @@ def test_small_layers_on_clusters(scheme, B, H, n, D, d):
         err = np.abs(out.cpu().numpy().astype(np.float64) - ref).max()
         assert err <= TOL_F32, (call, err)
         _check_counts(cnt, 3 * B * n * D * H * d)
+
+
+# How a cluster's CTA splits its work follows from the sizes: 8, 16 or 32 keys to a warp, one to eight parts of the sums, groups of four or eight
+# rows, an odd number of row tiles; more than 32 heads in clusters of 4 and 2, shared memory nearly full.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("B,H,n,D,d", [(1, 1, 9, 129, 128), (1, 2, 37, 65, 20), (1, 1, 150, 33, 8), (1, 3, 90, 7, 12), (1, 12, 64, 64, 24), (1, 1, 17, 252, 64),
+                                       (6, 8, 45, 64, 64), (16, 4, 100, 64, 64), (37, 2, 20, 30, 36), (1, 1, 167, 5, 52), (1, 1, 243, 3, 4)])
+def test_clusters_at_odd_sizes(scheme, B, H, n, D, d):
+    test_layer_shapes_and_schemes(scheme, B, H, n, D, d)
 
 
 @pytest.mark.parametrize("scheme", [oracle.FULL, oracle.SYMMETRIC, oracle.MASKED])
