@@ -29,6 +29,8 @@
 // TMEM columns, d = 128: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512); P_t (bf16, two keys per
 // column) overlays the first 64 columns of S_t.  d = 64: S0 S1 | P0 P1 [256,384) | O0 O1 [384,512): P has
 // its own columns, so S of the next key block is computed while the softmax of the current one runs.
+#include <type_traits>
+
 #include "psa_internal.h"
 #include "psa_sched.h"
 #include "psa_softmax.cuh"
@@ -70,10 +72,12 @@ constexpr int ISSUER1_WARP = CTRL_WARPS + 2 * SOFTMAX_WARPS_PER_TILE;
 template <int D> __host__ __device__ constexpr int persist_threads() { return ATTN_THREADS + (D == 64 ? 32 : 0); }
 template <int D> __host__ __device__ constexpr int item_readers() { return (D == 64 ? 2 : 1) + 2 * SOFTMAX_WARPS_PER_TILE; }   // issuers + one lane per softmax warp
 
+// D: columns of a tile in shared memory, KS: 16-column steps of phase 1, and of phase 3's output, that hold columns of the head (the rest are zeros,
+// which the census counts as issued: it goes by blocks of D columns).
 // KVS ("keys are the values"): K and V are one tensor (the case the paper mentions in Sec. 3.1 beside query = key =
 // value).  A key tile is then loaded once and serves phase 1 as the K-major operand and phase 3 as the MN-major
 // one; the shared-memory stages of the V ring extend the K ring, and a tile is released behind its PV.
-template <int D, bool KVS>
+template <int D, int KS, bool KVS>
 __global__ void __launch_bounds__(persist_threads<D>(), 1)
 attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ SchedParams sp, int H, int scheme,
                     int nitems, float sl2, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next) {
@@ -246,7 +250,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
             // order, sleeping on the barriers of each; the two slots' threads walk the item list independently.
             const int t = warp == 1 ? 0 : 1;
             const uint32_t idescS = umma_idesc_bf16(128, 128, UMMA_K_MAJOR, UMMA_K_MAJOR);
-            const uint32_t idescO = umma_idesc_bf16(128, D, UMMA_K_MAJOR, UMMA_MN_MAJOR);
+            const uint32_t idescO = umma_idesc_bf16(128, 16 * KS, UMMA_K_MAJOR, UMMA_MN_MAJOR);
             unsigned long long qk_blocks = 0, pv_blocks = 0;
             const uint32_t q_lo = umma_desc_lo_kmajor(smem_u32(sQ + t * Cfg::TILE_BYTES));
             const uint32_t k_lo = umma_desc_lo_kmajor(smem_u32(sK));
@@ -260,7 +264,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
             auto mma_S = [&](uint32_t kc) {     // S = Q K^T with K at ring position kc (phase 1, Eq. 1)
                 const uint32_t k = k_lo + (kc % KST) * (Cfg::TILE_BYTES >> 4);
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
+                for (int kk = 0; kk < KS; ++kk) {
                     const uint32_t off = ((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
                     umma_ss(dS, umma_desc_join(q_lo + off, UMMA_DESC_HI_SW128), umma_desc_join(k + off, UMMA_DESC_HI_SW128),
                             idescS, kk != 0);
@@ -350,7 +354,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
             // and S_{j+1} of a tile go back to back under one commit, and the thread sleeps on what each link
             // needs, tile 0 then tile 1 then tile 0 ...
             const uint32_t idescS = umma_idesc_bf16(128, 128, UMMA_K_MAJOR, UMMA_K_MAJOR);
-            const uint32_t idescO = umma_idesc_bf16(128, D, UMMA_K_MAJOR, UMMA_MN_MAJOR);
+            const uint32_t idescO = umma_idesc_bf16(128, 16 * KS, UMMA_K_MAJOR, UMMA_MN_MAJOR);
             unsigned long long qk_blocks = 0, pv_blocks = 0;
             const uint32_t q_lo[2] = {umma_desc_lo_kmajor(smem_u32(sQ)), umma_desc_lo_kmajor(smem_u32(sQ + Cfg::TILE_BYTES))};
             const uint32_t k_lo = umma_desc_lo_kmajor(smem_u32(sK));
@@ -365,7 +369,7 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
                 const uint32_t q = q_lo[t], k = k_lo + (kc % KST) * (Cfg::TILE_BYTES >> 4);
                 const uint32_t dS = tS0 + t * 128;
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
+                for (int kk = 0; kk < KS; ++kk) {
                     const uint32_t off = ((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
                     umma_ss(dS, umma_desc_join(q + off, UMMA_DESC_HI_SW128), umma_desc_join(k + off, UMMA_DESC_HI_SW128),
                             idescS, kk != 0);
@@ -638,15 +642,15 @@ attn_persist_kernel(const __grid_constant__ PMaps maps, const __grid_constant__ 
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// D: head size the kernel works with (64 or 128); d: the tensors' head size, d <= D, a multiple of 8 (the columns
+// D: columns that a tile is loaded with (64 or 128); d: the tensors' head size, d <= 16 KS <= D, a multiple of 8 (the columns
 // between d and D are zero-filled by the loads and dropped by the stores).
-template <int D, bool KVS>
+template <int D, int KS, bool KVS>
 int launch_persist(const void* Q, const void* K, const void* V, void* out, int B, int H, int n, int d, float scale,
                    int scheme, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next, cudaStream_t stream) {
     using Cfg = PCfg<D>;
     static DeviceSetup setup;
     const int sm_count = device_setup(&setup, [] {
-        return cudaFuncSetAttribute(attn_persist_kernel<D, KVS>, cudaFuncAttributeMaxDynamicSharedMemorySize, PCfg<D>::SMEM);
+        return cudaFuncSetAttribute(attn_persist_kernel<D, KS, KVS>, cudaFuncAttributeMaxDynamicSharedMemorySize, PCfg<D>::SMEM);
     }, "attention kernel set-up");
     if (sm_count <= 0) return PSA_ERR_CUDA;
     PMaps maps;
@@ -670,7 +674,7 @@ int launch_persist(const void* Q, const void* K, const void* V, void* out, int B
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_persist_kernel<D, KVS>, maps, sp, H, scheme, (int)nitems,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_persist_kernel<D, KS, KVS>, maps, sp, H, scheme, (int)nitems,
                                              scale * LOG2E, dc, cursor, dc_next);
     if (e != cudaSuccess) { set_cuda_error(e, "attn_persist_kernel launch"); return PSA_ERR_CUDA; }
     return PSA_OK;
@@ -684,12 +688,24 @@ int bf16_attention_persist(const void* Q, const void* K, const void* V, void* ou
                            float scale, int scheme, DeviceCounters* dc, unsigned int* cursor, DeviceCounters* dc_next, cudaStream_t stream) {
     if (scheme != PSA_FULL && scheme != PSA_MASKED) return PSA_ERR_SCHEME_ARGS;
     if (d < 8 || d > 128 || d % 8) return PSA_ERR_UNSUPPORTED;
-    if (K == V) {     // one tensor for keys and values: each key tile is loaded once
-        if (d <= 64) return launch_persist<64, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
-        return launch_persist<128, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
+    auto launch = [&](auto width, auto steps) {
+        constexpr int D = decltype(width)::value, KS = decltype(steps)::value;
+        if (K == V) return launch_persist<D, KS, true>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);     // each key tile is loaded once
+        return launch_persist<D, KS, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
+    };
+    using std::integral_constant;
+    const integral_constant<int, 64> narrow;
+    const integral_constant<int, 128> wide;
+    // The products run over 16 KS columns of the 64 or 128 that a tile is loaded with.  Between 64 and 96 the chain of a row tile gets shorter (us, all 128
+    // columns / here): masked, 32 heads of n = 3001, d = 72 83.3 / 79.0, d = 80 84.1 / 77.4, d = 96 86.3 / 82.3; FULL, n = 4096, d = 80 240 / 232.  At
+    // 104 and 112 the eighth step costs nothing beyond noise.  Up to 64 the exponentials bound: 1-2 % at d <= 32, nothing at 40 and 48.
+    switch ((d + 15) / 16) {
+        case 1: case 2: return launch(narrow, integral_constant<int, 2>{});
+        case 3: case 4: return launch(narrow, integral_constant<int, 4>{});
+        case 5: return launch(wide, integral_constant<int, 5>{});
+        case 6: return launch(wide, integral_constant<int, 6>{});
+        default: return launch(wide, integral_constant<int, 8>{});
     }
-    if (d <= 64) return launch_persist<64, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
-    return launch_persist<128, false>(Q, K, V, out, B, H, n, d, scale, scheme, dc, cursor, dc_next, stream);
 }
 
 }  // namespace psa
