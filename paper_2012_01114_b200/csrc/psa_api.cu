@@ -19,6 +19,12 @@ namespace {
 
 thread_local char g_err_text[256] = "";
 
+// Marks of fp32 calls (heads and tiles that the tensor cores cannot take) are a number of the call's own, so that nothing has to be cleared ahead of
+// its first kernel (us, with a clear ahead / without: layer of 4 x 512 x 768 85.1 / 81.2, core of 16 heads of n = 300, d = 128 24.6 / 21.3, of 32
+// heads of n = 42 8.4 / 6.9).  What memory holds by chance or from an earlier call is another number; if it is the same after all, a head or
+// tile is worked on by the path for marked ones, which takes any.
+constexpr int MARK_BASE = 0x5a000000;
+
 struct Context {
     std::mutex mu;
     void* user_ws = nullptr;
@@ -26,13 +32,14 @@ struct Context {
     void* own_ws = nullptr;
     size_t own_bytes = 0;
     DeviceCounters* last_dc = nullptr;  // counters of the most recent call
-    // The workspace starts with three counter blocks.  The bf16 FULL / MASKED path uses the first two in turn: the
-    // attention kernel of a call clears the block of the next call, so that no clearing copy has to run ahead of the
+    // The workspace starts with three counter blocks.  All paths but the symmetric one in bf16 use the first two in turn: the
+    // last attention kernel of a call clears the block of the next call, so that no clearing copy has to run ahead of the
     // call's first kernel.  `clean_ws` is the workspace whose block `next_block` is known to be clear.  A call that is being
     // captured into a graph has the third to itself and clears it first: the graph may run any number of times, between
     // any other calls.
     char* clean_ws = nullptr;
     int next_block = 0;
+    int mark = MARK_BASE;               // see next_mark
     // Streams and events of the entry points on host buffers, created by the first such call and kept.
     struct HostPipe* pipe = nullptr;
     std::vector<cudaEvent_t> prof_events;  // 3 per profiled call
@@ -86,8 +93,10 @@ WsShape call_shape(int batch, int heads, int n, int d_model, int d_k, int scheme
     return WsShape{batch, heads, n, d_model, d_k, scheme, dtype, with_proj, staging, with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme), false};
 }
 
-F32Scratch f32_scratch(char* ws, const WsLayout& L, size_t first_head) {
-    return F32Scratch{reinterpret_cast<int*>(ws + L.bad) + first_head, reinterpret_cast<float*>(ws + L.ml), ws + L.parts};
+int next_mark(Context& cx) { return cx.mark = cx.mark == 0x7fffffff ? MARK_BASE : cx.mark + 1; }
+
+F32Scratch f32_scratch(char* ws, const WsLayout& L, size_t first_head, int mark) {
+    return F32Scratch{reinterpret_cast<int*>(ws + L.bad) + first_head, mark, reinterpret_cast<float*>(ws + L.ml), ws + L.parts};
 }
 
 // Whether copies from or to this host memory run beside the calling thread (memory that CUDA knows of).
@@ -223,7 +232,7 @@ int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv,
     if (between) cudaEventRecord(between, stream);
     if (dtype == PSA_F32) {
         e = f32_attention(static_cast<const float*>(Q), static_cast<const float*>(K), static_cast<const float*>(V),
-                          static_cast<float*>(out), S, fs, batch, heads, n, d_k, scale, scheme, dc, stream);
+                          static_cast<float*>(out), S, fs, batch, heads, n, d_k, scale, scheme, dc, dc_next, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "f32_attention"); return PSA_ERR_CUDA; }
         return PSA_OK;
     }
@@ -233,9 +242,8 @@ int enqueue_layer(const void* X, const void* Wq, const void* Wk, const void* Wv,
 int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const void* Wv, const void* Q, const void* K,
               const void* V, int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype, void* out,
               cudaStream_t stream, bool with_proj, char* ws, const WsLayout& L) {
-    // the paths whose last kernel clears the other counter block: the fused bf16 kernels and the one-launch fp32 layer
-    const bool turns = (dtype == PSA_BF16 && scheme != PSA_SYMMETRIC) ||
-                       (with_proj && dtype == PSA_F32 && f32_fused_fits(n, d_model, d_k, scheme));
+    // the paths whose last attention kernel clears the other counter block
+    const bool turns = dtype == PSA_F32 || scheme != PSA_SYMMETRIC;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(stream, &capture);
     if (e != cudaSuccess) { set_cuda_error(e, "cudaStreamIsCapturing"); return PSA_ERR_CUDA; }
@@ -252,7 +260,7 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     } else if (turns && cx.clean_ws == ws) {
         block = cx.next_block;
     } else {
-        e = cudaMemsetAsync(ws, 0, L.clear_bytes ? L.clear + L.clear_bytes : TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
+        e = cudaMemsetAsync(ws, 0, TURN_BLOCKS * COUNTER_BLOCK_BYTES, stream);
     }
     if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync(counters)"); return PSA_ERR_CUDA; }
     if (!captured) cx.clean_ws = nullptr;          // until this call's kernels are known to be queued
@@ -269,8 +277,9 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     } tail{pev, stream};
     if (pev) cudaEventRecord(pev[0], stream);
     void* const qkv[3] = {ws + L.q, ws + L.k, ws + L.v};
-    const F32Scratch fs = f32_scratch(ws, L, 0);
-    const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in)};
+    const int mark = next_mark(cx);
+    const F32Scratch fs = f32_scratch(ws, L, 0, mark);
+    const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in), mark};
     const int rc = enqueue_layer(X, Wq, Wk, Wv, Q, K, V, batch, heads, n, d_model, d_k, scheme, dtype, out, stream, with_proj,
                                  qkv, S, L.s_bytes, s_clear, L.attn_tensor ? &fs : nullptr, L.in_bytes ? &ps : nullptr, dc, &dc->next_item, dc_next, pev ? pev[1] : nullptr);
     if (rc == PSA_OK && turns && !captured) {        // the other block will be clear once this call has run
@@ -440,6 +449,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     // further copy costs (16 x 512 x 768, 12 heads: 1597 us in one part, 1812 in eight; in fp32, whose kernels take longer, 4140
     // and 3310).  Asked here, under the copies of the matrices: the answer takes a few microseconds per buffer.
     if (dtype == PSA_BF16 && !(pinned(X_host) && pinned(out_host))) parts = 1;
+    const int mark = next_mark(cx);
     auto first = [&](int c) { return (int)((long long)batch * c / parts); };      // first sequence of part c
     for (int c = 0; c < parts && e == cudaSuccess; ++c) {
         const size_t b0 = first(c), nb = first(c + 1) - b0;
@@ -452,8 +462,8 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
         e = cudaStreamWaitEvent(stream, pipe->loaded[c], 0);
         if (e != cudaSuccess) break;
         void* const qkv[3] = {ws + L.q + b0 * ob, ws + L.k + b0 * ob, ws + L.v + b0 * ob};
-        const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in) + c * L.marks_pitch};
-        const F32Scratch fs = f32_scratch(ws, L, b0 * heads);       // (a part has marks of its own; the rest is used by one after another)
+        const F32ProjectScratch ps = {ws + L.parts, L.in_bytes, reinterpret_cast<int*>(ws + L.marks_in) + c * L.marks_pitch, mark};
+        const F32Scratch fs = f32_scratch(ws, L, b0 * heads, mark);       // (a part has marks of its own; the rest is used by one after another)
         rc = enqueue_layer(ws + L.xs + b0 * xb, ws + L.wq, ws + L.wk, ws + L.wv, nullptr, nullptr, nullptr, (int)nb, heads, n, d_model,
                            d_k, scheme, dtype, ws + L.outs + b0 * ob, stream, true, qkv,
                            sym ? reinterpret_cast<float*>(ws + L.s) : nullptr, L.s_bytes, false, L.attn_tensor ? &fs : nullptr, L.in_bytes ? &ps : nullptr, dc,
@@ -561,7 +571,7 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
     const void* Ws[3] = {Wo, Wo, Wo};
     void* outs[3] = {out, out, out};
     if (dtype == PSA_F32) {
-        const F32ProjectScratch ps = {ws + L.parts, L.out_bytes, reinterpret_cast<int*>(ws + L.marks_out)};
+        const F32ProjectScratch ps = {ws + L.parts, L.out_bytes, reinterpret_cast<int*>(ws + L.marks_out), cx.mark};
         cudaError_t e = cudaSuccess;
         if (L.out_bytes && !L.clear_bytes) e = cudaMemsetAsync(ps.marks, 0, f32_project_marks(batch * n, d_model, 1) * sizeof(int), stream);
         if (e == cudaSuccess) e = f32_project(static_cast<const float*>(y), reinterpret_cast<const float* const*>(Ws),

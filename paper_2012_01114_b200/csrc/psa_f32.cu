@@ -237,7 +237,7 @@ template <int DG, int KS, int MODE>
 __global__ void __launch_bounds__(FA_THREADS, DG == 1 ? 3 : 2)
 f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                  float* __restrict__ out, const float* __restrict__ S, int n, int H, int d, float scale, int masked,
-                 DeviceCounters* dc, const int* __restrict__ bad) {
+                 DeviceCounters* dc, DeviceCounters* dc_next, const int* __restrict__ bad, int mark) {
     using C = FACfg<DG, KS>;
     constexpr int U = C::U;
     extern __shared__ float4 fa_smem4[];
@@ -247,9 +247,11 @@ f32_flash_kernel(const float* __restrict__ Q, const float* __restrict__ K, const
     float* Ps = Vs + C::V_FLOATS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 15, ty = lane >> 4;
     const int bh = blockIdx.x, b = bh / H, h = bh - b * H;
+    if (MODE == 0) grid_dependency_wait();
+    // the counter block of the NEXT call on this workspace is cleared here, off that call's critical path
+    if (dc_next && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};
     if (MODE == 0) {
-        grid_dependency_wait();
-        if (bad && !bad[bh]) return;
+        if (bad && bad[bh] != mark) return;
     }
     const int rb = masked ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // the longest rows first
     const int r0 = rb * C::BR;
@@ -496,7 +498,7 @@ struct FDCfg {
 template <int DG>
 __global__ void __launch_bounds__(FD_THREADS, 3 - DG)
 f32_diagonal_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V, float* __restrict__ out, float* __restrict__ ml,
-                    const int* __restrict__ bad, int heads, int n, int H, int d, float scale, DeviceCounters* dc) {
+                    const int* __restrict__ bad, int mark, int heads, int n, int H, int d, float scale, DeviceCounters* dc) {
     using C = FDCfg<DG>;
     extern __shared__ float4 fd_smem4[];
     float* Qs = reinterpret_cast<float*>(fd_smem4);
@@ -508,7 +510,7 @@ f32_diagonal_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int bh = blockIdx.x % heads, tile = blockIdx.x / heads, b = bh / H, h = bh - b * H;
     grid_dependency_wait();
-    if (bad[bh]) return;
+    if (bad[bh] == mark) return;
     const size_t ld = (size_t)H * d, base = ((size_t)b * n + tile * 128) * ld + (size_t)h * d;
     const int rows = min(128, n - tile * 128), d4 = d >> 2;
     for (int t = tid; t < 128 * d4; t += FD_THREADS) {
@@ -760,7 +762,8 @@ template <int MODE>
 __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32)
 f32_attn_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                 float* __restrict__ out, float* __restrict__ S, int n, int H, int d, float scale, int masked,
-                DeviceCounters* dc) {
+                DeviceCounters* dc, DeviceCounters* dc_next) {
+    if (dc_next && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) *dc_next = DeviceCounters{0, 0, 0, 0, 0, 0, 0};      // (for the next call)
     extern __shared__ float sm[];
     float* ks = sm;                                   // [KEY_TILE][d + 1]
     float* qs = ks + KEY_TILE * (d + 1);              // [ROWS_PER_BLOCK][d]
@@ -1364,7 +1367,7 @@ cudaError_t project_general(const float* X, const float* const W[3], float* cons
 }
 
 cudaError_t attention_general(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H, int n, int d,
-                              float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+                              float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next, cudaStream_t stream) {
     const size_t smem = attn_smem_bytes(n, d);
     for (int b0 = 0; b0 < B; b0 += min(GRID_MAX, B - b0)) {
         const int nb = min(GRID_MAX, B - b0);
@@ -1372,12 +1375,12 @@ cudaError_t attention_general(const float* Q, const float* K, const float* V, fl
         const dim3 grid((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, H, nb), block(ROWS_PER_BLOCK * 32);
         if (scheme == PSA_SYMMETRIC) {
             float* s = S + (size_t)b0 * H * n * n;
-            f32_attn_kernel<1><<<grid, block, smem, stream>>>(Q + o, Q + o, Q + o, out + o, s, n, H, d, scale, 0, dc);
+            f32_attn_kernel<1><<<grid, block, smem, stream>>>(Q + o, Q + o, Q + o, out + o, s, n, H, d, scale, 0, dc, nullptr);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
-            f32_attn_kernel<2><<<grid, block, smem, stream>>>(Q + o, Q + o, Q + o, out + o, s, n, H, d, scale, 0, dc);
+            f32_attn_kernel<2><<<grid, block, smem, stream>>>(Q + o, Q + o, Q + o, out + o, s, n, H, d, scale, 0, dc, dc_next);
         } else {
-            f32_attn_kernel<0><<<grid, block, smem, stream>>>(Q + o, K + o, V + o, out + o, nullptr, n, H, d, scale, scheme == PSA_MASKED ? 1 : 0, dc);
+            f32_attn_kernel<0><<<grid, block, smem, stream>>>(Q + o, K + o, V + o, out + o, nullptr, n, H, d, scale, scheme == PSA_MASKED ? 1 : 0, dc, dc_next);
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1406,7 +1409,7 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
         // cores, 2048 x 768 x 3 x 768 171 / 70.
         const long long tiles = (long long)((rows + 31) / 32) * ((N + 31) / 32) * nW;
         if (ps && f32_project_pairs_fit(rows, D, N, nW, ps->bytes) && f32_project_pairs_pay(rows, D, N, nW, sms))
-            return f32_project_pairs(X, W, out, nW, rows, D, N, residual, ps->parts, ps->marks, dc, stream);
+            return f32_project_pairs(X, W, out, nW, rows, D, N, residual, ps->parts, ps->marks, ps->mark, dc, stream);
         if (tiles > 2 * sms) return f32_project_tensor(X, W, out, nW, rows, D, N, residual, dc, stream);
         const dim3 grid((N + GP_BN - 1) / GP_BN, (rows + GP_BM - 1) / GP_BM, nW);
         f32_project_tiled_kernel<<<grid, GP_THREADS, GP_SMEM, stream>>>(X, W[0], W[1], W[2], out[0], out[1], out[2], rows, D, N, residual, dc);
@@ -1483,7 +1486,7 @@ cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, co
 namespace {
 template <int DG, int KS, int MODE>
 cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n, int d,
-                         float scale, int masked, DeviceCounters* dc, const F32Scratch* fs, cudaStream_t stream) {
+                         float scale, int masked, DeviceCounters* dc, DeviceCounters* dc_next, const F32Scratch* fs, cudaStream_t stream) {
     using C = FACfg<DG, KS>;
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
@@ -1492,7 +1495,7 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
         return cudaErrorUnknown;
     const dim3 grid(B * H, (n + C::BR - 1) / C::BR);
     if (!fs) {
-        f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc, nullptr);
+        f32_flash_kernel<DG, KS, MODE><<<grid, FA_THREADS, C::SMEM, stream>>>(Q, K, V, out, S, n, H, d, scale, masked, dc, dc_next, nullptr, 0);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
@@ -1505,26 +1508,26 @@ cudaError_t launch_flash(const float* Q, const float* K, const float* V, float* 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f32_flash_kernel<DG, KS, MODE>, Q, K, V, out, S, n, H, d, scale, masked, dc, static_cast<const int*>(fs->bad));
+    return cudaLaunchKernelEx(&cfg, f32_flash_kernel<DG, KS, MODE>, Q, K, V, out, S, n, H, d, scale, masked, dc, dc_next, static_cast<const int*>(fs->bad), fs->mark);
 }
 template <int DG, int MODE>
 cudaError_t launch_flash_split(const float* Q, const float* K, const float* V, float* out, const float* S, int B, int H, int n,
-                               int d, float scale, int masked, DeviceCounters* dc, const F32Scratch* fs, int sms, cudaStream_t stream) {
+                               int d, float scale, int masked, DeviceCounters* dc, DeviceCounters* dc_next, const F32Scratch* fs, int sms, cudaStream_t stream) {
     auto ctas = [&](int br) { return (long long)B * H * ((n + br - 1) / br); };
     // Fewer rows per CTA cost efficiency (every warp rereads K for 16 rows, with 4 / KS keys to a load of q) and buy CTAs: the
     // line lies at two CTAs per SM (us for KS = 1 / 2 / 4).  16 heads of n = 300, d = 64, 80 tiles of 64 rows: 70 / 44 / 35; 16 of
     // n = 1024, d = 128, masked, 256 tiles: 210 / 166 / 216; 74 of n = 256, d = 64, 296 tiles: 46 / 54 / 70; 48 of n = 512, d = 64, 384
     // tiles: 110 / 124 / 159.  It is not exact: 16 heads of n = 1024, FULL, d = 64 161 / 179 / 208; 64 of n = 300, 320 tiles with a
     // nearly empty last one, 101 / 82 / 87.
-    if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, fs, stream);
-    if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, fs, stream);
-    return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, fs, stream);
+    if (ctas(64) >= 2 * sms) return launch_flash<DG, 1, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, dc_next, fs, stream);
+    if (ctas(32) >= 2 * sms) return launch_flash<DG, 2, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, dc_next, fs, stream);
+    return launch_flash<DG, 4, MODE>(Q, K, V, out, S, B, H, n, d, scale, masked, dc, dc_next, fs, stream);
 }
 template <int DG>
 cudaError_t tiled_attention(const float* Q, const float* K, const float* V, float* out, float* S, int B, int H, int n, int d,
-                            float scale, int scheme, DeviceCounters* dc, int sms, cudaStream_t stream) {
+                            float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next, int sms, cudaStream_t stream) {
     if (scheme != PSA_SYMMETRIC)
-        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, nullptr, sms, stream);
+        return launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, scheme == PSA_MASKED, dc, dc_next, nullptr, sms, stream);
     constexpr int SMEM = (FACfg<DG, 1>::Q_FLOATS + FACfg<DG, 1>::K_FLOATS) * (int)sizeof(float);
     static DeviceSetup setup;
     if (device_setup(&setup, [] {
@@ -1535,12 +1538,12 @@ cudaError_t tiled_attention(const float* Q, const float* K, const float* V, floa
     f32_sym_scores_kernel<DG><<<dim3(B * H, T * (T + 1) / 2), FA_THREADS, SMEM, stream>>>(Q, S, n, H, d, scale, dc);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, nullptr, sms, stream);
+    return launch_flash_split<DG, 2>(Q, Q, Q, out, S, B, H, n, d, scale, 0, dc, dc_next, nullptr, sms, stream);
 }
 // The call on the tensor cores (psa_f32_attn_tensor.cu), with the weights on the diagonal tiles and the heads that path cannot take here.
 template <int DG>
 cudaError_t tensor_attention(const float* Q, const float* K, const float* V, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale,
-                             int masked, DeviceCounters* dc, int sms, cudaStream_t stream) {
+                             int masked, DeviceCounters* dc, DeviceCounters* dc_next, int sms, cudaStream_t stream) {
     cudaError_t e = f32_attention_split(Q, K, V, fs, B, H, n, d, stream);
     if (e == cudaSuccess && masked) {
         static DeviceSetup setup;
@@ -1558,10 +1561,10 @@ cudaError_t tensor_attention(const float* Q, const float* K, const float* V, flo
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, f32_diagonal_kernel<DG>, Q, K, V, out, fs.ml, static_cast<const int*>(fs.bad), B * H, n, H, d, scale, dc);
+        e = cudaLaunchKernelEx(&cfg, f32_diagonal_kernel<DG>, Q, K, V, out, fs.ml, static_cast<const int*>(fs.bad), fs.mark, B * H, n, H, d, scale, dc);
     }
     if (e == cudaSuccess) e = f32_attention_tensor(Q, out, fs, B, H, n, d, scale, masked, dc, stream);
-    if (e == cudaSuccess) e = launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, masked, dc, &fs, sms, stream);
+    if (e == cudaSuccess) e = launch_flash_split<DG, 0>(Q, K, V, out, nullptr, B, H, n, d, scale, masked, dc, dc_next, &fs, sms, stream);
     return e;
 }
 }  // namespace
@@ -1596,19 +1599,19 @@ bool short_heads(long long heads, int n, int d, int scheme, int sms) {
 }  // namespace
 
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, const F32Scratch* fs, int B, int H,
-                          int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream) {
+                          int n, int d, float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next, cudaStream_t stream) {
     static DeviceSetup setup;
     const int sms = device_setup(&setup, [] { return cudaSuccess; }, "fp32 attention set-up");
     if (sms <= 0) return cudaErrorUnknown;
     if (fs && f32_tensor_attention_fits(B, H, n, d, scheme))
-        return d <= 64 ? tensor_attention<1>(Q, K, V, out, *fs, B, H, n, d, scale, scheme == PSA_MASKED, dc, sms, stream)
-                       : tensor_attention<2>(Q, K, V, out, *fs, B, H, n, d, scale, scheme == PSA_MASKED, dc, sms, stream);
+        return d <= 64 ? tensor_attention<1>(Q, K, V, out, *fs, B, H, n, d, scale, scheme == PSA_MASKED, dc, dc_next, sms, stream)
+                       : tensor_attention<2>(Q, K, V, out, *fs, B, H, n, d, scale, scheme == PSA_MASKED, dc, dc_next, sms, stream);
     if (H <= GRID_MAX && short_heads((long long)B * H, n, d, scheme, sms))
-        return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
+        return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, dc_next, stream);
     if (d % 4 == 0 && (long long)B * H <= 0x7fffffff && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(out))      // 16-byte rows
-        return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, sms, stream)
-                       : tiled_attention<2>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, sms, stream);
-    return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, stream);
+        return d <= 64 ? tiled_attention<1>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, dc_next, sms, stream)
+                       : tiled_attention<2>(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, dc_next, sms, stream);
+    return attention_general(Q, K, V, out, S, B, H, n, d, scale, scheme, dc, dc_next, stream);
 }
 
 }  // namespace psa

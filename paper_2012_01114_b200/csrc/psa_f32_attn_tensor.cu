@@ -71,7 +71,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t&
 // blockIdx.y: 0 K, 1 V, 2 Q (looked at only).  `count4`: groups of four numbers of a tensor.
 __global__ void __launch_bounds__(256)
 f32_split_kernel(const float4* __restrict__ Q, const float4* __restrict__ K, const float4* __restrict__ V, uint2* __restrict__ parts, uint32_t count4,
-                 int d, int H, int n, int* __restrict__ bad) {
+                 int d, int H, int n, int* __restrict__ bad, int mark) {
     const int which = blockIdx.y;
     const float4* src = which == 0 ? K : (which == 1 ? V : Q);
     uint2* dst = parts + (size_t)which * 3 * count4;
@@ -84,7 +84,7 @@ f32_split_kernel(const float4* __restrict__ Q, const float4* __restrict__ K, con
         const uint32_t least = min(min(2u * __float_as_uint(x.x) - 1u, 2u * __float_as_uint(x.y) - 1u), min(2u * __float_as_uint(x.z) - 1u, 2u * __float_as_uint(x.w) - 1u));
         if (most > (which == 1 ? FM_VALUE_MOST : FM_MOST) || (which == 1 && least < 2u * FM_VALUE_LEAST - 1u)) {
             const uint32_t row = i / (uint32_t)(d >> 2);
-            bad[(row / ((uint32_t)n * H)) * H + row % (uint32_t)H] = 1;
+            bad[(row / ((uint32_t)n * H)) * H + row % (uint32_t)H] = mark;
         }
         if (which == 2) continue;
         uint2 p[3];
@@ -98,7 +98,7 @@ f32_split_kernel(const float4* __restrict__ Q, const float4* __restrict__ K, con
 template <int D>
 __global__ void __launch_bounds__(FM_THREADS, 1)
 f32_attn_tensor_kernel(const __grid_constant__ FMMaps maps, const float* __restrict__ Q, float* __restrict__ out, const float* __restrict__ ml,
-                       const int* __restrict__ bad, int B, int H, int n, int d, int masked, int nitems, float scale, DeviceCounters* dc) {
+                       const int* __restrict__ bad, int mark, int B, int H, int n, int d, int masked, int nitems, float scale, DeviceCounters* dc) {
     using Cfg = FMCfg<D>;
     constexpr int ST = Cfg::STAGES;
     extern __shared__ uint8_t fm_smem_raw[];
@@ -149,7 +149,7 @@ f32_attn_tensor_kernel(const __grid_constant__ FMMaps maps, const float* __restr
             for (int idx = blockIdx.x; idx < nitems && ok; idx += gridDim.x) {
                 int bh, It, nblk;
                 item_work(idx, bh, It, nblk);
-                if (bad[bh]) continue;
+                if (bad[bh] == mark) continue;
                 const int b = bh / H, h = bh - b * H;
                 auto load = [&](const CUtensorMap* map, int j) {
                     const int s = rc % ST;
@@ -202,7 +202,7 @@ f32_attn_tensor_kernel(const __grid_constant__ FMMaps maps, const float* __restr
             for (int idx = blockIdx.x; idx < nitems && ok; idx += gridDim.x) {
                 int bh, It, nblk;
                 item_work(idx, bh, It, nblk);
-                if (bad[bh]) continue;
+                if (bad[bh] == mark) continue;
                 ok = mbar_wait(&q_ready, items & 1, abortp) && issue_S(blk > 0);
                 ++items;
                 for (int j = 0; j < nblk && ok; ++j) {
@@ -243,7 +243,7 @@ f32_attn_tensor_kernel(const __grid_constant__ FMMaps maps, const float* __restr
         for (int idx = blockIdx.x; idx < nitems && ok; idx += gridDim.x) {
             int bh, It, nblk;
             item_work(idx, bh, It, nblk);
-            if (bad[bh]) continue;
+            if (bad[bh] == mark) continue;
             const int b = bh / H, h = bh - b * H, gA = It * TILE + rA, gB = gA + 8;
             const size_t at = (((size_t)b * n + gA) * H + h) * d, down = (size_t)8 * H * d;
             // ---- the row tile's Q, split into tensor memory (every S of the item before has been waited for)
@@ -409,7 +409,7 @@ cudaError_t launch_main(const float* Q, float* out, const F32Scratch& fs, int B,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f32_attn_tensor_kernel<D>, maps, Q, out, static_cast<const float*>(fs.ml), static_cast<const int*>(fs.bad), B, H, n, d,
+    return cudaLaunchKernelEx(&cfg, f32_attn_tensor_kernel<D>, maps, Q, out, static_cast<const float*>(fs.ml), static_cast<const int*>(fs.bad), fs.mark, B, H, n, d,
                               masked, nitems, scale, dc);
 }
 
@@ -428,7 +428,7 @@ cudaError_t f32_attention_split(const float* Q, const float* K, const float* V, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, f32_split_kernel, reinterpret_cast<const float4*>(Q), reinterpret_cast<const float4*>(K), reinterpret_cast<const float4*>(V),
-                              static_cast<uint2*>(fs.parts), count4, d, H, n, fs.bad);
+                              static_cast<uint2*>(fs.parts), count4, d, H, n, fs.bad, fs.mark);
 }
 cudaError_t f32_attention_tensor(const float* Q, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale, int masked, DeviceCounters* dc,
                                  cudaStream_t stream) {

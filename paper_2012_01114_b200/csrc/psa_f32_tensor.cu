@@ -449,7 +449,8 @@ static_assert(sizeof(FtAgain) <= FP_STAGE, "does not fit the ring");
 // a nonzero number is below 2^-60.
 __global__ void __launch_bounds__(256)
 f32_split_operands_kernel(const float4* __restrict__ X, const float4* W0, const float4* W1, const float4* W2, uint2* __restrict__ xp, uint2* __restrict__ wp,
-                          uint32_t x4, uint32_t w4, uint32_t k4, uint32_t n4, int* __restrict__ x_small, int* __restrict__ w_small) {
+                          uint32_t x4, uint32_t w4, uint32_t k4, uint32_t n4, int* __restrict__ x_small, int* __restrict__ w_small,
+                          int mark) {
     const int which = blockIdx.y;
     const float4* src = which == 0 ? X : (which == 1 ? W0 : (which == 2 ? W1 : W2));
     const uint32_t count4 = which == 0 ? x4 : w4;
@@ -471,8 +472,8 @@ f32_split_operands_kernel(const float4* __restrict__ X, const float4* W0, const 
 #pragma unroll
         for (int k = 0; k < 3; ++k) dst[(size_t)k * count4 + i] = make_uint2(ft_pack(p[k][0], p[k][1]), ft_pack(p[k][2], p[k][3]));
         if (least < FT_SMALL) {
-            if (which == 0) x_small[i / k4 / FT_M] = 1;
-            else w_small[(which - 1) * blocks_n + (i % n4) / 64] = 1;
+            if (which == 0) x_small[i / k4 / FT_M] = mark;
+            else w_small[(which - 1) * blocks_n + (i % n4) / 64] = mark;
         }
     }
 }
@@ -480,7 +481,7 @@ f32_split_operands_kernel(const float4* __restrict__ X, const float4* W0, const 
 __global__ void __launch_bounds__(FP_THREADS, 1)
 f32_project_pairs_kernel(const __grid_constant__ FPMaps maps, const float* __restrict__ X, const float* W0, const float* W1, const float* W2, float* O0,
                          float* O1, float* O2, int M, int K, int N, int nW, const float* __restrict__ R, const int* __restrict__ x_small,
-                         const int* __restrict__ w_small, DeviceCounters* dc) {
+                         const int* __restrict__ w_small, int mark, DeviceCounters* dc) {
     extern __shared__ uint8_t fp_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(fp_smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t full_bar[FP_STAGES], empty_bar[FP_STAGES], acc_full[2], acc_empty[2];
@@ -608,7 +609,7 @@ f32_project_pairs_kernel(const __grid_constant__ FPMaps maps, const float* __res
                         *reinterpret_cast<float4*>(o + e) = y;
                     }
                 }
-                if (!finite || x_small[m0 / FT_M] || w_small[w * nt + t % nt]) atomicOr(&marks[mark_of(i) / 32], 1u << (mark_of(i) % 32));
+                if (!finite || x_small[m0 / FT_M] == mark || w_small[w * nt + t % nt] == mark) atomicOr(&marks[mark_of(i) / 32], 1u << (mark_of(i) % 32));
             }
         }
         // ---- tiles that were marked
@@ -655,7 +656,7 @@ bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms) {
 }
 
 cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N, const float* residual,
-                              void* parts, int* marks, DeviceCounters* dc, cudaStream_t stream) {
+                              void* parts, int* marks, int mark, DeviceCounters* dc, cudaStream_t stream) {
     static DeviceSetup setup;
     const int sms = device_setup(&setup, [] {
         return cudaFuncSetAttribute(f32_project_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FP_SMEM);
@@ -677,7 +678,7 @@ cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* co
     split.numAttrs = 1;
     const auto f4 = [&](int w) { return reinterpret_cast<const float4*>(W[nW == 3 ? w : 0]); };
     const cudaError_t e = cudaLaunchKernelEx(&split, f32_split_operands_kernel, reinterpret_cast<const float4*>(X), f4(0), f4(1), f4(2),
-                                             reinterpret_cast<uint2*>(xp), reinterpret_cast<uint2*>(wp), x4, w4, (uint32_t)(D / 4), (uint32_t)(N / 4), marks, w_small);
+                                             reinterpret_cast<uint2*>(xp), reinterpret_cast<uint2*>(wp), x4, w4, (uint32_t)(D / 4), (uint32_t)(N / 4), marks, w_small, mark);
     if (e != cudaSuccess) return e;
     FPMaps maps;
     if (!make_tensor_map_bf16_4d(&maps.a, xp, 3, rows, 1, D, 128)) return cudaErrorInvalidValue;
@@ -696,7 +697,7 @@ cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* co
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, f32_project_pairs_kernel, maps, X, W[0], W[nW == 3 ? 1 : 0], W[nW == 3 ? 2 : 0], out[0], out[nW == 3 ? 1 : 0],
-                              out[nW == 3 ? 2 : 0], rows, D, N, nW, residual, static_cast<const int*>(marks), static_cast<const int*>(w_small), dc);
+                              out[nW == 3 ? 2 : 0], rows, D, N, nW, residual, static_cast<const int*>(marks), static_cast<const int*>(w_small), mark, dc);
 }
 
 }  // namespace psa

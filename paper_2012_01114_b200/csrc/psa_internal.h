@@ -24,11 +24,13 @@ struct DeviceCounters {
 // ---- fp32 CUDA-core path (psa_f32.cu) ----
 // out[w][r, c] = sum_k X[r, k] W[w][k, c] for w < nW.
 // `residual` ([rows, N], may be null) is added to every output.
-// `ps` (may be null): scratch for the largest calls, see f32_project_pairs; `bytes`: room for the parts.
+// `ps` (may be null): scratch for the largest calls, see f32_project_pairs; `bytes`: room for the parts; `mark`: what a mark of this call is (any other
+// number is none, so that marks need not be clear when a call starts).
 struct F32ProjectScratch {
     void* parts;
     size_t bytes;
     int* marks;
+    int mark;
 };
 cudaError_t f32_project(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D,
                         int N, const float* residual, const F32ProjectScratch* ps, DeviceCounters* dc, cudaStream_t stream);
@@ -36,14 +38,15 @@ cudaError_t f32_project(const float* X, const float* const W[3], float* const ou
 cudaError_t f32_project_tensor(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N,
                                const float* residual, DeviceCounters* dc, cudaStream_t stream);
 // The same for the largest calls, operands split once into `parts` (f32_project_parts_bytes, psa_ws.h), on pairs of CTAs.  marks:
-// f32_project_marks ints, clear when the call's kernels start.
+// f32_project_marks ints, none of them `mark` when the call's kernels start.
 bool f32_project_pairs_pay(int rows, int D, int N, int nW, int sms);
 cudaError_t f32_project_pairs(const float* X, const float* const W[3], float* const out[3], int nW, int rows, int D, int N, const float* residual,
-                              void* parts, int* marks, DeviceCounters* dc, cudaStream_t stream);
-// Scratch of the tensor-core attention: marks of the heads it cannot take (B H ints, clear when the call's kernels start), maxima
+                              void* parts, int* marks, int mark, DeviceCounters* dc, cudaStream_t stream);
+// Scratch of the tensor-core attention: marks of the heads it cannot take (B H ints, set to `mark`, which none is when the call's kernels start), maxima
 // and sums of the rows on the diagonal tiles (2 B H n numbers), bf16 parts of K and V (6 B n H d each numbers of 16 bits, together).
 struct F32Scratch {
     int* bad;
+    int mark;
     float* ml;
     void* parts;
 };
@@ -51,9 +54,10 @@ struct F32Scratch {
 cudaError_t f32_attention_split(const float* Q, const float* K, const float* V, const F32Scratch& fs, int B, int H, int n, int d, cudaStream_t stream);
 cudaError_t f32_attention_tensor(const float* Q, float* out, const F32Scratch& fs, int B, int H, int n, int d, float scale, int masked, DeviceCounters* dc,
                                  cudaStream_t stream);
-// Q, K, V, out: [B, n, H, d] fp32.  S: scratch [B*H, n, n] fp32, used by PSA_SYMMETRIC only.  fs: may be null.
+// Q, K, V, out: [B, n, H, d] fp32.  S: scratch [B*H, n, n] fp32, used by PSA_SYMMETRIC only.  fs: may be null.  dc_next (may be null): a second
+// counter block, cleared by the last kernel.
 cudaError_t f32_attention(const float* Q, const float* K, const float* V, float* out, float* S, const F32Scratch* fs, int B, int H,
-                          int n, int d, float scale, int scheme, DeviceCounters* dc, cudaStream_t stream);
+                          int n, int d, float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next, cudaStream_t stream);
 
 // Small layers in one launch (projections and the three phases of a (batch, head) per CTA, all in shared memory):
 // f32_fused_fits says whether a shape qualifies.  X [B, n, D], W* [D, H*d] (Wk, Wv ignored for PSA_SYMMETRIC).

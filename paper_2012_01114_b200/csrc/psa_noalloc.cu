@@ -77,7 +77,7 @@ extern "C" int psa_attention_sym_f32_noalloc(const void* X, int batch, int heads
     float* S = reinterpret_cast<float*>(base + NOALLOC_COUNTER_BYTES);
     const float* x = static_cast<const float*>(X);
     e = f32_attention(x, x, x, static_cast<float*>(out), S, nullptr, batch, heads, n, d_k, 1.0f / sqrtf((float)d_k),
-                      PSA_SYMMETRIC, dc, stream);
+                      PSA_SYMMETRIC, dc, nullptr, stream);
     if (e != cudaSuccess) { set_cuda_error(e, "f32_attention(noalloc)"); return PSA_ERR_CUDA; }
     return PSA_OK;
 }

@@ -84,3 +84,35 @@ def test_too_small_even_for_the_lean_layout():
     finally:
         binding.psa_set_workspace(None)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("entry", ["core", "layer"])
+def test_nothing_is_left_from_call_to_call(entry):
+    # Nothing is cleared ahead of a call: heads marked by one call (values of 1e20, weights of 1e-30) are not marked in the next, memory full of anything is no
+    # mark, and the census of each call is its own.  The same kernels run on the same numbers, so outputs are equal bit by bit.
+    scheme = binding.MASKED if entry == "core" else binding.FULL
+    call, shape, _, (B, H, n, D, d) = _case(entry, scheme)
+    want = torch.empty(shape, device="cuda")
+    call(want)
+    bytes_ = binding.psa_workspace_bytes(B, H, n, D, d, scheme, binding.F32)
+    if entry == "core":
+        q, k, v = _inputs([((B, n, H, d), 1.0)] * 3)
+        v[0, 3, 2] = 1e20
+        odd = lambda: binding.psa_attention_core(q, k, v, scheme)
+    else:
+        t = _inputs([((B, n, D), 1.0)] + [((D, H * d), D ** -0.5)] * 3)
+        t[1][5, ::3] = 1e-30
+        odd = lambda: binding.psa_attention_f32(*t, H, scheme)
+    small = _inputs([((3, 40, 4, 32), 1.0)] * 3)
+    try:
+        for fill in (0x5a, 0x00, 0xff):
+            binding.psa_set_workspace(torch.full((bytes_,), fill, dtype=torch.uint8, device="cuda"))
+            for before in (lambda: None, odd, odd, lambda: binding.psa_attention_core(*small, binding.FULL), lambda: binding.psa_attention_core(small[0], None, None, binding.SYMMETRIC)):
+                before()
+                out = torch.full(shape, float("nan"), device="cuda")
+                call(out)
+                st, got = binding.psa_last_issued()
+                assert st == binding.OK and got == binding.psa_skip_count(B, H, n, D, d, scheme, binding.F32)
+                assert torch.equal(out.view(torch.int32), want.view(torch.int32))
+    finally:
+        binding.psa_set_workspace(None)
