@@ -183,3 +183,27 @@ def test_projection_tile_choices(rows, D, H, d):
     assert st == binding.OK and got["proj_macs"] == 4 * rows * D * H * d
     zref = y.double().view(rows, -1) @ Wo.double() + X.double().view(rows, D)
     assert ((z.double().view(rows, -1) - zref).abs() <= 2.0 ** -8 * zref.abs() + 1e-4).all()
+
+
+def _near(got, a, w, plus=0.0):
+    # a w + plus as summed in fp32 (K 2^-24 of the sum of sizes) and rounded to bf16 (2^-9)
+    a, w = a.double(), w.double()
+    ref = a @ w + plus
+    bound = 2.0 ** -8 * ref.abs() + a.shape[1] * 2.0 ** -24 * (a.abs() @ w.abs())
+    assert ((got.double() - ref).abs() <= bound).all()
+
+
+# One vector per sequence attends to itself: the layer's output is the projection X Wv, the block's that times Wo.  Sizes at which tiles of 192
+# columns are chosen, with ragged last tiles of rows and columns.
+@pytest.mark.parametrize("M,N,K", [(2048, 512, 512), (1990, 512, 576), (4000, 192, 512), (2700, 320, 512), (1000, 1024, 512), (4090, 768, 768)])
+def test_projections_on_tiles_of_192_columns(M, N, K):
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    X = torch.randn(M, 1, K, device="cuda", generator=g).bfloat16()
+    W = [(torch.randn(K, N, device="cuda", generator=g) * K ** -0.5).bfloat16() for _ in range(3)]
+    y = binding.psa_attention(X, *W, N // 64, binding.FULL)
+    _near(y[:, 0], X[:, 0], W[2])
+    if N == K:
+        Wo = (torch.randn(N, K, device="cuda", generator=g) * N ** -0.5).bfloat16()
+        for R in (None, X):
+            z = binding.psa_attention_block(X, *W, Wo, N // 64, binding.FULL, residual=R)
+            _near(z[:, 0], y[:, 0], Wo, 0.0 if R is None else R[:, 0].double())
