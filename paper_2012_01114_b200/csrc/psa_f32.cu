@@ -1091,6 +1091,7 @@ f32_fused_layer_kernel(const float* __restrict__ X, const float* __restrict__ Wq
 // step the projections took 4100, phase 1 3500), and k and v rows are pushed (fetched by the CTAs that need them they took two barriers of the
 // cluster and a pass of 3100 .. 4600).  The layout comes from the host, indices are divided by multiplication.
 // Measured (us a call, among calls with other inputs; before / now): 1 head of n = 64, d = 64 masked 12.9 / 8.3, FULL 11.2 / 8.4; 12 heads FULL 11.8 / 8.6, 20 heads 22.6 / 10.9.
+// Error against 64 bits (relative, 2-norm, 120 layers): 0.65 of that with undivided sums, nowhere more than 1 % larger.
 struct ClusterLayout {
     int ld, s_ld;                            // row pitches: q, k, v; weights, kept as [key][own row]
     int tiles, group;                        // row tiles of a CTA (at most), rows that a task of the projections takes
