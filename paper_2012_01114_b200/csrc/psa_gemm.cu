@@ -19,6 +19,7 @@
 #include <mutex>
 
 #include "psa_internal.h"
+#include "psa_sched.h"
 #include "psa_tma.h"
 #include "sm100.cuh"
 
@@ -388,23 +389,12 @@ int bf16_project(const void* A, const void* const Bw[3], void* const C[3], int n
     static DeviceSetup setup;
     const int sms = device_setup(&setup, [] { return cudaSuccess; }, "gemm set-up");
     if (sms <= 0) return PSA_ERR_CUDA;
-    // The tile with the shortest estimated run: start and last epilogue plus rounds of tiles over the SMs times their k-steps, in
-    // cycles as measured (K = 64 .. 3072).  A pair of CTAs takes 650 cycles per k-step of a 256 x 256 tile where a lone CTA
-    // takes 740 for 128 x 256, but its launch costs 2 us more; narrow tiles pay where wide ones leave SMs idle.  Projections
-    // with N = 768, K = 768 (us, pair / 256 / 128 columns): 200 rows 14.5 14.1 12.1, 600 rows 14.5 14.0 12.6, 2000 rows
-    // 16.2 14.5 16.7, 4096 rows 20.9 20.4 24.8, 8192 rows 30.5 32.4 41.1; K = 3072, 8192 rows 78.2 87.1 126.  192 columns pay where their tiles take as many
-    // rounds as wide ones: an output projection of 8192 x 768 x 768 with residual, 256 tiles for 192, two rounds either way (whole block of 8 x 1024,
-    // masked, 70.3 / 68.2), 16384 x 320 x 3 x 192, 384 tiles either way (layer 22.6 / 21.6).
-    const long long nk = (K + BK - 1) / BK;
-    auto cost = [&](int ctas, int bn, long long step, long long fixed) {
-        const long long tiles = (long long)((M + ctas * BM - 1) / (ctas * BM)) * ((N + bn - 1) / bn) * nW, slots = sms / ctas;
-        return fixed + ((tiles + slots - 1) / slots) * (nk * step);
-    };
-    const long long pair = cost(2, 256, 650, 7200), wide = cost(1, 256, 740, 3000), middle = cost(1, 192, 640, 2500), narrow = cost(1, 128, 570, 1500);
-    if (middle < wide && middle < narrow && middle < pair) return launch_gemm<1, 192>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
-    if (narrow <= wide && narrow <= pair) return launch_gemm<1, 128>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
-    if (wide <= pair) return launch_gemm<1, 256>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
-    return launch_gemm<2, 256>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+    switch (gemm_tile(M, K, N, nW, sms)) {
+        case GemmTile::LONE_128: return launch_gemm<1, 128>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+        case GemmTile::LONE_192: return launch_gemm<1, 192>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+        case GemmTile::LONE_256: return launch_gemm<1, 256>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+        default: return launch_gemm<2, 256>(A, Bw, C, nW, M, K, N, residual, sms, dc, stream);
+    }
 }
 
 }  // namespace psa

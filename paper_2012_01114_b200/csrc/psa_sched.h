@@ -208,4 +208,34 @@ inline int host_parts(int batch, size_t x_bytes, size_t out_bytes, const void* x
     return parts < 1 ? 1 : (int)(parts < most ? parts : most);
 }
 
+// ---- the output tile of a bf16 projection [M, K] by nW matrices [K, N] (psa_gemm.cu): 128 x 128, 192 or 256 on lone CTAs, 256 x 256 on pairs.
+// The one with the shortest estimated run: start and last epilogue plus rounds of tiles over the SMs times their k-steps of 64, in
+// cycles.  A pair of CTAs takes 650 cycles per k-step where a lone CTA takes 740 for 128 x 256, but its launch costs 2 us more; narrow
+// tiles pay where wide ones leave SMs idle.  Projections with N = 768, K = 768 (us, pair / 256 / 128 columns): 200 rows 14.5 14.1 12.1, 600 rows
+// 14.5 14.0 12.6, 2000 rows 16.2 14.5 16.7, 4096 rows 20.9 20.4 24.8, 8192 rows 30.5 32.4 41.1; K = 3072, 8192 rows 78.2 87.1 126.
+//
+// 192 columns pay where they take as many rounds as wide tiles or pairs.  Layers with three matrices (M x K x N, us, 128 / 192 / 256 columns / pair):
+// 2048 x 768 x 512 15.0 12.9 13.5 14.9; 4096 x 768 x 576 24.0 19.9 21.4 21.5; 8192 x 256 x 576 25.2 23.1 24.5 27.1; 8192 x 3072 x 576 105 90.5 102 96.8;
+// 16384 x 256 x 192 21.6 19.0 20.8 21.9.  Their k-step takes 680 cycles on a full chip (from K = 768 to 3072, us per step: 0.348, wide tiles 0.373, 128
+// columns 0.264); the 640 of the estimate is the line that short runs showed.  From 64 k-steps (rounds times steps) on a pair's later start no longer
+// counts, and 192 columns stay only where they leave out padding (N = 192, 320, 576; not 512, 768, 2560), those of few column tiles only up to
+// 4 rounds or 11 steps.  Time over that of a pair, beyond the line: 1280 x 2560 x 2560 1.03, 640 x 2560 x 2560 1.04, 4096 x 3072 x 512 1.03, 3072 x 3072 x 768
+// 1.02, 54144 x 768 x 192 1.03, 32768 x 1536 x 192 1.03; inside: 19328 x 3072 x 576 0.97, 60032 x 384 x 384 0.89, 9088 x 2048 x 576 0.97.
+enum class GemmTile { LONE_128, LONE_192, LONE_256, PAIR_256 };
+inline GemmTile gemm_tile(int M, int K, int N, int nW, int sms) {
+    const long long nk = (K + 63) / 64;
+    auto rounds = [&](int ctas, int bn) {
+        const long long tiles = (long long)((M + ctas * 128 - 1) / (ctas * 128)) * ((N + bn - 1) / bn) * nW, slots = sms / ctas;
+        return (tiles + slots - 1) / slots;
+    };
+    auto cost = [&](int ctas, int bn, long long step, long long fixed) { return fixed + rounds(ctas, bn) * nk * step; };
+    const long long pair = cost(2, 256, 650, 7200), wide = cost(1, 256, 740, 3000), middle = cost(1, 192, 640, 2500), narrow = cost(1, 128, 570, 1500);
+    if (middle < wide && middle < narrow && middle < pair) {
+        const bool brief = rounds(1, 192) * nk < 64, less_padding = (N + 191) / 192 * 192 < (N + 255) / 256 * 256;
+        if (brief || (less_padding && (N > 384 || nk < 12 || rounds(1, 192) < 5))) return GemmTile::LONE_192;
+    }
+    if (narrow <= wide && narrow <= pair) return GemmTile::LONE_128;
+    return wide <= pair ? GemmTile::LONE_256 : GemmTile::PAIR_256;
+}
+
 }  // namespace psa

@@ -207,3 +207,38 @@ def test_projections_on_tiles_of_192_columns(M, N, K):
         for R in (None, X):
             z = binding.psa_attention_block(X, *W, Wo, N // 64, binding.FULL, residual=R)
             _near(z[:, 0], y[:, 0], Wo, 0.0 if R is None else R[:, 0].double())
+
+
+# The same tiles where the output depends on all three projections, and an output projection with a last tile of columns that is cut short, with and
+# without residual: 192 columns at these sizes (tests/test_gemm_tile_cpu.py).  Reference: 64 bits from q, k, v rounded to bf16; bounds as
+# elsewhere on this path, 2e-2 and half a bf16 step of the output itself.
+@pytest.mark.parametrize("scheme,B,n,K,H", [(binding.FULL, 128, 16, 512, 8), (binding.MASKED, 20, 100, 576, 8), (binding.FULL, 40, 100, 512, 3),
+                                            (binding.MASKED, 21, 129, 512, 5), (binding.SYMMETRIC, 80, 100, 512, 11)])
+def test_layers_on_tiles_of_192_columns(scheme, B, n, K, H):
+    d, N, sym = 64, 64 * H, scheme == binding.SYMMETRIC
+    g = torch.Generator(device="cuda").manual_seed(B + n)
+    X = torch.randn(B, n, K, device="cuda", generator=g).bfloat16()
+    W = [(torch.randn(K, N, device="cuda", generator=g) * K ** -0.5).bfloat16() for _ in range(1 if sym else 3)]
+    y = binding.psa_attention(X, *(W + [None, None] if sym else W), H, scheme)
+    st, got = binding.psa_last_issued()
+    assert st == binding.OK and got == binding.psa_skip_count(B, H, n, K, d, scheme, binding.BF16)
+    q, k, v = [(X.double() @ w.double()).bfloat16().double().view(B, n, H, d).transpose(1, 2) for w in (W * 3)[:3]]
+    s = q @ k.transpose(2, 3) * d ** -0.5
+    if scheme == binding.MASKED:
+        s = s.masked_fill(torch.ones(n, n, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    ref = (s.softmax(3) @ v).transpose(1, 2).reshape(B, n, N)
+    assert ((y.double() - ref).abs() <= 2e-2 + 2.0 ** -8 * ref.abs()).all()
+
+
+def test_output_projection_on_tiles_of_192_columns_cut_short():
+    M, K, N = 8000, 512, 704
+    g = torch.Generator(device="cuda").manual_seed(3)
+    X = torch.randn(M, 1, N, device="cuda", generator=g).bfloat16()
+    W = [(torch.randn(N, K, device="cuda", generator=g) * N ** -0.5).bfloat16() for _ in range(3)]
+    Wo = (torch.randn(K, N, device="cuda", generator=g) * K ** -0.5).bfloat16()
+    y = binding.psa_attention(X, *W, K // 64, binding.FULL)
+    for R in (None, X):
+        z = binding.psa_attention_block(X, *W, Wo, K // 64, binding.FULL, residual=R)
+        st, got = binding.psa_last_issued()
+        assert st == binding.OK and got["proj_macs"] == 4 * M * K * N
+        _near(z[:, 0], y[:, 0], Wo, 0.0 if R is None else R[:, 0].double())
