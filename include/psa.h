@@ -64,12 +64,15 @@ typedef enum {
 /*
  * Multiply-accumulate census of one call (summed over batch and heads).
  *   proj_macs       projection MACs (paper Sec. 3.1; not part of the paper's own count)
- *   qk_macs         phase-1 MACs issued      pv_macs   phase-3 MACs issued
+ *   qk_macs         phase-1 MACs of the blocks issued      pv_macs   phase-3 MACs of the blocks issued
  *   exps            phase-2 exponentials evaluated
  *   useful_*        the paper's element-level counts for the scheme (Sec. 3.2, 4.2, 5.2):
  *                   FULL d*n^2 each; MASKED d*n(n+1)/2 each; SYMMETRIC d*n(n+1)/2 and d*n^2
  * The bf16 path issues whole 128x128 blocks of the weight matrix, so issued >= useful there (a
  * block on the diagonal, or a ragged last block, is issued in full); the fp32 path skips element by element, issued = useful.
+ * qk_macs and pv_macs say which blocks a scheme issued, 128 * 128 * (columns of the tiles that hold a head) each: 64 columns for
+ * d_k <= 64, 128 for d_k <= 128, else 256.  They are no count of what the tensor core multiplied beside that: FULL and MASKED with d_k <= 32
+ * or 64 < d_k <= 96 run over the first 32, 80 or 96 of those columns only, the others being zeros.
  * On the fp32 path every number is one multiply-accumulate of the plain product (in large calls six bf16 products are formed for
  * each, on tiles padded with zeros); so is proj_macs on either path.
  */
@@ -82,8 +85,7 @@ typedef struct {
  *   X, Wq, Wk, Wv, out   device, bf16, layouts above.
  *   PSA_SYMMETRIC: q = k = v = X*Wq (paper Sec. 4.1); Wk and Wv must be NULL or equal to Wq.
  * Supported: d_k any multiple of 8 up to 256 (PSA_SYMMETRIC: up to 128).  The kernels work on heads of 64, 128 or
- * 256 columns; a shorter head is zero-padded by the tile loads, and the census counts a block at the padded width (up to 96 columns the
- * products of FULL and MASKED leave whole 16-column steps of zeros out all the same); any n >= 1 (a last block of
+ * 256 columns; a shorter head is zero-padded by the tile loads, and the census counts a block at that width (see psa_counts); any n >= 1 (a last block of
  * fewer than 128 vectors is zero-filled and its keys carry no weight); d_model and heads*d_k multiples of 64.
  * Needs a workspace of psa_workspace_bytes(...) (grown on demand, see psa_set_workspace).
  */
@@ -162,7 +164,7 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
 size_t psa_block_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, int scheme, int dtype);
 
 /*
- * Analytic census: what the tile scheduler will issue for this shape and scheme (paper Sec. 3.2,
+ * Analytic census: which blocks the tile scheduler will issue for this shape and scheme, as psa_counts counts them (paper Sec. 3.2,
  * 4.2, 5.2 for the useful_* fields).  Host only, launches nothing.  d_model = 0 means "core only"
  * (proj_macs = 0).
  */
@@ -170,7 +172,7 @@ int psa_skip_count(int batch, int heads, int n, int d_model, int d_k, int scheme
 
 /*
  * Measured census: waits for `stream`, then returns the counters the kernels of the last call
- * accumulated on the device (one increment per block of work actually issued) and that call's
+ * accumulated on the device (one increment per block of work actually issued, of the size that psa_counts gives) and that call's
  * device status (PSA_OK or PSA_ERR_TIMEOUT).
  */
 int psa_last_issued(void* stream, psa_counts* counts);

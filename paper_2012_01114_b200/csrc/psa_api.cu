@@ -606,8 +606,8 @@ int psa_skip_count(int batch, int heads, int n, int d_model, int d_k, int scheme
     // pairs of a launch out as single row tiles, split_point in psa_sched.h, those are the same row tiles with the
     // same block lists taken one at a time: the census does not depend on the grouping.)
     const int T = row_tiles(n);
-    // (a head size below the 64, 128 or 256 columns the kernels work with is zero-padded by the loads: the padded
-    // width is what the tensor core is issued)
+    // (a head size below the 64, 128 or 256 columns of a tile is zero-padded by the loads; a block counts at that width, also where
+    // the products leave steps of zeros out)
     const uint64_t block_macs = (uint64_t)TILE * TILE * (d_k <= 64 ? 64 : (d_k <= 128 ? 128 : 256));
     uint64_t qk_blocks = 0, pv_blocks = 0, exps = 0;
     const int P = ctas_per_head(n);

@@ -72,8 +72,8 @@ constexpr int ISSUER1_WARP = CTRL_WARPS + 2 * SOFTMAX_WARPS_PER_TILE;
 template <int D> __host__ __device__ constexpr int persist_threads() { return ATTN_THREADS + (D == 64 ? 32 : 0); }
 template <int D> __host__ __device__ constexpr int item_readers() { return (D == 64 ? 2 : 1) + 2 * SOFTMAX_WARPS_PER_TILE; }   // issuers + one lane per softmax warp
 
-// D: columns of a tile in shared memory, KS: 16-column steps of phase 1, and of phase 3's output, that hold columns of the head (the rest are zeros,
-// which the census counts as issued: it goes by blocks of D columns).
+// D: columns of a tile in shared memory, KS: 16-column steps of phase 1, and of phase 3's output, that hold columns of the head (the rest are zeros;
+// the census counts blocks, each of D columns).
 // KVS ("keys are the values"): K and V are one tensor (the case the paper mentions in Sec. 3.1 beside query = key =
 // value).  A key tile is then loaded once and serves phase 1 as the K-major operand and phase 3 as the MN-major
 // one; the shared-memory stages of the V ring extend the K ring, and a tile is released behind its PV.
@@ -698,7 +698,8 @@ int bf16_attention_persist(const void* Q, const void* K, const void* V, void* ou
     const integral_constant<int, 128> wide;
     // The products run over 16 KS columns of the 64 or 128 that a tile is loaded with.  Between 64 and 96 the chain of a row tile gets shorter (us, all 128
     // columns / here): masked, 32 heads of n = 3001, d = 72 83.3 / 79.0, d = 80 84.1 / 77.4, d = 96 86.3 / 82.3; FULL, n = 4096, d = 80 240 / 232.  At
-    // 104 and 112 the eighth step costs nothing beyond noise.  Up to 64 the exponentials bound: 1-2 % at d <= 32, nothing at 40 and 48.
+    // 104 and 112 the eighth step costs nothing beyond noise.  Up to 64 the exponentials bound: 1 to 2 % at d <= 32 (128 heads of n = 200 8.78 / 8.51, 96 of n = 512 16.2 / 15.9,
+    // masked 14.9 / 14.6, 4096 of n = 128 64.9 / 63.9; one to four long heads FULL lose up to 1 %, one of n = 8192 71.6 / 72.3), nothing at 40 and 48.
     switch ((d + 15) / 16) {
         case 1: case 2: return launch(narrow, integral_constant<int, 2>{});
         case 3: case 4: return launch(narrow, integral_constant<int, 4>{});

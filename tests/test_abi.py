@@ -80,7 +80,7 @@ def test_argument_errors_launch_nothing(lib):
     assert lib.psa_skip_count(1, 1, 128, 0, 264, 0, binding.BF16, ctypes.byref(c)) == binding.ERR_UNSUPPORTED   # d_k > 256
     assert lib.psa_skip_count(1, 1, 128, 0, 256, 1, binding.BF16, ctypes.byref(c)) == binding.ERR_UNSUPPORTED   # symmetric: up to 128
     assert lib.psa_skip_count(1, 1, 128, 0, 96, 0, binding.BF16, ctypes.byref(c)) == binding.OK
-    assert c.qk_macs == 128 * 128 * 128 and c.useful_qk_macs == 128 * 128 * 96    # issued at the padded width of 128
+    assert c.qk_macs == 128 * 128 * 128 and c.useful_qk_macs == 128 * 128 * 96    # a block counts at the width of its tiles, 128
     assert lib.psa_skip_count(1, 1, 2048, 0, 64, 0, binding.F32, ctypes.byref(c)) == binding.ERR_UNSUPPORTED
     assert lib.psa_skip_count(0, 1, 128, 0, 64, 0, binding.BF16, ctypes.byref(c)) == binding.ERR_SHAPE
     assert lib.psa_skip_count(1, 1, 128, 0, 64, 0, binding.BF16, None) == binding.ERR_NULL
