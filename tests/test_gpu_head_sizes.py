@@ -1,8 +1,8 @@
 """Head sizes other than 64 and 128 on the bf16 path.  The kernels work on 64-column boxes: a head of d_k columns
 (any multiple of 8 up to 128) is described to TMA as its own axis of the tensor, so the columns between d_k and the
 next multiple of 64 are out of bounds -- zero-filled when a tile is loaded, dropped when the output is stored.
-Values against the oracle at the path's tolerance; the census counts what the tensor core is issued, which is the
-padded width (64 for d_k <= 64, 128 up to 128, 256 above), while the useful counts are the paper's, with d_k itself.
+Values against the oracle at the path's tolerance; the census counts the blocks issued, each at the width of its tiles (64 for d_k <= 64,
+128 up to 128, 256 above; the kernel itself leaves 16-column steps of zeros out), while the useful counts are the paper's, with d_k itself.
 Heads of more than 128 columns (full and masked schemes) run on a kernel of their own, one row tile per CTA."""
 import numpy as np
 import pytest
@@ -161,3 +161,47 @@ def test_wide_heads_work_list(scheme, B, H, n, d):
         assert st == binding.OK and got == binding.psa_skip_count(B, H, n, 0, d, scheme, binding.BF16)
         err = np.abs(out.float().cpu().numpy().astype(np.float64).reshape(ref.shape) - ref)
         assert (err <= 2e-2 + 2.0 ** -8 * np.abs(ref)).all()
+
+
+# The kernel's products run over 32, 64, 80, 96 or 128 columns by the head size: the head sizes at both ends of each, under the schemes that it serves.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("d", [24, 32, 40, 64, 72, 80, 88, 96, 104])
+def test_ends_of_the_column_steps(scheme, d):
+    test_core_with_other_head_sizes(scheme, 2, 3, 300, d)
+
+
+# One tensor for keys and values at these widths: a tile is then an operand of both products, with the columns of the one and of the other.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("d", [8, 32, 72, 80, 88, 96])
+def test_one_tensor_for_keys_and_values(scheme, d):
+    B, H, n = 2, 3, 421
+    qv, qb = inputs.tensor(43 * n + d, 4, (B, n, H, d), 1.0, "bf16")
+    kv, kb = inputs.tensor(43 * n + d, 5, (B, n, H, d), 1.0, "bf16")
+    q, k = _dev(qb), _dev(kb)
+    out = binding.psa_attention_core(q, k, k, scheme)
+    _census(B, H, n, 0, d, scheme)
+    ref, _ = oracle.attention_core(qv, kv, kv, scheme)
+    err = np.abs(_f64(out) - ref)
+    assert (err <= TOL_BF16 + 2.0 ** -8 * np.abs(ref)).all(), err.max()
+    apart = binding.psa_attention_core(q, k, k.clone(), scheme)
+    assert torch.equal(out.view(torch.int16), apart.view(torch.int16))
+
+
+# Keys that grow from block to block, by more than the threshold of the lazy rescale each time: it multiplies whole accumulators, also the columns that no
+# product has written.  With one tensor for keys and values the outputs grow by the same factors, and the tolerance with them.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("one", [False, True])
+@pytest.mark.parametrize("d", [16, 32, 72, 80, 88, 96])
+def test_rescale_at_column_steps(scheme, one, d):
+    B, H, n = 1, 2, 640
+    factors = np.repeat(1.0 + 3.0 * np.arange(5), 128)
+    qv, qb = inputs.tensor(47 * n + d, 4, (B, n, H, d), 1.0, "bf16")
+    kv, kb = inputs.tensor(47 * n + d, 5, (B, n, H, d), 1.0, "bf16", row_scale=factors)
+    vv, vb = (kv, kb) if one else inputs.tensor(47 * n + d, 6, (B, n, H, d), 1.0, "bf16")
+    k = _dev(kb)
+    out = binding.psa_attention_core(_dev(qb), k, k if one else _dev(vb), scheme)
+    assert binding.psa_last_rescales() > B * H * (n - 128) // 2
+    _census(B, H, n, 0, d, scheme)
+    ref, _ = oracle.attention_core(qv, kv, vv, scheme)
+    err = np.abs(_f64(out) - ref)
+    assert (err <= TOL_BF16 * (factors.max() if one else 1.0) + 2.0 ** -8 * np.abs(ref)).all(), err.max()
