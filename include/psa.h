@@ -202,6 +202,9 @@ size_t psa_workspace_bytes(int batch, int heads, int n, int d_model, int d_k, in
  * until replaced or until psa_set_workspace(NULL, 0).  Without a registered workspace, or when it
  * is too small (for an fp32 call: without the parts of psa_workspace_bytes), the library keeps a private one and grows it with
  * cudaMalloc (synchronously, on the first call that needs more).
+ * The library keeps counters in the first 256 bytes from call to call (a call clears those of the next one, in bf16 and in fp32): a program that
+ * writes there between two calls registers the memory again before the second, or that call's results, census and status are undefined.
+ * The memory behind them holds nothing between calls and may be used for anything in the meantime.
  */
 int psa_set_workspace(void* dev_ptr, size_t bytes);
 

@@ -116,3 +116,41 @@ def test_nothing_is_left_from_call_to_call(entry):
                 assert torch.equal(out.view(torch.int32), want.view(torch.int32))
     finally:
         binding.psa_set_workspace(None)
+
+
+# What a program may do with a registered workspace between calls: write anywhere but into the first 256 bytes, and there too if it registers the memory again.
+@pytest.mark.parametrize("dtype,scheme,entry,B,H,n,D,d", [
+    (binding.F32, binding.MASKED, "core", 2, 20, 520, 0, 64), (binding.F32, binding.FULL, "layer", 4, 12, 520, 768, 64), (binding.F32, binding.MASKED, "layer", 1, 1, 64, 64, 64),
+    (binding.F32, binding.SYMMETRIC, "core", 2, 3, 100, 0, 32), (binding.F32, binding.FULL, "core", 2, 3, 30, 0, 20), (binding.F32, binding.FULL, "block", 4, 12, 520, 768, 64),
+    (binding.BF16, binding.MASKED, "core", 10, 16, 300, 0, 64), (binding.BF16, binding.FULL, "layer", 3, 2, 200, 128, 192), (binding.BF16, binding.SYMMETRIC, "core", 20, 16, 300, 0, 128)])
+def test_memory_used_for_other_things_between_calls(dtype, scheme, entry, B, H, n, D, d):
+    sym, dt = scheme == binding.SYMMETRIC, torch.bfloat16 if dtype == binding.BF16 else torch.float32
+    if entry == "core":
+        t = [x.to(dt) for x in _inputs([((B, n, H, d), 1.0)] * (1 if sym else 3))]
+        call = lambda: binding.psa_attention_core(*(t + [None, None] if sym else t), scheme)
+    else:
+        t = [x.to(dt) for x in _inputs([((B, n, D), 1.0)] + [((D, H * d), D ** -0.5)] * 3 + [((H * d, D), (H * d) ** -0.5)])]
+        layer = binding.psa_attention if dtype == binding.BF16 else binding.psa_attention_f32
+        call = (lambda: binding.psa_attention_block(*t, H, scheme)) if entry == "block" else (lambda: layer(*t[:4], H, scheme))
+    size = binding.psa_block_workspace_bytes if entry == "block" else binding.psa_workspace_bytes
+    ws = torch.zeros(size(B, H, n, D, d, scheme, dtype), dtype=torch.uint8, device="cuda")
+
+    def checked():
+        out = call()
+        st, got = binding.psa_last_issued()
+        census = binding.psa_skip_count(B, H, n, D, d, scheme, dtype)
+        if entry == "block":
+            census["proj_macs"] += B * n * H * d * D
+        assert st == binding.OK and got == census
+        return out.view(torch.int16)
+    try:
+        binding.psa_set_workspace(ws)
+        want = checked()
+        for fill in (0xff, 0x5a, 0x00, 0xff):
+            ws[COUNTERS:] = fill
+            assert torch.equal(checked(), want)
+            ws[:] = fill
+            binding.psa_set_workspace(ws)
+            assert torch.equal(checked(), want)
+    finally:
+        binding.psa_set_workspace(None)
