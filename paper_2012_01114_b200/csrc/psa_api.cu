@@ -253,8 +253,9 @@ int run_layer(Context& cx, const void* X, const void* Wq, const void* Wk, const 
     int block = 0;
     if (captured) {
         block = CAPTURE_BLOCK;
-        e = cudaMemsetAsync(ws + CAPTURE_BLOCK * COUNTER_BLOCK_BYTES, 0, COUNTER_BLOCK_BYTES, stream);
-        if (e == cudaSuccess && L.clear_bytes) e = cudaMemsetAsync(ws + L.clear, 0, L.clear_bytes, stream);
+        // (its mark stays the same in every replay, so that marks are cleared too; the cursors between are those of host calls, which clear them)
+        const size_t first = CAPTURE_BLOCK * COUNTER_BLOCK_BYTES;
+        e = cudaMemsetAsync(ws + first, 0, (L.clear_bytes ? L.clear + L.clear_bytes : first + COUNTER_BLOCK_BYTES) - first, stream);
     } else if (s_clear) {
         e = bf16_symmetric_clear(S, L.s_bytes, batch, heads, n, L.s, stream);
     } else if (turns && cx.clean_ws == ws) {
@@ -433,7 +434,7 @@ int psa_attention_host(const void* X_host, const void* Wq_host, const void* Wk_h
     cudaError_t e = cudaEventRecord(pipe->start, stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->start, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->out, pipe->start, 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, L.clear_bytes ? L.clear + L.clear_bytes : COUNTER_BYTES, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, COUNTER_BYTES, stream);
     cx.clean_ws = nullptr;
     DeviceCounters* dc = reinterpret_cast<DeviceCounters*>(ws);
     cx.last_dc = dc;
@@ -572,11 +573,9 @@ int psa_attention_block_residual(const void* X, const void* Wq, const void* Wk, 
     void* outs[3] = {out, out, out};
     if (dtype == PSA_F32) {
         const F32ProjectScratch ps = {ws + L.parts, L.out_bytes, reinterpret_cast<int*>(ws + L.marks_out), cx.mark};
-        cudaError_t e = cudaSuccess;
-        if (L.out_bytes && !L.clear_bytes) e = cudaMemsetAsync(ps.marks, 0, f32_project_marks(batch * n, d_model, 1) * sizeof(int), stream);
-        if (e == cudaSuccess) e = f32_project(static_cast<const float*>(y), reinterpret_cast<const float* const*>(Ws),
-                                    reinterpret_cast<float* const*>(outs), 1, batch * n, heads * d_k, d_model,
-                                    static_cast<const float*>(R), L.out_bytes ? &ps : nullptr, cx.last_dc, stream);
+        const cudaError_t e = f32_project(static_cast<const float*>(y), reinterpret_cast<const float* const*>(Ws),
+                                          reinterpret_cast<float* const*>(outs), 1, batch * n, heads * d_k, d_model,
+                                          static_cast<const float*>(R), L.out_bytes ? &ps : nullptr, cx.last_dc, stream);
         if (e != cudaSuccess) { set_cuda_error(e, "f32_project(Wo)"); return PSA_ERR_CUDA; }
         return PSA_OK;
     }

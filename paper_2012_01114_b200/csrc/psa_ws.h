@@ -81,7 +81,7 @@ inline WsLayout ws_layout(const WsShape& c) {
     WsLayout L;
     memset(&L, 0, sizeof(L));
     size_t off = COUNTER_BYTES;
-    if (c.dtype == PSA_F32 && !c.lean) {      // marks right behind the counters: one clear serves both
+    if (c.dtype == PSA_F32 && !c.lean) {      // marks right behind the counters: a captured call, the only one that clears marks, clears both in one go
         const size_t bh = (size_t)c.batch * c.heads;
         L.attn_tensor = !c.one_launch && f32_tensor_attention_fits(c.batch, c.heads, c.n, c.d_k, c.scheme);
         L.in_bytes = c.with_proj && !c.one_launch ? f32_project_parts_bytes(rows, c.d_model, hd, c.scheme == PSA_SYMMETRIC ? 1 : 3) : 0;
@@ -93,7 +93,7 @@ inline WsLayout ws_layout(const WsShape& c) {
             off += align_up((c.staging ? HOST_CHUNKS : 1) * L.marks_pitch * sizeof(int), 256);
         }
         if (L.out_bytes) { L.marks_out = off; off += align_up(f32_project_marks(rows, c.d_model, 1) * sizeof(int), 256); }
-        L.clear_bytes = c.one_launch ? 0 : off - L.clear;
+        L.clear_bytes = off - L.clear;
         if (L.attn_tensor) { L.ml = off; off += align_up(2 * bh * c.n * sizeof(float), 256); }
         L.parts = off;           // (used by one kernel after another)
         off += align_up(std::max(std::max(L.in_bytes, L.out_bytes), L.attn_tensor ? 12 * bh * c.n * c.d_k : (size_t)0), 256);

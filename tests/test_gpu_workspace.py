@@ -154,3 +154,43 @@ def test_memory_used_for_other_things_between_calls(dtype, scheme, entry, B, H, 
             assert torch.equal(checked(), want)
     finally:
         binding.psa_set_workspace(None)
+
+
+# Marks of an output projection: those of one call (entries of 1e-30 in Wo) are none in the next, nor in a replay of a graph that has run with
+# such entries; the layer in several launches and, 400 sequences of 64 vectors, in one.
+@pytest.mark.parametrize("B,H,n,D,d", [(4, 12, 520, 768, 64), (400, 16, 64, 256, 16)])
+def test_marks_of_an_output_projection_from_call_to_call(B, H, n, D, d):
+    t = _inputs([((B, n, D), 1.0)] + [((D, H * d), D ** -0.5)] * 3 + [((H * d, D), (H * d) ** -0.5)])
+    Wo, out = t[4], torch.empty((B, n, D), device="cuda")
+    odd = Wo.clone()
+    odd[5, ::3] = 1e-30
+    call = lambda wo: binding.psa_attention_block(*t[:4], wo, H, binding.FULL, out=out, residual=t[0])
+    call(odd)
+    marked = out.clone()
+    for _ in range(3):
+        call(Wo)
+    want = out.clone()
+    bytes_ = binding.psa_block_workspace_bytes(B, H, n, D, d, binding.FULL, binding.F32)
+    try:
+        for fill in (0x5a, 0x00, 0xff):
+            binding.psa_set_workspace(torch.full((bytes_,), fill, dtype=torch.uint8, device="cuda"))
+            for before in ((), (odd,), (odd, odd)):
+                for w in before:
+                    call(w)
+                    assert torch.equal(out, marked)
+                call(Wo)
+                assert torch.equal(out, want)
+        moving = Wo.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            call(moving)
+        for wo, expected in ((Wo, want), (odd, marked), (Wo, want), (odd, marked), (Wo, want)):
+            moving.copy_(wo)
+            out.fill_(float("nan"))
+            graph.replay()
+            assert torch.equal(out, expected)
+            call(wo)
+            assert torch.equal(out, expected)
+    finally:
+        torch.cuda.synchronize()
+        binding.psa_set_workspace(None)

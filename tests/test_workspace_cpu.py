@@ -73,7 +73,7 @@ int main() {
                             if (!f32_project_pairs_fit(nb * c.n, c.d_model, hd, nW, L.in_bytes)) { ++refused; continue; }
                             ++used;
                             if (need > L.in_bytes) return 4;
-                            // marks of part k, cleared once ahead of all parts: behind those of the part before, before those of the next
+                            // marks of part k: behind those of the part before, before those of the next
                             if (f32_project_marks(nb * c.n, hd, nW) > L.marks_pitch) return 5;
                             const size_t last = L.marks_in + (k * L.marks_pitch + f32_project_marks(nb * c.n, hd, nW)) * 4;
                             if (L.marks_in < L.clear || last > L.clear + L.clear_bytes || (L.marks_out && L.marks_in < L.marks_out && last > L.marks_out)) return 8;
@@ -156,3 +156,25 @@ def test_calls_with_little_off_the_diagonal_tiles_stay_on_cuda_cores(tmp_path):
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", ROOT, "-o", str(tmp_path / "fits"), str(tmp_path / "fits.cpp")])
     got = subprocess.check_output([str(tmp_path / "fits")] + [str(x) for c in cuda + tensor for x in c]).split()
     assert [int(x) for x in got] == [0] * len(cuda) + [1] * len(tensor)
+
+
+MARKS = r"""
+#include <cstdio>
+#include "paper_2012_01114_b200/csrc/psa_ws.h"
+using namespace psa;
+int main() {
+    // a block whose layer runs in one launch, and one whose layer does not: marks behind the counters, all in the range that a captured call clears
+    for (bool one_launch : {true, false}) {
+        const WsLayout L = ws_layout(WsShape{400, 16, 64, 256, 16, PSA_FULL, PSA_F32, true, false, one_launch, false});
+        const size_t marks = f32_project_marks(400 * 64, 256, 1) * sizeof(int);
+        if (!L.out_bytes || L.clear != COUNTER_BYTES || L.marks_out < L.clear || L.marks_out + marks > L.clear + L.clear_bytes) return 1;
+    }
+    return 0;
+}
+"""
+
+
+def test_marks_of_an_output_projection_lie_in_what_a_captured_call_clears(tmp_path):
+    (tmp_path / "marks.cpp").write_text(MARKS)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", ROOT, "-o", str(tmp_path / "marks"), str(tmp_path / "marks.cpp")])
+    assert subprocess.call([str(tmp_path / "marks")]) == 0
