@@ -1299,7 +1299,9 @@ f32_fused_cluster_kernel(const float* __restrict__ X, const float* __restrict__ 
     const int width = d <= 8 ? 8 : d <= 16 ? 16 : 32, blocks = (d + 31) / 32, ysplits = L.y_splits;
     for (int unit = warp; unit < own_tiles * blocks * ysplits; unit += WARPS) {
         const int rest = unit >> __ffs(ysplits) - 1, p = unit - rest * ysplits, tile = fastdiv(rest, L.by_blocks), c = 32 * (rest - tile * blocks) + (lane & (width - 1));
-        // keys that all four rows keep, that any row keeps (of rows beyond n nothing is read)
+        // keys that all four rows keep, that any row keeps; neither goes beyond n, so that no v row beyond the sequence is read.  (Where n is no multiple
+        // of 4, the last tile's rows beyond n have q and weights of whatever shared memory held before, here as in phase 1: each row has an
+        // accumulator of its own, and those rows' are never stored.)
         const int i0 = own_row(4 * tile), whole = masked ? i0 + 1 : n, jend = masked ? min(i0 + 4, n) : n, step = ysplits * (32 / width);
         const float* w = S + 4 * tile;
         const float* v = vs + min(c, d - 1);
