@@ -316,7 +316,7 @@ int layer_entry(const void* X, const void* Wq, const void* Wk, const void* Wv, i
 
 }  // namespace
 
-int device_setup(DeviceSetup* st, cudaError_t (*configure)(), const char* what) {
+int device_setup(DeviceSetup* st, cudaError_t (*configure)(), const char* what, int* device) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) { set_cuda_error(e, what); return 0; }
@@ -329,6 +329,7 @@ int device_setup(DeviceSetup* st, cudaError_t (*configure)(), const char* what) 
         st->sm_count[dev] = sms;
         st->done[dev] = true;
     }
+    if (device) *device = dev;
     return st->sm_count[dev];
 }
 

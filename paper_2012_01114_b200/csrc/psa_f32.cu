@@ -1103,6 +1103,7 @@ struct ClusterLayout {
 };
 constexpr int FC_SPLITS = 8;
 constexpr size_t FC_HALF_SM = 113 * 1024;     // shared memory of a CTA that leaves room for a second one
+constexpr size_t FC_ALONE = FC_HALF_SM + 2048;     // that leaves none
 inline ClusterLayout cluster_layout(int n, int D, int d, int C) {
     ClusterLayout L;
     L.tiles = ((n + 3) / 4 + C - 1) / C;
@@ -1426,47 +1427,69 @@ bool f32_fused_fits(int n, int D, int d, int scheme) {
     return fused_layout(n, D, d, scheme == PSA_SYMMETRIC ? 1 : 3).total <= (size_t)FS_MAX_FLOATS;
 }
 
-// Heads few enough that one CTA each would leave SMs idle are spread over clusters of up to 8 CTAs.  `*alone`: a CTA keeps others off its SM, by
-// the shared memory that it asks for.  Left to themselves the clusters of a call, and those of the next one that come in early, share SMs while
-// others are idle (12 heads of n = 64, d = 64: 13.0 us a call, 8.6 alone; a CTA per head 11.8).  The clusters that fit are fewer than the SMs divided by
-// their size, as a cluster stays inside a part of the GPU: 16 heads in clusters of 8 16.4 us alone and 12.2 sharing, in clusters of 4 10.8 alone.
-// Measured (us, a CTA per head / clusters of 2 / 4 / 8, sharing SMs; d_model = 64): 48 heads of n = 30, d = 32 16.4 11.1 9.1 16.1, of n = 64, d = 64 24.6
-// 20.9 19.4 25.9, of n = 100, d = 64 (too much shared memory for two on an SM) 47.1 40.9 52.5 59.4; 100 of n = 64, d = 64 26.7 41.3 29.7 45.6, of n = 64,
-// d = 16 14.4 16.8 18.0 29.8; 74 of n = 64, d = 8 12.3 14.2 14.2.  Many heads of up to 16 vectors gain nothing (48 of n = 16, d = 16 8.0 7.6 7.6).
-int f32_fused_cluster_size(int B, int H, int n, int D, int d, int scheme, int sms, bool* alone) {
+// Heads few enough that one CTA each would leave SMs idle are spread over clusters: of the largest size of which all clusters of the call fit the GPU at
+// once, each CTA alone on its SM (by the shared memory that it asks for).  A cluster stays inside a part of the GPU, so that fewer fit than SMs / size; the
+// runtime says how many, and steps lie where it says: 15 of 8, 33 of 4 and 74 of 2 on 148 SMs.  Masked, n = 64, d_model = d = 64, us for a CTA per head / clusters of
+// 2 / 4 / 8 alone: 15 heads 24.6 15.2 10.5 8.5, 16 24.6 15.2 10.5 15.9, 33 24.6 15.4 10.5 23.9, 34 24.6 15.4 19.8 23.9, 74 24.6 15.3 29.7 40.2, 80 24.6 29.6 29.8.
+// Clusters that share SMs pack while others are idle (12 heads 8.5 alone, 12.5 sharing), but 71 of 4 fit then, and up to 64 heads, a tenth of the GPU left free, take
+// these before clusters of 2: 34 heads of n = 150, d = 16 18.1 against 19.4, 48 of n = 96, d = 48 20.6 against 20.9 (short heads lose, 48 of n = 64, d = 64 16.2 against
+// 15.3, d = 16 10.2 against 9.5, but with half as many CTAs to a head sums are split less and the error against 64 bits grows by up to a fifth).
+// Many heads of up to 16 vectors gain nothing (48 of n = 16, d = 16 8.0, clusters of 2 or 4 7.6).
+struct ClusterFits {
+    int alone[3], sharing4;                  // clusters of 2, 4, 8 CTAs alone on their SMs; of 4, two CTAs to an SM
+};
+ClusterFits g_cluster_fits[MAX_DEVICES];
+cudaError_t clusters_that_fit(int c, size_t bytes, int* clusters) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(FS_THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = c;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(clusters, f32_fused_cluster_kernel, &cfg);
+}
+cudaError_t fused_setup() {
+    constexpr int bytes = FS_MAX_FLOATS * (int)sizeof(float);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_fused_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f32_fused_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    ClusterFits& f = g_cluster_fits[dev];
+    for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = clusters_that_fit(2 << i, FC_ALONE, &f.alone[i]);
+    if (e == cudaSuccess) e = clusters_that_fit(4, FC_HALF_SM, &f.sharing4);
+    return e;
+}
+int f32_fused_cluster_size(int B, int H, int n, int D, int d, int scheme, const ClusterFits& f, bool* alone) {
     const long long heads = (long long)B * H;
     *alone = true;
     if (scheme == PSA_SYMMETRIC || (heads > 32 && n <= 16)) return 1;      // (the symmetric scheme's mirrored store crosses row owners)
-    const int tn = (n + 3) / 4;
-    auto floats = [&](int c) { return cluster_layout(n, D, d, c).total; };
-    auto fits = [&](int c) { return c <= tn && floats(c) <= (size_t)FS_MAX_FLOATS; };
-    if (fits(8) && 12 * heads <= sms) return 8;
-    if (fits(4) && 9 * heads <= 2 * sms) return 4;
-    *alone = false;
-    for (int c = 8; c > 2; c /= 2)
-        if (fits(c) && floats(c) * sizeof(float) <= FC_HALF_SM && 4 * heads * c <= 7 * sms) return c;
-    *alone = true;
-    return fits(2) && 2 * heads <= sms && (d >= 32 || heads <= 32) ? 2 : 1;
+    auto bytes = [&](int c) { return cluster_layout(n, D, d, c).total * sizeof(float); };
+    auto fits = [&](int c) { return c <= (n + 3) / 4 && bytes(c) <= FS_MAX_FLOATS * sizeof(float); };
+    if (heads <= f.alone[2] && fits(8)) return 8;
+    if (heads <= f.alone[1] && fits(4)) return 4;
+    if (heads <= f.sharing4 - f.sharing4 / 10 && fits(4) && bytes(4) <= FC_HALF_SM) { *alone = false; return 4; }
+    return heads <= f.alone[0] && fits(2) ? 2 : 1;
 }
 
 cudaError_t f32_fused_layer(const float* X, const float* Wq, const float* Wk, const float* Wv, float* out, int B, int H,
                             int n, int D, int d, float scale, int scheme, DeviceCounters* dc, DeviceCounters* dc_next,
                             cudaStream_t stream) {
     static DeviceSetup setup;
-    const int sms = device_setup(&setup, [] {
-        constexpr int bytes = FS_MAX_FLOATS * (int)sizeof(float);
-        const cudaError_t e = cudaFuncSetAttribute(f32_fused_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        return e != cudaSuccess ? e : cudaFuncSetAttribute(f32_fused_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    }, "fp32 fused layer set-up");
-    if (sms <= 0) return cudaErrorUnknown;
+    int dev = 0;
+    if (device_setup(&setup, fused_setup, "fp32 fused layer set-up", &dev) <= 0) return cudaErrorUnknown;
     bool alone;
-    const int C = f32_fused_cluster_size(B, H, n, D, d, scheme, sms, &alone);
+    const int C = f32_fused_cluster_size(B, H, n, D, d, scheme, g_cluster_fits[dev], &alone);
     if (C > 1) {
         const ClusterLayout L = cluster_layout(n, D, d, C);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(B * H * C);
         cfg.blockDim = dim3(FS_THREADS);
-        cfg.dynamicSmemBytes = std::max(L.total * sizeof(float), alone ? FC_HALF_SM + 2048 : 0);
+        cfg.dynamicSmemBytes = std::max(L.total * sizeof(float), alone ? FC_ALONE : 0);
         cfg.stream = stream;
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;

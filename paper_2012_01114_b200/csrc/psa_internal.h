@@ -93,13 +93,13 @@ int bf16_attention_persist(const void* Q, const void* K, const void* V, void* ou
 // Once-per-device set-up of a kernel family.  Function attributes (the dynamic shared-memory limit) belong to the
 // device that is current when they are set, and the SM count differs between devices, so both are kept per
 // device ordinal.  device_setup() returns the current device's SM count (> 0), having run `configure` (which sets
-// the family's attributes) the first time that device is seen; 0 on failure (error text set).  Thread-safe.
+// the family's attributes) the first time that device is seen; 0 on failure (error text set).  `device` (may be null): its ordinal.  Thread-safe.
 constexpr int MAX_DEVICES = 64;
 struct DeviceSetup {
     bool done[MAX_DEVICES];
     int sm_count[MAX_DEVICES];
 };
-int device_setup(DeviceSetup* st, cudaError_t (*configure)(), const char* what);
+int device_setup(DeviceSetup* st, cudaError_t (*configure)(), const char* what, int* device = nullptr);
 
 // Self-test of the bounded-wait failure path (psa_selftest.cu): a one-CTA kernel whose barrier nobody completes.
 cudaError_t launch_wait_expiry(DeviceCounters* dc, unsigned limit_us, cudaStream_t stream);

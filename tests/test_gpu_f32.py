@@ -80,6 +80,14 @@ def test_clusters_at_odd_sizes(scheme, B, H, n, D, d):
     test_layer_shapes_and_schemes(scheme, B, H, n, D, d)
 
 
+# The cluster size changes where the clusters of a call no longer fit the GPU at once: 15 of 8 CTAs, 33 of 4 (64 that share SMs), 74 of 2.
+@pytest.mark.parametrize("scheme", [oracle.FULL, oracle.MASKED])
+@pytest.mark.parametrize("heads", [13, 15, 16, 33, 34, 64, 65, 74, 75])
+@pytest.mark.parametrize("n,D,d", [(38, 24, 12), (97, 16, 20)])
+def test_numbers_of_heads_around_cluster_sizes(scheme, heads, n, D, d):
+    test_layer_shapes_and_schemes(scheme, heads, 1, n, D, d)
+
+
 @pytest.mark.parametrize("scheme", [oracle.FULL, oracle.SYMMETRIC, oracle.MASKED])
 def test_core_entry(scheme):
     rng = np.random.default_rng(5)
